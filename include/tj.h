@@ -77,7 +77,7 @@ enum { TJ_W_FP32 = 0,      /* FP32 FMA in one fixed rounding order: outputs (and
 enum { TJ_K_ACTOR_FUSED = 0,  /* MLP + selection + env step + insert in one kernel (FP32 path, or the fused tensor-core actor) */
        TJ_K_MLP_TENSOR = 1,   /* tensor-core MLP forward alone (the learner's two forwards; the actor's where it is not fused) */
        TJ_K_ENV = 2,          /* selection + env step + insert fed by the tensor-core MLP */
-       TJ_K_SAMPLE = 3,       /* eligible list + sample + gather */
+       TJ_K_SAMPLE = 3,       /* draw + gather */
        TJ_K_TD = 4,           /* TD error (FP32 forward, or the elementwise pass after tensor-core forwards) */
        TJ_K_PUBLISH = 5, TJ_K_GAE = 6,
        TJ_K_SGD = 7,          /* learner update: forward with kept activations, backward, parameter update */

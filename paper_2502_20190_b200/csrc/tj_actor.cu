@@ -69,6 +69,7 @@ __global__ void __launch_bounds__(NT) actor_small_env_kernel(const ActorParams p
   const int e = blockIdx.x * TE + tid;
   const bool owner = tid < TE && e < p.N;
   const bool on_policy = p.C == 0;
+  chain_begin();
   if (STAGE > 0) {
     if (tid == 0) mbar_init(&wbar, 1);
     __syncthreads();
@@ -221,6 +222,7 @@ __global__ void __launch_bounds__(NT) actor_lingauss_kernel(const ActorParams p)
   const int e0 = blockIdx.x * TE;
   const int D = p.D, Dp = (p.D + 3) & ~3;
   const int n_here = min(TE, p.N - e0);
+  chain_begin();
 
   // state -> xs[k][e]
   for (int i = tid; i < TE * D; i += NT) {
@@ -346,6 +348,7 @@ __global__ void __launch_bounds__(NT) actor_lingauss_kernel(const ActorParams p)
 }
 
 __global__ void init_env_kernel(int env_kind, int N, int S_d, uint2 seed, float* state, int* ep_step, float* ep_return) {
+  chain_begin();
   const int nb = S_d / 4;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (long long)N * nb) return;
@@ -358,25 +361,15 @@ __global__ void init_env_kernel(int env_kind, int N, int S_d, uint2 seed, float*
   }
 }
 
-template <typename K>
-cudaError_t launch_with_smem(K kernel, int grid, int threads, size_t smem_bytes, const ActorParams& p, cudaStream_t s) {
-  if (smem_bytes > 48 * 1024) {
-    cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
-    if (err != cudaSuccess) return err;
-  }
-  kernel<<<grid, threads, smem_bytes, s>>>(p);
-  return cudaGetLastError();
-}
-
 constexpr size_t kSmemMax = 227 * 1024 - 1024;   // per block, leaving room for static shared memory
 constexpr size_t kSmemTwoPerSm = 112 * 1024;     // two resident blocks per SM
 
 template <int TE, int NT, int EPT, int NPT, int ENV>
 cudaError_t launch_small(int stage, size_t smem, const ActorParams& p, cudaStream_t s) {
   const int grid = (p.N + TE - 1) / TE;
-  if (stage == 2) return launch_with_smem(actor_small_env_kernel<TE, NT, EPT, NPT, ENV, 2>, grid, NT, smem, p, s);
-  if (stage == 1) return launch_with_smem(actor_small_env_kernel<TE, NT, EPT, NPT, ENV, 1>, grid, NT, smem, p, s);
-  return launch_with_smem(actor_small_env_kernel<TE, NT, EPT, NPT, ENV, 0>, grid, NT, smem, p, s);
+  if (stage == 2) return launch_chained(actor_small_env_kernel<TE, NT, EPT, NPT, ENV, 2>, grid, NT, smem, s, p);
+  if (stage == 1) return launch_chained(actor_small_env_kernel<TE, NT, EPT, NPT, ENV, 1>, grid, NT, smem, s, p);
+  return launch_chained(actor_small_env_kernel<TE, NT, EPT, NPT, ENV, 0>, grid, NT, smem, s, p);
 }
 
 }  // namespace
@@ -384,8 +377,7 @@ cudaError_t launch_small(int stage, size_t smem, const ActorParams& p, cudaStrea
 cudaError_t launch_init_env(int env_kind, int N, int S_d, uint2 seed, float* state, int* ep_step, float* ep_return,
                             cudaStream_t s) {
   const long long n = (long long)N * (S_d / 4);
-  init_env_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(env_kind, N, S_d, seed, state, ep_step, ep_return);
-  return cudaGetLastError();
+  return launch_chained(init_env_kernel, (unsigned)((n + 255) / 256), 256, 0, s, env_kind, N, S_d, seed, state, ep_step, ep_return);
 }
 
 cudaError_t launch_actor(int env_kind, const ActorParams& p, cudaStream_t s) {
@@ -394,7 +386,7 @@ cudaError_t launch_actor(int env_kind, const ActorParams& p, cudaStream_t s) {
     const bool ext = p.logits_in != nullptr;
     const size_t smem = actor_smem_floats(TE, p.D, ext ? 0 : p.Hp, ext ? 0 : p.Ap, true, 0) * sizeof(float);
     if (smem > kSmemMax) return cudaErrorInvalidConfiguration;
-    return launch_with_smem(actor_lingauss_kernel<TE, NT>, (p.N + TE - 1) / TE, NT, smem, p, s);
+    return launch_chained(actor_lingauss_kernel<TE, NT>, (p.N + TE - 1) / TE, NT, smem, s, p);
   }
   // Tile: 16 envs x 128 threads while that still leaves SMs short of two blocks each, else 32 x 256.
   const bool small_tile = p.N < 148 * 2 * 32;

@@ -102,8 +102,7 @@ size_t carve(tj_ctx* x, void* base) {
     const size_t nb = (size_t)(c.replay_capacity / N);
     x->ring = cv.take<float>((size_t)c.replay_capacity * (2 * D + 4));
     x->block_ver = cv.take<int>(nb);
-    x->elig_list = cv.take<int>(nb);
-    x->elig_count = cv.take<int>(1);
+    x->sample_slots = cv.take<int>(c.minibatch);
     x->sgd_rows = 0;
     x->sgd_scratch = nullptr;
     if (c.policy_kind == TJ_POLICY_EPS_GREEDY && sgd_supported(D, c.hidden, c.n_actions)) {
@@ -294,7 +293,6 @@ int tj_create(const tj_config* cfg, void* workspace, size_t bytes, void* cuda_st
   if (cfg->replay_capacity > 0) {
     if ((e = cudaMemsetAsync(x->block_ver, 0, sizeof(int) * x->h_block_ver.size(), x->stream)) != cudaSuccess)
       return bail(e, "memset block versions");
-    if ((e = cudaMemsetAsync(x->elig_count, 0, sizeof(int), x->stream)) != cudaSuccess) return bail(e, "memset count");
   }
   if (cfg->env_kind == TJ_ENV_LINGAUSS) {
     // stage A and B as given, then transpose/pad A on the device
@@ -403,33 +401,22 @@ int tj_publish_weights(tj_ctx* x, const void* blob, size_t nbytes, int32_t on_de
       return cuda_fail(x, e, "publish: host to device copy");
     src = x->blob_stage;
   }
-  LaunchScope scope(x, TJ_K_PUBLISH, x->use_tc_pipelined ? 3 : (x->use_tc ? 2 : (x->use_split ? 2 : 1)), true, true);
-  const int next = x->active ^ 1;
-  float* dst = x->version == 0 ? x->wbuf[x->active] : x->wbuf[next];
-  if ((e = launch_pack_weights(src, dst, x->wl, x->value_head, x->cfg.weight_dtype == TJ_W_BF16, x->lstream)) != cudaSuccess)
-    return cuda_fail(x, e, "publish: repack");
-  if (x->use_split) {
-    const int slot = x->version == 0 ? x->active : next;
-    if ((e = launch_pack_split_weights(src, x->D, x->H, x->wsplit[slot], x->wsplit_scale[slot], x->lstream)) != cudaSuccess)
-      return cuda_fail(x, e, "publish: split of the hidden x hidden matrix");
-  }
-  uint16_t* dst_tc = nullptr;
-  if (x->use_tc) {
-    dst_tc = x->version == 0 ? x->wtc[x->active] : x->wtc[next];
-    if ((e = launch_pack_tc_weights(src, dst_tc, x->D, x->H, x->A, x->value_head, x->lstream)) != cudaSuccess)
-      return cuda_fail(x, e, "publish: tensor-core repack");
-    if (x->use_tc_pipelined &&
-        (e = launch_pack_pipelined_weights(src, x->version == 0 ? x->wtc_pipe[x->active] : x->wtc_pipe[next], x->D, x->H, x->A,
-                                           x->lstream)) != cudaSuccess)
-      return cuda_fail(x, e, "publish: tensor-core repack (pipelined actor)");
-  }
+  LaunchScope scope(x, TJ_K_PUBLISH, 1, true, true);
+  const int next = x->active ^ 1, slot = x->version == 0 ? x->active : next;
+  float* dst = x->wbuf[slot];
+  uint16_t* dst_tc = x->use_tc ? x->wtc[slot] : nullptr;
+  PublishParams pp{};
+  pp.blob = src; pp.L = x->wl; pp.value_head = x->value_head; pp.bf16 = x->cfg.weight_dtype == TJ_W_BF16;
+  pp.dst = dst; pp.tc = dst_tc;
+  if (x->use_tc_pipelined) pp.tc_pipe = x->wtc_pipe[slot];
+  if (x->use_split) { pp.split = x->wsplit[slot]; pp.split_scale = x->wsplit_scale[slot]; pp.split_h_scale = split_hidden_scale(); }
+  if ((e = launch_publish(pp, x->lstream)) != cudaSuccess) return cuda_fail(x, e, "publish: repack");
   if (x->version != 0) x->active = next;
   x->version += 1;
   if (!x->has_target || (x->cfg.target_sync_interval > 0 && x->k - x->k_last_sync >= x->cfg.target_sync_interval)) {
     if ((e = cudaMemcpyAsync(x->wtarget, dst, x->wl.total * sizeof(float), cudaMemcpyDeviceToDevice, x->lstream)) != cudaSuccess)
       return cuda_fail(x, e, "publish: target refresh");
     if (x->use_split) {
-      const int slot = x->active;
       if ((e = cudaMemcpyAsync(x->wsplit_target, x->wsplit[slot], split_weight_halfs(x->H) * sizeof(uint16_t), cudaMemcpyDeviceToDevice,
                                x->lstream)) != cudaSuccess ||
           (e = cudaMemcpyAsync(x->wsplit_scale_target, x->wsplit_scale[slot], 2 * sizeof(float), cudaMemcpyDeviceToDevice, x->lstream)) !=
@@ -568,9 +555,15 @@ int tj_replay_sample(tj_ctx* x, int32_t staleness_bound, int32_t* idx_out, const
   const int64_t valid = (int64_t)std::min<uint64_t>(x->cursor, (uint64_t)c.replay_capacity);
   if (valid < c.warmup) return fail(x, TJ_ERR_WARMUP, "fewer resident records than warmup");
   const int n_blocks = (int)(valid / x->N);
-  int64_t n_elig = 0;
-  for (int b = 0; b < n_blocks; ++b)
-    if (x->version - (int64_t)x->h_block_ver[(size_t)b] <= S) ++n_elig;
+  // versions never decrease in the order the blocks were written, so the eligible ones are the newest n_elig blocks
+  const uint64_t nb = (uint64_t)(c.replay_capacity / x->N), written = x->cursor / (uint64_t)x->N;
+  uint64_t lo = written - (uint64_t)n_blocks, hi = written;      // write numbers of the resident blocks
+  while (lo < hi) {
+    const uint64_t mid = lo + (hi - lo) / 2;
+    if (x->version - (int64_t)x->h_block_ver[(size_t)(mid % nb)] <= S) hi = mid;
+    else lo = mid + 1;
+  }
+  const int64_t n_elig = (int64_t)(written - lo);
   if (n_elig == 0) {
     x->hs.starved_calls += 1;
     return fail(x, TJ_ERR_STARVED, "no resident record within the staleness bound");
@@ -578,17 +571,19 @@ int tj_replay_sample(tj_ctx* x, int32_t staleness_bound, int32_t* idx_out, const
   if ((uint64_t)n_elig * (uint64_t)x->N > 0xFFFFFFFFull) return fail(x, TJ_ERR_UNSUPPORTED, "eligible set too large");
   learner_waits_for_actor(x);
   LaunchScope scope(x, TJ_K_SAMPLE, 2, true, true);
-  cudaError_t e = launch_eligible(x->block_ver, n_blocks, x->version, S, x->elig_list, x->elig_count, x->lstream);
-  if (e != cudaSuccess) return cuda_fail(x, e, "eligible list");
   SampleParams p{};
   p.B = c.minibatch; p.D = x->D; p.N = x->N; p.rec_words = x->rec_words;
   p.seed = make_uint2((uint32_t)c.seed, (uint32_t)(c.seed >> 32));
   p.k = x->k; p.v_learner = x->version;
-  p.ring = x->ring; p.elig_list = x->elig_list; p.elig_count = x->elig_count;
-  p.idx_out = idx_out;
+  p.ring = x->ring; p.slots = x->sample_slots; p.idx_out = idx_out;
+  const uint64_t first = lo % nb;                                // slot (in blocks) of the oldest eligible block
+  p.n_elig = (uint32_t)(n_elig * x->N);
+  p.n_lo = first + (uint64_t)n_elig > nb ? (int)(first + (uint64_t)n_elig - nb) : 0;
+  p.b_hi = (int)first;
   p.obs = out->obs; p.act = out->act; p.rew = out->rew; p.next_obs = out->next_obs; p.done = out->done; p.ver = out->ver;
   p.stats = x->dstats;
-  if ((e = launch_sample_gather(p, x->lstream)) != cudaSuccess) return cuda_fail(x, e, "sample and gather");
+  cudaError_t e = launch_sample_gather(p, x->lstream);
+  if (e != cudaSuccess) return cuda_fail(x, e, "sample and gather");
   if (x->two_stream) { cudaEventRecord(x->ev_sample, x->lstream); x->has_sample = true; }
   x->k += 1;
   x->hs.learner_steps += 1;

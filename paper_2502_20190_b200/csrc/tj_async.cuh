@@ -54,6 +54,28 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
   return false;
 }
 
+// Start of a kernel launched by launch_chained: waits until the kernel before it has finished and its writes are visible.
+// A kernel that allocates tensor memory calls this after the allocation: a successor resident on the same SM may ask for
+// tensor memory too, and must find this block's share already taken.
+__device__ __forceinline__ void chain_begin() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the next kernel of the stream become resident once every block has come this far (or left).  Short kernels call it
+// right after chain_begin(); kernels that fill the SMs leave it to their blocks' exits: a successor placed while they run
+// would crowd onto the few SMs that are idle (the FP32 learner lost 10 % to that).
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// all threads of the cluster's blocks meet (arrive has release, wait acquire semantics over distributed shared memory)
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+}
+// a float at this block's shared-memory address `p` in block `rank` of the cluster
+__device__ __forceinline__ float cluster_load_f32(const float* p, uint32_t rank) {
+  uint32_t a;
+  float v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+  return v;
+}
+
 // One thread queues `bytes` (multiple of 16) in chunks; the barrier must expect the same total.
 __device__ __forceinline__ void bulk_copy_chunks(void* dst, const void* src, size_t bytes, uint64_t* bar) {
   constexpr size_t kChunk = 16384;

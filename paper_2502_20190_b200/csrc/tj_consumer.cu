@@ -1,5 +1,6 @@
 // On-policy consumer kernels (App. C, synchronous mode; Table 2's PPO batch settings): per-segment advantage normalisation
 // and shuffled minibatches of segment rows.
+#include "tj_async.cuh"
 #include "tj_device.cuh"
 #include "tj_internal.h"
 
@@ -36,6 +37,8 @@ __device__ __forceinline__ double sum_partials(const double* partial, int n_bloc
 
 // pass 1: partial[b] = sum of x over the block's slice (slices are contiguous, fixed by n and the grid)
 __global__ void __launch_bounds__(NORM_THREADS) norm_sum_kernel(const float* __restrict__ x, long long n, double* __restrict__ partial) {
+  chain_begin();
+  chain_next();
   __shared__ double ws[NORM_THREADS / 32];
   const long long per = (n + gridDim.x - 1) / gridDim.x, lo = per * blockIdx.x, hi = lo + per < n ? lo + per : n;
   double v = 0.0;
@@ -47,6 +50,8 @@ __global__ void __launch_bounds__(NORM_THREADS) norm_sum_kernel(const float* __r
 // pass 2: partial2[b] = sum of (x - mean)^2 over the block's slice
 __global__ void __launch_bounds__(NORM_THREADS) norm_sqdev_kernel(const float* __restrict__ x, long long n, const double* __restrict__ partial,
                                                                 double* __restrict__ partial2) {
+  chain_begin();
+  chain_next();
   __shared__ double ws[NORM_THREADS / 32];
   __shared__ double tot;
   const double mean = sum_partials(partial, gridDim.x, &tot) / (double)n;
@@ -63,6 +68,8 @@ __global__ void __launch_bounds__(NORM_THREADS) norm_sqdev_kernel(const float* _
 // pass 3: out = (x - mean) / (sqrt(var) + eps)
 __global__ void __launch_bounds__(NORM_THREADS) norm_apply_kernel(const float* __restrict__ x, long long n, const double* __restrict__ partial,
                                                                 const double* __restrict__ partial2, double eps, float* __restrict__ out) {
+  chain_begin();
+  chain_next();
   __shared__ double tot, tot2;
   const double mean = sum_partials(partial, gridDim.x, &tot) / (double)n;
   const double var = sum_partials(partial2, gridDim.x, &tot2) / (double)n;
@@ -95,6 +102,8 @@ __device__ __forceinline__ long long shuffle_index(uint2 seed, unsigned long lon
 
 // one thread per minibatch row: position first + j of the shuffled order -> source row -> dense copies
 __global__ void segment_minibatch_kernel(const MinibatchParams p) {
+  chain_begin();
+  chain_next();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= p.n) return;
   const long long src = shuffle_index(p.seed, p.shuffle_id, p.hb, p.R, p.first + j);
@@ -130,16 +139,15 @@ cudaError_t launch_normalize(const float* x, long long n, double eps, float* out
   if (blocks < 1) blocks = 1;
   double* p1 = scratch;
   double* p2 = scratch + NORM_MAX_BLOCKS;
-  norm_sum_kernel<<<(unsigned)blocks, NORM_THREADS, 0, s>>>(x, n, p1);
-  norm_sqdev_kernel<<<(unsigned)blocks, NORM_THREADS, 0, s>>>(x, n, p1, p2);
-  norm_apply_kernel<<<(unsigned)blocks, NORM_THREADS, 0, s>>>(x, n, p1, p2, eps, out);
-  return cudaGetLastError();
+  cudaError_t e = launch_chained(norm_sum_kernel, (unsigned)blocks, NORM_THREADS, 0, s, x, n, p1);
+  if (e == cudaSuccess) e = launch_chained(norm_sqdev_kernel, (unsigned)blocks, NORM_THREADS, 0, s, x, n, p1, p2);
+  if (e == cudaSuccess) e = launch_chained(norm_apply_kernel, (unsigned)blocks, NORM_THREADS, 0, s, x, n, p1, p2, eps, out);
+  return e;
 }
 
 cudaError_t launch_segment_minibatch(const MinibatchParams& p, cudaStream_t s) {
   if (p.n <= 0) return cudaSuccess;
-  segment_minibatch_kernel<<<(p.n + 127) / 128, 128, 0, s>>>(p);
-  return cudaGetLastError();
+  return launch_chained(segment_minibatch_kernel, (p.n + 127) / 128, 128, 0, s, p);
 }
 
 }  // namespace tj

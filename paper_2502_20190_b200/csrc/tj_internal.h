@@ -4,11 +4,35 @@
 #include <stdint.h>
 
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/tj.h"
 
 namespace tj {
+
+// Launch with programmatic stream serialisation: the kernel's blocks may become resident as soon as every block of the
+// kernel before it in the stream has called chain_next() or left (tj_async.cuh), and each waits in chain_begin() until that
+// kernel has finished, so set-up and launch latency overlap the tail of the one before.  Every kernel launched this way
+// calls chain_begin() before it touches global memory.
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  if (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
 
 // Policy parameters as the kernels read them: every matrix transposed to [in][out_padded] so that a thread
 // fetches four consecutive output neurons with one 128-bit load; the value head (if any) is column A of the
@@ -133,8 +157,9 @@ struct SampleParams {
   long long k;
   long long v_learner;
   const float* ring;
-  const int* elig_list;
-  const int* elig_count;
+  uint32_t n_elig;           // |E| in records
+  int n_lo, b_hi;            // eligible ring blocks in slot order: 0 .. n_lo - 1, then b_hi, b_hi + 1, ...
+  int* slots;                // scratch [B]: the drawn slots, between the two kernels
   int* idx_out;
   float* obs;
   int* act;
@@ -161,6 +186,19 @@ struct MinibatchParams {
   float* adv;
   float* ret;
   int* row;
+};
+
+// one publish: the blob into every layout the context's kernels read (null: the context has no use for it)
+struct PublishParams {
+  const float* blob;
+  WeightLayout L;
+  int value_head, bf16;
+  float* dst;                // FP32 layout
+  uint16_t* tc;              // BF16 chunks of the general tensor-core kernel
+  uint16_t* tc_pipe;         // BF16 chunks of the pipelined actor
+  uint16_t* split;           // FP16 parts of W2 of the split-operand kernels
+  float* split_scale;        // [0] the power of two W2 was multiplied by, [1] 1 / (that x split_h_scale)
+  float split_h_scale;
 };
 
 struct TcEnvParams {
@@ -198,13 +236,11 @@ struct TcMlpParams {
 
 bool tc_mlp_supported(int D, int H, int Aout);
 size_t tc_weight_elems(int D, int H);
-cudaError_t launch_pack_tc_weights(const float* blob, uint16_t* dst, int D, int H, int A, int value_head, cudaStream_t s);
 cudaError_t launch_tc_mlp(const TcMlpParams& p, int sm_count, cudaStream_t s);
 cudaError_t launch_pack_env_matrix(const float* A, uint32_t* hi, uint32_t* lo, int D, cudaStream_t s);
 bool tc_fused_supported(int D, int H, int A);
 // pipelined fused actor (obs_dim 128, hidden a multiple of 128): its own weight chunk order
 bool tc_pipelined_supported(int D, int H, int A);
-cudaError_t launch_pack_pipelined_weights(const float* blob, uint16_t* dst, int D, int H, int A, cudaStream_t s);
 cudaError_t launch_actor_tc_pipelined(const TcMlpParams& p, int sm_count, cudaStream_t s);
 size_t tc_pipelined_scratch_floats();   // z scratch for the largest grid the launcher uses
 size_t tc_pipelined_env_halfs();        // FP16 high / low chunks of the env matrix
@@ -219,11 +255,8 @@ cudaError_t launch_td_finish(const float* partial, int n_partial, int n, float* 
 // launchers (each returns the cudaGetLastError() of its launches)
 cudaError_t launch_init_env(int env_kind, int N, int S_d, uint2 seed, float* state, int* ep_step, float* ep_return,
                             cudaStream_t s);
-cudaError_t launch_pack_weights(const float* blob, float* dst, const WeightLayout& L, int value_head, int bf16,
-                                cudaStream_t s);
+cudaError_t launch_publish(const PublishParams& p, cudaStream_t s);
 cudaError_t launch_actor(int env_kind, const ActorParams& p, cudaStream_t s);
-cudaError_t launch_eligible(const int* block_ver, int n_blocks, long long v_learner, long long bound, int* elig_list,
-                            int* elig_count, cudaStream_t s);
 cudaError_t launch_sample_gather(const SampleParams& p, cudaStream_t s);
 cudaError_t launch_td(const TdParams& p, cudaStream_t s);
 int td_grid(int n);
@@ -271,7 +304,7 @@ cudaError_t launch_segment_minibatch(const MinibatchParams& p, cudaStream_t s);
 // FP32-accuracy tensor-core actor for the small envs (hidden x hidden layer as three FP16 products of split operands)
 bool split_actor_supported(int env_kind, int D, int H, int Aout);
 size_t split_weight_halfs(int H);
-cudaError_t launch_pack_split_weights(const float* blob, int D, int H, uint16_t* dst, float* scale, cudaStream_t s);
+float split_hidden_scale();   // power of two the hidden activations are multiplied by before their FP16 split
 cudaError_t launch_actor_split(int env_kind, const ActorParams& p, const uint16_t* w2parts, const float* w2scale, int sm_count,
                                cudaStream_t s);
 int td_split_grid(int n);   // loss partials (one per 128 rows) of launch_td_split
@@ -311,8 +344,7 @@ struct tj_ctx {
   float* blob_stage;    // staging for host blobs
   float* ring;
   int* block_ver;
-  int* elig_list;
-  int* elig_count;
+  int* sample_slots;    // slots of the minibatch being sampled, [minibatch]
   float* td_partial;
   double* norm_scratch;  // per-block partial sums of tj_normalize
   float* sgd_scratch;   // learner update: activations and their gradients for one minibatch (FP32 replay contexts)

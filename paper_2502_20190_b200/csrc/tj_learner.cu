@@ -1,5 +1,4 @@
-// Learner-side kernels: parameter publish (repack), eligible-block list, staleness-bounded sampling with
-// gather, TD error / Huber loss, and the GAE reverse scan.
+// Learner-side kernels: staleness-bounded sampling and gather, TD error / Huber loss, and the GAE reverse scan.
 #include <mutex>
 
 #include "tj_async.cuh"
@@ -11,57 +10,6 @@ namespace tj {
 
 namespace {
 
-__device__ __forceinline__ float bf16_round_rne(float x) {
-  uint32_t u = __float_as_uint(x);
-  if ((u & 0x7F800000u) == 0x7F800000u) return x;
-  u += 0x7FFFu + ((u >> 16) & 1u);
-  return __uint_as_float(u & 0xFFFF0000u);
-}
-
-// blob [W1 HxD, b1 H, W2 HxH, b2 H, W3 AxH, b3 A (, Wv H, bv 1)] -> transposed, padded kernel layout
-__global__ void pack_weights_kernel(const float* __restrict__ blob, float* __restrict__ dst, WeightLayout L,
-                                    int value_head, int bf16) {
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= L.total) return;
-  const int D = L.D, H = L.H, A = L.A;
-  const float* W1 = blob;
-  const float* b1 = W1 + (size_t)H * D;
-  const float* W2 = b1 + H;
-  const float* b2 = W2 + (size_t)H * H;
-  const float* W3 = b2 + H;
-  const float* b3 = W3 + (size_t)A * H;
-  const float* Wv = b3 + A;
-  const float* bv = Wv + H;
-  float v = 0.f;
-  bool is_weight = false;
-  if (i >= L.off_W1t && i < L.off_W1t + (size_t)D * L.Hp) {
-    const size_t j = i - L.off_W1t;
-    const int k = (int)(j / L.Hp), n = (int)(j % L.Hp);
-    if (n < H) { v = W1[(size_t)n * D + k]; is_weight = true; }
-  } else if (i >= L.off_b1 && i < L.off_b1 + L.Hp) {
-    const int n = (int)(i - L.off_b1);
-    if (n < H) v = b1[n];
-  } else if (i >= L.off_W2t && i < L.off_W2t + (size_t)H * L.Hp) {
-    const size_t j = i - L.off_W2t;
-    const int k = (int)(j / L.Hp), n = (int)(j % L.Hp);
-    if (n < H) { v = W2[(size_t)n * H + k]; is_weight = true; }
-  } else if (i >= L.off_b2 && i < L.off_b2 + L.Hp) {
-    const int n = (int)(i - L.off_b2);
-    if (n < H) v = b2[n];
-  } else if (i >= L.off_W3t && i < L.off_W3t + (size_t)H * L.Ap) {
-    const size_t j = i - L.off_W3t;
-    const int k = (int)(j / L.Ap), n = (int)(j % L.Ap);
-    if (n < A) { v = W3[(size_t)n * H + k]; is_weight = true; }
-    else if (value_head && n == A) { v = Wv[k]; is_weight = true; }
-  } else if (i >= L.off_b3 && i < L.off_b3 + L.Ap) {
-    const int n = (int)(i - L.off_b3);
-    if (n < A) v = b3[n];
-    else if (value_head && n == A) v = bv[0];
-  }
-  if (bf16 && is_weight) v = bf16_round_rne(v);
-  dst[i] = v;
-}
-
 __global__ void transpose_pad_kernel(const float* __restrict__ src, float* __restrict__ dst, int rows, int cols,
                                      int ld_dst) {
   // dst[c][r] = src[r][c], dst rows padded to ld_dst with zeros
@@ -71,98 +19,91 @@ __global__ void transpose_pad_kernel(const float* __restrict__ src, float* __res
   dst[i] = r < rows ? src[(size_t)r * cols + c] : 0.f;
 }
 
-// Ascending list of ring blocks (one block = the N records of one actor step, all with one version) whose
-// version is at most `bound` behind the learner.  One thread block, stable compaction by chunks.
-__global__ void eligible_kernel(const int* __restrict__ block_ver, int n_blocks, long long v_learner, long long bound,
-                                int* __restrict__ elig_list, int* __restrict__ elig_count) {
-  __shared__ int warp_tot[32];
-  __shared__ int base;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) base = 0;
-  __syncthreads();
-  for (int c0 = 0; c0 < n_blocks; c0 += blockDim.x) {
-    const int b = c0 + tid;
-    const int flag = (b < n_blocks && v_learner - (long long)block_ver[b] <= bound) ? 1 : 0;
-    const unsigned m = __ballot_sync(0xffffffffu, flag);
-    const int before = __popc(m & ((1u << lane) - 1u));
-    if (lane == 0) warp_tot[warp] = __popc(m);
-    __syncthreads();
-    int woff = 0, tot = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-      if (w < warp) woff += warp_tot[w];
-      tot += warp_tot[w];
-    }
-    if (flag) elig_list[base + woff + before] = b;
-    __syncthreads();
-    if (tid == 0) base += tot;
-    __syncthreads();
-  }
-  if (tid == 0) *elig_count = base;
+// Staleness-bounded sampling in two kernels.  One ring block = the N records of one actor step, all with one version, and
+// blocks are written with non-decreasing versions, so the blocks within the bound are the newest ones: in slot order one
+// interval of blocks, or two where it wraps round the ring's end (p.n_lo blocks from 0, the rest from p.b_hi on).  The host
+// knows both from its own bookkeeping, and E[r] is arithmetic: no list of eligible blocks is built or read.
+//
+// draw_slots_kernel: draw j takes E[mulhi(x0, |E|)]; one thread per draw, bound by one launch's latency.
+__device__ __forceinline__ int eligible_slot(const SampleParams& p, uint32_t r) {
+  const uint32_t i = r / (uint32_t)p.N, e = r % (uint32_t)p.N;
+  const uint32_t block = i < (uint32_t)p.n_lo ? i : (uint32_t)p.b_hi + (i - (uint32_t)p.n_lo);
+  return (int)(block * (uint32_t)p.N + e);
 }
 
-// One warp per draw: slot = E[mulhi(x0, |E|)] with E enumerated block by block, then the record is copied
-// word for word into the dense minibatch arrays.
-__global__ void sample_gather_kernel(const SampleParams p) {
-  const int warp = (int)(((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-  if (warp >= p.B) return;
-  const int j = warp;
-  const unsigned long long nE = (unsigned long long)(*p.elig_count) * (unsigned long long)p.N;
-  const uint4 w = stream_words(p.seed, STREAM_SAMPLE, 0, (uint32_t)j, (unsigned long long)p.k);
-  const uint32_t r = __umulhi(w.x, (uint32_t)nE);
-  const int slot = p.elig_list[r / (uint32_t)p.N] * p.N + (int)(r % (uint32_t)p.N);
-  const float* rec = p.ring + (size_t)slot * p.rec_words;
-  const int D = p.D;
-  for (int i = lane; i < p.rec_words; i += 32) {
-    const float v = rec[i];
-    if (i < D) p.obs[(size_t)j * D + i] = v;
-    else if (i < 2 * D) p.next_obs[(size_t)j * D + (i - D)] = v;
-    else if (i == 2 * D) p.act[j] = __float_as_int(v);
-    else if (i == 2 * D + 1) p.rew[j] = v;
-    else if (i == 2 * D + 2) p.done[j] = __float_as_int(v);
-    else {
-      const int ver = __float_as_int(v);
-      p.ver[j] = ver;
-      long long stale = p.v_learner - (long long)ver;
-      if (stale < 0) stale = 0;
-      atomicAdd(&p.stats->hist[stale > 32 ? 32 : stale], 1ull);
-      atomicMax(&p.stats->max_stale, (unsigned long long)stale);
-    }
-  }
-  if (lane == 0 && p.idx_out) p.idx_out[j] = slot;
-}
-
-// The same gather with 128-bit accesses (obs_dim a multiple of 4, 16-byte aligned outputs): LPD lanes share one
-// draw and copy the record's 16-byte chunks -- obs, next_obs, then the (act, rew, done, ver) tail.
-template <int LPD>
-__global__ void sample_gather_vec_kernel(const SampleParams p) {
-  const int lane = threadIdx.x & 31, sub = lane % LPD;
-  const int j = (int)((((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (32 / LPD)) + lane / LPD;
+__global__ void __launch_bounds__(256) draw_slots_kernel(const SampleParams p) {
+  chain_begin();
+  chain_next();
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= p.B) return;
-  const unsigned long long nE = (unsigned long long)(*p.elig_count) * (unsigned long long)p.N;
   const uint4 w = stream_words(p.seed, STREAM_SAMPLE, 0, (uint32_t)j, (unsigned long long)p.k);
-  const uint32_t r = __umulhi(w.x, (uint32_t)nE);
-  const int slot = p.elig_list[r / (uint32_t)p.N] * p.N + (int)(r % (uint32_t)p.N);
-  const float4* rec = reinterpret_cast<const float4*>(p.ring + (size_t)slot * p.rec_words);
-  const int dq = p.D / 4;                         // chunks per observation
-  float4* obs = reinterpret_cast<float4*>(p.obs + (size_t)j * p.D);
-  float4* nxt = reinterpret_cast<float4*>(p.next_obs + (size_t)j * p.D);
-  for (int c = sub; c <= 2 * dq; c += LPD) {
-    const float4 v = __ldcs(rec + c);             // sampled rows are not reused: streaming load
-    if (c < dq) obs[c] = v;
-    else if (c < 2 * dq) nxt[c - dq] = v;
-    else {
-      const int ver = __float_as_int(v.w);
-      p.act[j] = __float_as_int(v.x);
-      p.rew[j] = v.y;
-      p.done[j] = __float_as_int(v.z);
-      p.ver[j] = ver;
-      long long stale = p.v_learner - (long long)ver;
-      if (stale < 0) stale = 0;
-      atomicAdd(&p.stats->hist[stale > 32 ? 32 : stale], 1ull);
-      atomicMax(&p.stats->max_stale, (unsigned long long)stale);
+  const int slot = eligible_slot(p, __umulhi(w.x, p.n_elig));
+  p.slots[j] = slot;
+  if (p.idx_out) p.idx_out[j] = slot;
+}
+
+// gather_kernel: LPD lanes share a draw and copy its record in 16-byte chunks -- obs, next_obs, then the (act, rew, done, ver)
+// tail -- into the dense arrays (whole chunks where the rows allow it, word by word for obs_dim 6 or unaligned arrays).  The
+// loads of UNR draws are in flight at once: bound by the latency of the scattered rows for short records, by HBM for the
+// 1,040-byte ones.  The staleness counts are taken per block in shared memory first: one global atomic per draw on the
+// handful of bins in use serialised in L2 (8,192 draws of 1,040 bytes: 10.4 us before, 4.9 us with the counts per block).
+template <int LPD, int UNR, bool VEC>
+__global__ void __launch_bounds__(256) gather_kernel(const SampleParams p) {
+  chain_begin();
+  chain_next();
+  __shared__ unsigned int bins[33];
+  __shared__ unsigned long long most;
+  constexpr int DPW = 32 / LPD;                              // draws a warp covers at a time
+  const int lane = threadIdx.x & 31, sub = lane % LPD, warp = threadIdx.x >> 5;
+  for (int i = threadIdx.x; i < 33; i += blockDim.x) bins[i] = 0u;
+  if (threadIdx.x == 0) most = 0ull;
+  __syncthreads();
+  const int chunks = p.rec_words / 4, dq = p.D / 4;
+  const int j0 = (blockIdx.x * (int)(blockDim.x >> 5) + warp) * (DPW * UNR) + lane / LPD;
+  int slot[UNR];
+#pragma unroll
+  for (int u = 0; u < UNR; ++u) {
+    const int j = j0 + u * DPW;
+    slot[u] = j < p.B ? p.slots[j] : -1;
+  }
+  for (int c = sub; c < chunks; c += LPD) {
+    float4 v[UNR];
+#pragma unroll
+    for (int u = 0; u < UNR; ++u)                            // sampled rows are not reused: streaming loads
+      if (slot[u] >= 0) v[u] = __ldcs(reinterpret_cast<const float4*>(p.ring + (size_t)slot[u] * p.rec_words) + c);
+#pragma unroll
+    for (int u = 0; u < UNR; ++u) {
+      if (slot[u] < 0) continue;
+      const size_t j = (size_t)(j0 + u * DPW);
+      if (c == chunks - 1) {
+        const int ver = __float_as_int(v[u].w);
+        p.act[j] = __float_as_int(v[u].x);
+        p.rew[j] = v[u].y;
+        p.done[j] = __float_as_int(v[u].z);
+        p.ver[j] = ver;
+        long long stale = p.v_learner - (long long)ver;
+        if (stale < 0) stale = 0;
+        atomicAdd(&bins[stale > 32 ? 32 : stale], 1u);
+        if (stale >= 32) atomicMax(&most, (unsigned long long)stale);
+      } else if (VEC) {
+        if (c < dq) reinterpret_cast<float4*>(p.obs + j * p.D)[c] = v[u];
+        else reinterpret_cast<float4*>(p.next_obs + j * p.D)[c - dq] = v[u];
+      } else {
+        const float w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int k = 4 * c + i;
+          if (k < p.D) p.obs[j * p.D + k] = w[i];
+          else p.next_obs[j * p.D + (k - p.D)] = w[i];
+        }
+      }
     }
   }
-  if (sub == 0 && p.idx_out) p.idx_out[j] = slot;
+  __syncthreads();
+  if (threadIdx.x < 33 && bins[threadIdx.x]) {
+    atomicAdd(&p.stats->hist[threadIdx.x], (unsigned long long)bins[threadIdx.x]);
+    atomicMax(&p.stats->max_stale, threadIdx.x < 32 ? (unsigned long long)threadIdx.x : most);
+  }
 }
 
 // TD error on a tile of TE samples: online forward on obs, target forward on next_obs.
@@ -195,6 +136,7 @@ __global__ void __launch_bounds__(NT) td_kernel(const TdParams p) {
   float* qsel = out + (size_t)p.Ap * TE;
   float* hub = qsel + TE;
   const int tid = threadIdx.x, j0 = blockIdx.x * TE, n_here = min(TE, p.n - j0), D = p.D;
+  chain_begin();
   if (STAGE > 0) {
     if (tid == 0) mbar_init(&wbar, 1);
     __syncthreads();
@@ -249,6 +191,8 @@ __global__ void __launch_bounds__(NT) td_kernel(const TdParams p) {
 // (a single thread walking the array pays one memory latency per element, a warp fetching one chunk per iteration one per
 // chunk), then lane 0 adds them in index order -- the same sum, term by term
 __global__ void td_finish_kernel(const float* __restrict__ partial, int n_partial, int n, float* __restrict__ loss_out) {
+  chain_begin();
+  chain_next();
   if (blockIdx.x != 0 || threadIdx.x >= 32) return;
   const int lane = threadIdx.x;
   float sum = 0.f;
@@ -277,6 +221,7 @@ constexpr int GAE_U = 8;
 __global__ void __launch_bounds__(128) gae_kernel(const float* __restrict__ rew, const float* __restrict__ val,
                                                   const uint8_t* __restrict__ done, int T, int N, float gamma,
                                                   float lambda, float* __restrict__ adv, float* __restrict__ ret) {
+  chain_begin();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= N) return;
   float next_adv = 0.f;
@@ -323,51 +268,35 @@ constexpr int kTdThreads = 128;
 
 }  // namespace
 
-cudaError_t launch_pack_weights(const float* blob, float* dst, const WeightLayout& L, int value_head, int bf16,
-                                cudaStream_t s) {
-  pack_weights_kernel<<<(unsigned)((L.total + 255) / 256), 256, 0, s>>>(blob, dst, L, value_head, bf16);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_transpose_pad(const float* src, float* dst, int rows, int cols, int ld_dst, cudaStream_t s) {
   const size_t n = (size_t)cols * ld_dst;
   transpose_pad_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(src, dst, rows, cols, ld_dst);
   return cudaGetLastError();
 }
 
-cudaError_t launch_eligible(const int* block_ver, int n_blocks, long long v_learner, long long bound, int* elig_list,
-                            int* elig_count, cudaStream_t s) {
-  eligible_kernel<<<1, 1024, 0, s>>>(block_ver, n_blocks, v_learner, bound, elig_list, elig_count);
-  return cudaGetLastError();
+template <int LPD, int UNR>
+static cudaError_t launch_gather(const SampleParams& p, bool vec, cudaStream_t s) {
+  const int per_block = 8 * (32 / LPD) * UNR;                // draws of a block of eight warps
+  const int grid = (p.B + per_block - 1) / per_block;
+  return launch_chained(vec ? gather_kernel<LPD, UNR, true> : gather_kernel<LPD, UNR, false>, grid, 256, 0, s, p);
 }
 
 cudaError_t launch_sample_gather(const SampleParams& p, cudaStream_t s) {
-  const int warps_per_block = 8;
-  const bool aligned = ((reinterpret_cast<uintptr_t>(p.obs) | reinterpret_cast<uintptr_t>(p.next_obs)) & 15) == 0;
-  if (p.D % 4 == 0 && aligned) {
-    if (p.rec_words <= 32) {      // a few chunks per record: four lanes per draw, eight draws per warp
-      const int draws_per_block = warps_per_block * 8;
-      sample_gather_vec_kernel<4><<<(p.B + draws_per_block - 1) / draws_per_block, warps_per_block * 32, 0, s>>>(p);
-    } else {
-      sample_gather_vec_kernel<32><<<(p.B + warps_per_block - 1) / warps_per_block, warps_per_block * 32, 0, s>>>(p);
-    }
-    return cudaGetLastError();
-  }
-  sample_gather_kernel<<<(p.B + warps_per_block - 1) / warps_per_block, warps_per_block * 32, 0, s>>>(p);
-  return cudaGetLastError();
+  const cudaError_t e = launch_chained(draw_slots_kernel, (p.B + 255) / 256, 256, 0, s, p);
+  if (e != cudaSuccess) return e;
+  const bool vec = p.D % 4 == 0 && ((reinterpret_cast<uintptr_t>(p.obs) | reinterpret_cast<uintptr_t>(p.next_obs)) & 15) == 0;
+  // lanes per draw by the record's length in 16-byte chunks (3 or 4 for the small envs, 65 for obs_dim 128), so that few
+  // lanes idle and a warp's loads stay contiguous per record
+  if (p.rec_words <= 16) return launch_gather<4, 1>(p, vec, s);
+  if (p.rec_words <= 64) return launch_gather<8, 2>(p, vec, s);
+  return launch_gather<32, 4>(p, vec, s);
 }
 
 int td_grid(int n) { return (n + kTdTile - 1) / kTdTile; }
 
 template <int TE, int NT, int EPT, int NPT, int STAGE>
 cudaError_t launch_td_stage(const TdParams& p, size_t smem, int grid, cudaStream_t s) {
-  auto kernel = td_kernel<TE, NT, EPT, NPT, STAGE>;
-  if (smem > 48 * 1024) {
-    cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
-  }
-  kernel<<<grid, NT, smem, s>>>(p);
-  return cudaGetLastError();
+  return launch_chained(td_kernel<TE, NT, EPT, NPT, STAGE>, grid, NT, smem, s, p);
 }
 
 // tile: 16 rows x 128 threads with 4 x 4 register tiles; wide layers (hidden >= 192) 32 rows x 128 threads, 8 x 8
@@ -392,8 +321,7 @@ cudaError_t launch_td(const TdParams& p, cudaStream_t s) {
   cudaError_t err = p.H >= 192 ? launch_td_tile<32, 128, 8, 8>(p, s, &grid) : launch_td_tile<kTdTile, kTdThreads, 4, 4>(p, s, &grid);
   if (err != cudaSuccess) return err;
   if (p.loss_out) {
-    td_finish_kernel<<<1, 32, 0, s>>>(p.partial, grid, p.n, p.loss_out);
-    err = cudaGetLastError();
+    err = launch_td_finish(p.partial, grid, p.n, p.loss_out, s);
   }
   return err;
 }
@@ -434,14 +362,12 @@ cudaError_t launch_td_static(const TdParams& p_in, int device, cudaStream_t s, b
 }
 
 cudaError_t launch_td_finish(const float* partial, int n_partial, int n, float* loss_out, cudaStream_t s) {
-  td_finish_kernel<<<1, 32, 0, s>>>(partial, n_partial, n, loss_out);
-  return cudaGetLastError();
+  return launch_chained(td_finish_kernel, 1, 32, 0, s, partial, n_partial, n, loss_out);
 }
 
 cudaError_t launch_gae(const float* rew, const float* val, const uint8_t* done, int T, int N, float gamma, float lambda,
                        float* adv, float* ret, cudaStream_t s) {
-  gae_kernel<<<(N + 127) / 128, 128, 0, s>>>(rew, val, done, T, N, gamma, lambda, adv, ret);
-  return cudaGetLastError();
+  return launch_chained(gae_kernel, (N + 127) / 128, 128, 0, s, rew, val, done, T, N, gamma, lambda, adv, ret);
 }
 
 }  // namespace tj

@@ -60,6 +60,7 @@ __device__ __forceinline__ void sg_dense(const float* __restrict__ W, const floa
 
 // shared memory: xs [D][16] | a1 [H][16] | a2 [H][16] | qs [A][16] | weight tile [256][33]
 __global__ void __launch_bounds__(SG_THREADS) sgd_forward_kernel(const SgdParams p) {
+  chain_begin();
   extern __shared__ __align__(16) float sg_sm[];
   const int D = p.D, H = p.H, A = p.A;
   float* xs = sg_sm;
@@ -258,6 +259,7 @@ template <bool B_KN, int EPI, int BM>
 __global__ void __launch_bounds__(GM_THREADS) sg_gemm_kernel(const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb,
                                                              float* __restrict__ C, int ldc, int M, int N, int K,
                                                              const float* __restrict__ bias, const float* __restrict__ mask, int ldm) {
+  chain_begin();
   sg_gemm_body<B_KN, EPI, BM>(A, lda, B, ldb, C, ldc, M, N, K, bias, mask, ldm);
 }
 
@@ -265,6 +267,7 @@ __global__ void __launch_bounds__(GM_THREADS) sg_gemm_kernel(const float* __rest
 struct GemmPair { const float* A[2]; const float* B[2]; float* C[2]; const float* bias[2]; };
 template <bool B_KN, int EPI, int BM>
 __global__ void __launch_bounds__(GM_THREADS) sg_gemm_pair_kernel(const GemmPair pr, int lda, int ldb, int ldc, int M, int N, int K) {
+  chain_begin();
   const int z = blockIdx.z;
   sg_gemm_body<B_KN, EPI, BM>(pr.A[z], lda, pr.B[z], ldb, pr.C[z], ldc, M, N, K, pr.bias[z], nullptr, 0);
 }
@@ -276,6 +279,7 @@ __global__ void __launch_bounds__(GM_THREADS) sg_gemm_pair_kernel(const GemmPair
 // the 16 x 32 partials are summed by a fixed halving exchange (16 shuffles).  blockIdx.y picks the network.
 constexpr int HD_ROWS = 64;   // rows per block: eight per warp
 __global__ void __launch_bounds__(256) sg_heads_kernel(const GemmPair pr, int n_rows, int H, int A, int ldc) {
+  chain_begin();
   extern __shared__ __align__(16) float4 hd_w[];       // [(j * 4 + kk) * 4 + aq][lane]: W[aq * 4 .. + 3][4 (32 j + lane) + kk]
   const int z = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const float* __restrict__ W = pr.B[z];
@@ -336,8 +340,8 @@ __global__ void __launch_bounds__(256) sg_heads_kernel(const GemmPair pr, int n_
 template <bool B_KN, int EPI, int BM = GM_BM>
 void sg_gemm(const float* A, int lda, const float* B, int ldb, float* C, int ldc, int M, int N, int K, const float* bias,
              const float* mask, int ldm, cudaStream_t s) {
-  sg_gemm_kernel<B_KN, EPI, BM><<<dim3((N + GM_BN - 1) / GM_BN, (M + BM - 1) / BM), GM_THREADS, 0, s>>>(A, lda, B, ldb, C, ldc, M, N, K,
-                                                                                                     bias, mask, ldm);
+  launch_chained(sg_gemm_kernel<B_KN, EPI, BM>, dim3((N + GM_BN - 1) / GM_BN, (M + BM - 1) / BM), GM_THREADS, 0, s, A, lda, B, ldb, C, ldc, M, N, K,
+                 bias, mask, ldm);
 }
 
 // ---------------------------------------------------------------------------------------------------------------------
@@ -379,6 +383,7 @@ __global__ void __launch_bounds__(TG_THREADS, 2) sg_gemm_tc_kernel(const float* 
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_base;
+  chain_begin();
 
   // loader mapping: a warp instruction covers eight rows x four 16-byte pieces (64 contiguous bytes per row); warp w
   // owns rows 16 w .. 16 w + 15 of both operands' tiles, a thread two pieces of each
@@ -502,6 +507,7 @@ __global__ void __launch_bounds__(TG_THREADS, 2) sg_gemm_tc_kernel(const float* 
 
 // dst[c][r] = src[r][c] for an n x n matrix (32 x 32 tiles through shared memory, both sides coalesced)
 __global__ void __launch_bounds__(256) sg_transpose_kernel(const float* __restrict__ src, float* __restrict__ dst, int n) {
+  chain_begin();
   __shared__ float tile[32][33];
   const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   for (int i = ty; i < 32; i += 8)
@@ -524,10 +530,8 @@ template <int EPI>
 cudaError_t sg_layer(const float* A, int lda, const float* B, int ldb, float* C, int ldc, int M, int N, int K, const float* bias,
                      const float* mask, int ldm, unsigned long long* error, cudaStream_t s) {
   if (tc_gemm_ok(A, lda, B, ldb, M, N, K)) {
-    cudaError_t e = cudaFuncSetAttribute(sg_gemm_tc_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, TG_SMEM_BYTES);
-    if (e != cudaSuccess) return e;
-    sg_gemm_tc_kernel<EPI><<<dim3((N + TG_N - 1) / TG_N, (M + TG_M - 1) / TG_M), TG_THREADS, TG_SMEM_BYTES, s>>>(A, lda, B, ldb, C, ldc, M, N, K,
-                                                                                                         bias, mask, ldm, error);
+    return launch_chained(sg_gemm_tc_kernel<EPI>, dim3((N + TG_N - 1) / TG_N, (M + TG_M - 1) / TG_M), TG_THREADS, TG_SMEM_BYTES, s, A, lda, B, ldb,
+                          C, ldc, M, N, K, bias, mask, ldm, error);
   } else {
     sg_gemm<false, EPI>(A, lda, B, ldb, C, ldc, M, N, K, bias, mask, ldm, s);
   }
@@ -538,6 +542,8 @@ cudaError_t sg_layer(const float* A, int lda, const float* B, int ldb, float* C,
 // ([n][A]: a row is read, then overwritten by its own thread), qt [n][A]; loss partials per SG_ROWS rows as in the
 // fused forward kernel
 __global__ void __launch_bounds__(32) sgd_loss_kernel(const SgdParams p, const float* __restrict__ qt) {
+  chain_begin();
+  chain_next();
   __shared__ float hub[SG_ROWS];
   const int r = threadIdx.x, j = blockIdx.x * SG_ROWS + r, A = p.A;
   if (r < SG_ROWS) {
@@ -570,6 +576,7 @@ __global__ void __launch_bounds__(32) sgd_loss_kernel(const SgdParams p, const f
 // loss and the entropy, and their gradients at the outputs: g[j][0..A) for the logits, g[j][A] for the value.
 // shared memory: xs [D][16] | a1 [H][16] | a2 [H][16] | qs [A + 1][16] | weight tile [256][33]
 __global__ void __launch_bounds__(SG_THREADS) ppo_forward_kernel(const SgdParams p) {
+  chain_begin();
   extern __shared__ __align__(16) float sg_sm[];
   const int D = p.D, H = p.H, A = p.A;
   float* xs = sg_sm;
@@ -649,6 +656,8 @@ __global__ void __launch_bounds__(SG_THREADS) ppo_forward_kernel(const SgdParams
 
 // out[k] = (sum over the blocks of partial k) / n, k = 0..4, blocks in ascending order
 __global__ void ppo_finish_kernel(const float* __restrict__ stat_partial, int n_blocks, int n, float* __restrict__ out) {
+  chain_begin();
+  chain_next();
   const int k = threadIdx.x;
   if (k >= 5) return;
   float s = 0.f;
@@ -658,6 +667,7 @@ __global__ void ppo_finish_kernel(const float* __restrict__ stat_partial, int n_
 
 // backward through the activations, SG_ROWS rows per block: shared memory d2 [H][16]
 __global__ void __launch_bounds__(SG_THREADS) sgd_backward_kernel(const SgdParams p) {
+  chain_begin();
   extern __shared__ __align__(16) float sg_sm[];
   const int D = p.D, H = p.H, A = p.A;
   float* d2 = sg_sm;
@@ -809,6 +819,7 @@ __device__ __forceinline__ void grad_tile(float* __restrict__ P, const GradProdu
 // No atomics: the apply kernel adds the ranges in order.
 __global__ void __launch_bounds__(256) sgd_grad_partial_kernel(float* __restrict__ P, const GradProducts gp, int count, int n_rows,
                                                                int rows_per_range) {
+  chain_begin();
   __shared__ __align__(16) float As[GP_ROWS][128 + 4], Bs[GP_ROWS][GP_TILE + 4];
   int q = 0;
   while (q + 1 < gp.n && (int)blockIdx.x >= gp.g[q + 1].tile_begin) ++q;
@@ -820,6 +831,8 @@ __global__ void __launch_bounds__(256) sgd_grad_partial_kernel(float* __restrict
 
 // C[i] -= lr * (P[0][i] + P[1][i] + ...), the partial sums added in range order
 __global__ void sgd_apply_kernel(float* __restrict__ Cm, const float* __restrict__ P, int count, int n_ranges, float lr) {
+  chain_begin();
+  chain_next();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   float s = 0.f;
@@ -832,6 +845,8 @@ __global__ void sgd_apply_kernel(float* __restrict__ Cm, const float* __restrict
 __global__ void sgd_apply_adam_kernel(float* __restrict__ Cm, float* __restrict__ m, float* __restrict__ v,
                                       const float* __restrict__ P, int count, int n_ranges, float lr, float beta1, float beta2,
                                       float eps, float c1, float c2) {
+  chain_begin();
+  chain_next();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   float g = 0.f;
@@ -890,14 +905,13 @@ cudaError_t backward_and_update(const SgdParams& p, float lr, const AdamParams* 
       if ((e = launch_gemm_tc2(b, GM_MASK, p.error, s)) != cudaSuccess) return e;
     } else if (tc_gemm_ok(p.dh2, H, p.w2t, H, p.n, H, H)) {
       // the tensor-core product wants both operands K-major: dh1 = dh2 (W2^T)^T with W2^T written out first
-      sg_transpose_kernel<<<dim3((H + 31) / 32, (H + 31) / 32), 256, 0, s>>>(W2m, p.w2t, H);
+      if ((e = launch_chained(sg_transpose_kernel, dim3((H + 31) / 32, (H + 31) / 32), 256, 0, s, W2m, p.w2t, H)) != cudaSuccess) return e;
       if ((e = sg_layer<GM_MASK>(p.dh2, H, p.w2t, H, p.dh1, H, p.n, H, H, nullptr, p.h1, H, p.error, s)) != cudaSuccess) return e;
     } else {
       sg_gemm<true, GM_MASK>(p.dh2, H, W2m, H, p.dh1, H, p.n, H, H, nullptr, p.h1, H, s);
     }
   } else {
-    if ((e = cudaFuncSetAttribute(sgd_backward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_b)) != cudaSuccess) return e;
-    sgd_backward_kernel<<<grid, SG_THREADS, smem_b, s>>>(p);
+    if ((e = launch_chained(sgd_backward_kernel, grid, SG_THREADS, smem_b, s, p)) != cudaSuccess) return e;
   }
   float* W1 = p.theta;
   float* b1 = W1 + (size_t)H * D;
@@ -955,13 +969,13 @@ cudaError_t backward_and_update(const SgdParams& p, float lr, const AdamParams* 
   n_ranges = (p.n + rows_per_range - 1) / rows_per_range;
   const int count = (int)((p.value_head ? bv + 1 : b3 + A) - p.theta);
   if (tb.n && (e = launch_wgrad_tc(tb, p.grad_partial, count, p.n, rows_per_range, n_ranges, p.error, s)) != cudaSuccess) return e;
-  if (gp.n_tiles > 0) sgd_grad_partial_kernel<<<dim3(gp.n_tiles, n_ranges), 256, 0, s>>>(p.grad_partial, gp, count, p.n, rows_per_range);
+  if (gp.n_tiles > 0 &&
+      (e = launch_chained(sgd_grad_partial_kernel, dim3(gp.n_tiles, n_ranges), 256, 0, s, p.grad_partial, gp, count, p.n, rows_per_range)) != cudaSuccess)
+    return e;
   if (adam)
-    sgd_apply_adam_kernel<<<(count + 255) / 256, 256, 0, s>>>(p.theta, adam->m, adam->v, p.grad_partial, count, n_ranges, lr, adam->beta1,
-                                                              adam->beta2, adam->eps, adam->c1, adam->c2);
-  else
-    sgd_apply_kernel<<<(count + 255) / 256, 256, 0, s>>>(p.theta, p.grad_partial, count, n_ranges, lr);
-  return cudaGetLastError();
+    return launch_chained(sgd_apply_adam_kernel, (count + 255) / 256, 256, 0, s, p.theta, adam->m, adam->v, p.grad_partial, count, n_ranges, lr,
+                          adam->beta1, adam->beta2, adam->eps, adam->c1, adam->c2);
+  return launch_chained(sgd_apply_kernel, (count + 255) / 256, 256, 0, s, p.theta, p.grad_partial, count, n_ranges, lr);
 }
 }  // namespace
 
@@ -1014,11 +1028,11 @@ cudaError_t launch_sgd_step(const SgdParams& p, float lr, const AdamParams* adam
       GemmPair heads{{p.h2, p.dh2}, {W3, T3}, {p.g, p.dh1}, {b3, tb3}};
       const size_t hd_smem = (size_t)H * 16 * sizeof(float);
       if (H % 128 == 0 && A <= 16 && hd_smem <= 96 * 1024) {
-        if ((e = cudaFuncSetAttribute(sg_heads_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hd_smem)) != cudaSuccess) return e;
-        sg_heads_kernel<<<dim3((n + HD_ROWS - 1) / HD_ROWS, 2), 256, hd_smem, s>>>(heads, n, H, A, A);
+        e = launch_chained(sg_heads_kernel, dim3((n + HD_ROWS - 1) / HD_ROWS, 2), 256, hd_smem, s, heads, n, H, A, A);
       } else {
-        sg_gemm_pair_kernel<false, GM_BIAS, 32><<<dim3((A + GM_BN - 1) / GM_BN, (n + 31) / 32, 2), GM_THREADS, 0, s>>>(heads, H, H, A, n, A, H);
+        e = launch_chained(sg_gemm_pair_kernel<false, GM_BIAS, 32>, dim3((A + GM_BN - 1) / GM_BN, (n + 31) / 32, 2), GM_THREADS, 0, s, heads, H, H, A, n, A, H);
       }
+      if (e != cudaSuccess) return e;
     } else {
       if ((e = sg_layer<GM_BIAS_RELU>(p.obs, D, W1, D, p.h1, H, n, H, D, b1, nullptr, 0, p.error, s)) != cudaSuccess) return e;
       if ((e = sg_layer<GM_BIAS_RELU>(p.h1, H, W2, H, p.h2, H, n, H, H, b2, nullptr, 0, p.error, s)) != cudaSuccess) return e;
@@ -1027,22 +1041,20 @@ cudaError_t launch_sgd_step(const SgdParams& p, float lr, const AdamParams* adam
       if ((e = sg_layer<GM_BIAS_RELU>(p.dh1, H, T2, H, p.dh2, H, n, H, H, tb2, nullptr, 0, p.error, s)) != cudaSuccess) return e;
       sg_gemm<false, GM_BIAS, 32>(p.dh2, H, T3, H, p.dh1, A, n, A, H, tb3, nullptr, 0, s);
     }
-    sgd_loss_kernel<<<sgd_partial_count(n), 32, 0, s>>>(p, p.dh1);
+    if ((e = launch_chained(sgd_loss_kernel, sgd_partial_count(n), 32, 0, s, p, (const float*)p.dh1)) != cudaSuccess) return e;
     return backward_and_update(p, lr, adam, s);
   }
   const size_t smem_f = (((size_t)p.D + 2 * (size_t)p.H + p.A) * SG_ROWS + (size_t)SG_THREADS * (SG_KT + 1)) * sizeof(float);
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(sgd_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_f)) != cudaSuccess) return e;
-  sgd_forward_kernel<<<sgd_partial_count(p.n), SG_THREADS, smem_f, s>>>(p);
+  if ((e = launch_chained(sgd_forward_kernel, sgd_partial_count(p.n), SG_THREADS, smem_f, s, p)) != cudaSuccess) return e;
   return backward_and_update(p, lr, adam, s);
 }
 
 cudaError_t launch_ppo_step(const SgdParams& p, float lr, const AdamParams* adam, float* stats_out, cudaStream_t s) {
   const size_t smem_f = (((size_t)p.D + 2 * (size_t)p.H + p.A + 1) * SG_ROWS + (size_t)SG_THREADS * (SG_KT + 1)) * sizeof(float);
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(ppo_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_f)) != cudaSuccess) return e;
-  ppo_forward_kernel<<<sgd_partial_count(p.n), SG_THREADS, smem_f, s>>>(p);
-  if (stats_out) ppo_finish_kernel<<<1, 32, 0, s>>>(p.stat_partial, sgd_partial_count(p.n), p.n, stats_out);
+  if ((e = launch_chained(ppo_forward_kernel, sgd_partial_count(p.n), SG_THREADS, smem_f, s, p)) != cudaSuccess) return e;
+  if (stats_out && (e = launch_chained(ppo_finish_kernel, 1, 32, 0, s, p.stat_partial, sgd_partial_count(p.n), p.n, stats_out)) != cudaSuccess) return e;
   return backward_and_update(p, lr, adam, s);
 }
 

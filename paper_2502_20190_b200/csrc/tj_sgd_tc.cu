@@ -84,6 +84,7 @@ __global__ void __launch_bounds__(T2_THREADS, 1) sg_gemm_tc2_kernel(const TcGemm
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = ctl->tmem_base;
+  chain_begin();
   volatile int* abort_flag = &ctl->abort_flag;
 
   if (tid < T2_WORKERS) {
@@ -278,6 +279,7 @@ __global__ void __launch_bounds__(T2_THREADS, 1) sg_wgrad_tc_kernel(const TcWgra
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = ctl->tmem_base;
+  chain_begin();
   volatile int* abort_flag = &ctl->abort_flag;
 
   if (tid < T2_WORKERS) {
@@ -431,6 +433,7 @@ __global__ void __launch_bounds__(T2_THREADS, 1) sg_wgrad_tc_kernel(const TcWgra
 // them: per tile of 256 rows and chunk of 16 columns one 32 KB block [high 256 x 16 | low 256 x 16], each part as K-major
 // core matrices (8 rows x 4 columns contiguous; element (n, k) at ((n / 8) * 4 + k / 4) * 32 + (n % 8) * 4 + k % 4).
 __global__ void __launch_bounds__(256) sg_pack_tf32_kernel(const TcPackJobs jobs) {
+  chain_begin();
   const TcPackJob& jb = jobs.j[blockIdx.y];
   const int total = jb.N * jb.K, nk = jb.K / T2_K;
   constexpr int PER = T2_N * T2_K;
@@ -458,8 +461,7 @@ size_t tc_pack_floats(int N, int K) { return (size_t)2 * N * K; }
 
 cudaError_t launch_pack_tf32_operands(const TcPackJobs& jobs, cudaStream_t s) {
   if (jobs.n <= 0) return cudaSuccess;
-  sg_pack_tf32_kernel<<<dim3(128, jobs.n), 256, 0, s>>>(jobs);
-  return cudaGetLastError();
+  return launch_chained(sg_pack_tf32_kernel, dim3(128, jobs.n), 256, 0, s, jobs);
 }
 
 cudaError_t launch_gemm_tc2(const TcGemmBatch& batch, int epi, unsigned long long* error, cudaStream_t s) {
@@ -467,10 +469,7 @@ cudaError_t launch_gemm_tc2(const TcGemmBatch& batch, int epi, unsigned long lon
   const TcGemm& g0 = batch.g[0];
   for (int i = 1; i < batch.n; ++i)
     if (batch.g[i].M != g0.M || batch.g[i].N != g0.N) return cudaErrorInvalidValue;   // one grid for all problems of a launch
-  cudaError_t e = cudaFuncSetAttribute(sg_gemm_tc2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, T2_SMEM_BYTES);
-  if (e != cudaSuccess) return e;
-  sg_gemm_tc2_kernel<<<dim3(g0.N / T2_N, (g0.M + T2_M - 1) / T2_M, batch.n), T2_THREADS, T2_SMEM_BYTES, s>>>(batch, epi, error);
-  return cudaGetLastError();
+  return launch_chained(sg_gemm_tc2_kernel, dim3(g0.N / T2_N, (g0.M + T2_M - 1) / T2_M, batch.n), T2_THREADS, T2_SMEM_BYTES, s, batch, epi, error);
 }
 
 bool tc_wgrad_ok(int N, int rows) { return N % 128 == 0 && rows >= 1024; }
@@ -480,10 +479,7 @@ int tc_wgrad_tiles(int M, int N) { return ((M + T2_M - 1) / T2_M) * (N / (N % T2
 cudaError_t launch_wgrad_tc(const TcWgradBatch& batch, float* P, int count, int n_rows, int rows_per_range, int n_ranges,
                             unsigned long long* error, cudaStream_t s) {
   if (batch.n <= 0 || batch.n_tiles <= 0) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(sg_wgrad_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, WG_SMEM_BYTES);
-  if (e != cudaSuccess) return e;
-  sg_wgrad_tc_kernel<<<dim3(batch.n_tiles, n_ranges), T2_THREADS, WG_SMEM_BYTES, s>>>(batch, P, count, n_rows, rows_per_range, error);
-  return cudaGetLastError();
+  return launch_chained(sg_wgrad_tc_kernel, dim3(batch.n_tiles, n_ranges), T2_THREADS, WG_SMEM_BYTES, s, batch, P, count, n_rows, rows_per_range, error);
 }
 
 }  // namespace tj

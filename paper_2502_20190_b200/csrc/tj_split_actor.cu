@@ -248,11 +248,12 @@ __global__ void __launch_bounds__(SA_NT, 1) actor_split_tc_kernel(const ActorPar
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&ctl->tmem_base)), "r"(256u) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  const MlpWeights mw = stage_mlp_weights<1>(p, p.W, wsm, &ctl->wbar, tid == 0);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = ctl->tmem_base;
+  chain_begin();
+  const MlpWeights mw = stage_mlp_weights<1>(p, p.W, wsm, &ctl->wbar, tid == 0);
   volatile int* abort_flag = &ctl->abort_flag;
   bool ok = tc_wait_elect(&ctl->wbar, 0, abort_flag);
   ok = __syncthreads_and(ok);
@@ -437,15 +438,16 @@ __global__ void __launch_bounds__(SA_NT, 1) td_split_tc_kernel(const TdParams p,
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&ctl->tmem_base)), "r"(256u) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = ctl->tmem_base;
+  chain_begin();
   MlpWeights mw = stage_mlp_weights<1>(p, p.Wonline, wsm, &ctl->wbar, tid == 0);
   for (int i = tid; i < SA_TE * D; i += SA_NT) {
     const int el = i / D, k = i % D;
     sh.xs[k * SA_TE + el] = el < n_here ? p.obs[(size_t)(j0 + el) * D + k] : 0.f;
   }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = ctl->tmem_base;
   volatile int* abort_flag = &ctl->abort_flag;
   bool ok = tc_wait_elect(&ctl->wbar, 0, abort_flag);
   ok = __syncthreads_and(ok);
@@ -527,52 +529,9 @@ __global__ void __launch_bounds__(SA_NT, 1) td_split_tc_kernel(const TdParams p,
   }
 }
 
-// W2 [H][H] (row = neuron) -> scaled FP16 high and low parts as the stream the kernel consumes: for each K chunk kc of 32
-// columns first the high parts' chunk, then the low parts', each H rows x 32 columns in the K-major core-matrix layout:
-// element (n, k) sits at ((n / 8) * 4 + (k % 32) / 8) * 64 + (n % 8) * 8 + k % 8 inside its chunk.
-// scale_out[0] = the power of two the weights were multiplied by, scale_out[1] = 1 / (that x the activation scale).
-// One launch of a few large blocks: every block finds the largest |entry| of the matrix itself (64 K floats from L2 at most,
-// 64 per thread), so no block waits for another; block 0 records the scale; then each block packs its share.
-constexpr int SPLIT_PACK_BLOCKS = 32, SPLIT_PACK_THREADS = 1024;
-__global__ void __launch_bounds__(SPLIT_PACK_THREADS) split_pack_kernel(const float* __restrict__ blob, int D, int H, float* __restrict__ scale_out,
-                                                                        uint16_t* __restrict__ dst) {
-  __shared__ float wmax[32];
-  const float* W2 = blob + (size_t)H * D + H;
-  float m = 0.f;
-  for (int i = threadIdx.x; i < H * H; i += blockDim.x) m = fmaxf(m, fabsf(W2[i]));   // the caller's pointer may be only 4-byte aligned
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
-  __syncthreads();
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = fmaxf(m, wmax[w]);
-  // largest entry into [1024, 2048): far inside FP16's range, low parts of all but the tiniest entries normal
-  int e = 0;
-  if (m > 0.f && isfinite(m)) e = 10 - (int)floorf(log2f(m));
-  e = e < -24 ? -24 : (e > 24 ? 24 : e);
-  const float sc = exp2f((float)e);
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    scale_out[0] = sc;
-    scale_out[1] = 1.0f / (sc * SA_H_SCALE);
-  }
-  const int chunk_elems = H * SA_KC;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < H * H; i += gridDim.x * blockDim.x) {
-    const int kc = i / chunk_elems, within = i % chunk_elems;
-    const int core = within / 64, in_core = within % 64;
-    const int rg = core / (SA_KC / 8), kg = core % (SA_KC / 8);
-    const int n = rg * 8 + in_core / 8, k = kc * SA_KC + kg * 8 + in_core % 8;
-    const float v = W2[(size_t)n * H + k] * sc;
-    const __half hi = __float2half_rn(v);
-    const __half lo = __float2half_rn(v - __half2float(hi));
-    dst[(size_t)(2 * kc) * chunk_elems + within] = __half_as_ushort(hi);
-    dst[(size_t)(2 * kc + 1) * chunk_elems + within] = __half_as_ushort(lo);
-  }
-}
-
 template <int ENV, int H>
 cudaError_t launch_split(const ActorParams& p, const uint16_t* w2parts, const float* w2scale, int grid, size_t smem, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(actor_split_tc_kernel<ENV, H>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  actor_split_tc_kernel<ENV, H><<<grid, SA_NT, smem, s>>>(p, w2parts, w2scale);
-  return cudaGetLastError();
+  return launch_chained(actor_split_tc_kernel<ENV, H>, grid, SA_NT, smem, s, p, w2parts, w2scale);
 }
 
 template <int ENV>
@@ -595,10 +554,7 @@ bool split_actor_supported(int env_kind, int D, int H, int Aout) {
 
 size_t split_weight_halfs(int H) { return (size_t)2 * H * H; }
 
-cudaError_t launch_pack_split_weights(const float* blob, int D, int H, uint16_t* dst, float* scale, cudaStream_t s) {
-  split_pack_kernel<<<SPLIT_PACK_BLOCKS, SPLIT_PACK_THREADS, 0, s>>>(blob, D, H, scale, dst);
-  return cudaGetLastError();
-}
+float split_hidden_scale() { return SA_H_SCALE; }
 
 cudaError_t launch_actor_split(int env_kind, const ActorParams& p, const uint16_t* w2parts, const float* w2scale, int sm_count,
                                cudaStream_t s) {
@@ -617,13 +573,8 @@ cudaError_t launch_actor_split(int env_kind, const ActorParams& p, const uint16_
 template <int D>
 static cudaError_t launch_td_split_d(const TdParams& p, const uint16_t* po, const float* so, const uint16_t* pt, const float* st, int grid,
                                      size_t smem, cudaStream_t s) {
-#define TJ_TD_SPLIT_CASE(HH)                                                                                                      \
-  case HH: {                                                                                                                      \
-    cudaError_t e = cudaFuncSetAttribute(td_split_tc_kernel<D, HH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);      \
-    if (e != cudaSuccess) return e;                                                                                               \
-    td_split_tc_kernel<D, HH><<<grid, SA_NT, smem, s>>>(p, po, so, pt, st);                                                        \
-    return cudaGetLastError();                                                                                                    \
-  }
+#define TJ_TD_SPLIT_CASE(HH) \
+  case HH: return launch_chained(td_split_tc_kernel<D, HH>, grid, SA_NT, smem, s, p, po, so, pt, st);
   switch (p.H) {
     TJ_TD_SPLIT_CASE(64)
     TJ_TD_SPLIT_CASE(128)

@@ -74,13 +74,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
     mbar_init(&ctl->pair_sync, TC_EPI_THREADS);
     ctl->abort_flag = 0;
   }
-  for (int i = tid; i < 2 * H + TC_N3; i += TC_THREADS) {
-    float v;
-    if (i < H) v = p.b1[i];
-    else if (i < 2 * H) v = p.b2[i - H];
-    else v = (i - 2 * H) < p.Aout ? p.b3[i - 2 * H] : 0.f;
-    bias[i] = v;
-  }
   __syncthreads();
   if (warp == 1) {   // one warp allocates all 512 TMEM columns (one block per SM) and publishes the base address
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&ctl->tmem_base)), "r"(512u) : "memory");
@@ -91,6 +84,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
   tc_fence_after();
   const uint32_t tmem = ctl->tmem_base;
   volatile int* abort_flag = &ctl->abort_flag;
+  chain_begin();
+  for (int i = tid; i < 2 * H + TC_N3; i += TC_THREADS) {
+    float v;
+    if (i < H) v = p.b1[i];
+    else if (i < 2 * H) v = p.b2[i - H];
+    else v = (i - 2 * H) < p.Aout ? p.b3[i - 2 * H] : 0.f;
+    bias[i] = v;
+  }
+  __syncthreads();
 
   // chunk schedule of one tile, the same for producer and MMA issuer:
   //   layer 1: n_blocks x (D/KC) chunks of NB rows; layer 2: n_blocks x (H/KC) chunks of NB rows;
@@ -447,48 +449,13 @@ done:
   }
 }
 
-// FP32 blob -> BF16 chunks in the order the producer streams them; within a chunk of R rows x KC columns
-// element (r, k) sits at ((r/8) * (KC/8) + k/8) * 64 + (r%8) * 8 + k%8.  Hidden layers: R = NB, KC = 32;
-// head: one chunk with R = 16, KC = H.
-__global__ void pack_tc_weights_kernel(const float* __restrict__ blob, uint16_t* __restrict__ dst, int D, int H, int A,
-                                       int value_head) {
-  const int n_blocks = H > 256 ? 2 : 1, NB = H / n_blocks;
-  const size_t n1 = (size_t)H * D, n2 = (size_t)H * H, n3 = (size_t)TC_N3 * H;
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n1 + n2 + n3) return;
-  const float* W1 = blob;
-  const float* W2 = W1 + n1 + H;
-  const float* W3 = W2 + n2 + H;
-  const float* Wv = W3 + (size_t)A * H + A;
-  size_t j = i;
-  const float* W;
-  int K, R, rows_total, n_off;
-  if (j < n1) { W = W1; K = D; R = NB; rows_total = H; }
-  else if (j < n1 + n2) { j -= n1; W = W2; K = H; R = NB; rows_total = H; }
-  else { j -= n1 + n2; W = W3; K = H; R = TC_N3; rows_total = A; }
-  const int KCc = W == W3 ? H : TC_KC;               // columns per chunk (the head is one chunk)
-  const size_t chunk_elems = (size_t)R * KCc;
-  const size_t chunk = j / chunk_elems, within = j % chunk_elems;
-  const int chunks_per_block = K / KCc;
-  const int nb = (int)(chunk / chunks_per_block), kc = (int)(chunk % chunks_per_block);
-  n_off = nb * R;
-  const int core = (int)(within / 64), in_core = (int)(within % 64);
-  const int rg = core / (KCc / 8), kg = core % (KCc / 8);
-  const int r = rg * 8 + in_core / 8, k = kc * KCc + kg * 8 + in_core % 8;
-  const int n = n_off + r;
-  float v = 0.f;
-  if (n < rows_total) v = W[(size_t)n * K + k];
-  else if (W == W3 && value_head && n == A) v = Wv[k];
-  uint32_t u = __float_as_uint(v);
-  u += 0x7FFFu + ((u >> 16) & 1u);
-  dst[i] = (uint16_t)(u >> 16);
-}
-
 // TD error from precomputed Q rows: q = Qo[j][act], q' = max_a Qt[j][a]; per-block partial sums of the Huber loss
 __global__ void td_from_q_kernel(const float* __restrict__ q_online, const float* __restrict__ q_target, int n, int A,
                                  const int* __restrict__ act, const float* __restrict__ rew,
                                  const int* __restrict__ done, float gamma, float kappa, float* __restrict__ td_out,
                                  float* __restrict__ huber_out, float* __restrict__ partial) {
+  chain_begin();
+  chain_next();
   __shared__ float hub[16];
   const int j = blockIdx.x * 16 + threadIdx.x;
   float h = 0.f;
@@ -524,25 +491,15 @@ bool tc_mlp_supported(int D, int H, int Aout) {
 
 size_t tc_weight_elems(int D, int H) { return (size_t)H * D + (size_t)H * H + (size_t)TC_N3 * H; }
 
-cudaError_t launch_pack_tc_weights(const float* blob, uint16_t* dst, int D, int H, int A, int value_head, cudaStream_t s) {
-  const size_t n = tc_weight_elems(D, H);
-  pack_tc_weights_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(blob, dst, D, H, A, value_head);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_tc_mlp(const TcMlpParams& p, int sm_count, cudaStream_t s) {
   if (p.n <= 0) return cudaSuccess;
   const bool fused = p.env.fused != 0;
   const size_t smem = tc_abuf_bytes(p.D, p.H, fused) + (size_t)TC_STAGES * TC_STAGE_BYTES + (size_t)(2 * p.H + TC_N3) * 4 +
                       sizeof(TcSmem) + 64;
   if (smem > 227 * 1024) return cudaErrorInvalidConfiguration;
-  auto kernel = fused ? mlp_bf16_tc_kernel<true> : mlp_bf16_tc_kernel<false>;
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   const int n_tiles = (p.n + TC_M - 1) / TC_M;
   const int grid = n_tiles < sm_count ? n_tiles : sm_count;
-  kernel<<<grid, TC_THREADS, smem, s>>>(p);
-  return cudaGetLastError();
+  return launch_chained(fused ? mlp_bf16_tc_kernel<true> : mlp_bf16_tc_kernel<false>, grid, TC_THREADS, smem, s, p);
 }
 
 // the env matrix A [D][D] as TF32 high and low parts, tiled in chunks of D rows x KC columns:
@@ -574,9 +531,8 @@ bool tc_fused_supported(int D, int H, int A) {
 cudaError_t launch_td_from_q(const float* q_online, const float* q_target, int n, int A, const int* act, const float* rew,
                              const int* done, float gamma, float kappa, float* td_out, float* huber_out, float* partial,
                              cudaStream_t s) {
-  td_from_q_kernel<<<(n + 15) / 16, 32, 0, s>>>(q_online, q_target, n, A, act, rew, done, gamma, kappa, td_out, huber_out,
-                                                partial);
-  return cudaGetLastError();
+  return launch_chained(td_from_q_kernel, (n + 15) / 16, 32, 0, s, q_online, q_target, n, A, act, rew, done, gamma, kappa, td_out,
+                        huber_out, partial);
 }
 
 }  // namespace tj

@@ -103,6 +103,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = ctl->tmem_base;
+  chain_begin();
   volatile int* abort_flag = &ctl->abort_flag;
   const TcEnvParams& ev = p.env;
 
@@ -504,40 +505,6 @@ done:
   }
 }
 
-// FP32 blob -> BF16 chunks in the order the pipelined actor streams them.  Hidden layers: per 128-neuron block, chunks of
-// 128 rows x 128 columns; element (r, k) of a chunk sits at ((r/8) * 16 + k/8) * 64 + (r%8) * 8 + k%8.  Head: one chunk of
-// 16 rows x H columns, element (r, k) at ((r/8) * (H/8) + k/8) * 64 + (r%8) * 8 + k%8.
-__global__ void pack_pipelined_weights_kernel(const float* __restrict__ blob, uint16_t* __restrict__ dst, int D, int H, int A) {
-  const size_t n1 = (size_t)H * D, n2 = (size_t)H * H, n3 = (size_t)PA_N3 * H;
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n1 + n2 + n3) return;
-  const float* W1 = blob;
-  const float* W2 = W1 + n1 + H;
-  const float* W3 = W2 + n2 + H;
-  float v = 0.f;
-  if (i < n1 + n2) {
-    const bool first = i < n1;
-    const size_t j = first ? i : i - n1;
-    const int K = first ? D : H;
-    const int chunks_per_block = K / PA_KC;
-    const size_t chunk = j / (PA_NB * PA_KC), within = j % (PA_NB * PA_KC);
-    const int b = (int)(chunk / chunks_per_block), c = (int)(chunk % chunks_per_block);
-    const int core = (int)(within / 64), in_core = (int)(within % 64);
-    const int rg = core / (PA_KC / 8), kg = core % (PA_KC / 8);
-    const int n = b * PA_NB + rg * 8 + in_core / 8, k = c * PA_KC + kg * 8 + in_core % 8;
-    v = (first ? W1 : W2)[(size_t)n * K + k];
-  } else {
-    const size_t j = i - n1 - n2;
-    const int core = (int)(j / 64), in_core = (int)(j % 64);
-    const int rg = core / (H / 8), kg = core % (H / 8);
-    const int n = rg * 8 + in_core / 8, k = kg * 8 + in_core % 8;
-    if (n < A) v = W3[(size_t)n * H + k];
-  }
-  uint32_t u = __float_as_uint(v);
-  u += 0x7FFFu + ((u >> 16) & 1u);
-  dst[i] = (uint16_t)(u >> 16);
-}
-
 // The env matrix A [128][128] scaled by `scale` (a power of two) as two FP16 chunks, high parts then low parts, each in the
 // layout of a weight chunk (row = component of z, column = component of s); B [n_actions][128] times 2 log2(e).
 __global__ void pack_env_f16_kernel(const float* __restrict__ A, const float* __restrict__ B, float scale, int n_b,
@@ -566,12 +533,6 @@ size_t tc_pipelined_scratch_floats() { return (size_t)PA_MAX_GRID * 2 * PA_M * P
 size_t tc_pipelined_env_halfs() { return (size_t)2 * PA_D * PA_D; }
 float tc_pipelined_state_scale() { return PA_S_SCALE; }
 
-cudaError_t launch_pack_pipelined_weights(const float* blob, uint16_t* dst, int D, int H, int A, cudaStream_t s) {
-  const size_t n = tc_weight_elems(D, H);
-  pack_pipelined_weights_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(blob, dst, D, H, A);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_pack_pipelined_env(const float* A, const float* B, float scale, int n_actions, uint16_t* dst, float* b_t,
                                       cudaStream_t s) {
   const int n = PA_D * PA_D > n_actions * PA_D ? PA_D * PA_D : n_actions * PA_D;
@@ -583,14 +544,11 @@ cudaError_t launch_actor_tc_pipelined(const TcMlpParams& p, int sm_count, cudaSt
   if (p.n <= 0) return cudaSuccess;
   if (!tc_pipelined_supported(p.D, p.H, p.Aout) || !p.env.fused) return cudaErrorInvalidConfiguration;
   const size_t smem = (size_t)PA_X_BYTES + PA_U_BYTES + (size_t)PA_STAGES * PA_STAGE_BYTES + sizeof(PaSmem) + 64;
-  cudaError_t e = cudaFuncSetAttribute(actor_tc_pipelined_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   const int n_tiles = (p.n + PA_M - 1) / PA_M;
   int grid = n_tiles < sm_count ? n_tiles : sm_count;
   if (grid > PA_MAX_GRID) grid = PA_MAX_GRID;
   if (!p.env.z_scratch || !p.env.lgA16 || !p.env.lgB_t) return cudaErrorInvalidValue;
-  actor_tc_pipelined_kernel<<<grid, PA_THREADS, smem, s>>>(p);
-  return cudaGetLastError();
+  return launch_chained(actor_tc_pipelined_kernel, grid, PA_THREADS, smem, s, p);
 }
 
 }  // namespace tj
