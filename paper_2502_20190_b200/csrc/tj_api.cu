@@ -695,14 +695,14 @@ void lay_out_update_scratch(const tj_ctx* x, tj::SgdParams& p) {
   p.h1 = x->sgd_scratch; p.h2 = p.h1 + RH; p.dh1 = p.h2 + RH; p.dh2 = p.dh1 + RH;
   p.g = p.dh2 + RH;
   p.partial = p.g + rows * 17;
-  p.stat_partial = p.partial + rows / 16 + 8;
+  p.stat_partial = p.partial + sgd_partial_floats(x->sgd_rows);
   p.w2t = p.stat_partial + 5 * (rows / 16) + 8;
   p.w2t += (4 - ((reinterpret_cast<uintptr_t>(p.w2t) / sizeof(float)) & 3)) & 3;   // 16-byte rows for the vector loads
   p.grad_partial = p.w2t + (size_t)x->H * x->H;
+  p.grad_partial += (4 - ((reinterpret_cast<uintptr_t>(p.grad_partial) / sizeof(float)) & 3)) & 3;
   {
     // after the partial gradients: split weight copies for the tensor-core products, 128-byte aligned for the bulk copies
-    const size_t blob = (size_t)x->H * x->D + x->H + (size_t)x->H * x->H + x->H + 17 * (size_t)x->H + 17;
-    float* w = p.grad_partial + (size_t)tj::SG_SPLITS * blob;
+    float* w = p.grad_partial + sgd_grad_partial_floats(x->sgd_rows, x->D, x->H);
     w += (32 - ((reinterpret_cast<uintptr_t>(w) / sizeof(float)) & 31)) & 31;
     p.wpack = w;
     p.sm_count = x->sm_count;
@@ -726,11 +726,9 @@ int learner_update(tj_ctx* x, const tj_batch* b, float lr, float* theta, const f
   lay_out_update_scratch(x, p);
   p.ldg = x->A; p.value_head = 0;
   p.error = &x->dstats->error;
-  LaunchScope scope(x, TJ_K_SGD, tj::sgd_step_launches(p) + (loss_mean_out ? 1 : 0), true, true);
-  cudaError_t e = launch_sgd_step(p, lr, adam, x->lstream);
+  LaunchScope scope(x, TJ_K_SGD, tj::sgd_step_launches(p, loss_mean_out != nullptr), true, true);
+  cudaError_t e = launch_sgd_step(p, lr, adam, loss_mean_out, x->lstream);
   if (e != cudaSuccess) return cuda_fail(x, e, "learner update");
-  if (loss_mean_out && (e = launch_td_finish(p.partial, sgd_partial_count(b->n), b->n, loss_mean_out, x->lstream)) != cudaSuccess)
-    return cuda_fail(x, e, "learner update (loss reduction)");
   learner_launched(x);
   return TJ_OK;
 }

@@ -285,11 +285,19 @@ bool tc_gemm2_ok(const float* A, int lda, int M, int N, int K);
 size_t tc_pack_floats(int N, int K);
 cudaError_t launch_pack_tf32_operands(const TcPackJobs& jobs, cudaStream_t s);
 cudaError_t launch_gemm_tc2(const TcGemmBatch& batch, int epi, unsigned long long* error, cudaStream_t s);
+// small networks: forward, backward and gradients fused (csrc/tj_sgd_small.cu)
+constexpr int SGD_FUSED_MAX_PARTS = 256;   // at most this many blocks, each with a partial gradient of its own
+bool sgd_fused_ok(int D, int H, int A, int value_head);
+int sgd_fused_stride(int D, int H);        // floats from one partial gradient to the next
+cudaError_t launch_sgd_fused(const SgdParams& p, float lr, const AdamParams* adam, float* loss_out, cudaStream_t s);
+size_t sgd_partial_floats(int max_rows);   // loss partials: one per 16 rows, or five per block of the fused kernel
+size_t sgd_grad_partial_floats(int max_rows, int D, int H);
 size_t sgd_scratch_floats(int max_rows, int D, int H);   // activations, deltas and 32 partial gradients of the blob
 int sgd_partial_count(int n);
 bool sgd_supported(int D, int H, int A);
-cudaError_t launch_sgd_step(const SgdParams& p, float lr, const AdamParams* adam /* nullable: plain SGD */, cudaStream_t s);
-int sgd_step_launches(const SgdParams& p);   // kernels one launch_sgd_step call launches (the path depends on the shape)
+cudaError_t launch_sgd_step(const SgdParams& p, float lr, const AdamParams* adam /* nullable: plain SGD */, float* loss_out /* nullable */,
+                            cudaStream_t s);
+int sgd_step_launches(const SgdParams& p, bool with_loss);   // kernels one launch_sgd_step call launches (the path depends on the shape)
 int ppo_step_launches(const SgdParams& p, bool with_stats);
 cudaError_t launch_ppo_step(const SgdParams& p, float lr, const AdamParams* adam, float* stats_out /* device [5], nullable */,
                             cudaStream_t s);

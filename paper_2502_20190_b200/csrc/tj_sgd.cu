@@ -860,14 +860,29 @@ __global__ void sgd_apply_adam_kernel(float* __restrict__ Cm, float* __restrict_
 
 }  // namespace
 
+size_t sgd_partial_floats(int max_rows) {
+  const size_t per16 = ((size_t)max_rows + SG_ROWS - 1) / SG_ROWS, fused = 5 * (size_t)SGD_FUSED_MAX_PARTS;
+  return (per16 > fused ? per16 : fused) + 8;
+}
+
+// the partial gradients: one per row range of the layered path, or one per block of the fused kernel
+size_t sgd_grad_partial_floats(int max_rows, int D, int H) {
+  const size_t blob = (size_t)H * D + H + (size_t)H * H + H + 17 * (size_t)H + 17 + 3;
+  size_t parts = SG_SPLITS;
+  if (sgd_fused_ok(D, H, 1, 0)) {
+    const size_t most = ((size_t)max_rows + 3) / 4;            // blocks of the fewest rows
+    parts = most < SG_SPLITS ? SG_SPLITS : (most > SGD_FUSED_MAX_PARTS ? SGD_FUSED_MAX_PARTS : most);
+  }
+  return parts * blob;
+}
+
 size_t sgd_scratch_floats(int max_rows, int D, int H) {
   const size_t rows = ((size_t)max_rows + SG_ROWS - 1) / SG_ROWS * SG_ROWS;
-  // h1, h2, dh1, dh2, g [rows][<= 16 actions + value], loss partials (1 + 5 per 16 rows), and per row range one partial
-  // gradient of the whole parameter blob (at most 16 actions and a value head); W2 transposed
-  const size_t blob = (size_t)H * D + H + (size_t)H * H + H + 17 * (size_t)H + 17;
+  // h1, h2, dh1, dh2, g [rows][<= 16 actions + value], loss partials, PPO's five per 16 rows, partial gradients of the whole
+  // parameter blob (at most 16 actions and a value head); W2 transposed
   // + split copies of W1 (x 2 networks), W2 (x 2) and W2^T for the tensor-core products
-  return 4 * rows * (size_t)H + rows * 17 + 6 * (rows / SG_ROWS) + 64 + (size_t)H * H + (size_t)SG_SPLITS * blob +
-         2 * tc_pack_floats(H, D) + 3 * tc_pack_floats(H, H) + 64;
+  return 4 * rows * (size_t)H + rows * 17 + sgd_partial_floats(max_rows) + 5 * (rows / SG_ROWS) + 64 + (size_t)H * H +
+         sgd_grad_partial_floats(max_rows, D, H) + 2 * tc_pack_floats(H, D) + 3 * tc_pack_floats(H, H) + 64;
 }
 
 int sgd_partial_count(int n) { return (n + SG_ROWS - 1) / SG_ROWS; }
@@ -987,11 +1002,17 @@ static int backward_launches(const SgdParams& p) {
   return (tc_gemm_ok(p.dh2, p.H, p.w2t, p.H, p.n, p.H, p.H) ? 3 : 2) + 2;
 }
 
-int sgd_step_launches(const SgdParams& p) { return (use_tiled(p) ? (use_tc2(p) ? 5 : 7) : 1) + backward_launches(p); }
+int sgd_step_launches(const SgdParams& p, bool with_loss) {
+  if (sgd_fused_ok(p.D, p.H, p.A, 0)) return 2;
+  return (use_tiled(p) ? (use_tc2(p) ? 5 : 7) : 1) + backward_launches(p) + (with_loss ? 1 : 0);
+}
 
-int ppo_step_launches(const SgdParams& p, bool with_stats) { return 1 + (with_stats ? 1 : 0) + backward_launches(p); }
+int ppo_step_launches(const SgdParams& p, bool with_stats) {
+  if (sgd_fused_ok(p.D, p.H, p.A, 1)) return 2;
+  return 1 + (with_stats ? 1 : 0) + backward_launches(p);
+}
 
-cudaError_t launch_sgd_step(const SgdParams& p, float lr, const AdamParams* adam, cudaStream_t s) {
+static cudaError_t sgd_step_layered(const SgdParams& p, float lr, const AdamParams* adam, cudaStream_t s) {
   if (use_tiled(p)) {
     const int n = p.n, D = p.D, H = p.H, A = p.A;
     const float *W1 = p.theta, *b1 = W1 + (size_t)H * D, *W2 = b1 + H, *b2 = W2 + (size_t)H * H, *W3 = b2 + H, *b3 = W3 + (size_t)A * H;
@@ -1050,7 +1071,15 @@ cudaError_t launch_sgd_step(const SgdParams& p, float lr, const AdamParams* adam
   return backward_and_update(p, lr, adam, s);
 }
 
+cudaError_t launch_sgd_step(const SgdParams& p, float lr, const AdamParams* adam, float* loss_out, cudaStream_t s) {
+  if (sgd_fused_ok(p.D, p.H, p.A, 0)) return launch_sgd_fused(p, lr, adam, loss_out, s);
+  cudaError_t e = sgd_step_layered(p, lr, adam, s);
+  if (e == cudaSuccess && loss_out) e = launch_td_finish(p.partial, sgd_partial_count(p.n), p.n, loss_out, s);
+  return e;
+}
+
 cudaError_t launch_ppo_step(const SgdParams& p, float lr, const AdamParams* adam, float* stats_out, cudaStream_t s) {
+  if (sgd_fused_ok(p.D, p.H, p.A, 1)) return launch_sgd_fused(p, lr, adam, stats_out, s);
   const size_t smem_f = (((size_t)p.D + 2 * (size_t)p.H + p.A + 1) * SG_ROWS + (size_t)SG_THREADS * (SG_KT + 1)) * sizeof(float);
   cudaError_t e;
   if ((e = launch_chained(ppo_forward_kernel, sgd_partial_count(p.n), SG_THREADS, smem_f, s, p)) != cudaSuccess) return e;
