@@ -510,14 +510,14 @@ int tj_actor_step(tj_ctx* x, int32_t n_steps, float* dbg_logits) {
       q.logits_in = x->logits_buf;
       q.dbg_logits = dbg_logits ? dbg_logits + (size_t)i * x->N * x->A : nullptr;
       LaunchScope scope(x, TJ_K_ENV, 1);
-      e = launch_actor(c.env_kind, q, x->stream);
+      e = launch_actor(c.env_kind, q, x->sm_count, x->stream);
     }
   } else if (x->use_split) {
     LaunchScope scope(x, TJ_K_ACTOR_FUSED, 1);
     e = launch_actor_split(c.env_kind, p, x->wsplit[x->active], x->wsplit_scale[x->active], x->sm_count, x->stream);
   } else {
     LaunchScope scope(x, TJ_K_ACTOR_FUSED, 1);
-    e = launch_actor(c.env_kind, p, x->stream);
+    e = launch_actor(c.env_kind, p, x->sm_count, x->stream);
   }
   if (e != cudaSuccess) return cuda_fail(x, e, "actor step");
   actor_launched(x);

@@ -256,7 +256,8 @@ cudaError_t launch_td_finish(const float* partial, int n_partial, int n, float* 
 cudaError_t launch_init_env(int env_kind, int N, int S_d, uint2 seed, float* state, int* ep_step, float* ep_return,
                             cudaStream_t s);
 cudaError_t launch_publish(const PublishParams& p, cudaStream_t s);
-cudaError_t launch_actor(int env_kind, const ActorParams& p, cudaStream_t s);
+cudaError_t launch_actor(int env_kind, const ActorParams& p, int sm_count, cudaStream_t s);
+cudaError_t launch_actor_fma(int env_kind, const ActorParams& p, int sm_count, cudaStream_t s);   // CartPole / Acrobot on the FP32 pipes
 cudaError_t launch_sample_gather(const SampleParams& p, cudaStream_t s);
 cudaError_t launch_td(const TdParams& p, cudaStream_t s);
 int td_grid(int n);

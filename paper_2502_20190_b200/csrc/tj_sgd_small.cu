@@ -10,6 +10,7 @@
 // has fewer 4 x 4 output tiles than threads the contraction is split over the idle ones.
 // Gradients leave as one partial per block, laid out like the parameter blob; the apply kernel adds them in a fixed order.
 #include "tj_async.cuh"
+#include "tj_fma.cuh"
 #include "tj_internal.h"
 
 namespace tj {
@@ -19,21 +20,6 @@ namespace {
 constexpr int FS_NT = 512;
 constexpr int FS_MAX_H = 128;
 constexpr int FS_MAX_PARTS = SGD_FUSED_MAX_PARTS;
-
-typedef unsigned long long f32x2;
-
-__device__ __forceinline__ void fma2(f32x2& acc, f32x2 a, f32x2 b) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b)); }
-__device__ __forceinline__ f32x2 dup2(float x) {
-  f32x2 d;
-  asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(x));
-  return d;
-}
-__device__ __forceinline__ float2 halves(f32x2 v) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-  return r;
-}
-__device__ __forceinline__ ulonglong2 ld_pairs(const float* p) { return *reinterpret_cast<const ulonglong2*>(p); }
 
 // row strides: a multiple of four floats, odd in 16-byte units, so that eight lanes on consecutive rows touch all banks
 __host__ __device__ inline int fs_ld(int k) {
