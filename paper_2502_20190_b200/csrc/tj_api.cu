@@ -662,7 +662,7 @@ int tj_td_error(tj_ctx* x, const tj_batch* b, float* td_out, float* huber_out, f
     return TJ_OK;
   }
   LaunchScope scope(x, TJ_K_TD, loss_mean_out ? 2 : 1, true, true);
-  e = launch_td(p, x->lstream);
+  e = launch_td(p, x->sm_count, x->lstream);
   if (e != cudaSuccess) return cuda_fail(x, e, "TD error");
   learner_launched(x);
   return TJ_OK;
@@ -680,7 +680,7 @@ int tj_td_error_static(tj_ctx* x, const tj_batch* b, float* td_out, float* huber
   const TdParams p = td_params(x, b, td_out, huber_out, loss_mean_out, nullptr);
   bool too_large = false;
   LaunchScope scope(x, TJ_K_TD, loss_mean_out ? 2 : 1, /*may_create=*/false, true);
-  cudaError_t e = launch_td_static(p, x->cfg.device, x->lstream, &too_large);
+  cudaError_t e = launch_td_static(p, x->cfg.device, x->sm_count, x->lstream, &too_large);
   if (too_large) return fail(x, TJ_ERR_INVALID_ARG, "tj_td_error_static: batch too large for the library's scratch");
   if (e == cudaErrorInvalidDevice) return fail(x, TJ_ERR_INVALID_ARG, "tj_td_error_static: the context's device must be the current device");
   if (e != cudaSuccess) return cuda_fail(x, e, "TD error (library scratch)");

@@ -259,7 +259,8 @@ cudaError_t launch_publish(const PublishParams& p, cudaStream_t s);
 cudaError_t launch_actor(int env_kind, const ActorParams& p, int sm_count, cudaStream_t s);
 cudaError_t launch_actor_fma(int env_kind, const ActorParams& p, int sm_count, cudaStream_t s);   // CartPole / Acrobot on the FP32 pipes
 cudaError_t launch_sample_gather(const SampleParams& p, cudaStream_t s);
-cudaError_t launch_td(const TdParams& p, cudaStream_t s);
+cudaError_t launch_td(const TdParams& p, int sm_count, cudaStream_t s);
+cudaError_t launch_td_fma(const TdParams& p, int sm_count, int* grid_out, cudaStream_t s);
 int td_grid(int n);
 constexpr int SG_SPLITS = 32;     // at most this many row ranges per gradient product (partial sums go through scratch)
 // tensor-core products of the update (csrc/tj_sgd_tc.cu): C = epilogue(A B^T), B split and laid out once per update
@@ -303,7 +304,7 @@ int ppo_step_launches(const SgdParams& p, bool with_stats);
 cudaError_t launch_ppo_step(const SgdParams& p, float lr, const AdamParams* adam, float* stats_out /* device [5], nullable */,
                             cudaStream_t s);
 int td_static_max_rows();
-cudaError_t launch_td_static(const TdParams& p, int device, cudaStream_t s, bool* too_large);
+cudaError_t launch_td_static(const TdParams& p, int device, int sm_count, cudaStream_t s, bool* too_large);
 cudaError_t launch_gae(const float* rew, const float* val, const uint8_t* done, int T, int N, float gamma, float lambda,
                        float* adv, float* ret, cudaStream_t s);
 int shuffle_half_bits(long long R);

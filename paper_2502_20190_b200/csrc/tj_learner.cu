@@ -187,30 +187,24 @@ __global__ void __launch_bounds__(NT) td_kernel(const TdParams p) {
   }
 }
 
-// fixed-order sum of the per-block partial losses: one warp fetches 16 x 32 partials with independent coalesced loads
-// (a single thread walking the array pays one memory latency per element, a warp fetching one chunk per iteration one per
-// chunk), then lane 0 adds them in index order -- the same sum, term by term
-__global__ void td_finish_kernel(const float* __restrict__ partial, int n_partial, int n, float* __restrict__ loss_out) {
+// Fixed-order sum of the per-block partial losses: thread i adds partials i, i + 256, ... (independent loads), then a tree.  One block,
+// bound by one memory latency (a warp that added them in index order, one shuffle each, took 6-8 us for 512 partials).
+__global__ void __launch_bounds__(256) td_finish_kernel(const float* __restrict__ partial, int n_partial, int n, float* __restrict__ loss_out) {
+  __shared__ float ws[8];
   chain_begin();
   chain_next();
-  if (blockIdx.x != 0 || threadIdx.x >= 32) return;
-  const int lane = threadIdx.x;
-  float sum = 0.f;
-  for (int base = 0; base < n_partial; base += 16 * 32) {
-    float mine[16];
+  float s = 0.f;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < n_partial; i += 256) s += __ldcg(partial + i);
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    s = 0.f;
 #pragma unroll
-    for (int c = 0; c < 16; ++c) {
-      const int i = base + c * 32 + lane;
-      mine[c] = i < n_partial ? partial[i] : 0.f;
-    }
-#pragma unroll
-    for (int c = 0; c < 16; ++c) {
-      const int left = n_partial - (base + c * 32);
-      const int cnt = left < 0 ? 0 : (left < 32 ? left : 32);
-      for (int l = 0; l < cnt; ++l) sum += __shfl_sync(0xffffffffu, mine[c], l);
-    }
+    for (int w = 0; w < 8; ++w) s += ws[w];
+    *loss_out = s / (float)n;
   }
-  if (lane == 0) *loss_out = sum / (float)n;
 }
 
 // GAE: one thread per environment walks its column backwards; a warp reads 32 consecutive environments, so
@@ -316,9 +310,11 @@ cudaError_t launch_td_tile(const TdParams& p, cudaStream_t s, int* grid_out) {
   return cudaErrorInvalidConfiguration;
 }
 
-cudaError_t launch_td(const TdParams& p, cudaStream_t s) {
+cudaError_t launch_td(const TdParams& p, int sm_count, cudaStream_t s) {
   int grid = 0;
-  cudaError_t err = p.H >= 192 ? launch_td_tile<32, 128, 8, 8>(p, s, &grid) : launch_td_tile<kTdTile, kTdThreads, 4, 4>(p, s, &grid);
+  cudaError_t err = launch_td_fma(p, sm_count, &grid, s);
+  if (err == cudaSuccess && grid == 0)     // more outputs or parameters than that kernel holds
+    err = p.H >= 192 ? launch_td_tile<32, 128, 8, 8>(p, s, &grid) : launch_td_tile<kTdTile, kTdThreads, 4, 4>(p, s, &grid);
   if (err != cudaSuccess) return err;
   if (p.loss_out) {
     err = launch_td_finish(p.partial, grid, p.n, p.loss_out, s);
@@ -333,7 +329,7 @@ static __device__ __align__(256) float g_td_static_partial[kStaticTdPartials];
 
 int td_static_max_rows() { return 65536; }
 
-cudaError_t launch_td_static(const TdParams& p_in, int device, cudaStream_t s, bool* too_large) {
+cudaError_t launch_td_static(const TdParams& p_in, int device, int sm_count, cudaStream_t s, bool* too_large) {
   *too_large = p_in.n > td_static_max_rows() || td_grid(p_in.n) > kStaticTdPartials;
   if (*too_large) return cudaSuccess;
   // In host code the array's name is only a stand-in; the device address has to be asked for, once per device, with
@@ -358,11 +354,11 @@ cudaError_t launch_td_static(const TdParams& p_in, int device, cudaStream_t s, b
   }
   TdParams p = p_in;
   p.partial = scratch;
-  return launch_td(p, s);
+  return launch_td(p, sm_count, s);
 }
 
 cudaError_t launch_td_finish(const float* partial, int n_partial, int n, float* loss_out, cudaStream_t s) {
-  return launch_chained(td_finish_kernel, 1, 32, 0, s, partial, n_partial, n, loss_out);
+  return launch_chained(td_finish_kernel, 1, 256, 0, s, partial, n_partial, n, loss_out);
 }
 
 cudaError_t launch_gae(const float* rew, const float* val, const uint8_t* done, int T, int N, float gamma, float lambda,
