@@ -76,6 +76,12 @@ __device__ __forceinline__ float cluster_load_f32(const float* p, uint32_t rank)
   return v;
 }
 
+__device__ __forceinline__ void cluster_store_f32(float* p, uint32_t rank, float v) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr(p)), "r"(rank));
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+
 // One thread queues `bytes` (multiple of 16) in chunks; the barrier must expect the same total.
 __device__ __forceinline__ void bulk_copy_chunks(void* dst, const void* src, size_t bytes, uint64_t* bar) {
   constexpr size_t kChunk = 16384;

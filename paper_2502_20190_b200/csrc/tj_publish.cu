@@ -29,14 +29,15 @@ __device__ __forceinline__ size_t core_offset(int row, int k, int kc) {
   return ((size_t)(row >> 3) * (kc >> 3) + (k >> 3)) * 64 + (size_t)(row & 7) * 8;
 }
 
-// NT threads; SPLIT: split-operand context, launched as clusters of eight blocks.  Cluster 0 owns W2: its blocks first agree
-// on the largest |entry| (each scans an eighth; a scan of the whole matrix by every block took 14 us), then pack.
+// NT threads; SPLIT: split-operand context, launched as clusters of eight blocks.  Cluster 0 owns W2: each of its blocks
+// reads an eighth into shared memory, they agree on the largest |entry| (a scan of the whole matrix by every block took 14 us), then
+// pack what they hold (7.3 us with a second read of it).
 template <int NT, bool SPLIT>
 __global__ void __launch_bounds__(NT) publish_kernel(const PublishParams p) {
   chain_begin();
   chain_next();
   constexpr int KT = NT / 8;                      // inputs per tile
-  __shared__ float tile[32][KT + 1];
+  extern __shared__ float pub_sm[];               // one tile [32][KT + 1], or a cluster-0 block's tiles of W2
   __shared__ float red[NT / 32];
   __shared__ float cluster_max;
   const int D = p.L.D, H = p.L.H, A = p.L.A, Hp = p.L.Hp, Ap = p.L.Ap, tid = threadIdx.x;
@@ -51,16 +52,22 @@ __global__ void __launch_bounds__(NT) publish_kernel(const PublishParams p) {
   const int row_tiles = (Hp + 31) / 32, k_tiles1 = (D + KT - 1) / KT, k_tiles2 = (H + KT - 1) / KT;
   const int n1 = row_tiles * k_tiles1, n2 = row_tiles * k_tiles2;
 
-  // one tile of W (H x K): load, then one write per layout
-  auto do_tile = [&](const float* W, int K, int t, float* dst, int layer, float split_scale) {
+  // tile t of W (H x K) -> shared memory; returns this thread's largest |entry|
+  auto load_tile = [&](float (*tile)[KT + 1], const float* W, int K, int t) {
     const int n0 = (t % row_tiles) * 32, k0 = (t / row_tiles) * KT;
-    __syncthreads();
+    float m = 0.f;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int r = tid / KT + i * 8, c = tid % KT;
-      tile[r][c] = n0 + r < H && k0 + c < K ? W[(size_t)(n0 + r) * K + k0 + c] : 0.f;
+      const float v = n0 + r < H && k0 + c < K ? W[(size_t)(n0 + r) * K + k0 + c] : 0.f;
+      tile[r][c] = v;
+      m = fmaxf(m, fabsf(v));
     }
-    __syncthreads();
+    return m;
+  };
+  // the tile in shared memory -> every layout
+  auto write_tile = [&](const float (*tile)[KT + 1], int K, int t, float* dst, int layer, float split_scale) {
+    const int n0 = (t % row_tiles) * 32, k0 = (t / row_tiles) * KT;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int n = n0 + (tid & 31), k = k0 + (tid >> 5) + i * (NT / 32);
@@ -105,11 +112,12 @@ __global__ void __launch_bounds__(NT) publish_kernel(const PublishParams p) {
     }
   };
 
+  float (*tile)[KT + 1] = reinterpret_cast<float (*)[KT + 1]>(pub_sm);
   int job = blockIdx.x;
   if (SPLIT) {
-    if (job < 8) {                                 // cluster 0: the hidden x hidden matrix
+    if (job < 8) {                                 // cluster 0: the hidden x hidden matrix, every block's share read once
       float m = 0.f;
-      for (int i = job * NT + tid; i < H * H; i += 8 * NT) m = fmaxf(m, fabsf(W2[i]));
+      for (int t = job, i = 0; t < n2; t += 8, ++i) m = fmaxf(m, load_tile(tile + 32 * i, W2, H, t));
       for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
       if ((tid & 31) == 0) red[tid >> 5] = m;
       __syncthreads();
@@ -135,18 +143,19 @@ __global__ void __launch_bounds__(NT) publish_kernel(const PublishParams p) {
         p.split_scale[0] = sc;
         p.split_scale[1] = 1.0f / (sc * p.split_h_scale);
       }
-      for (int t = job; t < n2; t += 8) do_tile(W2, H, t, p.dst + p.L.off_W2t, 1, sc);
+      for (int t = job, i = 0; t < n2; t += 8, ++i) write_tile(tile + 32 * i, H, t, p.dst + p.L.off_W2t, 1, sc);
       return;
     }
     job -= 8;
-    if (job < n1) { do_tile(W1, D, job, p.dst + p.L.off_W1t, 0, 0.f); return; }
-    job -= n1;
-  } else {
-    if (job < n1) { do_tile(W1, D, job, p.dst + p.L.off_W1t, 0, 0.f); return; }
-    job -= n1;
-    if (job < n2) { do_tile(W2, H, job, p.dst + p.L.off_W2t, 1, 0.f); return; }
-    job -= n2;
   }
+  if (job < n1 || (!SPLIT && job < n1 + n2)) {
+    const int layer = job < n1 ? 0 : 1, t = job - layer * n1, K = layer ? H : D;
+    load_tile(tile, layer ? W2 : W1, K, t);
+    __syncthreads();
+    write_tile(tile, K, t, p.dst + (layer ? p.L.off_W2t : p.L.off_W1t), layer, 0.f);
+    return;
+  }
+  job -= n1 + (SPLIT ? 0 : n2);
   // biases and the head, element by element
   int i = job * NT + tid;
   if (i < 2 * Hp) {
@@ -185,7 +194,11 @@ cudaError_t launch_publish(const PublishParams& p, cudaStream_t s) {
   const int NT = split ? 1024 : 256, KT = NT / 8, row_tiles = (L.Hp + 31) / 32;
   const int n1 = row_tiles * ((L.D + KT - 1) / KT), n2 = row_tiles * ((L.H + KT - 1) / KT);
   const int rest = 2 * L.Hp + L.H * L.Ap + L.Ap + (p.tc ? 16 * L.H : 0), n_rest = (rest + NT - 1) / NT;
-  if (!split) return launch_chained(publish_kernel<256, false>, n1 + n2 + n_rest, 256, 0, s, p);
+  const size_t tile_bytes = (size_t)32 * (KT + 1) * sizeof(float);
+  if (!split) return launch_chained(publish_kernel<256, false>, n1 + n2 + n_rest, 256, tile_bytes, s, p);
+  const size_t smem = tile_bytes * ((n2 + 7) / 8);
+  const cudaError_t e = cudaFuncSetAttribute(publish_kernel<1024, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute at[2];
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -194,6 +207,7 @@ cudaError_t launch_publish(const PublishParams& p, cudaStream_t s) {
   at[0].val.clusterDim.x = 8; at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
   cfg.gridDim = dim3((8 + n1 + n_rest + 7) / 8 * 8);
   cfg.blockDim = dim3(1024);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cfg.attrs = at;
   cfg.numAttrs = 2;

@@ -5,16 +5,17 @@
 // with FP32 accumulation in tensor memory (error about 2^-22 per term, the dropped lo x lo term; FP16 runs at twice the rate
 // of the 3 x TF32 form of the same idea).  Layer 1 (4 or 6 inputs) and the head (2-4 outputs) stay on the FP32 pipes.
 //
-// One thread block keeps a tile of 128 environments for all n_steps of the call (environments are independent): thread e
-// owns env e's state in registers.  Eight worker warps, one MMA-issuing warp, one copy warp; per step:
-//   observation -> shared memory;
+// One thread block keeps its tiles of 128 environments for all n_steps of the call (environments are independent): eight worker
+// warps, one MMA-issuing warp, one copy warp; per step and tile:
 //   workers: layer 1 in the fixed FMA order of the FP32 path, ReLU, split -> FP16 A operand, 32 hidden units (one K chunk of
 //     the next layer) at a time, each chunk handed to the issuing lane through its own mbarrier;
 //   copy lane: streams W2's parts in 32-column chunks (bulk copies, four ring slots, the stream running on across steps);
 //   issuing lane: per K chunk, issues W_hi x (h_hi, h_lo) and W_lo x h_hi (M = 128, N = H) as soon as that chunk of h1 exists, so
 //     the tensor pipe works underneath layer 1;
-//   workers: accumulator -> + b2, ReLU, head partial sums by two threads per row -> outputs;
+//   workers: accumulator -> + b2, ReLU, head sums in column order -> outputs;
 //   then exactly the FP32 kernel's selection, env step, record / segment write and reset.
+// The FP32 work per step (layer 1 with its split, drain, env step: about 14,000 warp instructions a tile) and the MMAs (6,100 cycles at
+// hidden 256) are of one size; what a step takes beyond them is latency.
 // Every wait is bounded; a timeout latches the context's error word and the block leaves after freeing its tensor memory.
 #include <cuda_fp16.h>
 
@@ -28,22 +29,9 @@ namespace tj {
 namespace {
 
 constexpr int SA_TE = 128;            // envs per tile = rows of the MMA
-constexpr int SA_WORKERS = 256;       // threads of the worker warps; one more warp issues
-constexpr int SA_NT = SA_WORKERS + 64;   // + the MMA-issuing warp and the copy warp
 constexpr int SA_KC = 32;             // K columns per streamed chunk of W2
 constexpr int SA_SLOTS = 4;
-constexpr int SA_MAX_KC = 256 / SA_KC;
 constexpr float SA_H_SCALE = 16.0f;   // hidden activations are split after this scaling (|h1| < 4,094 stays inside FP16)
-
-struct SaCtl {
-  uint64_t full[SA_SLOTS], empty[SA_SLOTS];
-  uint64_t a_ready[SA_MAX_KC];   // K chunk of the A operand written (one arrival per worker warp)
-  uint64_t wbar;                 // small parameters staged
-  uint64_t acc_full;             // all MMAs of a forward pass complete
-  uint32_t tmem_base;
-  int abort_flag;
-  int range_flag;               // a scaled hidden activation left FP16's range: the outputs of that pass are meaningless
-};
 
 __device__ __forceinline__ float4 sa_reset4(uint2 seed, uint32_t e, unsigned long long step, float lo, float width) {
   const uint4 w = stream_words(seed, STREAM_RESET, 0, e, step);
@@ -63,156 +51,6 @@ __device__ __forceinline__ void sa_observe(float4 s, float* obs) {
   }
 }
 
-struct SaShared {
-  uint8_t *a_hi, *a_lo, *ring;
-  float *xs, *out, *part;
-  SaCtl* ctl;
-};
-
-// eight hidden units n0 .. n0+7 of layer 1 for one env, in the canonical order (bias, then inputs in index order), ReLU,
-// scaling, split; one 16-byte row segment of each part of the A operand
-template <int D>
-__device__ __forceinline__ float sa_layer1_block(const MlpWeights& mw, int Hp, const float* x, int n0, uint8_t* a_hi, uint8_t* a_lo, size_t off) {
-  float acc[8];
-  const float4 b0 = *reinterpret_cast<const float4*>(mw.b1 + n0), b1 = *reinterpret_cast<const float4*>(mw.b1 + n0 + 4);
-  acc[0] = b0.x; acc[1] = b0.y; acc[2] = b0.z; acc[3] = b0.w; acc[4] = b1.x; acc[5] = b1.y; acc[6] = b1.z; acc[7] = b1.w;
-#pragma unroll
-  for (int k = 0; k < D; ++k) {
-    const float4 w0 = *reinterpret_cast<const float4*>(mw.W1t + (size_t)k * Hp + n0);
-    const float4 w1 = *reinterpret_cast<const float4*>(mw.W1t + (size_t)k * Hp + n0 + 4);
-    acc[0] = fmaf(w0.x, x[k], acc[0]); acc[1] = fmaf(w0.y, x[k], acc[1]); acc[2] = fmaf(w0.z, x[k], acc[2]); acc[3] = fmaf(w0.w, x[k], acc[3]);
-    acc[4] = fmaf(w1.x, x[k], acc[4]); acc[5] = fmaf(w1.y, x[k], acc[5]); acc[6] = fmaf(w1.z, x[k], acc[6]); acc[7] = fmaf(w1.w, x[k], acc[7]);
-  }
-  uint32_t hi2[4], lo2[4];
-  float vmax = 0.f;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float v0 = fmaxf(acc[2 * i], 0.f) * SA_H_SCALE, v1 = fmaxf(acc[2 * i + 1], 0.f) * SA_H_SCALE;
-    vmax = fmaxf(vmax, fmaxf(v0, v1));
-    const float h0 = __uint_as_float(__float_as_uint(v0) & 0xFFFFE000u), h1 = __uint_as_float(__float_as_uint(v1) & 0xFFFFE000u);
-    hi2[i] = pack_f16x2(h0, h1);
-    lo2[i] = pack_f16x2(v0 - h0, v1 - h1);
-  }
-  *reinterpret_cast<uint4*>(a_hi + off) = make_uint4(hi2[0], hi2[1], hi2[2], hi2[3]);
-  *reinterpret_cast<uint4*>(a_lo + off) = make_uint4(lo2[0], lo2[1], lo2[2], lo2[3]);
-  return vmax;
-}
-
-// Network outputs of the observations in xs -> out[i][e], i < Aout.  Called by every thread of the block; `pass` counts the
-// calls, `copied` is the copy lane's position in the chunk stream: pass q reads the split matrix parts[q & 1] (the actor
-// passes the same matrix twice, the TD kernel the online and the target network's).  Returns false after a timeout.
-template <int D, int H>
-__device__ __forceinline__ bool sa_forward(int Hp, int Aout, const MlpWeights& mw, const SaShared& sh, const uint16_t* parts0,
-                                           const uint16_t* parts1, float inv_scale, uint32_t tmem, uint32_t pass, uint32_t& copied,
-                                           volatile int* abort_flag) {
-  constexpr int NKC = H / SA_KC;                 // K chunks of the hidden x hidden layer
-  constexpr uint32_t NSTREAM = 2 * NKC;          // chunks of W2 per pass: (high, low) per K chunk
-  constexpr uint32_t CHUNK_BYTES = H * SA_KC * 2;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  SaCtl* ctl = sh.ctl;
-  if (tid < SA_WORKERS) {
-    const int e = tid & (SA_TE - 1), half = tid >> 7;
-    float x[D];
-#pragma unroll
-    for (int k = 0; k < D; ++k) x[k] = sh.xs[k * SA_TE + e];
-    tc_fence_before();                            // this thread's accumulator reads of the previous pass are complete
-    float vmax = 0.f;
-#pragma unroll 1
-    for (int kc = 0; kc < NKC; ++kc) {
-#pragma unroll
-      for (int b = 0; b < 2; ++b) {
-        const int n0 = kc * SA_KC + half * 16 + b * 8;
-        const size_t off = ((size_t)(e >> 3) * (H / 8) + (n0 >> 3)) * 128 + (e & 7) * 16;
-        vmax = fmaxf(vmax, sa_layer1_block<D>(mw, Hp, x, n0, sh.a_hi, sh.a_lo, off));
-      }
-      fence_async_smem();
-      mbar_arrive_warp(&ctl->a_ready[kc]);
-    }
-    // 65,504 is FP16's largest finite value (a NaN activation also lands here: the comparison is written to catch it)
-    if (!(vmax <= 65504.f)) ctl->range_flag = 1;
-  } else if (warp == SA_WORKERS / 32) {
-    // The issuing lane's warp-mates wait at the warp barrier, not in a polling loop: lanes of one warp that poll while
-    // another lane of it issues take turns with that lane, and every blocked poll then stalls the issue.
-    if (lane == 0) {
-      // The stream position at the start of a pass is pass x NSTREAM, a multiple of the slot count: chunk c of any pass sits
-      // in slot c % SLOTS, and only the barrier parities depend on the pass.
-      const uint32_t idesc = make_idesc_f16(H);
-      const uint32_t ahi_lo = desc_lo(smem_addr(sh.a_hi), 128u), alo_lo = desc_lo(smem_addr(sh.a_lo), 128u);
-      const uint32_t a_hiword = desc_hi((uint32_t)(H / 8) * 128u), b_hiword = desc_hi((uint32_t)(SA_KC / 8) * 128u);
-      const uint32_t ring_lo = desc_lo(smem_addr(sh.ring), 128u);
-      const uint32_t round0 = pass * (NSTREAM / SA_SLOTS);           // trips around the ring before this pass
-      bool alive = true;
-#pragma unroll
-      for (int kc = 0; kc < NKC; ++kc) {
-        if (!alive) break;
-        if (!tc_wait(&ctl->a_ready[kc], pass & 1, abort_flag)) { alive = false; break; }
-        tc_fence_after();
-        const uint32_t a_off = (uint32_t)kc * (SA_KC / 8) * 8u;     // in 16-byte units: 8 per core matrix, 4 core matrices per chunk
-#pragma unroll
-        for (int part = 0; part < 2; ++part) {
-          const int c = 2 * kc + part, s = c % SA_SLOTS;
-          if (!tc_wait(&ctl->full[s], (round0 + c / SA_SLOTS) & 1, abort_flag)) { alive = false; break; }
-          tc_fence_after();
-          const uint32_t b_lo = ring_lo + (uint32_t)s * (CHUNK_BYTES / 16);
-#pragma unroll
-          for (int j = 0; j < SA_KC / 16; ++j) {
-            umma_ss(tmem, ahi_lo + a_off + 16u * j, a_hiword, b_lo + 16u * j, b_hiword, idesc, (c | j) != 0);
-            if (part == 0) umma_ss(tmem, alo_lo + a_off + 16u * j, a_hiword, b_lo + 16u * j, b_hiword, idesc, 1u);
-          }
-          umma_commit(&ctl->empty[s]);
-        }
-      }
-      umma_commit(&ctl->acc_full);
-    }
-    __syncwarp();
-  } else {
-    // copy lane: keeps the ring full -- chunk g of the stream follows chunk g - SLOTS into its slot once that one is consumed
-    if (lane == 0) {
-#pragma unroll 1
-      for (uint32_t c = 0; c < NSTREAM; ++c, ++copied) {
-        const uint32_t sp = copied % SA_SLOTS;
-        if (!tc_wait(&ctl->empty[sp], ((copied / SA_SLOTS) - 1) & 1, abort_flag)) break;
-        mbar_expect_tx(&ctl->full[sp], CHUNK_BYTES);
-        const uint16_t* src = ((copied / NSTREAM) & 1u) ? parts1 : parts0;
-        bulk_copy_g2s(sh.ring + (size_t)sp * CHUNK_BYTES, reinterpret_cast<const uint8_t*>(src) + (size_t)(copied % NSTREAM) * CHUNK_BYTES,
-                      CHUNK_BYTES, &ctl->full[sp]);
-      }
-    }
-    __syncwarp();
-  }
-  // after a timeout the abort flag is up: the pass runs to its end on meaningless numbers (every thread keeps to the same
-  // barriers) and the caller leaves
-  tc_wait_elect(&ctl->acc_full, pass & 1, abort_flag);
-  tc_fence_after();
-  // drain: two threads per row (the two column halves); h2 = relu(acc / scale + b2), head partial sums in column order
-  if (tid < SA_WORKERS) {
-    const int q = warp & 3, half = warp >> 2, r = q * 32 + lane;
-    float pa[4] = {0.f, 0.f, 0.f, 0.f};
-    const uint32_t t_row = tmem + ((uint32_t)(q * 32) << 16);
-#pragma unroll 2
-    for (int c0 = half * (H / 2); c0 < (half + 1) * (H / 2); c0 += 16) {
-      uint32_t v[16];
-      tmem_ld16(t_row + (uint32_t)c0, v);
-      tmem_ld_wait();
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const float h2 = fmaxf(fmaf(__uint_as_float(v[i]), inv_scale, mw.b2[c0 + i]), 0.f);
-        const float4 w = *reinterpret_cast<const float4*>(mw.W3t + (size_t)(c0 + i) * 4);   // a row of W3t (Ap = 4)
-        pa[0] = fmaf(w.x, h2, pa[0]); pa[1] = fmaf(w.y, h2, pa[1]); pa[2] = fmaf(w.z, h2, pa[2]); pa[3] = fmaf(w.w, h2, pa[3]);
-      }
-    }
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-      if (a < Aout) sh.part[((size_t)half * 4 + a) * SA_TE + r] = pa[a];
-  }
-  __syncthreads();
-  if (tid < SA_TE)
-    for (int a = 0; a < Aout; ++a)
-      sh.out[a * SA_TE + tid] = (mw.b3[a] + sh.part[(size_t)a * SA_TE + tid]) + sh.part[((size_t)4 + a) * SA_TE + tid];
-  __syncthreads();
-  return *abort_flag == 0;
-}
-
 // ------------------------------------------------------------------------------------------------------------------------
 // The actor.  A thread owns an environment for the whole call: observation, layer 1, head sums, selection and environment step stay
 // in its registers, so the workers meet nobody but the issuing lane.  TPR threads per environment:
@@ -220,8 +58,11 @@ __device__ __forceinline__ bool sa_forward(int Hp, int Aout, const MlpWeights& m
 //      compute layer 1 (calls with more tiles than SMs);
 //   2  eight warps on one tile: each thread takes half the neurons and half the columns of the drain, the two exchange their head
 //      sums once per step and both step the environment (one tile per SM: the chain of one step is the bound).
+// With two tiles in flight shared memory is the bound: the MMAs read 96 of its 128 bytes per cycle while they run (40 % of the time) and
+// the broadcast weights and the A operand take another 53 %.  65,536 CartPole envs, hidden 256, 128 steps: 3.71 ms (one tile at a time
+// 5.16; two threads per env and two tiles, 18 warps: 4.19).
 // Layer 1 hands 32 hidden units (one K chunk) at a time to the issuing lane through a ring of A-operand slots.
-constexpr int S2_NT = 320;                // eight worker warps, the issuing warp, the copy warp
+constexpr int S2_NT = 320;                // eight worker warps on one tile, the issuing warp, the copy warp
 constexpr int S2_A_SLOTS = 8;             // A-operand slots of a block, 16 KB each: four per group, or eight for the one tile
 constexpr int S2_A_PART = SA_TE * SA_KC * 2;
 constexpr int S2_A_SLOT = 2 * S2_A_PART;  // high part, low part
@@ -247,23 +88,27 @@ __device__ __forceinline__ f32x2 pair2(float a, float b) {
   return d;
 }
 
-// eight hidden units n0 .. n0 + 7 of layer 1 in the canonical order (bias, then inputs in index order; weights and biases come scaled by
-// SA_H_SCALE, a power of two, which leaves every rounding where it was), ReLU, split; returns the largest scaled activation
-template <int D, int H>
-__device__ __forceinline__ float s2_layer1_block(const float* w1, const float* b1, const f32x2 (&x)[D], int n0, uint8_t* hi_dst, uint8_t* lo_dst, float vmax) {
-  f32x2 acc[4];
-  {
-    const ulonglong2 b0 = ld_pairs(b1 + n0), b4 = ld_pairs(b1 + n0 + 4);
-    acc[0] = b0.x; acc[1] = b0.y; acc[2] = b4.x; acc[3] = b4.y;
+// 8 NB hidden units from n0 of layer 1 in the canonical order (bias, then inputs in index order; weights and biases come scaled by
+// SA_H_SCALE, a power of two, which leaves every rounding where it was), ReLU, split -> NB 16-byte row segments of each part of the A
+// operand; returns the largest scaled activation.  All units are computed before the first store: a store orders the loads after it.
+template <int D, int H, int NB>
+__device__ __forceinline__ float s2_layer1(const float* w1, const float* b1, const f32x2 (&x)[D], int n0, uint8_t* hi_dst, float vmax) {
+  f32x2 acc[4 * NB];
+#pragma unroll
+  for (int i = 0; i < 2 * NB; ++i) {
+    const ulonglong2 b = ld_pairs(b1 + n0 + 4 * i);
+    acc[2 * i] = b.x; acc[2 * i + 1] = b.y;
   }
 #pragma unroll
-  for (int k = 0; k < D; ++k) {
-    const ulonglong2 w0 = ld_pairs(w1 + k * H + n0), w4 = ld_pairs(w1 + k * H + n0 + 4);
-    fma2(acc[0], w0.x, x[k]); fma2(acc[1], w0.y, x[k]); fma2(acc[2], w4.x, x[k]); fma2(acc[3], w4.y, x[k]);
-  }
-  uint32_t hi[4], lo[4];
+  for (int k = 0; k < D; ++k)
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < 2 * NB; ++i) {
+      const ulonglong2 w = ld_pairs(w1 + k * H + n0 + 4 * i);
+      fma2(acc[2 * i], w.x, x[k]); fma2(acc[2 * i + 1], w.y, x[k]);
+    }
+  uint32_t hi[4 * NB], lo[4 * NB];
+#pragma unroll
+  for (int i = 0; i < 4 * NB; ++i) {
     const float2 a = halves(acc[i]);
     const float v0 = fmaxf(a.x, 0.f), v1 = fmaxf(a.y, 0.f);
     vmax = fmaxf(vmax, fmaxf(a.x, a.y));
@@ -271,163 +116,200 @@ __device__ __forceinline__ float s2_layer1_block(const float* w1, const float* b
     hi[i] = pack_f16x2(h0, h1);
     lo[i] = pack_f16x2(v0 - h0, v1 - h1);
   }
-  *reinterpret_cast<uint4*>(hi_dst) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-  *reinterpret_cast<uint4*>(lo_dst) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    *reinterpret_cast<uint4*>(hi_dst + b * 128) = make_uint4(hi[4 * b], hi[4 * b + 1], hi[4 * b + 2], hi[4 * b + 3]);
+    *reinterpret_cast<uint4*>(hi_dst + S2_A_PART + b * 128) = make_uint4(lo[4 * b], lo[4 * b + 1], lo[4 * b + 2], lo[4 * b + 3]);
+  }
   return vmax;
 }
 
-template <int ENV, int H, int TPR>
-__global__ void __launch_bounds__(S2_NT, 1) actor_split_tc_kernel(const ActorParams p, const S2Plan pl, const uint16_t* __restrict__ w2parts,
-                                                                 const float* __restrict__ w2scale) {
-  extern __shared__ __align__(1024) uint8_t smem_raw[];
-  constexpr int D = ENV == TJ_ENV_CARTPOLE ? 4 : 6;
-  constexpr uint32_t CHUNK_BYTES = H * SA_KC * 2;             // one chunk of one part of W2
-  constexpr int NKC = H / SA_KC, NSTREAM = 2 * NKC;
-  constexpr int GROUPS = 3 - TPR, AS = S2_A_SLOTS / GROUPS;   // tiles in flight; A slots of each
-  constexpr uint32_t ACC_COLS = H <= 128 ? 128 : 256;
-  uint8_t* a_ring = smem_raw;
-  uint8_t* w_ring = a_ring + S2_A_SLOTS * S2_A_SLOT;
-  float* w1 = reinterpret_cast<float*>(w_ring + SA_SLOTS * CHUNK_BYTES);   // [D][H], scaled
-  float* b1 = w1 + D * H;                                     // [H], scaled
-  float* b2 = b1 + H;                                         // [H]
-  float* w3 = b2 + H;                                         // TPR 1: [4][H / 2] pairs (column c, column c + H / 2); 2: [H][4]
-  float* b3 = w3 + 4 * H;                                     // [4]
-  float* part = b3 + 4;                                       // TPR 2: head sums [step parity][half][TE][4]
-  S2Ctl* ctl = reinterpret_cast<S2Ctl*>(part + (TPR == 2 ? 2 * 2 * SA_TE * 4 : 0));
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int n_tiles = (p.N + SA_TE - 1) / SA_TE;
-  const bool on_policy = p.C == 0;
-  if (tid == 0) {
-    for (int s = 0; s < SA_SLOTS; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
-    for (int s = 0; s < S2_A_SLOTS; ++s) { mbar_init(&ctl->a_ready[s], 4 * TPR); mbar_init(&ctl->a_free[s], 1); }
-    mbar_init(&ctl->acc_full[0], 1);
-    mbar_init(&ctl->acc_full[1], 1);
-    ctl->abort_flag = ctl->range_flag = 0;
+// where everything lies in shared memory
+template <int D, int H, int TPR, int GROUPS>
+struct S2Smem {
+  static constexpr uint32_t CHUNK_BYTES = H * SA_KC * 2;      // one chunk of one part of W2
+  static constexpr int NKC = H / SA_KC, NSTREAM = 2 * NKC;
+  static constexpr int AS = S2_A_SLOTS / GROUPS, NT = 128 * TPR * GROUPS + 64;   // A slots of a tile in flight; threads
+  static constexpr uint32_t ACC_COLS = H <= 128 ? 128 : 256;
+  uint8_t *a_ring, *w_ring;
+  float *w1, *b1, *b2;    // [D][H] and [H], scaled; [H]
+  float* w3;              // TPR 1: [4][H / 2] pairs (column c, column c + H / 2); 2: [H][4]
+  float* b3;              // [4]
+  float* part;            // TPR 2: head sums [tile in flight][pass parity][half][TE][4]
+  S2Ctl* ctl;
+  __device__ __forceinline__ explicit S2Smem(uint8_t* base) {
+    a_ring = base;
+    w_ring = a_ring + S2_A_SLOTS * S2_A_SLOT;
+    w1 = reinterpret_cast<float*>(w_ring + SA_SLOTS * CHUNK_BYTES);
+    b1 = w1 + D * H; b2 = b1 + H; w3 = b2 + H; b3 = w3 + 4 * H; part = b3 + 4;
+    ctl = reinterpret_cast<S2Ctl*>(part + (TPR == 2 ? GROUPS * 2 * 2 * SA_TE * 4 : 0));
   }
-  __syncthreads();
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&ctl->tmem_base)), "r"(GROUPS * ACC_COLS) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  static size_t bytes() {
+    return (size_t)S2_A_SLOTS * S2_A_SLOT + (size_t)SA_SLOTS * CHUNK_BYTES +
+           ((size_t)(D + 6) * H + 4 + (TPR == 2 ? GROUPS * 2 * 2 * SA_TE * 4 : 0)) * sizeof(float) + sizeof(S2Ctl) + 64;
   }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = ctl->tmem_base;
-  volatile int* abort_flag = &ctl->abort_flag;
-  chain_begin();
-  for (int i = tid; i < D * H; i += S2_NT) w1[i] = SA_H_SCALE * __ldg(p.W + p.off_W1t + i);
-  for (int i = tid; i < H; i += S2_NT) {
-    b1[i] = SA_H_SCALE * __ldg(p.W + p.off_b1 + i);
-    b2[i] = __ldg(p.W + p.off_b2 + i);
-    const float4 w = __ldg(reinterpret_cast<const float4*>(p.W + p.off_W3t) + i);
-    if (TPR == 2) {
-      reinterpret_cast<float4*>(w3)[i] = w;
-    } else {
-      float* d = w3 + 2 * (i % (H / 2)) + i / (H / 2);
-      d[0] = w.x; d[H] = w.y; d[2 * H] = w.z; d[3 * H] = w.w;
-    }
-  }
-  if (tid < 4) b3[tid] = tid < p.Aout ? __ldg(p.W + p.off_b3 + tid) : 0.f;
-  __syncthreads();
-  const int my_tiles = ((int)blockIdx.x < n_tiles) ? (n_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
 
-  if (warp == 8) {
-    // The issuing lane's warp-mates wait at the block's last barrier: lanes of one warp that poll while another lane of it issues
-    // take turns with that lane, and every blocked poll then stalls the issue.
-    if (lane == 0) {
-      const uint32_t idesc = make_idesc_f16(H);
-      const uint32_t a0 = desc_lo(smem_addr(a_ring), 128u), w0 = desc_lo(smem_addr(w_ring), 128u);
-      const uint32_t hiword = desc_hi((uint32_t)(SA_KC / 8) * 128u);          // A slots and W2 chunks: 32 columns wide
-      uint32_t wc = 0, ac[2] = {0, 0};
-      bool alive = true;
-      for (int r = 0; r * GROUPS < my_tiles && alive; ++r)
-        for (int i = 0; i < pl.n_pass && alive; ++i)
-#pragma unroll
-          for (int g = 0; g < GROUPS; ++g) {
-            if (!alive || r * GROUPS + g >= my_tiles) break;
-            const uint32_t acc = tmem + (uint32_t)g * ACC_COLS;
-#pragma unroll 1
-            for (int kc = 0; kc < NKC; ++kc, ++ac[g]) {
-              const uint32_t as = (uint32_t)g * AS + ac[g] % AS;
-              if (!tc_wait(&ctl->a_ready[as], (ac[g] / AS) & 1, abort_flag)) { alive = false; break; }
-              tc_fence_after();
-              const uint32_t a_hi = a0 + as * (S2_A_SLOT / 16), a_lo = a_hi + S2_A_PART / 16;
-#pragma unroll
-              for (int half = 0; half < 2; ++half, ++wc) {
-                const uint32_t s = wc % SA_SLOTS;
-                if (!tc_wait(&ctl->full[s], (wc / SA_SLOTS) & 1, abort_flag)) { alive = false; break; }
-                tc_fence_after();
-                const uint32_t b = w0 + s * (CHUNK_BYTES / 16);
-#pragma unroll
-                for (int j = 0; j < SA_KC / 16; ++j) {
-                  umma_ss(acc, a_hi + 16u * j, hiword, b + 16u * j, hiword, idesc, (kc | half | j) != 0);
-                  if (half == 0) umma_ss(acc, a_lo + 16u * j, hiword, b + 16u * j, hiword, idesc, 1u);
-                }
-                umma_commit(&ctl->empty[s]);
-              }
-              if (!alive) break;
-              umma_commit(&ctl->a_free[as]);
-            }
-            umma_commit(&ctl->acc_full[g]);
-          }
+  // barriers and tensor memory; returns its base.  Ends with a block barrier.
+  __device__ __forceinline__ uint32_t set_up() const {
+    if (threadIdx.x == 0) {
+      for (int s = 0; s < SA_SLOTS; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
+      for (int s = 0; s < S2_A_SLOTS; ++s) { mbar_init(&ctl->a_ready[s], 4 * TPR); mbar_init(&ctl->a_free[s], 1); }
+      mbar_init(&ctl->acc_full[0], 1);
+      mbar_init(&ctl->acc_full[1], 1);
+      ctl->abort_flag = ctl->range_flag = 0;
     }
-    __syncwarp();
-  } else if (warp == 9) {
-    // copy lane: W2's parts, chunk by chunk and pass after pass (the same for every tile)
-    if (lane == 0) {
-      const uint32_t total = (uint32_t)my_tiles * (uint32_t)pl.n_pass * NSTREAM;
-      uint32_t c = 0;
-      for (uint32_t in_pass = 0; c < total; ++c, in_pass = in_pass + 1 == NSTREAM ? 0 : in_pass + 1) {
-        const uint32_t s = c % SA_SLOTS;
-        if (c >= SA_SLOTS && !tc_wait(&ctl->empty[s], ((c / SA_SLOTS) - 1) & 1, abort_flag)) break;
-        mbar_expect_tx(&ctl->full[s], CHUNK_BYTES);
-        bulk_copy_g2s(w_ring + s * CHUNK_BYTES, reinterpret_cast<const uint8_t*>(w2parts) + (size_t)in_pass * CHUNK_BYTES, CHUNK_BYTES, &ctl->full[s]);
-      }
-      // after a timeout the last copies may still be on their way: they must land before the block gives its shared memory back
-      if (*abort_flag)
-        for (uint32_t i = c > SA_SLOTS ? c - SA_SLOTS : 0; i < c; ++i)
-          if (!mbar_wait_bounded(&ctl->full[i % SA_SLOTS], (i / SA_SLOTS) & 1)) break;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&ctl->tmem_base)), "r"(GROUPS * ACC_COLS) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    __syncwarp();
-  } else {
-    const int g = TPR == 1 ? warp >> 2 : 0, half = TPR == 2 ? warp >> 2 : 0;
-    const int row = tid & (SA_TE - 1);                        // row of the tile = TMEM lane
-    const uint32_t t_row = tmem + (uint32_t)g * ACC_COLS + ((uint32_t)((warp & 3) * 32) << 16);
-    const float inv_scale = __ldg(w2scale + 1);               // 1 / (activation scale x weight scale)
-    uint32_t ac = 0, pass = 0;
-    bool ok = true;
-    float vmax = 0.f;
-
-    // network outputs of one observation
-    auto forward = [&](const float (&obs)[6], float (&out)[4]) {
-      tc_fence_before();                                      // this thread's accumulator reads of the previous pass are complete
-      f32x2 x[D];
-#pragma unroll
-      for (int k = 0; k < D; ++k) x[k] = dup2(obs[k]);
-#pragma unroll 1
-      for (int kc = 0; kc < NKC; ++kc, ++ac) {
-        const uint32_t as = (uint32_t)g * AS + ac % AS;
-        if (ac >= AS) ok = ok && tc_wait_elect(&ctl->a_free[as], ((ac / AS) - 1) & 1, abort_flag);
-        uint8_t* dst = a_ring + as * S2_A_SLOT + (row >> 3) * ((SA_KC / 8) * 128) + (row & 7) * 16;
-#pragma unroll
-        for (int b = 0; b < 4 / TPR; ++b) {
-          const int kg = half * 2 + b;
-          vmax = s2_layer1_block<D, H>(w1, b1, x, kc * SA_KC + kg * 8, dst + kg * 128, dst + S2_A_PART + kg * 128, vmax);
-        }
-        fence_async_smem();
-        mbar_arrive_warp(&ctl->a_ready[as]);
-      }
-      ok = ok && tc_wait_elect(&ctl->acc_full[g], pass & 1, abort_flag);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    return ctl->tmem_base;
+  }
+  __device__ __forceinline__ void tear_down(uint32_t tmem) const {
+    tc_fence_before();
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      __syncwarp();
       tc_fence_after();
-      if (TPR == 1) {
-        // h2 = relu(acc / scale + b2); the sums over the two halves of the columns side by side, each in column order
-        f32x2 s[4] = {0ull, 0ull, 0ull, 0ull};
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(GROUPS * ACC_COLS) : "memory");
+    }
+  }
+  // the parameters around the hidden matrix, from the packed FP32 layout P describes
+  template <typename P>
+  __device__ __forceinline__ void stage(const P& p, const float* W, int Aout) const {
+    for (int i = threadIdx.x; i < H; i += NT) {
+      float wk[D];
+#pragma unroll
+      for (int k = 0; k < D; ++k) wk[k] = __ldg(W + p.off_W1t + k * H + i);
+      const float c1 = __ldg(W + p.off_b1 + i), c2 = __ldg(W + p.off_b2 + i);
+      const float4 w = __ldg(reinterpret_cast<const float4*>(W + p.off_W3t) + i);
+#pragma unroll
+      for (int k = 0; k < D; ++k) w1[k * H + i] = SA_H_SCALE * wk[k];
+      b1[i] = SA_H_SCALE * c1;
+      b2[i] = c2;
+      if (TPR == 2) {
+        reinterpret_cast<float4*>(w3)[i] = w;
+      } else {
+        float* d = w3 + 2 * (i % (H / 2)) + i / (H / 2);
+        d[0] = w.x; d[H] = w.y; d[2 * H] = w.z; d[3 * H] = w.w;
+      }
+    }
+    if (threadIdx.x >= NT - 4) {
+      const int a = threadIdx.x - (NT - 4);
+      b3[a] = a < Aout ? __ldg(W + p.off_b3 + a) : 0.f;
+    }
+  }
+  // Issuing lane: the MMAs of n_pass passes over each of `tiles` tiles, the groups' passes in turn.  Its warp-mates wait at the block's
+  // last barrier: lanes of one warp that poll while another lane of it issues take turns with that lane, and every blocked poll then
+  // stalls the issue.
+  __device__ __forceinline__ void issue(uint32_t tmem, int tiles, int n_pass) const {
+    volatile int* abort_flag = &ctl->abort_flag;
+    const uint32_t idesc = make_idesc_f16(H);
+    const uint32_t a0 = desc_lo(smem_addr(a_ring), 128u), w0 = desc_lo(smem_addr(w_ring), 128u);
+    const uint32_t hiword = desc_hi((uint32_t)(SA_KC / 8) * 128u);            // A slots and W2 chunks: 32 columns wide
+    uint32_t wc = 0, ac[2] = {0, 0};
+    bool alive = true;
+    for (int r = 0; r * GROUPS < tiles && alive; ++r)
+      for (int i = 0; i < n_pass && alive; ++i)
+#pragma unroll
+        for (int g = 0; g < GROUPS; ++g) {
+          if (!alive || r * GROUPS + g >= tiles) break;
+          const uint32_t acc = tmem + (uint32_t)g * ACC_COLS;
 #pragma unroll 1
-        for (int c0 = 0; c0 < H / 2; c0 += 16) {
-          uint32_t u[16], v[16];
-          tmem_ld16(t_row + (uint32_t)c0, u);
-          tmem_ld16(t_row + (uint32_t)(c0 + H / 2), v);
-          tmem_ld_wait();
+          for (int kc = 0; kc < NKC; ++kc, ++ac[g]) {
+            const uint32_t as = (uint32_t)g * AS + ac[g] % AS;
+            if (!tc_wait(&ctl->a_ready[as], (ac[g] / AS) & 1, abort_flag)) { alive = false; break; }
+            tc_fence_after();
+            const uint32_t a_hi = a0 + as * (S2_A_SLOT / 16), a_lo = a_hi + S2_A_PART / 16;
+#pragma unroll
+            for (int half = 0; half < 2; ++half, ++wc) {
+              const uint32_t s = wc % SA_SLOTS;
+              if (!tc_wait(&ctl->full[s], (wc / SA_SLOTS) & 1, abort_flag)) { alive = false; break; }
+              tc_fence_after();
+              const uint32_t b = w0 + s * (CHUNK_BYTES / 16);
+#pragma unroll
+              for (int j = 0; j < SA_KC / 16; ++j) {
+                umma_ss(acc, a_hi + 16u * j, hiword, b + 16u * j, hiword, idesc, (kc | half | j) != 0);
+                if (half == 0) umma_ss(acc, a_lo + 16u * j, hiword, b + 16u * j, hiword, idesc, 1u);
+              }
+              umma_commit(&ctl->empty[s]);
+            }
+            if (!alive) break;
+            umma_commit(&ctl->a_free[as]);
+          }
+          umma_commit(&ctl->acc_full[g]);
+        }
+  }
+  // Copy lane: W2's parts, chunk by chunk, `passes` times
+  __device__ __forceinline__ void copy(const uint16_t* parts, uint32_t passes) const {
+    volatile int* abort_flag = &ctl->abort_flag;
+    const uint32_t total = passes * NSTREAM;
+    uint32_t c = 0;
+    for (uint32_t in_pass = 0; c < total; ++c, in_pass = in_pass + 1 == NSTREAM ? 0 : in_pass + 1) {
+      const uint32_t s = c % SA_SLOTS;
+      if (c >= SA_SLOTS && !tc_wait(&ctl->empty[s], ((c / SA_SLOTS) - 1) & 1, abort_flag)) break;
+      mbar_expect_tx(&ctl->full[s], CHUNK_BYTES);
+      bulk_copy_g2s(w_ring + s * CHUNK_BYTES, reinterpret_cast<const uint8_t*>(parts) + (size_t)in_pass * CHUNK_BYTES, CHUNK_BYTES, &ctl->full[s]);
+    }
+    // after a timeout the last copies may still be on their way: they must land before the block gives its shared memory back
+    if (*abort_flag)
+      for (uint32_t i = c > SA_SLOTS ? c - SA_SLOTS : 0; i < c; ++i)
+        if (!mbar_wait_bounded(&ctl->full[i % SA_SLOTS], (i / SA_SLOTS) & 1)) break;
+  }
+};
+
+// A worker thread's side of the forward passes.  After a timeout the abort flag is up: the waits return at once and the thread runs to
+// its end on meaningless numbers, through the same barriers as the others.
+template <int D, int H, int TPR, int GROUPS>
+struct S2Worker {
+  using M = S2Smem<D, H, TPR, GROUPS>;
+  const M& m;
+  int g, half, row;                                           // tile in flight, half of the columns, row of the tile = TMEM lane
+  uint32_t t_row, ac = 0, pass = 0;
+  float inv_scale, vmax = 0.f;                                // 1 / (activation scale x weight scale); largest scaled activation
+  bool ok = true;
+  __device__ __forceinline__ S2Worker(const M& mm, uint32_t tmem, float inv) : m(mm) {
+    const int warp = threadIdx.x >> 5;
+    g = warp / (4 * TPR);
+    half = TPR == 2 ? (warp >> 2) & 1 : 0;
+    row = threadIdx.x & (SA_TE - 1);
+    t_row = tmem + (uint32_t)g * M::ACC_COLS + ((uint32_t)((warp & 3) * 32) << 16);
+    inv_scale = inv;
+  }
+  // network outputs of one observation
+  __device__ __forceinline__ void forward(const float (&obs)[6], int Aout, float (&out)[4]) {
+    volatile int* abort_flag = &m.ctl->abort_flag;
+    tc_fence_before();                                        // this thread's accumulator reads of the previous pass are complete
+    f32x2 x[D];
+#pragma unroll
+    for (int k = 0; k < D; ++k) x[k] = dup2(obs[k]);
+#pragma unroll 1
+    for (int kc = 0; kc < M::NKC; ++kc, ++ac) {
+      const uint32_t as = (uint32_t)g * M::AS + ac % M::AS;
+      if (ac >= M::AS) ok = ok && tc_wait_elect(&m.ctl->a_free[as], ((ac / M::AS) - 1) & 1, abort_flag);
+      uint8_t* dst = m.a_ring + as * S2_A_SLOT + (row >> 3) * ((SA_KC / 8) * 128) + (row & 7) * 16 + half * 256;
+#pragma unroll
+      for (int b = 0; b < 4 / TPR; b += 2) vmax = s2_layer1<D, H, 2>(m.w1, m.b1, x, kc * SA_KC + half * 16 + 8 * b, dst + 128 * b, vmax);
+      fence_async_smem();
+      mbar_arrive_warp(&m.ctl->a_ready[as]);
+    }
+    ok = ok && tc_wait_elect(&m.ctl->acc_full[g], pass & 1, abort_flag);
+    tc_fence_after();
+    const float* b2 = m.b2;
+    const float* w3 = m.w3;
+    if (TPR == 1) {
+      // h2 = relu(acc / scale + b2); the sums over the two halves of the columns side by side, each in column order
+      // (fetching the next columns ahead took 17 % longer: the registers for it spill)
+      f32x2 s[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll 1
+      for (int c0 = 0; c0 < H / 2; c0 += 16) {
+        uint32_t u[16], v[16];
+        tmem_ld16(t_row + (uint32_t)c0, u);
+        tmem_ld16(t_row + (uint32_t)(c0 + H / 2), v);
+        tmem_ld_wait();
 #pragma unroll
           for (int i = 0; i < 16; i += 4) {
             const float4 ba = *reinterpret_cast<const float4*>(b2 + c0 + i), bb = *reinterpret_cast<const float4*>(b2 + c0 + i + H / 2);
@@ -438,46 +320,75 @@ __global__ void __launch_bounds__(S2_NT, 1) actor_split_tc_kernel(const ActorPar
               h[j] = pair2(fmaxf(fmaf(__uint_as_float(u[i + j]), inv_scale, b_lo[j]), 0.f), fmaxf(fmaf(__uint_as_float(v[i + j]), inv_scale, b_hi[j]), 0.f));
 #pragma unroll
             for (int a = 0; a < 4; ++a) {
-              if (a >= 3 && p.Aout <= 3) break;
+              if (a == 3 && Aout <= 3) break;
               const ulonglong2 wa = ld_pairs(w3 + a * H + 2 * (c0 + i)), wb = ld_pairs(w3 + a * H + 2 * (c0 + i) + 4);
               fma2(s[a], wa.x, h[0]); fma2(s[a], wa.y, h[1]); fma2(s[a], wb.x, h[2]); fma2(s[a], wb.y, h[3]);
             }
           }
         }
 #pragma unroll
-        for (int a = 0; a < 4; ++a) { const float2 t = halves(s[a]); out[a] = (b3[a] + t.x) + t.y; }
-      } else {
-        f32x2 s01 = 0ull, s23 = 0ull;
-        const int c_begin = half * (H / 2);
+      for (int a = 0; a < 4; ++a) { const float2 t = halves(s[a]); out[a] = (m.b3[a] + t.x) + t.y; }
+    } else {
+      f32x2 s01 = 0ull, s23 = 0ull;
+      const int c_begin = half * (H / 2);
+      uint32_t u[2][16];
+      tmem_ld16(t_row + (uint32_t)c_begin, u[0]);
 #pragma unroll 1
-        for (int c0 = c_begin; c0 < c_begin + H / 2; c0 += 32) {
-          uint32_t u[32];
-          tmem_ld16(t_row + (uint32_t)c0, u);
-          tmem_ld16(t_row + (uint32_t)c0 + 16u, u + 16);
-          tmem_ld_wait();
+      for (int c1 = c_begin; c1 < c_begin + H / 2; c1 += 32)
 #pragma unroll
-          for (int i = 0; i < 32; i += 4) {
+        for (int q = 0; q < 2; ++q) {
+          const int c0 = c1 + 16 * q;
+          tmem_ld_wait();
+          if (c0 + 16 < c_begin + H / 2) tmem_ld16(t_row + (uint32_t)(c0 + 16), u[q ^ 1]);
+#pragma unroll
+          for (int i = 0; i < 16; i += 4) {
             const float4 ba = *reinterpret_cast<const float4*>(b2 + c0 + i);
             const float bv[4] = {ba.x, ba.y, ba.z, ba.w};
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-              const f32x2 h = dup2(fmaxf(fmaf(__uint_as_float(u[i + j]), inv_scale, bv[j]), 0.f));
+              const f32x2 h = dup2(fmaxf(fmaf(__uint_as_float(u[q][i + j]), inv_scale, bv[j]), 0.f));
               const ulonglong2 w = ld_pairs(w3 + 4 * (c0 + i + j));
               fma2(s01, w.x, h);
               fma2(s23, w.y, h);
             }
           }
         }
-        const float2 a = halves(s01), b = halves(s23);
-        float4* px = reinterpret_cast<float4*>(part) + (size_t)(pass & 1) * 2 * SA_TE;
-        px[half * SA_TE + row] = make_float4(a.x, a.y, b.x, b.y);
-        asm volatile("bar.sync 1, 256;" ::: "memory");
-        const float4 l = px[row], h = px[SA_TE + row];
-        out[0] = (b3[0] + l.x) + h.x; out[1] = (b3[1] + l.y) + h.y; out[2] = (b3[2] + l.z) + h.z; out[3] = (b3[3] + l.w) + h.w;
-      }
-      ++pass;
-    };
+      const float2 a = halves(s01), b = halves(s23);
+      float4* px = reinterpret_cast<float4*>(m.part) + (size_t)(2 * g + (pass & 1)) * 2 * SA_TE;
+      px[half * SA_TE + row] = make_float4(a.x, a.y, b.x, b.y);
+      asm volatile("bar.sync %0, 256;" ::"r"(1 + g) : "memory");
+      const float4 l = px[row], h = px[SA_TE + row];
+      const float* b3 = m.b3;
+      out[0] = (b3[0] + l.x) + h.x; out[1] = (b3[1] + l.y) + h.y; out[2] = (b3[2] + l.z) + h.z; out[3] = (b3[3] + l.w) + h.w;
+    }
+    ++pass;
+  }
+};
 
+template <int ENV, int H, int TPR, int GROUPS>
+__global__ void __launch_bounds__(128 * TPR * GROUPS + 64, 1) actor_split_tc_kernel(const ActorParams p, const S2Plan pl, const uint16_t* __restrict__ w2parts,
+                                                                 const float* __restrict__ w2scale) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  constexpr int D = ENV == TJ_ENV_CARTPOLE ? 4 : 6;
+  constexpr int WW = 4 * TPR * GROUPS;                        // worker warps, then the issuing warp and the copy warp
+  const S2Smem<D, H, TPR, GROUPS> m(smem_raw);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int n_tiles = (p.N + SA_TE - 1) / SA_TE;
+  const bool on_policy = p.C == 0;
+  const uint32_t tmem = m.set_up();
+  chain_begin();
+  m.stage(p, p.W, p.Aout);
+  const int my_tiles = ((int)blockIdx.x < n_tiles) ? (n_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+  __syncthreads();
+  if (warp == WW + 1) {
+    if (lane == 0) m.copy(w2parts, (uint32_t)my_tiles * (uint32_t)pl.n_pass);
+    __syncwarp();
+  } else if (warp == WW) {
+    if (lane == 0) m.issue(tmem, my_tiles, pl.n_pass);
+    __syncwarp();
+  } else {
+    S2Worker<D, H, TPR, GROUPS> wk(m, tmem, __ldg(w2scale + 1));
+    const int g = wk.g, half = wk.half, row = wk.row;
     unsigned long long n_episodes = 0;
     double ret_sum = 0.0;
     const bool first = half == 0;                             // of an environment's threads the one that writes what is written once
@@ -502,7 +413,7 @@ __global__ void __launch_bounds__(S2_NT, 1) actor_split_tc_kernel(const ActorPar
         const unsigned long long t = (unsigned long long)p.t0 + step;
         float out[4];
         const uint4 w = stream_words(p.seed, STREAM_ACTION, 0, (uint32_t)e, t);
-        forward(obs, out);
+        wk.forward(obs, p.Aout, out);
         auto logit = [&](int i) { return i == 0 ? out[0] : (i == 1 ? out[1] : (i == 2 ? out[2] : out[3])); };
         if (p.dbg_logits && owner && first) {
           float* dl = p.dbg_logits + ((size_t)step * p.N + e) * p.A;
@@ -564,7 +475,7 @@ __global__ void __launch_bounds__(S2_NT, 1) actor_split_tc_kernel(const ActorPar
         }
         if (on_policy) {
           if (++pos == p.T) {                                 // bootstrap value of the state each env is now in
-            forward(obs, out);
+            wk.forward(obs, p.Aout, out);
             if (owner && first) p.seg_val[((size_t)seg * (p.T + 1) + p.T) * p.N + e] = logit(p.A);
             pos = 0;
             seg = seg + 1 == p.G ? 0 : seg + 1;
@@ -592,167 +503,105 @@ __global__ void __launch_bounds__(S2_NT, 1) actor_split_tc_kernel(const ActorPar
       ret_sum = 0.0;
     }
     // 65,504 is FP16's largest finite value (the comparison is written to catch a NaN too)
-    if (!(vmax <= 65504.f)) ctl->range_flag = 1;
+    if (!(wk.vmax <= 65504.f)) m.ctl->range_flag = 1;
   }
-  tc_fence_before();
-  __syncthreads();
+  m.tear_down(tmem);
   if (tid == 0) {
-    if (ctl->abort_flag) atomicExch(&p.stats->error, 4ull);
-    else if (ctl->range_flag) atomicExch(&p.stats->error, 5ull);
-  }
-  if (warp == 0) {
-    __syncwarp();
-    tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(GROUPS * ACC_COLS) : "memory");
+    if (m.ctl->abort_flag) atomicExch(&p.stats->error, 4ull);
+    else if (m.ctl->range_flag) atomicExch(&p.stats->error, 5ull);
   }
 }
 
-// TD error (Algorithm 1, TD-error line; Huber loss on it) for a context in this weight mode: a tile of 128 sampled rows per
-// block, the online network on obs (pass 0), the target network on next_obs (pass 1), both with the split-operand hidden
-// layer above; the small parameters are staged twice, the chunk stream alternates between the two split matrices.
-// Outputs and the per-block loss partial as in the FP32 TD kernel (one partial per 128 rows, summed in row order).
+// TD error (Algorithm 1, TD-error line; Huber loss on it) for a context in this weight mode: a pair of thread blocks (a cluster) per 128
+// sampled rows, block 0 with the online network on obs, block 1 with the target network on next_obs at the same time; block 1 leaves
+// max_a q' in block 0's shared memory.  (One block that ran the two networks one after the other took 25 us for 4,096 rows.)
+// Outputs and the per-tile loss partial as in the FP32 TD kernel.
 template <int D, int H>
-__global__ void __launch_bounds__(SA_NT, 1) td_split_tc_kernel(const TdParams p, const uint16_t* __restrict__ parts_online,
+__global__ void __launch_bounds__(S2_NT, 1) td_split_tc_kernel(const TdParams p, const uint16_t* __restrict__ parts_online,
                                                               const float* __restrict__ scale_online,
                                                               const uint16_t* __restrict__ parts_target,
                                                               const float* __restrict__ scale_target) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  constexpr int A_BYTES = SA_TE * H * 2;
-  constexpr uint32_t CHUNK_BYTES = H * SA_KC * 2;
-  constexpr uint32_t NSTREAM = 2 * (H / SA_KC);
-  SaShared sh;
-  sh.a_hi = smem_raw;
-  sh.a_lo = sh.a_hi + A_BYTES;
-  sh.ring = sh.a_lo + A_BYTES;
-  float* wsm = reinterpret_cast<float*>(sh.ring + SA_SLOTS * CHUNK_BYTES);
-  const size_t staged = p.w_total - (p.off_b2 - p.off_W2t);
-  sh.xs = wsm + staged;
-  sh.out = sh.xs + (size_t)8 * SA_TE;
-  sh.part = sh.out + (size_t)4 * SA_TE;
-  sh.ctl = reinterpret_cast<SaCtl*>(sh.part + 2 * (size_t)4 * SA_TE);
-  SaCtl* ctl = sh.ctl;
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const int j0 = blockIdx.x * SA_TE, n_here = min(SA_TE, p.n - j0);
-  if (tid == 0) {
-    for (int s = 0; s < SA_SLOTS; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
-    for (int k = 0; k < SA_MAX_KC; ++k) mbar_init(&ctl->a_ready[k], SA_WORKERS / 32);
-    mbar_init(&ctl->wbar, 1);
-    mbar_init(&ctl->acc_full, 1);
-    ctl->abort_flag = 0;
-    ctl->range_flag = 0;
-  }
-  __syncthreads();
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&ctl->tmem_base)), "r"(256u) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = ctl->tmem_base;
+  const S2Smem<D, H, 2, 1> m(smem_raw);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int net = (int)(blockIdx.x & 1u), tile = (int)(blockIdx.x >> 1);   // the cluster is blocks 2 t and 2 t + 1
+  const int j = tile * SA_TE + (tid & (SA_TE - 1));
+  float* qmax = m.part + 2 * SA_TE * 4;                       // the exchange area of the pass that never comes
+  const uint32_t tmem = m.set_up();
   chain_begin();
-  MlpWeights mw = stage_mlp_weights<1>(p, p.Wonline, wsm, &ctl->wbar, tid == 0);
-  for (int i = tid; i < SA_TE * D; i += SA_NT) {
-    const int el = i / D, k = i % D;
-    sh.xs[k * SA_TE + el] = el < n_here ? p.obs[(size_t)(j0 + el) * D + k] : 0.f;
-  }
-  volatile int* abort_flag = &ctl->abort_flag;
-  bool ok = tc_wait_elect(&ctl->wbar, 0, abort_flag);
-  ok = __syncthreads_and(ok);
-  uint32_t copied = 0;
-  if (tid == SA_WORKERS + 32 && ok) {
-    for (; copied < SA_SLOTS; ++copied) {
-      mbar_expect_tx(&ctl->full[copied], CHUNK_BYTES);
-      bulk_copy_g2s(sh.ring + (size_t)copied * CHUNK_BYTES, reinterpret_cast<const uint8_t*>(parts_online) + (size_t)copied * CHUNK_BYTES,
-                    CHUNK_BYTES, &ctl->full[copied]);
-    }
-  }
-  uint32_t passes = 0;
-  float qsel = 0.f;
-  if (ok) {
-    ok = sa_forward<D, H>(p.Hp, p.A, mw, sh, parts_online, parts_target, scale_online[1], tmem, 0u, copied, abort_flag);
-    passes = 1;
-    ok = __syncthreads_and(ok);
-  }
-  if (ok) {
-    if (tid < n_here) {
-      int a = p.act[j0 + tid];
-      a = a < 0 ? 0 : (a >= p.A ? p.A - 1 : a);
-      qsel = sh.out[a * SA_TE + tid];
-    }
-    __syncthreads();   // every thread is done with the online parameters and outputs: the staging buffer may be refilled
-    mw = stage_mlp_weights<1>(p, p.Wtarget, wsm, &ctl->wbar, tid == 0);
-    for (int i = tid; i < SA_TE * D; i += SA_NT) {
-      const int el = i / D, k = i % D;
-      sh.xs[k * SA_TE + el] = el < n_here ? p.next_obs[(size_t)(j0 + el) * D + k] : 0.f;
-    }
-    ok = tc_wait_elect(&ctl->wbar, 1, abort_flag);
-    ok = __syncthreads_and(ok);
-  }
-  if (ok) {
-    ok = sa_forward<D, H>(p.Hp, p.A, mw, sh, parts_online, parts_target, scale_target[1], tmem, 1u, copied, abort_flag);
-    passes = 2;
-    ok = __syncthreads_and(ok);
-  }
-  const float nan = __int_as_float(0x7FC00000);
-  float* hub = sh.part;                       // free again after the pass
-  if (tid < SA_TE) {
-    float h = 0.f;
-    if (tid < n_here) {
-      const int j = j0 + tid;
-      float delta = nan;
-      h = nan;
-      if (ok) {
-        float qmax = sh.out[tid];
-        for (int i = 1; i < p.A; ++i) qmax = fmaxf(qmax, sh.out[i * SA_TE + tid]);
-        const float y = p.rew[j] + p.gamma * (p.done[j] ? 0.f : 1.f) * qmax;
-        delta = y - qsel;
-        const float ad = fabsf(delta);
-        h = ad <= p.kappa ? 0.5f * delta * delta : p.kappa * (ad - 0.5f * p.kappa);
+  m.stage(p, net ? p.Wtarget : p.Wonline, p.A);
+  cluster_sync_all();                                         // block 0 is running before block 1 writes to it
+  float out[4] = {0.f, 0.f, 0.f, 0.f};
+  const bool row_thread = tid < SA_TE, live = j < p.n;
+  int act = 0, done = 0;
+  float rew = 0.f;
+  if (warp == 9) {
+    if (lane == 0) m.copy(net ? parts_target : parts_online, 1u);
+    __syncwarp();
+  } else if (warp == 8) {
+    if (lane == 0) m.issue(tmem, 1, 1);
+    __syncwarp();
+  } else {
+    S2Worker<D, H, 2, 1> wk(m, tmem, __ldg((net ? scale_target : scale_online) + 1));
+    const float* x = net ? p.next_obs : p.obs;
+    float obs[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (live) {
+#pragma unroll
+      for (int k = 0; k < D; ++k) obs[k] = __ldg(x + (size_t)j * D + k);
+      if (row_thread && net == 0) {
+        act = p.act[j];
+        rew = p.rew[j];
+        done = p.done[j];
       }
-      if (p.td_out) p.td_out[j] = delta;        // after a timeout: defined outputs (NaN), never what an earlier call left
+    }
+    wk.forward(obs, p.A, out);
+    if (!(wk.vmax <= 65504.f)) m.ctl->range_flag = 1;
+    if (row_thread && net == 1) {
+      float q = out[0];
+      for (int i = 1; i < p.A; ++i) q = fmaxf(q, i == 1 ? out[1] : (i == 2 ? out[2] : out[3]));
+      if (!wk.ok) q = __int_as_float(0x7FC00000);             // after a timeout: defined outputs (NaN), never what an earlier call left
+      cluster_store_f32(qmax + tid, 0u, q);
+    }
+    if (!wk.ok) out[0] = out[1] = out[2] = out[3] = __int_as_float(0x7FC00000);
+  }
+  cluster_sync_all();
+  if (row_thread && net == 0) {
+    float h = 0.f;
+    if (live) {
+      act = act < 0 ? 0 : (act >= p.A ? p.A - 1 : act);
+      const float q = act == 0 ? out[0] : (act == 1 ? out[1] : (act == 2 ? out[2] : out[3]));
+      const float y = rew + p.gamma * (done ? 0.f : 1.f) * qmax[tid];
+      const float delta = y - q, ad = fabsf(delta);
+      h = ad <= p.kappa ? 0.5f * delta * delta : p.kappa * (ad - 0.5f * p.kappa);
+      if (p.td_out) p.td_out[j] = delta;
       if (p.huber_out) p.huber_out[j] = h;
     }
-    hub[tid] = h;
+    for (int o = 16; o > 0; o >>= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
+    if (lane == 0) m.part[warp] = h;
   }
-  __syncthreads();
+  m.tear_down(tmem);
   if (tid == 0) {
-    float sum = 0.f;
-    for (int i = 0; i < n_here; ++i) sum += hub[i];
-    p.partial[blockIdx.x] = sum;
-    if (ctl->abort_flag && p.error) atomicExch(p.error, 4ull);
-    else if (ctl->range_flag && p.error) atomicExch(p.error, 5ull);
-  }
-  // the copies still in flight must land before the block gives its shared memory back
-  if (tid == SA_WORKERS + 32) {
-    for (uint32_t g = passes * NSTREAM; g < copied; ++g)
-      if (!tc_wait(&ctl->full[g % SA_SLOTS], (g / SA_SLOTS) & 1, abort_flag)) break;
-  }
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 0) {
-    __syncwarp();
-    tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256u) : "memory");
+    if (net == 0) p.partial[tile] = (m.part[0] + m.part[1]) + (m.part[2] + m.part[3]);
+    if (m.ctl->abort_flag && p.error) atomicExch(p.error, 4ull);
+    else if (m.ctl->range_flag && p.error) atomicExch(p.error, 5ull);
   }
 }
 
 template <int ENV, int H>
-cudaError_t launch_split(const ActorParams& p, const S2Plan& pl, const uint16_t* w2parts, const float* w2scale, int grid, int tpr, cudaStream_t s) {
+cudaError_t launch_split(const ActorParams& p, const S2Plan& pl, const uint16_t* w2parts, const float* w2scale, int grid, int groups, cudaStream_t s) {
   constexpr int D = ENV == TJ_ENV_CARTPOLE ? 4 : 6;
-  const size_t smem = (size_t)S2_A_SLOTS * S2_A_SLOT + (size_t)SA_SLOTS * H * SA_KC * 2 +
-                      ((size_t)(D + 6) * H + 4 + (tpr == 2 ? 2 * 2 * SA_TE * 4 : 0)) * sizeof(float) + sizeof(S2Ctl) + 64;
-  return tpr == 1 ? launch_chained(actor_split_tc_kernel<ENV, H, 1>, grid, S2_NT, smem, s, p, pl, w2parts, w2scale)
-                  : launch_chained(actor_split_tc_kernel<ENV, H, 2>, grid, S2_NT, smem, s, p, pl, w2parts, w2scale);
+#define TJ_SPLIT(T, G) launch_chained(actor_split_tc_kernel<ENV, H, T, G>, grid, S2Smem<D, H, T, G>::NT, S2Smem<D, H, T, G>::bytes(), s, p, pl, w2parts, w2scale)
+  return groups == 1 ? TJ_SPLIT(2, 1) : TJ_SPLIT(1, 2);
+#undef TJ_SPLIT
 }
 
 template <int ENV>
-cudaError_t launch_split_env(const ActorParams& p, const S2Plan& pl, const uint16_t* w2parts, const float* w2scale, int grid, int tpr, cudaStream_t s) {
+cudaError_t launch_split_env(const ActorParams& p, const S2Plan& pl, const uint16_t* w2parts, const float* w2scale, int grid, int groups, cudaStream_t s) {
   switch (p.H) {
-    case 64: return launch_split<ENV, 64>(p, pl, w2parts, w2scale, grid, tpr, s);
-    case 128: return launch_split<ENV, 128>(p, pl, w2parts, w2scale, grid, tpr, s);
-    case 192: return launch_split<ENV, 192>(p, pl, w2parts, w2scale, grid, tpr, s);
-    case 256: return launch_split<ENV, 256>(p, pl, w2parts, w2scale, grid, tpr, s);
+    case 64: return launch_split<ENV, 64>(p, pl, w2parts, w2scale, grid, groups, s);
+    case 128: return launch_split<ENV, 128>(p, pl, w2parts, w2scale, grid, groups, s);
+    case 192: return launch_split<ENV, 192>(p, pl, w2parts, w2scale, grid, groups, s);
+    case 256: return launch_split<ENV, 256>(p, pl, w2parts, w2scale, grid, groups, s);
     default: return cudaErrorInvalidConfiguration;
   }
 }
@@ -785,39 +634,50 @@ cudaError_t launch_actor_split(int env_kind, const ActorParams& p, const uint16_
     pl.seg0 = (int)((p.t0 / p.T) % p.G);
     pl.n_pass += (pl.pos0 + p.n_steps) / p.T;
   }
-  const int tpr = n_tiles > sm_count ? 1 : 2;                // a second tile per SM hides the first one's chain
-  return env_kind == TJ_ENV_CARTPOLE ? launch_split_env<TJ_ENV_CARTPOLE>(p, pl, w2parts, w2scale, grid, tpr, s)
-                                     : launch_split_env<TJ_ENV_ACROBOT>(p, pl, w2parts, w2scale, grid, tpr, s);
-}
-
-template <int D>
-static cudaError_t launch_td_split_d(const TdParams& p, const uint16_t* po, const float* so, const uint16_t* pt, const float* st, int grid,
-                                     size_t smem, cudaStream_t s) {
-#define TJ_TD_SPLIT_CASE(HH) \
-  case HH: return launch_chained(td_split_tc_kernel<D, HH>, grid, SA_NT, smem, s, p, po, so, pt, st);
-  switch (p.H) {
-    TJ_TD_SPLIT_CASE(64)
-    TJ_TD_SPLIT_CASE(128)
-    TJ_TD_SPLIT_CASE(192)
-    TJ_TD_SPLIT_CASE(256)
-    default: return cudaErrorInvalidConfiguration;
-  }
-#undef TJ_TD_SPLIT_CASE
+  const int groups = n_tiles > sm_count ? 2 : 1;             // a second tile per SM runs in the first one's gaps
+  return env_kind == TJ_ENV_CARTPOLE ? launch_split_env<TJ_ENV_CARTPOLE>(p, pl, w2parts, w2scale, grid, groups, s)
+                                     : launch_split_env<TJ_ENV_ACROBOT>(p, pl, w2parts, w2scale, grid, groups, s);
 }
 
 int td_split_grid(int n) { return (n + SA_TE - 1) / SA_TE; }
+
+template <int D, int H>
+static cudaError_t launch_td_split_dh(const TdParams& p, const uint16_t* po, const float* so, const uint16_t* pt, const float* st, cudaStream_t s) {
+  const size_t smem = S2Smem<D, H, 2, 1>::bytes();
+  const cudaError_t e = cudaFuncSetAttribute(td_split_tc_kernel<D, H>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = dim3(2 * td_split_grid(p.n));
+  cfg.blockDim = dim3(S2_NT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, td_split_tc_kernel<D, H>, p, po, so, pt, st);
+}
+
+template <int D>
+static cudaError_t launch_td_split_d(const TdParams& p, const uint16_t* po, const float* so, const uint16_t* pt, const float* st, cudaStream_t s) {
+  switch (p.H) {
+    case 64: return launch_td_split_dh<D, 64>(p, po, so, pt, st, s);
+    case 128: return launch_td_split_dh<D, 128>(p, po, so, pt, st, s);
+    case 192: return launch_td_split_dh<D, 192>(p, po, so, pt, st, s);
+    case 256: return launch_td_split_dh<D, 256>(p, po, so, pt, st, s);
+    default: return cudaErrorInvalidConfiguration;
+  }
+}
 
 cudaError_t launch_td_split(const TdParams& p, const uint16_t* parts_online, const float* scale_online, const uint16_t* parts_target,
                             const float* scale_target, cudaStream_t s) {
   if (p.n <= 0) return cudaSuccess;
   if (!(p.D == 4 || p.D == 6) || p.A > 4 || p.Ap != 4) return cudaErrorInvalidConfiguration;
-  const size_t staged = p.w_total - (p.off_b2 - p.off_W2t);
-  const size_t smem = (size_t)2 * SA_TE * p.H * 2 + (size_t)SA_SLOTS * p.H * SA_KC * 2 +
-                      (staged + (size_t)(8 + 4 + 8) * SA_TE) * sizeof(float) + sizeof(SaCtl) + 64;
-  if (smem > 227 * 1024) return cudaErrorInvalidConfiguration;
-  const int grid = td_split_grid(p.n);
-  return p.D == 4 ? launch_td_split_d<4>(p, parts_online, scale_online, parts_target, scale_target, grid, smem, s)
-                  : launch_td_split_d<6>(p, parts_online, scale_online, parts_target, scale_target, grid, smem, s);
+  return p.D == 4 ? launch_td_split_d<4>(p, parts_online, scale_online, parts_target, scale_target, s)
+                  : launch_td_split_d<6>(p, parts_online, scale_online, parts_target, scale_target, s);
 }
 
 }  // namespace tj
