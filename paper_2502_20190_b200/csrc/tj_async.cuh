@@ -49,6 +49,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 
 // Waits for the phase with the given parity; gives up after a fixed number of polls and reports false.
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity) {
+#pragma unroll 1
   for (int i = 0; i < (1 << 22); ++i)
     if (mbar_try_wait(bar, parity)) return true;
   return false;

@@ -440,11 +440,11 @@ __global__ void __launch_bounds__(TG_THREADS, 2) sg_gemm_tc_kernel(const float* 
 #pragma unroll
       for (int j = 0; j < TG_K / 8; ++j) {
         const uint32_t o = (uint32_t)j * 256u;
-        umma_tf32(tmem, make_desc(a_hi + o, 128u, SBO), make_desc(b_hi + o, 128u, SBO), idesc, (i | j) != 0);
-        umma_tf32(tmem, make_desc(a_lo + o, 128u, SBO), make_desc(b_hi + o, 128u, SBO), idesc, true);
-        umma_tf32(tmem, make_desc(a_hi + o, 128u, SBO), make_desc(b_lo + o, 128u, SBO), idesc, true);
+        umma_tf32(tmem, make_desc(a_hi + o, 128u, SBO), make_desc(b_hi + o, 128u, SBO), idesc, (i | j) != 0, 1u);
+        umma_tf32(tmem, make_desc(a_lo + o, 128u, SBO), make_desc(b_hi + o, 128u, SBO), idesc, true, 1u);
+        umma_tf32(tmem, make_desc(a_hi + o, 128u, SBO), make_desc(b_lo + o, 128u, SBO), idesc, true, 1u);
       }
-      umma_commit(&done[s]);
+      umma_commit(&done[s], 1u);
     }
     if (i + TG_PF < nk) fetch((i + TG_PF) * TG_K, fa, fb);
     return true;

@@ -202,11 +202,10 @@ struct S2Smem {
       b3[a] = a < Aout ? __ldg(W + p.off_b3 + a) : 0.f;
     }
   }
-  // Issuing lane: the MMAs of n_pass passes over each of `tiles` tiles, the groups' passes in turn.  Its warp-mates wait at the block's
-  // last barrier: lanes of one warp that poll while another lane of it issues take turns with that lane, and every blocked poll then
-  // stalls the issue.
+  // Issuing warp: the MMAs of n_pass passes over each of `tiles` tiles, the groups' passes in turn
   __device__ __forceinline__ void issue(uint32_t tmem, int tiles, int n_pass) const {
     volatile int* abort_flag = &ctl->abort_flag;
+    const uint32_t leader = elect_one();
     const uint32_t idesc = make_idesc_f16(H);
     const uint32_t a0 = desc_lo(smem_addr(a_ring), 128u), w0 = desc_lo(smem_addr(w_ring), 128u);
     const uint32_t hiword = desc_hi((uint32_t)(SA_KC / 8) * 128u);            // A slots and W2 chunks: 32 columns wide
@@ -221,26 +220,26 @@ struct S2Smem {
 #pragma unroll 1
           for (int kc = 0; kc < NKC; ++kc, ++ac[g]) {
             const uint32_t as = (uint32_t)g * AS + ac[g] % AS;
-            if (!tc_wait(&ctl->a_ready[as], (ac[g] / AS) & 1, abort_flag)) { alive = false; break; }
+            if (!tc_wait_warp(&ctl->a_ready[as], (ac[g] / AS) & 1, abort_flag)) { alive = false; break; }
             tc_fence_after();
             const uint32_t a_hi = a0 + as * (S2_A_SLOT / 16), a_lo = a_hi + S2_A_PART / 16;
 #pragma unroll
             for (int half = 0; half < 2; ++half, ++wc) {
               const uint32_t s = wc % SA_SLOTS;
-              if (!tc_wait(&ctl->full[s], (wc / SA_SLOTS) & 1, abort_flag)) { alive = false; break; }
+              if (!tc_wait_warp(&ctl->full[s], (wc / SA_SLOTS) & 1, abort_flag)) { alive = false; break; }
               tc_fence_after();
               const uint32_t b = w0 + s * (CHUNK_BYTES / 16);
 #pragma unroll
               for (int j = 0; j < SA_KC / 16; ++j) {
-                umma_ss(acc, a_hi + 16u * j, hiword, b + 16u * j, hiword, idesc, (kc | half | j) != 0);
-                if (half == 0) umma_ss(acc, a_lo + 16u * j, hiword, b + 16u * j, hiword, idesc, 1u);
+                umma_ss(acc, a_hi + 16u * j, hiword, b + 16u * j, hiword, idesc, (kc | half | j) != 0, leader);
+                if (half == 0) umma_ss(acc, a_lo + 16u * j, hiword, b + 16u * j, hiword, idesc, 1u, leader);
               }
-              umma_commit(&ctl->empty[s]);
+              umma_commit(&ctl->empty[s], leader);
             }
             if (!alive) break;
-            umma_commit(&ctl->a_free[as]);
+            umma_commit(&ctl->a_free[as], leader);
           }
-          umma_commit(&ctl->acc_full[g]);
+          umma_commit(&ctl->acc_full[g], leader);
         }
   }
   // Copy lane: W2's parts, chunk by chunk, `passes` times
@@ -384,8 +383,7 @@ __global__ void __launch_bounds__(128 * TPR * GROUPS + 64, 1) actor_split_tc_ker
     if (lane == 0) m.copy(w2parts, (uint32_t)my_tiles * (uint32_t)pl.n_pass);
     __syncwarp();
   } else if (warp == WW) {
-    if (lane == 0) m.issue(tmem, my_tiles, pl.n_pass);
-    __syncwarp();
+    m.issue(tmem, my_tiles, pl.n_pass);
   } else {
     S2Worker<D, H, TPR, GROUPS> wk(m, tmem, __ldg(w2scale + 1));
     const int g = wk.g, half = wk.half, row = wk.row;
@@ -539,8 +537,7 @@ __global__ void __launch_bounds__(S2_NT, 1) td_split_tc_kernel(const TdParams p,
     if (lane == 0) m.copy(net ? parts_target : parts_online, 1u);
     __syncwarp();
   } else if (warp == 8) {
-    if (lane == 0) m.issue(tmem, 1, 1);
-    __syncwarp();
+    m.issue(tmem, 1, 1);
   } else {
     S2Worker<D, H, 2, 1> wk(m, tmem, __ldg((net ? scale_target : scale_online) + 1));
     const float* x = net ? p.next_obs : p.obs;

@@ -124,7 +124,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
         }
       }
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
+    const uint32_t leader = elect_one();
     // ------------------------------------------------------------------ MMA issuer
     uint32_t it = 0, layer_count = 0;
     for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
@@ -134,61 +135,61 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
         const int rows = layer == 2 ? TC_N3 : NB;
         const uint32_t idesc = make_idesc(rows);
         const uint32_t a_sbo = (uint32_t)(K / 8) * 128u, b_sbo = (uint32_t)(TC_KC / 8) * 128u;
-        if (!tc_wait(&ctl->a_ready, layer_count & 1, abort_flag)) goto done;
+        if (!tc_wait_warp(&ctl->a_ready, layer_count & 1, abort_flag)) goto done;
         tc_fence_after();
         if (layer == 2) {
           // the head's weights arrive as one chunk: 16 rows x H columns
           const int s = it % TC_STAGES;
-          if (!tc_wait(&ctl->full[s], (it / TC_STAGES) & 1, abort_flag)) goto done;
+          if (!tc_wait_warp(&ctl->full[s], (it / TC_STAGES) & 1, abort_flag)) goto done;
           const uint32_t b_base = smem_addr(ring + (size_t)s * TC_STAGE_BYTES);
           for (int j = 0; j < H / 16; ++j)
             umma_bf16(tmem, make_desc(smem_addr(abuf) + j * 256u, 128u, a_sbo), make_desc(b_base + j * 256u, 128u, a_sbo), idesc,
-                      j != 0);
-          umma_commit(&ctl->empty[s]);
+                      j != 0, leader);
+          umma_commit(&ctl->empty[s], leader);
           ++it;
         } else {
           for (int nb = 0; nb < nb_count; ++nb) {
             for (int kc = 0; kc < K / TC_KC; ++kc, ++it) {
               const int s = it % TC_STAGES;
-              if (!tc_wait(&ctl->full[s], (it / TC_STAGES) & 1, abort_flag)) goto done;
+              if (!tc_wait_warp(&ctl->full[s], (it / TC_STAGES) & 1, abort_flag)) goto done;
               const uint32_t b_base = smem_addr(ring + (size_t)s * TC_STAGE_BYTES);
               const uint32_t a_base = smem_addr(abuf) + (uint32_t)(kc * (TC_KC / 8)) * 128u;
 #pragma unroll
               for (int j = 0; j < TC_KC / 16; ++j) {
                 umma_bf16(tmem + (uint32_t)(nb * NB), make_desc(a_base + j * 256u, 128u, a_sbo),
-                          make_desc(b_base + j * 256u, 128u, b_sbo), idesc, (kc | j) != 0);
+                          make_desc(b_base + j * 256u, 128u, b_sbo), idesc, (kc | j) != 0, leader);
               }
-              umma_commit(&ctl->empty[s]);    // the slot is free once these MMAs have read it
+              umma_commit(&ctl->empty[s], leader);    // the slot is free once these MMAs have read it
             }
           }
         }
-        umma_commit(&ctl->acc_full);        // accumulator of this layer complete
+        umma_commit(&ctl->acc_full, leader);        // accumulator of this layer complete
       }
       if (FUSED) {
         // z = A s as three TF32 products: (s_hi, A_hi), (s_lo, A_hi), (s_hi, A_lo)
         const uint32_t idesc = make_idesc_tf32(D);
         const uint32_t a_sbo = (uint32_t)(D / 4) * 128u, b_sbo = (uint32_t)(TC_KC / 4) * 128u;
         const uint32_t lo_off = (uint32_t)TC_M * D * 4;
-        if (!tc_wait(&ctl->a_ready, layer_count & 1, abort_flag)) goto done;
+        if (!tc_wait_warp(&ctl->a_ready, layer_count & 1, abort_flag)) goto done;
         tc_fence_after();
         for (int half = 0; half < 2; ++half) {       // chunks of A_hi (used with s_hi and s_lo), then of A_lo (with s_hi)
           for (int kc = 0; kc < ce; ++kc, ++it) {
             const int s = it % TC_STAGES;
-            if (!tc_wait(&ctl->full[s], (it / TC_STAGES) & 1, abort_flag)) goto done;
+            if (!tc_wait_warp(&ctl->full[s], (it / TC_STAGES) & 1, abort_flag)) goto done;
             const uint32_t b_base = smem_addr(ring + (size_t)s * TC_STAGE_BYTES);
             const uint32_t a_base = smem_addr(abuf) + (uint32_t)(kc * (TC_KC / 4)) * 128u;
 #pragma unroll
             for (int j = 0; j < TC_KC / 8; ++j) {
               umma_tf32(tmem, make_desc(a_base + j * 256u, 128u, a_sbo), make_desc(b_base + j * 256u, 128u, b_sbo), idesc,
-                        (half | kc | j) != 0);
+                        (half | kc | j) != 0, leader);
               if (half == 0)
                 umma_tf32(tmem, make_desc(a_base + lo_off + j * 256u, 128u, a_sbo), make_desc(b_base + j * 256u, 128u, b_sbo),
-                          idesc, true);
+                          idesc, true, leader);
             }
-            umma_commit(&ctl->empty[s]);
+            umma_commit(&ctl->empty[s], leader);
           }
         }
-        umma_commit(&ctl->acc_full);
+        umma_commit(&ctl->acc_full, leader);
         ++layer_count;
       }
     }

@@ -4,12 +4,11 @@
 // A thread block owns 128 rows (envs) per tile, one row per TMEM lane, and walks tiles persistently.  Roles:
 //   warp 0, one lane    producer: streams 32 KB operand chunks (weights, the env matrix) from L2 into a ring of two slots
 //   warp 1, one lane    MMA issuer (tcgen05.mma, M = 128, N = 128 per hidden block)
-//   warps 4-11          network warps (two threads per row): state rows -> BF16 (layer-1 operand); per 128-neuron block of a
-//                       hidden layer: accumulator -> bias, ReLU, BF16 -> next layer's operand; z -> a scratch tile in global
-//                       memory
-//   warps 12-19         env warps: the FP16 parts of the next tile's state rows and the record's observation; take the head
-//                       outputs out of TMEM, select the action, read z back and finish the step (tanh, Philox noise, reward,
-//                       done, record, reset or new state, counters), eight rows x four 16-byte pieces per warp instruction
+//   warps 4-19          network warps (four threads per row): per 128-neuron block of a hidden layer: accumulator -> bias, ReLU, BF16
+//                       -> next layer's operand; z -> a scratch tile in global memory
+//   warps 20-27         env warps: the next tile's state rows as BF16 (layer-1 operand) and, with the record's observation, as FP16
+//                       parts; take the head outputs out of TMEM, select the action, read z back and finish the step (tanh, Philox
+//                       noise, reward, done, record, reset or new state, counters), four rows x eight 16-byte pieces per instruction
 // The env warps work on tile i while the network warps and the tensor pipe are already on tile i + 1.
 //
 // Per tile the tensor pipe runs ten accumulator blocks that alternate between two 128-column accumulators:
@@ -21,6 +20,9 @@
 // Tensor memory (512 columns): [0, H/2) h1 as packed BF16 pairs; [256, 384) and [384, 512) the two accumulators.
 // Shared memory: X (BF16 state tile, 32 KB) | U (128 KB: the FP16 high and low parts of the state tile in its first 64 KB
 // until z is done, then h2, the head's A operand) | ring (64 KB) | barriers.
+// Code size counts here: five roles execute five different programs at once, and with everything unrolled the kernel no longer fitted
+// the instruction cache -- the issuing lane, which runs each line of its program once or a few times per tile, then took 446 cycles per
+// MMA of the z product (64 on the tensor pipe) fetching instructions from L2.  So loops are unrolled only as far as their latency asks.
 // Every wait is bounded: on a timeout the block raises an abort flag, records an error, frees its TMEM and leaves.
 #include <cuda_fp16.h>
 
@@ -40,8 +42,9 @@ constexpr int PA_STAGE_BYTES = PA_W_BYTES;
 constexpr int PA_STAGES = 65536 / PA_STAGE_BYTES;
 constexpr int PA_X_BYTES = PA_M * PA_D * 2;
 constexpr int PA_U_BYTES = 131072;
-constexpr int PA_THREADS = 640;            // warps 0-3: producer, MMA issuer, two idle; 4-11 network; 12-19 env
-constexpr int PA_GROUP_WARPS = 8;          // warps of the network group and of the env group (one barrier arrival each)
+constexpr int PA_NET_WARPS = 16, PA_ENV_WARPS = 8;   // one barrier arrival each
+constexpr int PA_ENV0 = 4 + PA_NET_WARPS;  // warps 0-3: producer, MMA issuer, two idle; then network, then env
+constexpr int PA_THREADS = 32 * (PA_ENV0 + PA_ENV_WARPS);
 constexpr uint32_t PA_COL_HB = 0, PA_COL_ACC0 = 256, PA_COL_ACC1 = 384;
 constexpr int PA_N3 = 16;                  // head width on the tensor cores
 constexpr int PA_MAX_GRID = 192;           // thread blocks the z scratch is sized for
@@ -49,7 +52,7 @@ constexpr float PA_S_SCALE = 256.0f;       // state values are split after this 
 
 struct PaSmem {
   uint64_t full[PA_STAGES], empty[PA_STAGES];
-  uint64_t x_ready;        // network -> MMA: X holds the tile's BF16 rows
+  uint64_t x_ready;        // env -> MMA: X holds the tile's BF16 rows
   uint64_t u_ready;        // env -> MMA: U holds the tile's FP16 high / low parts
   uint64_t acc_full[2];    // MMA -> network: an accumulator block is complete
   uint64_t acc_empty[2];   // network -> MMA: it has been drained (and its result stored)
@@ -82,15 +85,15 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
 
   if (tid == 0) {
     for (int s = 0; s < PA_STAGES; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
-    mbar_init(&ctl->x_ready, PA_GROUP_WARPS);
-    mbar_init(&ctl->u_ready, PA_GROUP_WARPS);
+    mbar_init(&ctl->x_ready, PA_ENV_WARPS);
+    mbar_init(&ctl->u_ready, PA_ENV_WARPS);
     mbar_init(&ctl->acc_full[0], 1);
     mbar_init(&ctl->acc_full[1], 1);
-    mbar_init(&ctl->acc_empty[0], PA_GROUP_WARPS);
-    mbar_init(&ctl->acc_empty[1], PA_GROUP_WARPS);
+    mbar_init(&ctl->acc_empty[0], PA_NET_WARPS);
+    mbar_init(&ctl->acc_empty[1], PA_NET_WARPS);
     mbar_init(&ctl->head_full, 1);
-    mbar_init(&ctl->env_taken, PA_GROUP_WARPS);
-    mbar_init(&ctl->z_stored, PA_GROUP_WARPS);
+    mbar_init(&ctl->env_taken, PA_ENV_WARPS);
+    mbar_init(&ctl->z_stored, PA_NET_WARPS);
     mbar_init(&ctl->act_ready, 4);
     ctl->abort_flag = 0;
   }
@@ -108,9 +111,8 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
   const TcEnvParams& ev = p.env;
 
   if (warp < 4) {
-    // registers: 640 threads x 96 at launch = 61,440; 128 x 64 + 256 x 96 + 256 x 112 = 61,440 after the two changes.  The
-    // issuing lane's loop is the pace-maker of the whole block: it must not spill, so its warpgroup keeps 64 registers.
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+    // registers: 896 threads x 72 at launch = 64,512; 128 x 56 + 512 x 56 + 256 x 112 = 64,512 after the changes
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
     if (warp == 0 && lane == 0) {
       // ---------------------------------------------------------------- producer
       // order per tile (the order the MMA issuer consumes): layer 1 (one chunk per block), env matrix (high part, low
@@ -138,7 +140,8 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
           bulk_copy_g2s_keep(ring + (size_t)s * PA_STAGE_BYTES, src, bytes, &ctl->full[s], keep_policy);
         }
       }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
+      const uint32_t leader = elect_one();
       // ---------------------------------------------------------------- MMA issuer
       // Accumulator uses of a tile: u = 0 .. n_hb-1 layer 1, n_hb z, n_hb+1 .. 2 n_hb layer 2, 2 n_hb + 1 head; use u
       // writes accumulator u & 1 (the count per tile is even, so the pattern repeats).  The network warps drain every use
@@ -154,44 +157,44 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
       // before use u may overwrite its accumulator, the previous use of that accumulator must have been read out
       auto acquire = [&](int u) -> bool {
         if (u == 0) return true;      // accumulator 0: its last drain was awaited before the previous tile's head
-        if (u == 1) return tiles == 0 || tc_wait(&ctl->env_taken, (tiles - 1) & 1, abort_flag);
-        return (u & 1) ? tc_wait(&ctl->acc_empty[1], (nwait1++) & 1, abort_flag) : tc_wait(&ctl->acc_empty[0], (nwait0++) & 1, abort_flag);
+        if (u == 1) return tiles == 0 || tc_wait_warp(&ctl->env_taken, (tiles - 1) & 1, abort_flag);
+        return (u & 1) ? tc_wait_warp(&ctl->acc_empty[1], (nwait1++) & 1, abort_flag) : tc_wait_warp(&ctl->acc_empty[0], (nwait0++) & 1, abort_flag);
       };
       for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++tiles) {
-        if (!tc_wait(&ctl->x_ready, tiles & 1, abort_flag)) goto done;
+        if (!tc_wait_warp(&ctl->x_ready, tiles & 1, abort_flag)) goto done;
         // layer 1: one chunk per 128-neuron block; A operand = X in shared memory
         for (int b = 0; b < n_hb; ++b, ++it) {
           const int u = b;
           if (!acquire(u)) goto done;
           const uint32_t acc = tmem + ((u & 1) ? PA_COL_ACC1 : PA_COL_ACC0);
           const uint32_t s = it % PA_STAGES;
-          if (!tc_wait(&ctl->full[s], (it / PA_STAGES) & 1, abort_flag)) goto done;
+          if (!tc_wait_warp(&ctl->full[s], (it / PA_STAGES) & 1, abort_flag)) goto done;
           tc_fence_after();
           const uint32_t b_lo = ring_lo + s * (PA_STAGE_BYTES / 16);
-#pragma unroll
-          for (int j = 0; j < PA_KC / 16; ++j) umma_ss(acc, x_lo + j * 16u, hi_k128, b_lo + j * 16u, hi_k128, idesc_h, j != 0);
-          umma_commit(&ctl->empty[s]);
-          umma_commit((u & 1) ? &ctl->acc_full[1] : &ctl->acc_full[0]);
+#pragma unroll 4
+          for (int j = 0; j < PA_KC / 16; ++j) umma_ss(acc, x_lo + j * 16u, hi_k128, b_lo + j * 16u, hi_k128, idesc_h, j != 0, leader);
+          umma_commit(&ctl->empty[s], leader);
+          umma_commit((u & 1) ? &ctl->acc_full[1] : &ctl->acc_full[0], leader);
         }
         // z = A s from the FP16 parts: (s_hi, A_hi) + (s_lo, A_hi) with the first chunk, (s_hi, A_lo) with the second
         {
           const int u = n_hb;
-          if (!tc_wait(&ctl->u_ready, tiles & 1, abort_flag)) goto done;
+          if (!tc_wait_warp(&ctl->u_ready, tiles & 1, abort_flag)) goto done;
           if (!acquire(u)) goto done;
           const uint32_t acc = tmem + ((u & 1) ? PA_COL_ACC1 : PA_COL_ACC0);
           for (int part = 0; part < 2; ++part, ++it) {
             const uint32_t s = it % PA_STAGES;
-            if (!tc_wait(&ctl->full[s], (it / PA_STAGES) & 1, abort_flag)) goto done;
+            if (!tc_wait_warp(&ctl->full[s], (it / PA_STAGES) & 1, abort_flag)) goto done;
             tc_fence_after();
             const uint32_t b_lo = ring_lo + s * (PA_STAGE_BYTES / 16);
-#pragma unroll
+#pragma unroll 2
             for (int j = 0; j < D / 16; ++j) {
-              umma_ss(acc, u_lo + j * 16u, hi_k128, b_lo + j * 16u, hi_k128, idesc_z, (part | j) != 0);
-              if (part == 0) umma_ss(acc, ulo_lo + j * 16u, hi_k128, b_lo + j * 16u, hi_k128, idesc_z, 1u);
+              umma_ss(acc, u_lo + j * 16u, hi_k128, b_lo + j * 16u, hi_k128, idesc_z, (part | j) != 0, leader);
+              if (part == 0) umma_ss(acc, ulo_lo + j * 16u, hi_k128, b_lo + j * 16u, hi_k128, idesc_z, 1u, leader);
             }
-            umma_commit(&ctl->empty[s]);
+            umma_commit(&ctl->empty[s], leader);
           }
-          umma_commit((u & 1) ? &ctl->acc_full[1] : &ctl->acc_full[0]);
+          umma_commit((u & 1) ? &ctl->acc_full[1] : &ctl->acc_full[0], leader);
         }
         // layer 2: per block H / PA_KC chunks; A operand = h1 in tensor memory (8 columns per K = 16); the drain of the last
         // layer-1 block (awaited by the first block here) completes h1
@@ -201,128 +204,83 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
           const uint32_t acc = tmem + ((u & 1) ? PA_COL_ACC1 : PA_COL_ACC0);
           for (int c = 0; c < n_kc2; ++c, ++it) {
             const uint32_t s = it % PA_STAGES;
-            if (!tc_wait(&ctl->full[s], (it / PA_STAGES) & 1, abort_flag)) goto done;
+            if (!tc_wait_warp(&ctl->full[s], (it / PA_STAGES) & 1, abort_flag)) goto done;
             tc_fence_after();
             const uint32_t b_lo = ring_lo + s * (PA_STAGE_BYTES / 16);
             const uint32_t a_col = tmem + PA_COL_HB + (uint32_t)(c * (PA_KC / 2));
-#pragma unroll
-            for (int j = 0; j < PA_KC / 16; ++j) umma_ts(acc, a_col + (uint32_t)(j * 8), b_lo + j * 16u, hi_k128, idesc_h, (c | j) != 0);
-            umma_commit(&ctl->empty[s]);
+#pragma unroll 4
+            for (int j = 0; j < PA_KC / 16; ++j) umma_ts(acc, a_col + (uint32_t)(j * 8), b_lo + j * 16u, hi_k128, idesc_h, (c | j) != 0, leader);
+            umma_commit(&ctl->empty[s], leader);
           }
-          umma_commit((u & 1) ? &ctl->acc_full[1] : &ctl->acc_full[0]);
+          umma_commit((u & 1) ? &ctl->acc_full[1] : &ctl->acc_full[0], leader);
         }
         // head: 16 outputs, K = H, A operand = h2 in shared memory; accumulator 1.  Both remaining drains complete h2.
         {
           if (!acquire(2 * n_hb + 1)) goto done;
-          if (!tc_wait(&ctl->acc_empty[0], (nwait0++) & 1, abort_flag)) goto done;
+          if (!tc_wait_warp(&ctl->acc_empty[0], (nwait0++) & 1, abort_flag)) goto done;
           const uint32_t s = it % PA_STAGES;
-          if (!tc_wait(&ctl->full[s], (it / PA_STAGES) & 1, abort_flag)) goto done;
+          if (!tc_wait_warp(&ctl->full[s], (it / PA_STAGES) & 1, abort_flag)) goto done;
           tc_fence_after();
           const uint32_t b_lo = ring_lo + s * (PA_STAGE_BYTES / 16);
-          for (int j = 0; j < H / 16; ++j) umma_ss(tmem + PA_COL_ACC1, u_lo + j * 16u, hi_head, b_lo + j * 16u, hi_head, idesc16, j != 0);
-          umma_commit(&ctl->empty[s]);
-          umma_commit(&ctl->head_full);
+#pragma unroll 4
+          for (int j = 0; j < H / 16; ++j) umma_ss(tmem + PA_COL_ACC1, u_lo + j * 16u, hi_head, b_lo + j * 16u, hi_head, idesc16, j != 0, leader);
+          umma_commit(&ctl->empty[s], leader);
+          umma_commit(&ctl->head_full, leader);
           ++it;
         }
       }
     }
-  } else if (warp < 12) {
+  } else if (warp < PA_ENV0) {
     // ------------------------------------------------------------------ network warps
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
     const int q = warp & 3;                       // TMEM lane quarter this warp may access
-    const int hsel = (warp - 4) >> 2;             // which half of a row / of a block's columns
+    const int hsel = (warp - 4) >> 2;             // which quarter of a block's columns
     const int r = q * 32 + lane;                  // row of the tile = TMEM lane
     const uint32_t t_lane = tmem + ((uint32_t)(q * 32) << 16);
     uint32_t tiles = 0, nfull0 = 0, nfull1 = 0;
-    // Conversions read the row-major state with eight rows x four 16-byte pieces per warp instruction (64 contiguous
-    // bytes per row) instead of one row per lane: a quarter of the memory wavefronts, and conflict-free stores.
-    const int nw = warp - 4, c_r8 = lane >> 2, c_kq = lane & 3;
-    // BF16 rows of a tile -> X (layer-1 A operand)
-    auto convert_x = [&](int tile) {
-#pragma unroll
-      for (int g = 0; g < 2; ++g) {
-        const int rr = nw * 16 + g * 8 + c_r8;
-        const long long row = (long long)tile * PA_M + rr;
-        const float* xr = p.x + (size_t)(row < p.n ? row : 0) * D;
-        float4 v[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-          v[i] = row < p.n ? __ldg(reinterpret_cast<const float4*>(xr + (c_kq + 4 * i) * 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
-        uint8_t* dx = xbuf + ((size_t)(rr >> 3) * (D / 8)) * 128 + (rr & 7) * 16;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int k4 = c_kq + 4 * i;
-          *reinterpret_cast<uint2*>(dx + (size_t)(k4 >> 1) * 128 + (k4 & 1) * 8) =
-              make_uint2(pack_bf16x2(v[i].x, v[i].y), pack_bf16x2(v[i].z, v[i].w));
-        }
-      }
-      fence_async_smem();
-      mbar_arrive_warp(&ctl->x_ready);
-    };
-    if ((int)blockIdx.x < n_tiles) convert_x(blockIdx.x);
     for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++tiles) {
-      const int next_tile = tile + (int)gridDim.x;
-      {
-        // pull the rows of the tile after the next towards L2
-        const long long prow = (long long)(next_tile + (int)gridDim.x) * PA_M + r;
-        if (prow < p.n) {
-          const float* xn = p.x + (size_t)prow * D + hsel * 64;
-          prefetch_l2(xn);
-          prefetch_l2(xn + 32);
-        }
-      }
       for (int u = 0; u <= 2 * n_hb; ++u) {
         const int buf = u & 1;
         if (!tc_wait_elect(buf ? &ctl->acc_full[1] : &ctl->acc_full[0], (buf ? nfull1++ : nfull0++) & 1, abort_flag)) goto done;
         tc_fence_after();
-        const uint32_t t_acc = t_lane + (buf ? PA_COL_ACC1 : PA_COL_ACC0) + (uint32_t)(hsel * 64);
+        const uint32_t t_acc = t_lane + (buf ? PA_COL_ACC1 : PA_COL_ACC0) + (uint32_t)(hsel * 32);
         if (u == n_hb) {
-          // z: this thread's 64 components go to the block's scratch tile, where the env warps pick them up
-          uint32_t v[64];
-#pragma unroll
-          for (int g = 0; g < 4; ++g) tmem_ld16(t_acc + (uint32_t)(g * 16), v + 16 * g);
+          // z: this thread's 32 components go to the block's scratch tile, where the env warps pick them up
+          uint32_t v[32];
+          tmem_ld16(t_acc, v);
+          tmem_ld16(t_acc + 16u, v + 16);
           tmem_ld_wait();
           tc_fence_before();
-          {
-            // scratch tile [k/4][row][4]: a warp's 32 rows are contiguous, for this store and for the env warps' loads
-            float* zs = ev.z_scratch + ((size_t)blockIdx.x * 2 + (tiles & 1)) * (PA_M * D);
+          // scratch tile [k/4][row][4]: a warp's 32 rows are contiguous
+          float* zs = ev.z_scratch + ((size_t)blockIdx.x * 2 + (tiles & 1)) * (PA_M * D);
 #pragma unroll
-            for (int i = 0; i < 16; ++i)
-              *reinterpret_cast<uint4*>(zs + ((size_t)(hsel * 16 + i) * PA_M + r) * 4) = make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-          }
+          for (int i = 0; i < 8; ++i)
+            *reinterpret_cast<uint4*>(zs + ((size_t)(hsel * 8 + i) * PA_M + r) * 4) = make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
           mbar_arrive_warp(&ctl->acc_empty[buf]);
           mbar_arrive_warp(&ctl->z_stored);
-          // layer 1 of this tile is complete, so X is free: the next tile's rows go in while layer 2 runs
-          if (next_tile < n_tiles) convert_x(next_tile);
           continue;
         }
         const int layer = u < n_hb ? 0 : 1;
         const int b = ((layer == 0 ? u : u - n_hb - 1) + rot) % n_hb;   // neuron block of this use
         const float* bias = layer == 0 ? p.b1 : p.b2;
-        const int c0 = b * PA_NB + hsel * 64;          // first of this thread's 64 columns
-        uint32_t v[64];
-#pragma unroll
-        for (int g = 0; g < 4; ++g) tmem_ld16(t_acc + (uint32_t)(g * 16), v + 16 * g);
+        const int c0 = b * PA_NB + hsel * 32;          // first of this thread's 32 columns
+        uint32_t v[32], o[16];
+        tmem_ld16(t_acc, v);
+        tmem_ld16(t_acc + 16u, v + 16);
         tmem_ld_wait();
 #pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-          uint32_t o[16];
+        for (int j4 = 0; j4 < 8; ++j4) {
+          const float4 bb = __ldg(reinterpret_cast<const float4*>(bias + c0 + 4 * j4));
+          o[2 * j4] = pack_bf16x2_relu(__uint_as_float(v[4 * j4]) + bb.x, __uint_as_float(v[4 * j4 + 1]) + bb.y);
+          o[2 * j4 + 1] = pack_bf16x2_relu(__uint_as_float(v[4 * j4 + 2]) + bb.z, __uint_as_float(v[4 * j4 + 3]) + bb.w);
+        }
+        if (layer == 0) {
+          tmem_st16(t_lane + PA_COL_HB + (uint32_t)(c0 / 2), o);
+        } else {
+          uint8_t* dst = ubuf + ((size_t)(r >> 3) * (H / 8)) * 128 + (r & 7) * 16 + (size_t)(c0 / 8) * 128;
 #pragma unroll
-          for (int j4 = 0; j4 < 8; ++j4) {
-            float f0 = __uint_as_float(v[hh * 32 + 4 * j4 + 0]), f1 = __uint_as_float(v[hh * 32 + 4 * j4 + 1]);
-            float f2 = __uint_as_float(v[hh * 32 + 4 * j4 + 2]), f3 = __uint_as_float(v[hh * 32 + 4 * j4 + 3]);
-            const float4 bb = __ldg(reinterpret_cast<const float4*>(bias + c0 + hh * 32 + 4 * j4));
-            f0 += bb.x; f1 += bb.y; f2 += bb.z; f3 += bb.w;
-            o[2 * j4] = pack_bf16x2_relu(f0, f1);
-            o[2 * j4 + 1] = pack_bf16x2_relu(f2, f3);
-          }
-          if (layer == 0) {
-            tmem_st16(t_lane + PA_COL_HB + (uint32_t)((c0 + hh * 32) / 2), o);
-          } else {
-            uint8_t* dst = ubuf + ((size_t)(r >> 3) * (H / 8)) * 128 + (r & 7) * 16 + (size_t)((c0 + hh * 32) / 8) * 128;
-#pragma unroll
-            for (int g = 0; g < 4; ++g)
-              *reinterpret_cast<uint4*>(dst + (size_t)g * 128) = make_uint4(o[4 * g], o[4 * g + 1], o[4 * g + 2], o[4 * g + 3]);
-          }
+          for (int g = 0; g < 4; ++g)
+            *reinterpret_cast<uint4*>(dst + (size_t)g * 128) = make_uint4(o[4 * g], o[4 * g + 1], o[4 * g + 2], o[4 * g + 3]);
         }
         if (layer == 0) tmem_st_wait();
         else fence_async_smem();
@@ -333,27 +291,49 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
   } else {
     // ------------------------------------------------------------------ env warps
     asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
-    const int ew = warp - 12;                      // 0..7; the first four also read the head outputs (one TMEM quarter each)
-    const int e_r8 = lane >> 2, e_kq = lane & 3;   // env step: eight rows x four 16-byte pieces per warp instruction
+    const int ew = warp - PA_ENV0;                 // 0..7; the first four also read the head outputs (one TMEM quarter each)
+    const int e_r4 = lane >> 3, e_kq = lane & 7;   // four rows x eight 16-byte pieces per warp instruction, four pieces per lane and row
     uint32_t tiles = 0;
     // FP16 high / low parts of a tile's scaled rows -> U (A operand of z = A s); the FP32 row is the record's observation
-    auto convert_u = [&](int tile) {
+    // BF16 rows of a tile -> X (layer-1 A operand)
+    auto convert_x = [&](int tile) {
+#pragma unroll 1
+      for (int g = 0; g < 4; ++g) {
+        const int rr = ew * 16 + g * 4 + e_r4;
+        const long long row = (long long)tile * PA_M + rr;
+        const float* xr = p.x + (size_t)(row < p.n ? row : 0) * D;
+        float4 v[4];
 #pragma unroll
-      for (int g = 0; g < 2; ++g) {
-        const int rr = ew * 16 + g * 8 + e_r8;
+        for (int i = 0; i < 4; ++i)
+          v[i] = row < p.n ? __ldg(reinterpret_cast<const float4*>(xr + (e_kq + 8 * i) * 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        uint8_t* dx = xbuf + ((size_t)(rr >> 3) * (D / 8)) * 128 + (rr & 7) * 16;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int k4 = e_kq + 8 * i;
+          *reinterpret_cast<uint2*>(dx + (size_t)(k4 >> 1) * 128 + (k4 & 1) * 8) =
+              make_uint2(pack_bf16x2(v[i].x, v[i].y), pack_bf16x2(v[i].z, v[i].w));
+        }
+      }
+      fence_async_smem();
+      mbar_arrive_warp(&ctl->x_ready);
+    };
+    auto convert_u = [&](int tile) {
+#pragma unroll 1
+      for (int g = 0; g < 4; ++g) {
+        const int rr = ew * 16 + g * 4 + e_r4;
         const long long row = (long long)tile * PA_M + rr;
         const bool live = row < p.n;
         const float* xr = p.x + (size_t)(live ? row : 0) * D;
-        float4 v[8];
+        float4 v[4];
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
-          v[i] = live ? __ldg(reinterpret_cast<const float4*>(xr + (e_kq + 4 * i) * 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int i = 0; i < 4; ++i)
+          v[i] = live ? __ldg(reinterpret_cast<const float4*>(xr + (e_kq + 8 * i) * 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
         uint8_t* dhi = ubuf + ((size_t)(rr >> 3) * (D / 8)) * 128 + (rr & 7) * 16;
         uint8_t* dlo = dhi + PA_X_BYTES;
         float* rec = ev.ring + (ev.slot0 + (unsigned long long)(live ? row : 0)) * ev.rec_words;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int k4 = e_kq + 4 * i;
+        for (int i = 0; i < 4; ++i) {
+          const int k4 = e_kq + 8 * i;
           const float4 sv = v[i];
           // high part: the scaled value cut to 11 significant bits (exact in FP16); low part: the exact remainder, rounded
           float4 s4, hi, lo;
@@ -371,12 +351,27 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
       fence_async_smem();
       mbar_arrive_warp(&ctl->u_ready);
     };
-    if ((int)blockIdx.x < n_tiles) convert_u(blockIdx.x);
     unsigned long long n_episodes = 0;
     double ret_sum = 0.0;
     const float zc = ev.z_to_t;                    // accumulator -> 2 log2(e) * z
-    for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++tiles) {
-      if (ew < 4) {
+    // the first round has no tile to finish, it only converts: one copy of the conversion's code (see the note on code size above)
+    bool warm = false;
+    for (int tile = (int)blockIdx.x - (int)gridDim.x; tile < n_tiles; tile += gridDim.x) {
+      // layer 1 and z of this tile are complete, so X is free: the next tile's rows go in while layer 2 runs
+      const int next_tile = tile + (int)gridDim.x;
+      if (warm && !tc_wait_elect(&ctl->z_stored, tiles & 1, abort_flag)) goto done;
+      if (next_tile < n_tiles) {
+        convert_x(next_tile);
+        // pull the rows of the tile after the next towards L2
+        const long long prow = (long long)(next_tile + (int)gridDim.x) * PA_M + ew * 16 + (lane >> 1);
+        if (prow < p.n) {
+          const float* xn = p.x + (size_t)prow * D + (lane & 1) * 64;
+          prefetch_l2(xn);
+          prefetch_l2(xn + 32);
+        }
+      }
+      if (!warm) {
+      } else if (ew < 4) {
         const int r = ew * 32 + lane;              // row of the tile = TMEM lane
         const long long row = (long long)tile * PA_M + r;
         if (!tc_wait_elect(&ctl->head_full, tiles & 1, abort_flag)) goto done;
@@ -409,14 +404,13 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
         if (!tc_wait_elect(&ctl->head_full, tiles & 1, abort_flag)) goto done;
       }
       // the head of this tile is complete, so U is free: the next tile's FP16 parts go in before this tile's env step
-      if (tile + (int)gridDim.x < n_tiles) convert_u(tile + (int)gridDim.x);
+      if (next_tile < n_tiles) convert_u(next_tile);
+      if (!warm) { warm = true; continue; }
       if (!tc_wait_elect(&ctl->act_ready, tiles & 1, abort_flag)) goto done;
-      // z was stored long before the head finished; the wait orders the loads below after those stores
-      if (!tc_wait_elect(&ctl->z_stored, tiles & 1, abort_flag)) goto done;
       const float* zs = ev.z_scratch + ((size_t)blockIdx.x * 2 + (tiles & 1)) * (PA_M * D);
 #pragma unroll 1
-      for (int g = 0; g < 2; ++g) {
-        const int rr = ew * 16 + g * 8 + e_r8;
+      for (int g = 0; g < 4; ++g) {
+        const int rr = ew * 16 + g * 4 + e_r4;
         const long long row = (long long)tile * PA_M + rr;
         const bool live = row < p.n;
         const int action = ctl->act[tiles & 1][rr];
@@ -425,13 +419,13 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
         const float ret0 = live ? ev.ep_return[row] : 0.f;
         const float* Ba = ev.lgB_t + (size_t)action * D;     // B[a] times 2 log2(e)
         // s' = tanh(z + B[a]) + noise; piece k4 = components 4 k4 .. 4 k4 + 3 = one Philox block
-        float4 zz[8], sn[8];
+        float4 zz[4], sn[4];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) zz[i] = __ldcg(reinterpret_cast<const float4*>(zs + ((size_t)(e_kq + 4 * i) * PA_M + rr) * 4));
+        for (int i = 0; i < 4; ++i) zz[i] = __ldcg(reinterpret_cast<const float4*>(zs + ((size_t)(e_kq + 8 * i) * PA_M + rr) * 4));
         float sq = 0.f;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int k4 = e_kq + 4 * i;
+        for (int i = 0; i < 4; ++i) {
+          const int k4 = e_kq + 8 * i;
           const uint4 w = stream_words(ev.seed, STREAM_NOISE, (uint32_t)k4, (uint32_t)row, ev.t);
           const float2 n01 = box_muller_scaled(w.x, w.y, ev.noise_std), n23 = box_muller_scaled(w.z, w.w, ev.noise_std);
           const float4 bb = __ldg(reinterpret_cast<const float4*>(Ba + 4 * k4));
@@ -444,9 +438,10 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
           sn[i] = o;
           if (live) __stcs(reinterpret_cast<float4*>(rec + D + 4 * k4), o);
         }
-        // the four lanes of a row add their partial squared norms (same order in every lane)
+        // the eight lanes of a row add their partial squared norms (same order in every lane)
         sq += __shfl_xor_sync(0xffffffffu, sq, 1);
         sq += __shfl_xor_sync(0xffffffffu, sq, 2);
+        sq += __shfl_xor_sync(0xffffffffu, sq, 4);
         if (live) {
           const float rew = -sq / (float)D;
           int ep = ep0 + 1;
@@ -456,16 +451,16 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
           if (done) {
             ep_ret = 0.f;
             ep = 0;
-#pragma unroll 4
-            for (int i = 0; i < 8; ++i) {
-              const int k4 = e_kq + 4 * i;
+#pragma unroll 1
+            for (int i = 0; i < 4; ++i) {
+              const int k4 = e_kq + 8 * i;
               const uint4 w = stream_words(ev.seed, STREAM_RESET, (uint32_t)k4, (uint32_t)row, ev.t);
               *reinterpret_cast<float4*>(st + 4 * k4) = make_float4(uniform_range(w.x, -0.1f, 0.2f), uniform_range(w.y, -0.1f, 0.2f),
                                                                     uniform_range(w.z, -0.1f, 0.2f), uniform_range(w.w, -0.1f, 0.2f));
             }
           } else {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) *reinterpret_cast<float4*>(st + 4 * (e_kq + 4 * i)) = sn[i];
+            for (int i = 0; i < 4; ++i) *reinterpret_cast<float4*>(st + 4 * (e_kq + 8 * i)) = sn[i];
           }
           if (e_kq == 0) {
             *reinterpret_cast<float4*>(rec + 2 * D) =
@@ -479,6 +474,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
           }
         }
       }
+      ++tiles;
     }
     // episode statistics: one atomic pair per warp
     {
@@ -492,7 +488,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
         atomicAdd(&ev.stats->episodes, n);
         atomicAdd(&ev.stats->return_sum, rs);
       }
-      if (blockIdx.x == 0 && tid == 12 * 32) ev.block_ver[ev.slot0 / (unsigned long long)p.n] = ev.version;
+      if (blockIdx.x == 0 && tid == PA_ENV0 * 32) ev.block_ver[ev.slot0 / (unsigned long long)p.n] = ev.version;
     }
   }
 done:
