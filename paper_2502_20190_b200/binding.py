@@ -1,6 +1,8 @@
-"""ctypes binding of ``libtj.so`` (see ``include/tj.h``): argument marshalling only.
+"""Binding of ``libtj.so`` (see ``include/tj.h``): argument marshalling only.
 
-The module-level ``tj_*`` functions mirror the C ABI one to one.  ``Context`` is a
+The module-level ``tj_*`` functions mirror the C ABI one to one through ctypes; the calls that a training loop
+makes every iteration go through a small extension module (``csrc/tj_python.cpp``), which marshals them in a
+tenth of the time.  ``Context`` is a
 convenience wrapper that allocates the workspace and the output arrays with torch
 (device memory and the stream are torch's; every computation runs in the library's
 CUDA kernels).  There is no CPU fallback: without the compiled library or without a
@@ -9,9 +11,13 @@ CUDA device the calls raise.
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
+import operator
 import os
 
 import numpy as np
+
+from . import build as _build
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 # TJ_LIB_PATH names another build of the library (same ABI), e.g. one compiled with different options
@@ -69,11 +75,27 @@ class TjStats(C.Structure):
 
 
 _lib = None
+_calls = None
+
+# in the order tj_python.cpp's init() takes them
+_FAST = ("tj_actor_step", "tj_replay_sample", "tj_td_error", "tj_publish_weights", "tj_sgd_step", "tj_adam_step", "tj_ppo_step", "tj_gae",
+         "tj_normalize", "tj_segment_minibatch")
+
+
+def _load_calls(lib):
+    """The extension module with the per-iteration calls, bound to this library's functions; raises when it is not built."""
+    if not os.path.exists(_build.CALLS):
+        raise RuntimeError("%s is missing: build it with `python -m paper_2502_20190_b200.build`" % os.path.basename(_build.CALLS))
+    spec = importlib.util.spec_from_file_location("_tjcall", _build.CALLS)
+    m = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(m)
+    m.init(*[C.cast(getattr(lib, n), C.c_void_p).value for n in _FAST])
+    return m
 
 
 def load_library():
     """Load libtj.so; raises (never falls back) when it has not been built."""
-    global _lib
+    global _lib, _calls
     if _lib is not None:
         return _lib
     if not os.path.exists(LIB_PATH):
@@ -110,6 +132,7 @@ def load_library():
     for name in EXPORTS:
         if name != "tj_last_error":
             getattr(L, name).restype = C.c_int
+    _calls = _load_calls(L)
     _lib = L
     return L
 
@@ -146,9 +169,8 @@ def tj_wait(h, which: int, timeout_ms: int):
 
 
 def tj_publish_weights(h, blob_ptr: int, nbytes: int, on_device: int):
-    v = C.c_int64()
-    st = load_library().tj_publish_weights(h, blob_ptr, nbytes, on_device, C.byref(v))
-    return st, v.value
+    load_library()
+    return _calls.publish_weights(getattr(h, "value", h), blob_ptr or None, nbytes, on_device)
 
 
 def tj_actor_step(h, n_steps: int, dbg_logits_ptr: int = 0):
@@ -295,6 +317,10 @@ class Context:
         st, self.h = tj_create(self.cfg, self._ws_ptr, nbytes, self.stream.cuda_stream)
         if st != TJ_OK:
             raise TjError(st, tj_last_error())
+        self._addr = self.h.value                      # what the extension module's calls take
+        self._blobs = self._ptrs = None                # parameter blobs of the last update, already checked
+        self._segments = {}                            # views of the segment slots
+        self._one = torch.empty(1, dtype=torch.float32, device=self.device)
         c = self.cfg
         self.N, self.D, self.A, self.H, self.B = c.n_envs, c.obs_dim, c.n_actions, c.hidden, c.minibatch
         self.S_d = c.obs_dim if c.env_kind == 2 else 4
@@ -316,7 +342,8 @@ class Context:
     def close(self):
         if getattr(self, "h", None):
             tj_destroy(self.h)
-            self.h = None
+            self.h = self._addr = self._blobs = None
+            self._segments = {}
 
     def __del__(self):
         try:
@@ -325,9 +352,19 @@ class Context:
             pass
 
     def _check(self, st, ok=(TJ_OK,)):
-        if st not in ok:
+        if st and st not in ok:
             raise TjError(st, tj_last_error(self.h))
         return st
+
+    def _blob_ptrs(self, blobs):
+        """Addresses of parameter blobs (float32, contiguous, of one size); those of the last call need no second look."""
+        ptrs = tuple([x.data_ptr() for x in blobs])
+        if self._blobs is None or ptrs != self._ptrs or len(blobs) != len(self._blobs) or not all(map(operator.is_, blobs, self._blobs)):
+            f32, n = self.torch.float32, blobs[0].numel()
+            for x in blobs:
+                assert x.dtype == f32 and x.is_contiguous() and x.numel() == n
+            self._blobs, self._ptrs = blobs, ptrs
+        return ptrs
 
     def _view(self, ptr, shape, dtype):
         """torch view of a workspace address."""
@@ -343,19 +380,20 @@ class Context:
         torch = self.torch
         if isinstance(blob, torch.Tensor):
             assert blob.is_cuda and blob.dtype == torch.float32 and blob.is_contiguous()
-            st, v = tj_publish_weights(self.h, blob.data_ptr(), blob.numel() * 4, 1)
+            st, v = _calls.publish_weights(self._addr, blob.data_ptr(), blob.numel() * 4, 1)
         else:
             blob = np.ascontiguousarray(blob, np.float32)
-            st, v = tj_publish_weights(self.h, blob.ctypes.data, blob.size * 4, 0)
-        self._check(st)
+            st, v = _calls.publish_weights(self._addr, blob.ctypes.data, blob.size * 4, 0)
+        if st:
+            self._check(st)
         return v
 
     def actor_step(self, n_steps=1, dbg_logits=None):
-        ptr = 0
+        ptr = None
         if dbg_logits is not None:
             assert dbg_logits.is_cuda and dbg_logits.numel() >= n_steps * self.N * self.A
             ptr = dbg_logits.data_ptr()
-        return self._check(tj_actor_step(self.h, n_steps, ptr))
+        return self._check(_calls.actor_step(self._addr, n_steps, ptr))
 
     def alloc_batch(self, n=None):
         torch = self.torch
@@ -377,52 +415,44 @@ class Context:
             if self._batch is None:
                 self._batch = self.alloc_batch()
             batch = self._batch
-        st = tj_replay_sample(self.h, staleness_bound, batch["idx"].data_ptr(), batch["c"])
+        st = _calls.replay_sample(self._addr, staleness_bound, batch["idx"].data_ptr(), batch["c"])
         self._check(st, allow)
         return st, batch
 
     def td_error(self, batch, out=None):
-        torch = self.torch
-        n = batch["c"].n
         if out is None:
+            torch, n = self.torch, batch["c"].n
             out = dict(td=torch.empty(n, dtype=torch.float32, device=self.device),
                        huber=torch.empty(n, dtype=torch.float32, device=self.device),
                        loss=torch.empty(1, dtype=torch.float32, device=self.device))
-        self._check(tj_td_error(self.h, batch["c"], out["td"].data_ptr(), out["huber"].data_ptr(),
-                                out["loss"].data_ptr()))
+        self._check(_calls.td_error(self._addr, batch["c"], out["td"].data_ptr(), out["huber"].data_ptr(), out["loss"].data_ptr()))
         return out
 
     def sgd_step(self, batch, lr, theta, theta_target):
         """theta (updated in place) and theta_target: float32 device tensors in the publish layout; returns the loss tensor"""
-        torch = self.torch
-        assert theta.dtype == torch.float32 and theta_target.dtype == torch.float32
-        assert theta.is_contiguous() and theta_target.is_contiguous() and theta.numel() == theta_target.numel()
-        loss = torch.empty(1, dtype=torch.float32, device=self.device)
-        self._check(tj_sgd_step(self.h, batch["c"], float(lr), theta.data_ptr(), theta_target.data_ptr(), loss.data_ptr()))
+        t, tt = self._blob_ptrs((theta, theta_target))
+        loss = self._one.new_empty(1)
+        self._check(_calls.sgd_step(self._addr, batch["c"], lr, t, tt, loss.data_ptr()))
         return loss
 
     def adam_step(self, batch, lr, theta, theta_target, m, v, t, beta1=0.9, beta2=0.999, eps=1e-8):
-        torch = self.torch
-        for x in (theta, theta_target, m, v):
-            assert x.dtype == torch.float32 and x.is_contiguous() and x.numel() == theta.numel()
-        loss = torch.empty(1, dtype=torch.float32, device=self.device)
-        self._check(tj_adam_step(self.h, batch["c"], float(lr), float(beta1), float(beta2), float(eps), int(t), theta.data_ptr(),
-                                 theta_target.data_ptr(), m.data_ptr(), v.data_ptr(), loss.data_ptr()))
+        p, pt, pm, pv = self._blob_ptrs((theta, theta_target, m, v))
+        loss = self._one.new_empty(1)
+        self._check(_calls.adam_step(self._addr, batch["c"], lr, beta1, beta2, eps, t, p, pt, pm, pv, loss.data_ptr()))
         return loss
 
     def ppo_step(self, obs, act, logp_old, adv, ret, lr, theta, m, v, t, clip_eps=0.2, c_v=0.5, c_e=0.01, beta1=0.9,
                  beta2=0.999, eps=1e-8):
         """obs [n][D], act (int32), logp_old, adv, ret [n]: contiguous device tensors (views of a segment are fine);
         returns the 5 statistics tensor (loss, policy, value, entropy, clip fraction)"""
-        torch = self.torch
         n = act.numel()
-        for x_ in (obs, act, logp_old, adv, ret, theta, m, v):
+        for x_ in (obs, act, logp_old, adv, ret):
             assert x_.is_contiguous()
-        assert obs.numel() == n * self.D and act.dtype == torch.int32
-        stats = torch.empty(5, dtype=torch.float32, device=self.device)
-        b = TjPpoBatch(n, obs.data_ptr(), act.data_ptr(), logp_old.data_ptr(), adv.data_ptr(), ret.data_ptr())
-        self._check(tj_ppo_step(self.h, b, float(lr), float(beta1), float(beta2), float(eps), int(t), float(clip_eps), float(c_v),
-                                float(c_e), theta.data_ptr(), m.data_ptr(), v.data_ptr(), stats.data_ptr()))
+        assert obs.numel() == n * self.D and act.dtype == self.torch.int32
+        p, pm, pv = self._blob_ptrs((theta, m, v))
+        stats = self._one.new_empty(5)
+        self._check(_calls.ppo_step(self._addr, n, obs.data_ptr(), act.data_ptr(), logp_old.data_ptr(), adv.data_ptr(), ret.data_ptr(), lr,
+                                    beta1, beta2, eps, t, clip_eps, c_v, c_e, p, pm, pv, stats.data_ptr()))
         return stats
 
     def gae(self, rew, val, done, gamma, lam, adv=None, ret=None):
@@ -434,8 +464,7 @@ class Context:
             adv = torch.empty_like(rew)
         if ret is None:
             ret = torch.empty_like(rew)
-        self._check(tj_gae(self.h, rew.data_ptr(), val.data_ptr(), done.data_ptr(), T, N, gamma, lam, adv.data_ptr(),
-                           ret.data_ptr()))
+        self._check(_calls.gae(self._addr, rew.data_ptr(), val.data_ptr(), done.data_ptr(), T, N, gamma, lam, adv.data_ptr(), ret.data_ptr()))
         return adv, ret
 
     def segment_acquire(self, allow=(TJ_OK,)):
@@ -444,19 +473,21 @@ class Context:
         self._check(st, allow)
         if st != TJ_OK:
             return st, None
-        T, N, D = seg.T, seg.N, self.D
-        return st, dict(T=T, N=N, version=seg.version, c=seg,
-                        obs=self._view(seg.obs, (T, N, D), torch.float32), act=self._view(seg.act, (T, N), torch.int32),
-                        rew=self._view(seg.rew, (T, N), torch.float32), done=self._view(seg.done, (T, N), torch.uint8),
-                        logp=self._view(seg.logp, (T, N), torch.float32),
-                        val=self._view(seg.val, (T + 1, N), torch.float32))
+        views = self._segments.get(seg.obs)            # a slot's arrays stay where they are
+        if views is None:
+            T, N, D = seg.T, seg.N, self.D
+            views = self._segments[seg.obs] = dict(
+                obs=self._view(seg.obs, (T, N, D), torch.float32), act=self._view(seg.act, (T, N), torch.int32),
+                rew=self._view(seg.rew, (T, N), torch.float32), done=self._view(seg.done, (T, N), torch.uint8),
+                logp=self._view(seg.logp, (T, N), torch.float32), val=self._view(seg.val, (T + 1, N), torch.float32))
+        return st, dict(T=seg.T, N=seg.N, version=seg.version, c=seg, **views)
 
     def normalize(self, x, eps=1e-8, out=None):
         """(x - mean) / (std + eps) over all entries of a float32 device tensor, in the library's kernels."""
         assert x.is_cuda and x.dtype == self.torch.float32 and x.is_contiguous()
         if out is None:
             out = self.torch.empty_like(x)
-        self._check(tj_normalize(self.h, x.data_ptr(), x.numel(), float(eps), out.data_ptr()))
+        self._check(_calls.normalize(self._addr, x.data_ptr(), x.numel(), eps, out.data_ptr()))
         return out
 
     def alloc_minibatch(self, n):
@@ -471,7 +502,7 @@ class Context:
     def segment_minibatch(self, seg, adv, ret, shuffle_id, first, mb):
         """Rows at positions first .. first + n - 1 of shuffle `shuffle_id` of the segment, copied into the minibatch arrays."""
         assert adv.is_contiguous() and ret.is_contiguous() and adv.numel() == seg["T"] * seg["N"] == ret.numel()
-        self._check(tj_segment_minibatch(self.h, seg["c"], adv.data_ptr(), ret.data_ptr(), int(shuffle_id), int(first), mb["c"]))
+        self._check(_calls.segment_minibatch(self._addr, seg["c"], adv.data_ptr(), ret.data_ptr(), shuffle_id, first, mb["c"]))
         return mb
 
     def segment_check(self, seg, allow=(TJ_OK, TJ_ERR_STALE_SEGMENT)):
