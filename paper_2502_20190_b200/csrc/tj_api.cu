@@ -689,12 +689,13 @@ int tj_td_error_static(tj_ctx* x, const tj_batch* b, float* td_out, float* huber
 }
 
 namespace {
-// h1, h2, dh1, dh2 [rows][H] | g [rows][17] | loss partials | PPO statistic partials | W2^T [H][H] | gradient partial sums
+// h1, h2, dh1, dh2 [rows][H] | g [rows][17] | qt [rows][16] | loss partials | PPO statistic partials | W2^T [H][H] | gradient partial sums
 void lay_out_update_scratch(const tj_ctx* x, tj::SgdParams& p) {
   const size_t rows = ((size_t)x->sgd_rows + 15) / 16 * 16, RH = rows * (size_t)x->H;
   p.h1 = x->sgd_scratch; p.h2 = p.h1 + RH; p.dh1 = p.h2 + RH; p.dh2 = p.dh1 + RH;
   p.g = p.dh2 + RH;
-  p.partial = p.g + rows * 17;
+  p.qt = p.g + rows * 17;
+  p.partial = p.qt + rows * 16;
   p.stat_partial = p.partial + sgd_partial_floats(x->sgd_rows);
   p.w2t = p.stat_partial + 5 * (rows / 16) + 8;
   p.w2t += (4 - ((reinterpret_cast<uintptr_t>(p.w2t) / sizeof(float)) & 3)) & 3;   // 16-byte rows for the vector loads
@@ -726,8 +727,11 @@ int learner_update(tj_ctx* x, const tj_batch* b, float lr, float* theta, const f
   lay_out_update_scratch(x, p);
   p.ldg = x->A; p.value_head = 0;
   p.error = &x->dstats->error;
-  LaunchScope scope(x, TJ_K_SGD, tj::sgd_step_launches(p, loss_mean_out != nullptr), true, true);
+  int launches = 0;
+  p.launches = &launches;
+  LaunchScope scope(x, TJ_K_SGD, 0, true, true);
   cudaError_t e = launch_sgd_step(p, lr, adam, loss_mean_out, x->lstream);
+  x->hs.kernel_launches += launches;
   if (e != cudaSuccess) return cuda_fail(x, e, "learner update");
   learner_launched(x);
   return TJ_OK;
@@ -779,8 +783,11 @@ int tj_ppo_step(tj_ctx* x, const tj_ppo_batch* b, float lr, float beta1, float b
   a.m = m; a.v = v; a.beta1 = beta1; a.beta2 = beta2; a.eps = eps;
   a.c1 = (float)(1.0 - std::pow((double)beta1, (double)t));
   a.c2 = (float)(1.0 - std::pow((double)beta2, (double)t));
-  LaunchScope scope(x, TJ_K_SGD, tj::ppo_step_launches(p, stats_out != nullptr), true, true);
+  int launches = 0;
+  p.launches = &launches;
+  LaunchScope scope(x, TJ_K_SGD, 0, true, true);
   cudaError_t e = launch_ppo_step(p, lr, &a, stats_out, x->lstream);
+  x->hs.kernel_launches += launches;
   if (e != cudaSuccess) return cuda_fail(x, e, "PPO update");
   learner_launched(x);
   return TJ_OK;

@@ -130,6 +130,7 @@ struct SgdParams {
   float gamma, kappa;
   float *h1, *h2, *dh1, *dh2;  // scratch [n][H] each
   float* g;                    // scratch [n][A]: dL/dq, non-zero at the selected action only
+  float* qt;                   // scratch [n][A]: the target network's Q values (more than four outputs)
   float* partial;              // scratch: one Huber partial sum per 16 rows
   float* grad_partial;         // scratch: per row range one partial gradient laid out like the parameter blob
   float* w2t;                  // scratch [H][H]: W2 transposed, the backward pass's operand on the older tensor-core path
@@ -144,6 +145,7 @@ struct SgdParams {
   float clip_eps, c_v, c_e;
   float* stat_partial;         // scratch: five partial sums per 16 rows (loss, policy, value, entropy, clipped rows)
   unsigned long long* error;   // device error word of the context (a bounded wait that ran out)
+  int* launches;               // host: raised by the kernels an update launches
 };
 
 struct AdamParams {
@@ -299,8 +301,6 @@ int sgd_partial_count(int n);
 bool sgd_supported(int D, int H, int A);
 cudaError_t launch_sgd_step(const SgdParams& p, float lr, const AdamParams* adam /* nullable: plain SGD */, float* loss_out /* nullable */,
                             cudaStream_t s);
-int sgd_step_launches(const SgdParams& p, bool with_loss);   // kernels one launch_sgd_step call launches (the path depends on the shape)
-int ppo_step_launches(const SgdParams& p, bool with_stats);
 cudaError_t launch_ppo_step(const SgdParams& p, float lr, const AdamParams* adam, float* stats_out /* device [5], nullable */,
                             cudaStream_t s);
 int td_static_max_rows();

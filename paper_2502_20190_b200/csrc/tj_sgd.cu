@@ -13,134 +13,15 @@ namespace tj {
 
 namespace {
 
-constexpr int SG_ROWS = 16;       // minibatch rows per thread block in the forward and backward kernels
-constexpr int SG_THREADS = 256;
-
-constexpr int SG_KT = 32;         // K columns of the weight tile staged in shared memory
-
-// one dense layer for SG_ROWS rows at once: out[i][r] = (relu)(b[i] + sum_k W[i][k] in[k][r]); activations live in shared
-// memory k-major, so a step of the inner loop is one weight times 16 broadcast values.  The weights (row-major out x in)
-// pass through a 256 x 32 shared-memory tile so that the global loads run along k, 128 contiguous bytes per row.
-template <bool RELU>
-__device__ __forceinline__ void sg_dense(const float* __restrict__ W, const float* __restrict__ b, int n_out, int n_in,
-                                         const float* in, float* out, float* wt) {
-  for (int i0 = 0; i0 < n_out; i0 += SG_THREADS) {
-    const int i = i0 + threadIdx.x;
-    float acc[SG_ROWS];
-    const float bi = i < n_out ? b[i] : 0.f;
-#pragma unroll
-    for (int r = 0; r < SG_ROWS; ++r) acc[r] = bi;
-    for (int k0 = 0; k0 < n_in; k0 += SG_KT) {
-      __syncthreads();
-      for (int t = threadIdx.x; t < SG_THREADS * SG_KT; t += SG_THREADS) {
-        const int ii = t / SG_KT, kk = t % SG_KT;
-        wt[ii * (SG_KT + 1) + kk] = (i0 + ii < n_out && k0 + kk < n_in) ? __ldg(W + (size_t)(i0 + ii) * n_in + k0 + kk) : 0.f;
-      }
-      __syncthreads();
-      const int kn = n_in - k0 < SG_KT ? n_in - k0 : SG_KT;
-      for (int kk = 0; kk < kn; ++kk) {
-        const float wk = wt[threadIdx.x * (SG_KT + 1) + kk];
-        const float4* a = reinterpret_cast<const float4*>(in + (size_t)(k0 + kk) * SG_ROWS);
-#pragma unroll
-        for (int r4 = 0; r4 < SG_ROWS / 4; ++r4) {
-          const float4 v = a[r4];
-          acc[4 * r4 + 0] = fmaf(wk, v.x, acc[4 * r4 + 0]);
-          acc[4 * r4 + 1] = fmaf(wk, v.y, acc[4 * r4 + 1]);
-          acc[4 * r4 + 2] = fmaf(wk, v.z, acc[4 * r4 + 2]);
-          acc[4 * r4 + 3] = fmaf(wk, v.w, acc[4 * r4 + 3]);
-        }
-      }
-    }
-    if (i < n_out) {
-#pragma unroll
-      for (int r = 0; r < SG_ROWS; ++r) out[(size_t)i * SG_ROWS + r] = RELU ? fmaxf(acc[r], 0.f) : acc[r];
-    }
-  }
-}
-
-// shared memory: xs [D][16] | a1 [H][16] | a2 [H][16] | qs [A][16] | weight tile [256][33]
-__global__ void __launch_bounds__(SG_THREADS) sgd_forward_kernel(const SgdParams p) {
-  chain_begin();
-  extern __shared__ __align__(16) float sg_sm[];
-  const int D = p.D, H = p.H, A = p.A;
-  float* xs = sg_sm;
-  float* a1 = xs + (size_t)D * SG_ROWS;
-  float* a2 = a1 + (size_t)H * SG_ROWS;
-  float* qs = a2 + (size_t)H * SG_ROWS;
-  float* wt = qs + (size_t)A * SG_ROWS;
-  __shared__ float qsel[SG_ROWS], hub[SG_ROWS];
-  const int row0 = blockIdx.x * SG_ROWS;
-  const float *W1 = p.theta, *b1 = W1 + (size_t)H * D, *W2 = b1 + H, *b2 = W2 + (size_t)H * H, *W3 = b2 + H, *b3 = W3 + (size_t)A * H;
-  const float *T1 = p.theta_target, *tb1 = T1 + (size_t)H * D, *T2 = tb1 + H, *tb2 = T2 + (size_t)H * H, *T3 = tb2 + H,
-              *tb3 = T3 + (size_t)A * H;
-  // ---- online network on obs; h1 and h2 are kept for the backward pass
-  for (int i = threadIdx.x; i < D * SG_ROWS; i += SG_THREADS) {
-    const int k = i / SG_ROWS, r = i % SG_ROWS;
-    xs[i] = row0 + r < p.n ? p.obs[(size_t)(row0 + r) * D + k] : 0.f;
-  }
-  __syncthreads();
-  sg_dense<true>(W1, b1, H, D, xs, a1, wt);
-  __syncthreads();
-  sg_dense<true>(W2, b2, H, H, a1, a2, wt);
-  __syncthreads();
-  sg_dense<false>(W3, b3, A, H, a2, qs, wt);
-  for (int i = threadIdx.x; i < H * SG_ROWS; i += SG_THREADS) {
-    const int k = i / SG_ROWS, r = i % SG_ROWS;
-    if (row0 + r < p.n) {
-      p.h1[(size_t)(row0 + r) * H + k] = a1[i];
-      p.h2[(size_t)(row0 + r) * H + k] = a2[i];
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x < SG_ROWS && row0 + threadIdx.x < p.n) {
-    int a = p.act[row0 + threadIdx.x];
-    a = a < 0 ? 0 : (a >= A ? A - 1 : a);
-    qsel[threadIdx.x] = qs[(size_t)a * SG_ROWS + threadIdx.x];
-  }
-  __syncthreads();
-  // ---- target network on next_obs
-  for (int i = threadIdx.x; i < D * SG_ROWS; i += SG_THREADS) {
-    const int k = i / SG_ROWS, r = i % SG_ROWS;
-    xs[i] = row0 + r < p.n ? p.next_obs[(size_t)(row0 + r) * D + k] : 0.f;
-  }
-  __syncthreads();
-  sg_dense<true>(T1, tb1, H, D, xs, a1, wt);
-  __syncthreads();
-  sg_dense<true>(T2, tb2, H, H, a1, a2, wt);
-  __syncthreads();
-  sg_dense<false>(T3, tb3, A, H, a2, qs, wt);
-  __syncthreads();
-  if (threadIdx.x < SG_ROWS) {
-    const int r = threadIdx.x, j = row0 + r;
-    float h = 0.f;
-    if (j < p.n) {
-      float qmax = qs[r];
-      for (int i = 1; i < A; ++i) qmax = fmaxf(qmax, qs[(size_t)i * SG_ROWS + r]);
-      const float y = p.rew[j] + p.gamma * (p.done[j] ? 0.f : 1.f) * qmax;
-      const float delta = y - qsel[r], ad = fabsf(delta);
-      h = ad <= p.kappa ? 0.5f * delta * delta : p.kappa * (ad - 0.5f * p.kappa);
-      const float gj = -fminf(fmaxf(delta, -p.kappa), p.kappa) / (float)p.n;
-      int a = p.act[j];
-      a = a < 0 ? 0 : (a >= A ? A - 1 : a);
-      for (int i = 0; i < A; ++i) p.g[(size_t)j * A + i] = i == a ? gj : 0.f;
-    }
-    hub[r] = h;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float s = 0.f;
-    for (int r = 0; r < SG_ROWS; ++r) s += hub[r];
-    p.partial[blockIdx.x] = s;
-  }
-}
+constexpr int SG_ROWS = 16;       // minibatch rows per loss partial
 
 // ---------------------------------------------------------------------------------------------------------------------
 // Wide networks and large minibatches: the layers as tiled FP32 matrix products (a weight element is reused for 128 rows
 // instead of 16).  C[m][n] = epi(sum_k A[m][k] Bop[k][n]): A row-major M x K.  B_KN false: B is N x K row-major (a weight
 // matrix as the forward pass uses it, Bop = B^T); true: B is K x N row-major (the same matrix in the backward pass).
-// 128 x 64 tile per block (32 x 64 for the heads, whose few outputs would leave most SMs idle with tall tiles), 16 k per
-// step, each thread 8 x 4 (2 x 4); k ascending, one accumulator per output: a fixed order.
-constexpr int GM_BM = 128, GM_BN = 64, GM_BK = 16, GM_THREADS = 256;
+// 128 x 64 tile per block (64 or 32 rows where tall tiles would leave SMs idle), 16 k per step, each thread 8 x 4 (4 x 4,
+// 2 x 4); k ascending, one accumulator per output: a fixed order.
+constexpr int GM_BN = 64, GM_BK = 16, GM_THREADS = 256;
 
 template <bool B_KN, int EPI, int BM>
 __device__ __forceinline__ void sg_gemm_body(const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb,
@@ -225,6 +106,9 @@ __device__ __forceinline__ void sg_gemm_body(const float* __restrict__ A, int ld
         const float4 a1 = *reinterpret_cast<const float4*>(&As[kk][ty * 8 + 4]);
         av[0] = a0.x; av[1] = a0.y; av[2] = a0.z; av[3] = a0.w;
         av[RM - 4] = a1.x; av[RM - 3] = a1.y; av[RM - 2] = a1.z; av[RM - 1] = a1.w;
+      } else if constexpr (RM == 4) {
+        const float4 a0 = *reinterpret_cast<const float4*>(&As[kk][ty * 4]);
+        av[0] = a0.x; av[1] = a0.y; av[2] = a0.z; av[3] = a0.w;
       } else {
 #pragma unroll
         for (int i = 0; i < RM; ++i) av[i] = As[kk][ty * RM + i];
@@ -255,21 +139,14 @@ __device__ __forceinline__ void sg_gemm_body(const float* __restrict__ A, int ld
   }
 }
 
-template <bool B_KN, int EPI, int BM>
-__global__ void __launch_bounds__(GM_THREADS) sg_gemm_kernel(const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb,
-                                                             float* __restrict__ C, int ldc, int M, int N, int K,
-                                                             const float* __restrict__ bias, const float* __restrict__ mask, int ldm) {
-  chain_begin();
-  sg_gemm_body<B_KN, EPI, BM>(A, lda, B, ldb, C, ldc, M, N, K, bias, mask, ldm);
-}
-
-// the same product for two operand sets of one shape in one launch (the two networks' heads): blockIdx.z picks the set
+// one product, or the same product for two operand sets of one shape (the two networks): blockIdx.z picks the set
 struct GemmPair { const float* A[2]; const float* B[2]; float* C[2]; const float* bias[2]; };
 template <bool B_KN, int EPI, int BM>
-__global__ void __launch_bounds__(GM_THREADS) sg_gemm_pair_kernel(const GemmPair pr, int lda, int ldb, int ldc, int M, int N, int K) {
+__global__ void __launch_bounds__(GM_THREADS) sg_gemm_kernel(const GemmPair pr, int lda, int ldb, int ldc, int M, int N, int K,
+                                                             const float* __restrict__ mask, int ldm) {
   chain_begin();
   const int z = blockIdx.z;
-  sg_gemm_body<B_KN, EPI, BM>(pr.A[z], lda, pr.B[z], ldb, pr.C[z], ldc, M, N, K, pr.bias[z], nullptr, 0);
+  sg_gemm_body<B_KN, EPI, BM>(pr.A[z], lda, pr.B[z], ldb, pr.C[z], ldc, M, N, K, pr.bias[z], mask, ldm);
 }
 
 // The heads of both networks for wide hidden layers: out[row][a] = bias[a] + sum_k h[row][k] W[a][k], a < A <= 16, H a
@@ -337,11 +214,19 @@ __global__ void __launch_bounds__(256) sg_heads_kernel(const GemmPair pr, int n_
   }
 }
 
-template <bool B_KN, int EPI, int BM = GM_BM>
-void sg_gemm(const float* A, int lda, const float* B, int ldb, float* C, int ldc, int M, int N, int K, const float* bias,
-             const float* mask, int ldm, cudaStream_t s) {
-  launch_chained(sg_gemm_kernel<B_KN, EPI, BM>, dim3((N + GM_BN - 1) / GM_BN, (M + BM - 1) / BM), GM_THREADS, 0, s, A, lda, B, ldb, C, ldc, M, N, K,
-                 bias, mask, ldm);
+// Tile height: the tallest of 128, 64, 32 rows that still gives every SM a block; a product that has too few tiles even so
+// is bound by its chain of k-steps.
+template <bool B_KN, int EPI>
+cudaError_t sg_gemm(const SgdParams& p, const GemmPair& pr, int sets, int lda, int ldb, int ldc, int M, int N, int K, const float* mask, int ldm,
+                    cudaStream_t s) {
+  const int cols = (N + GM_BN - 1) / GM_BN, sms = p.sm_count > 0 ? p.sm_count : 148;
+  ++*p.launches;
+  auto go = [&](auto kernel, int bm) {
+    return launch_chained(kernel, dim3(cols, (M + bm - 1) / bm, sets), GM_THREADS, 0, s, pr, lda, ldb, ldc, M, N, K, mask, ldm);
+  };
+  if ((long long)cols * ((M + 127) / 128) * sets >= sms) return go(sg_gemm_kernel<B_KN, EPI, 128>, 128);
+  if ((long long)cols * ((M + 63) / 64) * sets >= sms) return go(sg_gemm_kernel<B_KN, EPI, 64>, 64);
+  return go(sg_gemm_kernel<B_KN, EPI, 32>, 32);
 }
 
 // ---------------------------------------------------------------------------------------------------------------------
@@ -525,195 +410,202 @@ static bool tc_gemm_ok(const float* A, int lda, const float* B, int ldb, int M, 
          (reinterpret_cast<uintptr_t>(B) & 15) == 0 && K >= 32 && tiles >= 96;
 }
 
-// forward-layout product (B is N x K): tensor cores where the shape allows, the FMA tiles otherwise
+// forward-layout products (B is N x K) of both sets: tensor cores where the shape allows, the FMA tiles otherwise
 template <int EPI>
-cudaError_t sg_layer(const float* A, int lda, const float* B, int ldb, float* C, int ldc, int M, int N, int K, const float* bias,
-                     const float* mask, int ldm, unsigned long long* error, cudaStream_t s) {
-  if (tc_gemm_ok(A, lda, B, ldb, M, N, K)) {
-    return launch_chained(sg_gemm_tc_kernel<EPI>, dim3((N + TG_N - 1) / TG_N, (M + TG_M - 1) / TG_M), TG_THREADS, TG_SMEM_BYTES, s, A, lda, B, ldb,
-                          C, ldc, M, N, K, bias, mask, ldm, error);
-  } else {
-    sg_gemm<false, EPI>(A, lda, B, ldb, C, ldc, M, N, K, bias, mask, ldm, s);
+cudaError_t sg_layer(const SgdParams& p, const GemmPair& pr, int sets, int lda, int ldb, int ldc, int M, int N, int K, const float* mask, int ldm,
+                     cudaStream_t s) {
+  bool tc = N >= 128;
+  for (int z = 0; z < sets; ++z) tc = tc && tc_gemm_ok(pr.A[z], lda, pr.B[z], ldb, M, N, K);
+  if (!tc) return sg_gemm<false, EPI>(p, pr, sets, lda, ldb, ldc, M, N, K, mask, ldm, s);
+  for (int z = 0; z < sets; ++z) {
+    ++*p.launches;
+    const cudaError_t e = launch_chained(sg_gemm_tc_kernel<EPI>, dim3((N + TG_N - 1) / TG_N, (M + TG_M - 1) / TG_M), TG_THREADS, TG_SMEM_BYTES, s, pr.A[z],
+                                         lda, pr.B[z], ldb, pr.C[z], ldc, M, N, K, pr.bias[z], mask, ldm, p.error);
+    if (e != cudaSuccess) return e;
   }
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
-// TD error, Huber loss and its gradient at the outputs from the two networks' Q values: q (in) and g (out) share p.g
-// ([n][A]: a row is read, then overwritten by its own thread), qt [n][A]; loss partials per SG_ROWS rows as in the
-// fused forward kernel
-__global__ void __launch_bounds__(32) sgd_loss_kernel(const SgdParams p, const float* __restrict__ qt) {
+// Heads, loss, its gradient at the outputs and dh2 for at most four outputs, a warp per minibatch row: the row of h2 (and of the target
+// network's) against the few head rows, summed by shuffles; then dh2[i] = sum_a g[a] W3[a][i] (+ g[A] Wv[i]) where h2[i] > 0, the row
+// still in L1.  Bound by reading h2 twice and writing dh2 (as a 32-row product tile per head, a loss kernel and a product with K = A
+// this was four launches and 37 us for 4,096 rows x 256 units).  Loss partials per SG_ROWS rows.
+template <bool PPO>
+__global__ void __launch_bounds__(256) sgd_rows_kernel(const SgdParams p, const float* t2) {
+  __shared__ float part[5][SG_ROWS];
   chain_begin();
-  chain_next();
-  __shared__ float hub[SG_ROWS];
-  const int r = threadIdx.x, j = blockIdx.x * SG_ROWS + r, A = p.A;
-  if (r < SG_ROWS) {
-    float h = 0.f;
+  const int H = p.H, D = p.D, A = p.A, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const float *W3 = p.theta + (size_t)H * D + H + (size_t)H * H + H, *b3 = W3 + (size_t)A * H, *Wv = b3 + A;
+  const float *T3 = p.theta_target + (size_t)H * D + H + (size_t)H * H + H, *tb3 = T3 + (size_t)A * H;
+#pragma unroll 1
+  for (int r = warp; r < SG_ROWS; r += 8) {
+    const int j = blockIdx.x * SG_ROWS + r;
+    float l[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
     if (j < p.n) {
-      int a = p.act[j];
-      a = a < 0 ? 0 : (a >= A ? A - 1 : a);
-      float* gr = p.g + (size_t)j * A;
-      const float qsel = gr[a];
-      const float* tr = qt + (size_t)j * A;
-      float qmax = tr[0];
-      for (int i = 1; i < A; ++i) qmax = fmaxf(qmax, tr[i]);
-      const float y = p.rew[j] + p.gamma * (p.done[j] ? 0.f : 1.f) * qmax;
-      const float delta = y - qsel, ad = fabsf(delta);
-      h = ad <= p.kappa ? 0.5f * delta * delta : p.kappa * (ad - 0.5f * p.kappa);
-      const float gj = -fminf(fmaxf(delta, -p.kappa), p.kappa) / (float)p.n;
-      for (int i = 0; i < A; ++i) gr[i] = i == a ? gj : 0.f;
+      const float* h = p.h2 + (size_t)j * H;
+      const float* t = PPO ? h : t2 + (size_t)j * H;
+      const int act0 = p.act[j], act = act0 < 0 ? 0 : (act0 >= A ? A - 1 : act0);
+      const float s0 = PPO ? p.logp_old[j] : p.rew[j], s1 = PPO ? p.adv[j] : 0.f, s2 = PPO ? p.ret[j] : 0.f;
+      const int dn = PPO ? 0 : p.done[j];
+      float q[4] = {0.f, 0.f, 0.f, 0.f}, qt[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int i = lane; i < H; i += 32) {
+        const float x = h[i], y = PPO ? 0.f : t[i];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          if (a < A) {
+            q[a] = fmaf(x, __ldg(W3 + a * H + i), q[a]);
+            if (!PPO) qt[a] = fmaf(y, __ldg(T3 + a * H + i), qt[a]);
+          } else if (PPO && a == A) {
+            q[a] = fmaf(x, __ldg(Wv + i), q[a]);
+          }
+        }
+      }
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        for (int o = 16; o > 0; o >>= 1) {
+          q[a] += __shfl_xor_sync(0xffffffffu, q[a], o);
+          if (!PPO) qt[a] += __shfl_xor_sync(0xffffffffu, qt[a], o);
+        }
+        if (a < A) {
+          q[a] += __ldg(b3 + a);
+          if (!PPO) qt[a] += __ldg(tb3 + a);
+        } else if (PPO && a == A) {
+          q[a] += __ldg(Wv + H);
+        }
+      }
+      float g[4] = {0.f, 0.f, 0.f, 0.f};
+      if (PPO) {
+        float lmax = q[0];
+#pragma unroll
+        for (int a = 1; a < 4; ++a)
+          if (a < A) lmax = fmaxf(lmax, q[a]);
+        float Z = 0.f, ent = 0.f, logp = 0.f, val = 0.f;
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+          if (a < A) Z += expf(q[a] - lmax);
+        const float logZ = lmax + logf(Z);
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          if (a < A) {
+            const float lp = q[a] - logZ;
+            ent -= expf(lp) * lp;
+            if (a == act) logp = lp;
+          } else if (a == A) {
+            val = q[a];
+          }
+        }
+        const float ratio = expf(logp - s0);
+        const float rc = fminf(fmaxf(ratio, 1.f - p.clip_eps), 1.f + p.clip_eps);
+        const float t1 = ratio * s1, t3 = rc * s1;
+        const bool unclipped = t1 <= t3;
+        const float dv = val - s2, inv_n = 1.f / (float)p.n, g_logp = unclipped ? -s1 * ratio : 0.f;
+        l[1] = -(unclipped ? t1 : t3);
+        l[2] = 0.5f * dv * dv;
+        l[3] = ent;
+        l[4] = unclipped ? 0.f : 1.f;
+        l[0] = l[1] + p.c_v * l[2] - p.c_e * l[3];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          if (a < A) {
+            const float lp = q[a] - logZ, pi = expf(lp);
+            const float dlogp = (a == act ? 1.f : 0.f) - pi, dent = -pi * (lp + ent);
+            g[a] = (g_logp * dlogp - p.c_e * dent) * inv_n;
+          } else if (a == A) {
+            g[a] = p.c_v * dv * inv_n;
+          }
+        }
+      } else {
+        float qmax = qt[0], qs = 0.f;
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          if (a > 0 && a < A) qmax = fmaxf(qmax, qt[a]);
+          if (a == act) qs = q[a];
+        }
+        const float delta = s0 + p.gamma * (dn ? 0.f : 1.f) * qmax - qs, ad = fabsf(delta);
+        l[0] = ad <= p.kappa ? 0.5f * delta * delta : p.kappa * (ad - 0.5f * p.kappa);
+        const float gj = -fminf(fmaxf(delta, -p.kappa), p.kappa) / (float)p.n;
+#pragma unroll
+        for (int a = 0; a < 4; ++a) g[a] = a == act ? gj : 0.f;
+      }
+      if (lane == 0) {
+        float* gr = p.g + (size_t)j * p.ldg;
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+          if (a < p.ldg) gr[a] = g[a];
+      }
+      float* d = p.dh2 + (size_t)j * H;            // for the Q head t2 is this very row: every lane has read its entries above
+      __syncwarp();
+      for (int i = lane; i < H; i += 32) {
+        float v = 0.f;
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          if (a < A) v = fmaf(g[a], __ldg(W3 + a * H + i), v);
+          else if (PPO && a == A) v = fmaf(g[a], __ldg(Wv + i), v);
+        }
+        d[i] = h[i] > 0.f ? v : 0.f;
+      }
     }
-    hub[r] = h;
+    if (lane == 0)
+#pragma unroll
+      for (int k = 0; k < (PPO ? 5 : 1); ++k) part[k][r] = l[k];
   }
-  __syncwarp();
-  if (r == 0) {
+  __syncthreads();
+  if (threadIdx.x < (PPO ? 5 : 1)) {
     float s = 0.f;
-    for (int i = 0; i < SG_ROWS; ++i) s += hub[i];
+    for (int r = 0; r < SG_ROWS; ++r) s += part[threadIdx.x][r];
+    if (PPO) p.stat_partial[(size_t)blockIdx.x * 5 + threadIdx.x] = s;
+    else p.partial[blockIdx.x] = s;
+  }
+}
+
+// The same from Q values that other kernels computed, for more outputs: q (in) and g (out) share p.g ([n][A], a row is read before its
+// own warp overwrites it), qt [n][A]; dh2 has one term per entry, the selected action's.
+__global__ void __launch_bounds__(256) sgd_loss_kernel(const SgdParams p) {
+  __shared__ float part[SG_ROWS];
+  chain_begin();
+  const int H = p.H, D = p.D, A = p.A, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const float* W3 = p.theta + (size_t)H * D + H + (size_t)H * H + H;
+#pragma unroll 1
+  for (int r = warp; r < SG_ROWS; r += 8) {
+    const int j = blockIdx.x * SG_ROWS + r;
+    float l = 0.f;
+    if (j < p.n) {
+      const int act0 = p.act[j], act = act0 < 0 ? 0 : (act0 >= A ? A - 1 : act0);
+      float* gr = p.g + (size_t)j * A;
+      const float* tr = p.qt + (size_t)j * A;
+      float qmax = lane < A ? tr[lane] : -INFINITY;            // A <= 16 outputs
+      for (int o = 16; o > 0; o >>= 1) qmax = fmaxf(qmax, __shfl_xor_sync(0xffffffffu, qmax, o));
+      const float delta = p.rew[j] + p.gamma * (p.done[j] ? 0.f : 1.f) * qmax - gr[act], ad = fabsf(delta);
+      l = ad <= p.kappa ? 0.5f * delta * delta : p.kappa * (ad - 0.5f * p.kappa);
+      const float gj = -fminf(fmaxf(delta, -p.kappa), p.kappa) / (float)p.n;
+      __syncwarp();
+      if (lane < A) gr[lane] = lane == act ? gj : 0.f;
+      const float* h = p.h2 + (size_t)j * H;
+      const float* w = W3 + (size_t)act * H;
+      float* d = p.dh2 + (size_t)j * H;
+#pragma unroll 4
+      for (int i = lane; i < H; i += 32) d[i] = h[i] > 0.f ? gj * __ldg(w + i) : 0.f;
+    }
+    if (lane == 0) part[r] = l;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float s = 0.f;
+    for (int r = 0; r < SG_ROWS; ++r) s += part[r];
     p.partial[blockIdx.x] = s;
   }
 }
 
-// On-policy forward (PPO): trunk, policy head and value head of the one network; per row the clipped surrogate, the value
-// loss and the entropy, and their gradients at the outputs: g[j][0..A) for the logits, g[j][A] for the value.
-// shared memory: xs [D][16] | a1 [H][16] | a2 [H][16] | qs [A + 1][16] | weight tile [256][33]
-__global__ void __launch_bounds__(SG_THREADS) ppo_forward_kernel(const SgdParams p) {
-  chain_begin();
-  extern __shared__ __align__(16) float sg_sm[];
-  const int D = p.D, H = p.H, A = p.A;
-  float* xs = sg_sm;
-  float* a1 = xs + (size_t)D * SG_ROWS;
-  float* a2 = a1 + (size_t)H * SG_ROWS;
-  float* qs = a2 + (size_t)H * SG_ROWS;
-  float* wt = qs + (size_t)(A + 1) * SG_ROWS;
-  __shared__ float part[5][SG_ROWS];
-  const int row0 = blockIdx.x * SG_ROWS;
-  const float *W1 = p.theta, *b1 = W1 + (size_t)H * D, *W2 = b1 + H, *b2 = W2 + (size_t)H * H, *W3 = b2 + H, *b3 = W3 + (size_t)A * H,
-              *Wv = b3 + A, *bv = Wv + H;
-  for (int i = threadIdx.x; i < D * SG_ROWS; i += SG_THREADS) {
-    const int k = i / SG_ROWS, r = i % SG_ROWS;
-    xs[i] = row0 + r < p.n ? p.obs[(size_t)(row0 + r) * D + k] : 0.f;
-  }
-  __syncthreads();
-  sg_dense<true>(W1, b1, H, D, xs, a1, wt);
-  __syncthreads();
-  sg_dense<true>(W2, b2, H, H, a1, a2, wt);
-  __syncthreads();
-  sg_dense<false>(W3, b3, A, H, a2, qs, wt);
-  sg_dense<false>(Wv, bv, 1, H, a2, qs + (size_t)A * SG_ROWS, wt);
-  for (int i = threadIdx.x; i < H * SG_ROWS; i += SG_THREADS) {
-    const int k = i / SG_ROWS, r = i % SG_ROWS;
-    if (row0 + r < p.n) {
-      p.h1[(size_t)(row0 + r) * H + k] = a1[i];
-      p.h2[(size_t)(row0 + r) * H + k] = a2[i];
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x < SG_ROWS) {
-    const int r = threadIdx.x, j = row0 + r;
-    float l_tot = 0.f, l_pi = 0.f, l_v = 0.f, l_h = 0.f, l_c = 0.f;
-    if (j < p.n) {
-      int a = p.act[j];
-      a = a < 0 ? 0 : (a >= A ? A - 1 : a);
-      float lmax = qs[r];
-      for (int i = 1; i < A; ++i) lmax = fmaxf(lmax, qs[(size_t)i * SG_ROWS + r]);
-      float Z = 0.f;
-      for (int i = 0; i < A; ++i) Z += expf(qs[(size_t)i * SG_ROWS + r] - lmax);
-      const float logZ = lmax + logf(Z);
-      float ent = 0.f;
-      for (int i = 0; i < A; ++i) {
-        const float lp = qs[(size_t)i * SG_ROWS + r] - logZ;
-        ent -= expf(lp) * lp;
-      }
-      const float logp = qs[(size_t)a * SG_ROWS + r] - logZ;
-      const float ratio = expf(logp - p.logp_old[j]), Aj = p.adv[j];
-      const float rc = fminf(fmaxf(ratio, 1.f - p.clip_eps), 1.f + p.clip_eps);
-      const float t1 = ratio * Aj, t2 = rc * Aj;
-      const bool unclipped = t1 <= t2;
-      const float val = qs[(size_t)A * SG_ROWS + r], dv = val - p.ret[j];
-      l_pi = -(unclipped ? t1 : t2);
-      l_c = unclipped ? 0.f : 1.f;
-      l_v = 0.5f * dv * dv;
-      l_h = ent;
-      l_tot = l_pi + p.c_v * l_v - p.c_e * l_h;
-      const float g_logp = unclipped ? -Aj * ratio : 0.f, inv_n = 1.f / (float)p.n;
-      float* gr = p.g + (size_t)j * p.ldg;
-      for (int i = 0; i < A; ++i) {
-        const float lp = qs[(size_t)i * SG_ROWS + r] - logZ, pi = expf(lp);
-        const float dlogp = (i == a ? 1.f : 0.f) - pi;
-        const float dent = -pi * (lp + ent);
-        gr[i] = (g_logp * dlogp - p.c_e * dent) * inv_n;
-      }
-      gr[A] = p.c_v * dv * inv_n;
-    }
-    part[0][r] = l_tot; part[1][r] = l_pi; part[2][r] = l_v; part[3][r] = l_h; part[4][r] = l_c;
-  }
-  __syncthreads();
-  if (threadIdx.x < 5) {
-    float s = 0.f;
-    for (int r = 0; r < SG_ROWS; ++r) s += part[threadIdx.x][r];
-    p.stat_partial[(size_t)blockIdx.x * 5 + threadIdx.x] = s;
-  }
-}
-
-// out[k] = (sum over the blocks of partial k) / n, k = 0..4, blocks in ascending order
-__global__ void ppo_finish_kernel(const float* __restrict__ stat_partial, int n_blocks, int n, float* __restrict__ out) {
+// out[k] = (sum over the blocks of partial k) / n, k = 0..4: a warp per statistic, a fixed tree
+__global__ void __launch_bounds__(160) ppo_finish_kernel(const float* __restrict__ stat_partial, int n_blocks, int n, float* __restrict__ out) {
   chain_begin();
   chain_next();
-  const int k = threadIdx.x;
-  if (k >= 5) return;
+  const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float s = 0.f;
-  for (int b = 0; b < n_blocks; ++b) s += stat_partial[(size_t)b * 5 + k];
-  out[k] = s / (float)n;
+  for (int b = lane; b < n_blocks; b += 32) s += stat_partial[(size_t)b * 5 + k];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) out[k] = s / (float)n;
 }
-
-// backward through the activations, SG_ROWS rows per block: shared memory d2 [H][16]
-__global__ void __launch_bounds__(SG_THREADS) sgd_backward_kernel(const SgdParams p) {
-  chain_begin();
-  extern __shared__ __align__(16) float sg_sm[];
-  const int D = p.D, H = p.H, A = p.A;
-  float* d2 = sg_sm;
-  const int row0 = blockIdx.x * SG_ROWS;
-  const float* W2 = p.theta + (size_t)H * D + H;
-  const float* W3 = W2 + (size_t)H * H + H;
-  const float* Wv = W3 + (size_t)A * H + A;
-  // dh2[r][i] = sum_a g[r][a] W3[a][i] (+ g[r][A] Wv[i] with the value head) where h2 > 0; for the Q head g has one
-  // non-zero entry per row
-  for (int idx = threadIdx.x; idx < H * SG_ROWS; idx += SG_THREADS) {
-    const int r = idx / H, i = idx % H, j = row0 + r;
-    float v = 0.f;
-    if (j < p.n && p.h2[(size_t)j * H + i] > 0.f) {
-      const float* gr = p.g + (size_t)j * p.ldg;
-      for (int a = 0; a < A; ++a) v = fmaf(gr[a], W3[(size_t)a * H + i], v);
-      if (p.value_head) v = fmaf(gr[A], Wv[i], v);
-    }
-    d2[(size_t)i * SG_ROWS + r] = v;
-    if (j < p.n) p.dh2[(size_t)j * H + i] = v;
-  }
-  __syncthreads();
-  // dh1[r][k] = sum_i W2[i][k] dh2[r][i] where h1 > 0 (threads along k: the weight loads are coalesced)
-  for (int k = threadIdx.x; k < H; k += SG_THREADS) {
-    float acc[SG_ROWS];
-#pragma unroll
-    for (int r = 0; r < SG_ROWS; ++r) acc[r] = 0.f;
-    for (int i = 0; i < H; ++i) {
-      const float w = __ldg(W2 + (size_t)i * H + k);
-      const float4* a = reinterpret_cast<const float4*>(d2 + (size_t)i * SG_ROWS);
-#pragma unroll
-      for (int r4 = 0; r4 < SG_ROWS / 4; ++r4) {
-        const float4 v = a[r4];
-        acc[4 * r4 + 0] = fmaf(w, v.x, acc[4 * r4 + 0]);
-        acc[4 * r4 + 1] = fmaf(w, v.y, acc[4 * r4 + 1]);
-        acc[4 * r4 + 2] = fmaf(w, v.z, acc[4 * r4 + 2]);
-        acc[4 * r4 + 3] = fmaf(w, v.w, acc[4 * r4 + 3]);
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < SG_ROWS; ++r) {
-      const int j = row0 + r;
-      if (j < p.n) p.dh1[(size_t)j * H + k] = p.h1[(size_t)j * H + k] > 0.f ? acc[r] : 0.f;
-    }
-  }
-}
-
 
 // One gradient product of the update: C (M x N, at float offset `off` of the parameter blob) gets (Am rows)^T (Bm rows),
 // a bias (Bm == nullptr) a column of ones.  Tiles of all products are numbered in one list: tile_begin is this product's
@@ -813,14 +705,77 @@ __device__ __forceinline__ void grad_tile(float* __restrict__ P, const GradProdu
     }
 }
 
+// The gradients of narrow operands (obs_dim <= 8, at most four outputs): W1, both hidden biases, the head and its biases.  As 64-column
+// product tiles they were three of five tiles of an update and almost all padding.  Thread (s, n) sums neuron n of the block's 64
+// over rows s, s + 4, ... of the range; the four sums meet in shared memory.
+struct NarrowGrad {
+  const float *dh1, *dh2, *h2, *g, *obs;
+  int D, H, A, ldg, value_head, n_blocks;
+};
+
+__device__ __forceinline__ void grad_narrow_block(float* __restrict__ P, const NarrowGrad& d, int block, int j_begin, int j_end, float* sm) {
+  const int n = block * 64 + (threadIdx.x & 63), s = threadIdx.x >> 6, H = d.H, D = d.D, A = d.A;
+  float v[14];                                       // W1 [8] | b1 | b2 | head [4]
+#pragma unroll
+  for (int i = 0; i < 14; ++i) v[i] = 0.f;
+  if (n < H) {
+#pragma unroll 4
+    for (int j = j_begin + s; j < j_end; j += 4) {
+      const float d1 = d.dh1[(size_t)j * H + n], d2 = d.dh2[(size_t)j * H + n], h = d.h2[(size_t)j * H + n];
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (k < D) v[k] = fmaf(d1, __ldg(d.obs + (size_t)j * D + k), v[k]);
+      v[8] += d1;
+      v[9] += d2;
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+        if (a < d.ldg) v[10 + a] = fmaf(h, __ldg(d.g + (size_t)j * d.ldg + a), v[10 + a]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 14; ++i) sm[(s * 14 + i) * 64 + (threadIdx.x & 63)] = v[i];
+  __syncthreads();
+  const int o_b1 = H * D, o_b2 = o_b1 + H + H * H, o_W3 = o_b2 + H, o_b3 = o_W3 + A * H;
+  for (int i = threadIdx.x; i < 14 * 64; i += 256) {
+    const int c = i >> 6, nn = block * 64 + (i & 63);
+    const float t = (sm[i] + sm[i + 14 * 64]) + (sm[i + 2 * 14 * 64] + sm[i + 3 * 14 * 64]);
+    if (nn >= H) continue;
+    if (c < 8) {
+      if (c < D) P[nn * D + c] = t;
+    } else if (c < 10) {
+      P[(c == 8 ? o_b1 : o_b2) + nn] = t;
+    } else {
+      const int a = c - 10;
+      if (a < A) P[o_W3 + a * H + nn] = t;
+      else if (d.value_head && a == A) P[o_b3 + A + nn] = t;
+    }
+  }
+  if (block == 0 && threadIdx.x < 32 * 4) {          // output biases: a warp per output sums its column of g
+    const int a = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (a < d.ldg) {
+      float t = 0.f;
+      for (int j = j_begin + lane; j < j_end; j += 32) t += __ldg(d.g + (size_t)j * d.ldg + a);
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (lane == 0) P[a < A ? o_b3 + a : o_b3 + A + H] = t;
+    }
+  }
+}
+
 // Every gradient product of one update in a single launch: thread block (tile, range) sums, over its range of minibatch
 // rows, one tile of one product (128 x 64 where the product has at least 128 rows, else 64 x 64) and writes it to
 // P[range][off + m * N + n] -- a partial gradient laid out like the parameter blob itself, `count` floats per range.
 // No atomics: the apply kernel adds the ranges in order.
-__global__ void __launch_bounds__(256) sgd_grad_partial_kernel(float* __restrict__ P, const GradProducts gp, int count, int n_rows,
-                                                               int rows_per_range) {
+__global__ void __launch_bounds__(256) sgd_grad_partial_kernel(float* __restrict__ P, const GradProducts gp, const NarrowGrad narrow, int count,
+                                                               int n_rows, int rows_per_range) {
+  __shared__ __align__(16) float sm[4 * 14 * 64];
   chain_begin();
-  __shared__ __align__(16) float As[GP_ROWS][128 + 4], Bs[GP_ROWS][GP_TILE + 4];
+  if ((int)blockIdx.x >= gp.n_tiles) {
+    const int j_begin = blockIdx.y * rows_per_range, j_end = min(j_begin + rows_per_range, n_rows);
+    grad_narrow_block(P + (size_t)blockIdx.y * count, narrow, blockIdx.x - gp.n_tiles, j_begin, j_end, sm);
+    return;
+  }
+  float (*As)[128 + 4] = reinterpret_cast<float (*)[128 + 4]>(sm);
+  float (*Bs)[GP_TILE + 4] = reinterpret_cast<float (*)[GP_TILE + 4]>(sm + GP_ROWS * (128 + 4));
   int q = 0;
   while (q + 1 < gp.n && (int)blockIdx.x >= gp.g[q + 1].tile_begin) ++q;
   const GradProduct& d = gp.g[q];
@@ -878,56 +833,45 @@ size_t sgd_grad_partial_floats(int max_rows, int D, int H) {
 
 size_t sgd_scratch_floats(int max_rows, int D, int H) {
   const size_t rows = ((size_t)max_rows + SG_ROWS - 1) / SG_ROWS * SG_ROWS;
-  // h1, h2, dh1, dh2, g [rows][<= 16 actions + value], loss partials, PPO's five per 16 rows, partial gradients of the whole
+  // h1, h2, dh1, dh2, g [rows][<= 16 actions + value], qt [rows][<= 16], loss partials, PPO's five per 16 rows, partial gradients of the whole
   // parameter blob (at most 16 actions and a value head); W2 transposed
   // + split copies of W1 (x 2 networks), W2 (x 2) and W2^T for the tensor-core products
-  return 4 * rows * (size_t)H + rows * 17 + sgd_partial_floats(max_rows) + 5 * (rows / SG_ROWS) + 64 + (size_t)H * H +
+  return 4 * rows * (size_t)H + rows * 33 + sgd_partial_floats(max_rows) + 5 * (rows / SG_ROWS) + 64 + (size_t)H * H +
          sgd_grad_partial_floats(max_rows, D, H) + 2 * tc_pack_floats(H, D) + 3 * tc_pack_floats(H, H) + 64;
 }
 
 int sgd_partial_count(int n) { return (n + SG_ROWS - 1) / SG_ROWS; }
 
-bool sgd_supported(int D, int H, int A) {
-  const size_t smem = (((size_t)D + 2 * (size_t)H + A) * SG_ROWS + (size_t)SG_THREADS * (SG_KT + 1)) * sizeof(float);
-  return H >= 1 && D >= 1 && A >= 1 && A <= 16 && smem <= 200 * 1024;
-}
+bool sgd_supported(int D, int H, int A) { return H >= 1 && D >= 1 && A >= 1 && A <= 16; }
 
 namespace {
-// the tiled path pays off once a layer is a real matrix product; below that the fused per-16-rows kernels launch less
-bool use_tiled(const SgdParams& p) { return !p.value_head && p.H >= 128 && p.n >= 512; }
 // wide layers with enough 128 x 256 tiles: the pre-split tensor-core products (both hidden layers must qualify)
 bool use_tc2(const SgdParams& p) {
-  return use_tiled(p) && p.wpack && tc_gemm2_ok(p.obs, p.D, p.n, p.H, p.D) && tc_gemm2_ok(p.next_obs, p.D, p.n, p.H, p.D) &&
+  return !p.value_head && p.n >= 512 && p.wpack && tc_gemm2_ok(p.obs, p.D, p.n, p.H, p.D) && tc_gemm2_ok(p.next_obs, p.D, p.n, p.H, p.D) &&
          tc_gemm2_ok(p.h1, p.H, p.n, p.H, p.H);
 }
 
-// the backward pass and every parameter update: C -= lr * (gradient rows)^T (input rows), a bias with a column of ones
+// dh1 = (dh2 W2) where h1 > 0, and every parameter update: C -= lr * (gradient rows)^T (input rows), a bias with a column of ones
 cudaError_t backward_and_update(const SgdParams& p, float lr, const AdamParams* adam, cudaStream_t s) {
   const int D = p.D, H = p.H, A = p.A;
-  const int grid = sgd_partial_count(p.n);
-  const size_t smem_b = (size_t)H * SG_ROWS * sizeof(float);
+  const float* W2m = p.theta + (size_t)H * D + H;
   cudaError_t e;
-  if (use_tiled(p)) {
-    // dh2 = (g W3) where h2 > 0; dh1 = (dh2 W2) where h1 > 0
-    const float* W2m = p.theta + (size_t)H * D + H;
-    const float* W3m = W2m + (size_t)H * H + H;
-    sg_gemm<true, GM_MASK>(p.g, p.ldg, W3m, H, p.dh2, H, p.n, H, A, nullptr, p.h2, H, s);
-    if (use_tc2(p)) {
-      // W2^T was split with the other weight matrices at the start of the step
-      TcGemmBatch b{};
-      b.g[0] = TcGemm{p.dh2, H, p.wpack + 2 * tc_pack_floats(H, D) + 2 * tc_pack_floats(H, H), p.dh1, H, p.n, H, H, nullptr, p.h1, H};
-      b.n = 1;
-      if ((e = launch_gemm_tc2(b, GM_MASK, p.error, s)) != cudaSuccess) return e;
-    } else if (tc_gemm_ok(p.dh2, H, p.w2t, H, p.n, H, H)) {
-      // the tensor-core product wants both operands K-major: dh1 = dh2 (W2^T)^T with W2^T written out first
-      if ((e = launch_chained(sg_transpose_kernel, dim3((H + 31) / 32, (H + 31) / 32), 256, 0, s, W2m, p.w2t, H)) != cudaSuccess) return e;
-      if ((e = sg_layer<GM_MASK>(p.dh2, H, p.w2t, H, p.dh1, H, p.n, H, H, nullptr, p.h1, H, p.error, s)) != cudaSuccess) return e;
-    } else {
-      sg_gemm<true, GM_MASK>(p.dh2, H, W2m, H, p.dh1, H, p.n, H, H, nullptr, p.h1, H, s);
-    }
+  if (use_tc2(p)) {
+    // W2^T was split with the other weight matrices at the start of the step
+    TcGemmBatch b{};
+    b.g[0] = TcGemm{p.dh2, H, p.wpack + 2 * tc_pack_floats(H, D) + 2 * tc_pack_floats(H, H), p.dh1, H, p.n, H, H, nullptr, p.h1, H};
+    b.n = 1;
+    ++*p.launches;
+    e = launch_gemm_tc2(b, GM_MASK, p.error, s);
+  } else if (!p.value_head && H >= 128 && tc_gemm_ok(p.dh2, H, p.w2t, H, p.n, H, H)) {
+    // the tensor-core product wants both operands K-major: dh1 = dh2 (W2^T)^T with W2^T written out first
+    ++*p.launches;
+    if ((e = launch_chained(sg_transpose_kernel, dim3((H + 31) / 32, (H + 31) / 32), 256, 0, s, W2m, p.w2t, H)) != cudaSuccess) return e;
+    e = sg_layer<GM_MASK>(p, GemmPair{{p.dh2}, {p.w2t}, {p.dh1}, {nullptr}}, 1, H, H, H, p.n, H, H, p.h1, H, s);
   } else {
-    if ((e = launch_chained(sgd_backward_kernel, grid, SG_THREADS, smem_b, s, p)) != cudaSuccess) return e;
+    e = sg_gemm<true, GM_MASK>(p, GemmPair{{p.dh2}, {W2m}, {p.dh1}, {nullptr}}, 1, H, H, H, p.n, H, H, p.h1, H, s);
   }
+  if (e != cudaSuccess) return e;
   float* W1 = p.theta;
   float* b1 = W1 + (size_t)H * D;
   float* W2 = b1 + H;
@@ -966,10 +910,16 @@ cudaError_t backward_and_update(const SgdParams& p, float lr, const AdamParams* 
       add(bias, M, 1, G, ldg, nullptr, 0);
     }
   };
-  product(W1, b1, H, D, p.dh1, H, p.obs, D);
-  product(W2, b2, H, H, p.dh2, H, p.h1, H);
-  product(W3, b3, A, H, p.g, p.ldg, p.h2, H);
-  if (p.value_head) product(Wv, bv, 1, H, p.g + A, p.ldg, p.h2, H);
+  NarrowGrad narrow{};
+  if (!tc_grads && D <= 8 && A + p.value_head <= 4) {
+    add(W2, H, H, p.dh2, H, p.h1, H);
+    narrow = NarrowGrad{p.dh1, p.dh2, p.h2, p.g, p.obs, D, H, A, p.ldg, p.value_head, (H + 63) / 64};
+  } else {
+    product(W1, b1, H, D, p.dh1, H, p.obs, D);
+    product(W2, b2, H, H, p.dh2, H, p.h1, H);
+    product(W3, b3, A, H, p.g, p.ldg, p.h2, H);
+    if (p.value_head) product(Wv, bv, 1, H, p.g + A, p.ldg, p.h2, H);
+  }
   // row ranges: with tensor-core tiles about one thread block per SM in all (a block costs a fixed ~10 us beside its rows);
   // otherwise 128 rows or more per range
   int n_ranges;
@@ -983,9 +933,11 @@ cudaError_t backward_and_update(const SgdParams& p, float lr, const AdamParams* 
   const int rows_per_range = ((p.n + n_ranges - 1) / n_ranges + 31) / 32 * 32;
   n_ranges = (p.n + rows_per_range - 1) / rows_per_range;
   const int count = (int)((p.value_head ? bv + 1 : b3 + A) - p.theta);
+  *p.launches += (tb.n ? 1 : 0) + (gp.n_tiles + narrow.n_blocks > 0 ? 1 : 0) + 1;
   if (tb.n && (e = launch_wgrad_tc(tb, p.grad_partial, count, p.n, rows_per_range, n_ranges, p.error, s)) != cudaSuccess) return e;
-  if (gp.n_tiles > 0 &&
-      (e = launch_chained(sgd_grad_partial_kernel, dim3(gp.n_tiles, n_ranges), 256, 0, s, p.grad_partial, gp, count, p.n, rows_per_range)) != cudaSuccess)
+  if (gp.n_tiles + narrow.n_blocks > 0 &&
+      (e = launch_chained(sgd_grad_partial_kernel, dim3(gp.n_tiles + narrow.n_blocks, n_ranges), 256, 0, s, p.grad_partial, gp, narrow, count, p.n,
+                          rows_per_range)) != cudaSuccess)
     return e;
   if (adam)
     return launch_chained(sgd_apply_adam_kernel, (count + 255) / 256, 256, 0, s, p.theta, adam->m, adam->v, p.grad_partial, count, n_ranges, lr,
@@ -994,96 +946,90 @@ cudaError_t backward_and_update(const SgdParams& p, float lr, const AdamParams* 
 }
 }  // namespace
 
-// launches of the backward pass and the update: dh2 and dh1 (with W2's transpose on the tensor-core path) or the fused
-// backward kernel, the grouped gradient products, the apply pass
-static int backward_launches(const SgdParams& p) {
-  if (!use_tiled(p)) return 3;
-  if (use_tc2(p)) return 2 + 2 + (tc_wgrad_ok(p.D, p.n) ? 0 : 1);   // hidden-width products always qualify; W1's by obs_dim
-  return (tc_gemm_ok(p.dh2, p.H, p.w2t, p.H, p.n, p.H, p.H) ? 3 : 2) + 2;
-}
-
-int sgd_step_launches(const SgdParams& p, bool with_loss) {
-  if (sgd_fused_ok(p.D, p.H, p.A, 0)) return 2;
-  return (use_tiled(p) ? (use_tc2(p) ? 5 : 7) : 1) + backward_launches(p) + (with_loss ? 1 : 0);
-}
-
-int ppo_step_launches(const SgdParams& p, bool with_stats) {
-  if (sgd_fused_ok(p.D, p.H, p.A, 1)) return 2;
-  return 1 + (with_stats ? 1 : 0) + backward_launches(p);
-}
-
 static cudaError_t sgd_step_layered(const SgdParams& p, float lr, const AdamParams* adam, cudaStream_t s) {
-  if (use_tiled(p)) {
-    const int n = p.n, D = p.D, H = p.H, A = p.A;
-    const float *W1 = p.theta, *b1 = W1 + (size_t)H * D, *W2 = b1 + H, *b2 = W2 + (size_t)H * H, *W3 = b2 + H, *b3 = W3 + (size_t)A * H;
-    const float *T1 = p.theta_target, *tb1 = T1 + (size_t)H * D, *T2 = tb1 + H, *tb2 = T2 + (size_t)H * H, *T3 = tb2 + H,
-                *tb3 = T3 + (size_t)A * H;
-    // online network: h1, h2 kept, Q values into g; target network: its activations borrow dh1 / dh2 (free until the
-    // backward pass), its Q values then take dh1's place
-    cudaError_t e;
-    if (use_tc2(p)) {
-      // both networks' weight matrices (and W2^T for the backward pass) split once, then each layer of both networks in one launch
-      float* pk_W1 = p.wpack;
-      float* pk_T1 = pk_W1 + tc_pack_floats(H, D);
-      float* pk_W2 = pk_T1 + tc_pack_floats(H, D);
-      float* pk_T2 = pk_W2 + tc_pack_floats(H, H);
-      float* pk_W2t = pk_T2 + tc_pack_floats(H, H);
-      TcPackJobs jobs{};
-      jobs.j[jobs.n++] = TcPackJob{W1, D, 0, H, D, pk_W1};
-      jobs.j[jobs.n++] = TcPackJob{T1, D, 0, H, D, pk_T1};
-      jobs.j[jobs.n++] = TcPackJob{W2, H, 0, H, H, pk_W2};
-      jobs.j[jobs.n++] = TcPackJob{T2, H, 0, H, H, pk_T2};
-      jobs.j[jobs.n++] = TcPackJob{W2, H, 1, H, H, pk_W2t};
-      if ((e = launch_pack_tf32_operands(jobs, s)) != cudaSuccess) return e;
-      TcGemmBatch l1{};
-      l1.g[0] = TcGemm{p.obs, D, pk_W1, p.h1, H, n, H, D, b1, nullptr, 0};
-      l1.g[1] = TcGemm{p.next_obs, D, pk_T1, p.dh1, H, n, H, D, tb1, nullptr, 0};
-      l1.n = 2;
-      if ((e = launch_gemm_tc2(l1, GM_BIAS_RELU, p.error, s)) != cudaSuccess) return e;
-      TcGemmBatch l2{};
-      l2.g[0] = TcGemm{p.h1, H, pk_W2, p.h2, H, n, H, H, b2, nullptr, 0};
-      l2.g[1] = TcGemm{p.dh1, H, pk_T2, p.dh2, H, n, H, H, tb2, nullptr, 0};
-      l2.n = 2;
-      if ((e = launch_gemm_tc2(l2, GM_BIAS_RELU, p.error, s)) != cudaSuccess) return e;
-      // both heads in one launch: Q of the online network into g, of the target network into dh1's place
-      GemmPair heads{{p.h2, p.dh2}, {W3, T3}, {p.g, p.dh1}, {b3, tb3}};
-      const size_t hd_smem = (size_t)H * 16 * sizeof(float);
-      if (H % 128 == 0 && A <= 16 && hd_smem <= 96 * 1024) {
-        e = launch_chained(sg_heads_kernel, dim3((n + HD_ROWS - 1) / HD_ROWS, 2), 256, hd_smem, s, heads, n, H, A, A);
-      } else {
-        e = launch_chained(sg_gemm_pair_kernel<false, GM_BIAS, 32>, dim3((A + GM_BN - 1) / GM_BN, (n + 31) / 32, 2), GM_THREADS, 0, s, heads, H, H, A, n, A, H);
-      }
-      if (e != cudaSuccess) return e;
-    } else {
-      if ((e = sg_layer<GM_BIAS_RELU>(p.obs, D, W1, D, p.h1, H, n, H, D, b1, nullptr, 0, p.error, s)) != cudaSuccess) return e;
-      if ((e = sg_layer<GM_BIAS_RELU>(p.h1, H, W2, H, p.h2, H, n, H, H, b2, nullptr, 0, p.error, s)) != cudaSuccess) return e;
-      sg_gemm<false, GM_BIAS, 32>(p.h2, H, W3, H, p.g, A, n, A, H, b3, nullptr, 0, s);
-      if ((e = sg_layer<GM_BIAS_RELU>(p.next_obs, D, T1, D, p.dh1, H, n, H, D, tb1, nullptr, 0, p.error, s)) != cudaSuccess) return e;
-      if ((e = sg_layer<GM_BIAS_RELU>(p.dh1, H, T2, H, p.dh2, H, n, H, H, tb2, nullptr, 0, p.error, s)) != cudaSuccess) return e;
-      sg_gemm<false, GM_BIAS, 32>(p.dh2, H, T3, H, p.dh1, A, n, A, H, tb3, nullptr, 0, s);
-    }
-    if ((e = launch_chained(sgd_loss_kernel, sgd_partial_count(n), 32, 0, s, p, (const float*)p.dh1)) != cudaSuccess) return e;
+  const int n = p.n, D = p.D, H = p.H, A = p.A;
+  const float *W1 = p.theta, *b1 = W1 + (size_t)H * D, *W2 = b1 + H, *b2 = W2 + (size_t)H * H, *W3 = b2 + H, *b3 = W3 + (size_t)A * H;
+  const float *T1 = p.theta_target, *tb1 = T1 + (size_t)H * D, *T2 = tb1 + H, *tb2 = T2 + (size_t)H * H, *T3 = tb2 + H, *tb3 = T3 + (size_t)A * H;
+  // online network: h1, h2 kept; target network: its activations borrow dh1 / dh2 (free until the backward pass)
+  cudaError_t e;
+  if (use_tc2(p)) {
+    // both networks' weight matrices (and W2^T for the backward pass) split once, then each layer of both networks in one launch
+    float* pk_W1 = p.wpack;
+    float* pk_T1 = pk_W1 + tc_pack_floats(H, D);
+    float* pk_W2 = pk_T1 + tc_pack_floats(H, D);
+    float* pk_T2 = pk_W2 + tc_pack_floats(H, H);
+    float* pk_W2t = pk_T2 + tc_pack_floats(H, H);
+    TcPackJobs jobs{};
+    jobs.j[jobs.n++] = TcPackJob{W1, D, 0, H, D, pk_W1};
+    jobs.j[jobs.n++] = TcPackJob{T1, D, 0, H, D, pk_T1};
+    jobs.j[jobs.n++] = TcPackJob{W2, H, 0, H, H, pk_W2};
+    jobs.j[jobs.n++] = TcPackJob{T2, H, 0, H, H, pk_T2};
+    jobs.j[jobs.n++] = TcPackJob{W2, H, 1, H, H, pk_W2t};
+    if ((e = launch_pack_tf32_operands(jobs, s)) != cudaSuccess) return e;
+    TcGemmBatch l1{};
+    l1.g[0] = TcGemm{p.obs, D, pk_W1, p.h1, H, n, H, D, b1, nullptr, 0};
+    l1.g[1] = TcGemm{p.next_obs, D, pk_T1, p.dh1, H, n, H, D, tb1, nullptr, 0};
+    l1.n = 2;
+    if ((e = launch_gemm_tc2(l1, GM_BIAS_RELU, p.error, s)) != cudaSuccess) return e;
+    TcGemmBatch l2{};
+    l2.g[0] = TcGemm{p.h1, H, pk_W2, p.h2, H, n, H, H, b2, nullptr, 0};
+    l2.g[1] = TcGemm{p.dh1, H, pk_T2, p.dh2, H, n, H, H, tb2, nullptr, 0};
+    l2.n = 2;
+    if ((e = launch_gemm_tc2(l2, GM_BIAS_RELU, p.error, s)) != cudaSuccess) return e;
+    *p.launches += 3;
+  } else {
+    const GemmPair l1{{p.obs, p.next_obs}, {W1, T1}, {p.h1, p.dh1}, {b1, tb1}}, l2{{p.h1, p.dh1}, {W2, T2}, {p.h2, p.dh2}, {b2, tb2}};
+    if ((e = sg_layer<GM_BIAS_RELU>(p, l1, 2, D, D, H, n, H, D, nullptr, 0, s)) != cudaSuccess) return e;
+    if ((e = sg_layer<GM_BIAS_RELU>(p, l2, 2, H, H, H, n, H, H, nullptr, 0, s)) != cudaSuccess) return e;
+  }
+  if (A <= 4) {
+    ++*p.launches;
+    if ((e = launch_chained(sgd_rows_kernel<false>, sgd_partial_count(n), 256, 0, s, p, (const float*)p.dh2)) != cudaSuccess) return e;
     return backward_and_update(p, lr, adam, s);
   }
-  const size_t smem_f = (((size_t)p.D + 2 * (size_t)p.H + p.A) * SG_ROWS + (size_t)SG_THREADS * (SG_KT + 1)) * sizeof(float);
-  cudaError_t e;
-  if ((e = launch_chained(sgd_forward_kernel, sgd_partial_count(p.n), SG_THREADS, smem_f, s, p)) != cudaSuccess) return e;
+  // both heads in one launch: Q of the online network into g, of the target network into qt
+  const GemmPair heads{{p.h2, p.dh2}, {W3, T3}, {p.g, p.qt}, {b3, tb3}};
+  const size_t hd_smem = (size_t)H * 16 * sizeof(float);
+  if (H % 128 == 0 && hd_smem <= 96 * 1024) {
+    ++*p.launches;
+    e = launch_chained(sg_heads_kernel, dim3((n + HD_ROWS - 1) / HD_ROWS, 2), 256, hd_smem, s, heads, n, H, A, A);
+  } else {
+    e = sg_gemm<false, GM_BIAS>(p, heads, 2, H, H, A, n, A, H, nullptr, 0, s);
+  }
+  if (e != cudaSuccess) return e;
+  ++*p.launches;
+  if ((e = launch_chained(sgd_loss_kernel, sgd_partial_count(n), 256, 0, s, p)) != cudaSuccess) return e;
   return backward_and_update(p, lr, adam, s);
 }
 
 cudaError_t launch_sgd_step(const SgdParams& p, float lr, const AdamParams* adam, float* loss_out, cudaStream_t s) {
-  if (sgd_fused_ok(p.D, p.H, p.A, 0)) return launch_sgd_fused(p, lr, adam, loss_out, s);
+  if (sgd_fused_ok(p.D, p.H, p.A, 0)) {
+    *p.launches += 2;
+    return launch_sgd_fused(p, lr, adam, loss_out, s);
+  }
   cudaError_t e = sgd_step_layered(p, lr, adam, s);
-  if (e == cudaSuccess && loss_out) e = launch_td_finish(p.partial, sgd_partial_count(p.n), p.n, loss_out, s);
+  if (e == cudaSuccess && loss_out) {
+    ++*p.launches;
+    e = launch_td_finish(p.partial, sgd_partial_count(p.n), p.n, loss_out, s);
+  }
   return e;
 }
 
 cudaError_t launch_ppo_step(const SgdParams& p, float lr, const AdamParams* adam, float* stats_out, cudaStream_t s) {
-  if (sgd_fused_ok(p.D, p.H, p.A, 1)) return launch_sgd_fused(p, lr, adam, stats_out, s);
-  const size_t smem_f = (((size_t)p.D + 2 * (size_t)p.H + p.A + 1) * SG_ROWS + (size_t)SG_THREADS * (SG_KT + 1)) * sizeof(float);
+  if (sgd_fused_ok(p.D, p.H, p.A, 1)) {
+    *p.launches += 2;
+    return launch_sgd_fused(p, lr, adam, stats_out, s);
+  }
+  if (p.A > 3) return cudaErrorInvalidConfiguration;           // the segment environments have two or three actions
+  const int n = p.n, D = p.D, H = p.H;
+  const float *W1 = p.theta, *b1 = W1 + (size_t)H * D, *W2 = b1 + H, *b2 = W2 + (size_t)H * H;
   cudaError_t e;
-  if ((e = launch_chained(ppo_forward_kernel, sgd_partial_count(p.n), SG_THREADS, smem_f, s, p)) != cudaSuccess) return e;
-  if (stats_out && (e = launch_chained(ppo_finish_kernel, 1, 32, 0, s, p.stat_partial, sgd_partial_count(p.n), p.n, stats_out)) != cudaSuccess) return e;
+  if ((e = sg_gemm<false, GM_BIAS_RELU>(p, GemmPair{{p.obs}, {W1}, {p.h1}, {b1}}, 1, D, D, H, n, H, D, nullptr, 0, s)) != cudaSuccess) return e;
+  if ((e = sg_gemm<false, GM_BIAS_RELU>(p, GemmPair{{p.h1}, {W2}, {p.h2}, {b2}}, 1, H, H, H, n, H, H, nullptr, 0, s)) != cudaSuccess) return e;
+  *p.launches += stats_out ? 2 : 1;
+  if ((e = launch_chained(sgd_rows_kernel<true>, sgd_partial_count(n), 256, 0, s, p, (const float*)nullptr)) != cudaSuccess) return e;
+  if (stats_out && (e = launch_chained(ppo_finish_kernel, 1, 160, 0, s, (const float*)p.stat_partial, sgd_partial_count(n), n, stats_out)) != cudaSuccess)
+    return e;
   return backward_and_update(p, lr, adam, s);
 }
 
