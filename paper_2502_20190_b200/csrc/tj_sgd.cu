@@ -7,6 +7,7 @@
 //   update    W3[a] -= lr sum_j g_j h2_j, W2 -= lr dh2^T h1, W1 -= lr dh1^T x, biases likewise
 // Every sum runs in a fixed order (rows ascending), so a step is reproducible bit for bit.
 #include "tj_internal.h"
+#include "tj_fma.cuh"
 #include "tj_tc.cuh"
 
 namespace tj {
@@ -19,123 +20,188 @@ constexpr int SG_ROWS = 16;       // minibatch rows per loss partial
 // Wide networks and large minibatches: the layers as tiled FP32 matrix products (a weight element is reused for 128 rows
 // instead of 16).  C[m][n] = epi(sum_k A[m][k] Bop[k][n]): A row-major M x K.  B_KN false: B is N x K row-major (a weight
 // matrix as the forward pass uses it, Bop = B^T); true: B is K x N row-major (the same matrix in the backward pass).
-// 128 x 64 tile per block (64 or 32 rows where tall tiles would leave SMs idle), 16 k per step, each thread 8 x 4 (4 x 4,
-// 2 x 4); k ascending, one accumulator per output: a fixed order.
-constexpr int GM_BN = 64, GM_BK = 16, GM_THREADS = 256;
+// 64 x 64 tile per block (32 rows where that leaves SMs idle), 32 k per step in one of two stages.  Two groups of 128 threads take
+// alternate halves of each step, a thread 8 x 4 outputs (4 x 4 in the 32-row tile) with two rows per instruction, and add their sums
+// at the end: a fixed order.  An update has few tiles per SM, so what bounds a tile is latency: one group of four warps with
+// 16 k per step waited for shared and global memory two cycles of three (dh1 of
+// 4,096 x 256 outputs, K = 256: 23.6 us then, 17.9 now; W2's gradient 28.5 and 19.2; the FMA rate alone allows 7.3).
+constexpr int GM_BN = 64, GM_BK = 32, GM_THREADS = 256;
+template <int BM>
+constexpr int GM_STAGE = GM_BK * (BM + 4 + GM_BN + 4);   // floats of one of the two stages
+
+// acc (RM x 4, two rows per entry) += over K rows of As (RM values) and Bs (4 values), the next row's operands on their way meanwhile
+template <int RM, int K, int LDA, int LDB>
+__device__ __forceinline__ void multiply_step(const float* As, const float* Bs, f32x2 (&acc)[RM / 2][4]) {
+  f32x2 av[2][RM / 2];
+  float4 bq[2];
+  auto load = [&](int k, f32x2 (&a)[RM / 2], float4& b) {
+#pragma unroll
+    for (int i = 0; i < RM / 4; ++i) {
+      const ulonglong2 v = ld_pairs(As + k * LDA + i * 4);
+      a[i * 2] = v.x; a[i * 2 + 1] = v.y;
+    }
+    b = *reinterpret_cast<const float4*>(Bs + k * LDB);
+  };
+  load(0, av[0], bq[0]);
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    if (k + 1 < K) load(k + 1, av[(k + 1) & 1], bq[(k + 1) & 1]);
+    const float4 b = bq[k & 1];
+    const f32x2 bv[4] = {dup2(b.x), dup2(b.y), dup2(b.z), dup2(b.w)};
+#pragma unroll
+    for (int i = 0; i < RM / 2; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) fma2(acc[i][j], av[k & 1][i], bv[j]);
+  }
+}
+
+// four consecutive floats of a row from column c (zero beyond the matrix): a 16-byte load where the row allows it
+__device__ __forceinline__ float4 load_row4(const float* base, int ld, int row, int n_rows, int c, int n_cols, bool vec) {
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (row < n_rows && c < n_cols) {
+    const float* src = base + (size_t)row * ld + c;
+    if (vec && c + 3 < n_cols) {
+      v = __ldg(reinterpret_cast<const float4*>(src));
+    } else {
+      v.x = __ldg(src);
+      if (c + 1 < n_cols) v.y = __ldg(src + 1);
+      if (c + 2 < n_cols) v.z = __ldg(src + 2);
+      if (c + 3 < n_cols) v.w = __ldg(src + 3);
+    }
+  }
+  return v;
+}
+
+// One BM x 64 tile over k in [k_begin, k_end).  load_a(r, k) gives A[r][k .. k+3] (A_KM: A[r .. r+3][k]) with r counted from the tile's
+// first row, load_b likewise (B_KN: four columns of row k).  This thread's share of the result is out[RM / 2][4]: rows `row0` .. and
+// columns `col0` .. of the tile.
+template <int BM, bool A_KM, bool B_KN, class LoadA, class LoadB>
+__device__ __forceinline__ void tile_product(LoadA load_a, LoadB load_b, int k_begin, int k_end, float* sm, float (&out)[BM / 16][4], int& row0,
+                                             int& col0) {
+  constexpr int RM = BM / 8, LDA = BM + 4, LDB = GM_BN + 4, NA = BM * GM_BK / 4 / GM_THREADS, NB = GM_BN * GM_BK / 4 / GM_THREADS;
+  const int tid = threadIdx.x, kg = tid >> 7, ty = (tid & 127) >> 4, tx = tid & 15;
+  f32x2 acc[RM / 2][4];
+#pragma unroll
+  for (int i = 0; i < RM / 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+  // the next step's operands travel from global memory to registers while this one is multiplied.  Piece i of a row-major operand:
+  // four k of a row, four pieces (64 bytes) of eight rows per warp; of a k-major one: four columns of row k
+  auto piece_r = [](int i, int rows) { return (i >> 2) % rows; };
+  auto piece_k = [](int i, int rows) { return (i & 3) * 4 + 16 * (i / (4 * rows)); };
+  float4 ra[NA], rb[NB];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int u = 0; u < NA; ++u) {
+      const int i = tid + u * GM_THREADS;
+      ra[u] = A_KM ? load_a((i % (BM / 4)) * 4, k0 + i / (BM / 4)) : load_a(piece_r(i, BM), k0 + piece_k(i, BM));
+    }
+#pragma unroll
+    for (int u = 0; u < NB; ++u) {
+      const int i = tid + u * GM_THREADS;
+      rb[u] = B_KN ? load_b((i % 16) * 4, k0 + i / 16) : load_b(piece_r(i, GM_BN), k0 + piece_k(i, GM_BN));
+    }
+  };
+  fetch(k_begin);
+  int stage = 0;
+#pragma unroll 1
+  for (int k0 = k_begin; k0 < k_end; k0 += GM_BK, stage ^= 1) {
+    // two stages: whoever writes one has passed the barrier after which nobody reads it
+    float* As = sm + stage * GM_STAGE<BM>;
+    float* Bs = As + GM_BK * LDA;
+    auto put = [](float* dst, int ld, bool km, int r, int k, const float4 v) {
+      if (km) {
+        *reinterpret_cast<float4*>(dst + k * ld + r) = v;
+      } else {
+        dst[k * ld + r] = v.x; dst[(k + 1) * ld + r] = v.y; dst[(k + 2) * ld + r] = v.z; dst[(k + 3) * ld + r] = v.w;
+      }
+    };
+#pragma unroll
+    for (int u = 0; u < NA; ++u) {
+      const int i = tid + u * GM_THREADS;
+      if (A_KM) put(As, LDA, true, (i % (BM / 4)) * 4, i / (BM / 4), ra[u]);
+      else put(As, LDA, false, piece_r(i, BM), piece_k(i, BM), ra[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < NB; ++u) {
+      const int i = tid + u * GM_THREADS;
+      if (B_KN) put(Bs, LDB, true, (i % 16) * 4, i / 16, rb[u]);
+      else put(Bs, LDB, false, piece_r(i, GM_BN), piece_k(i, GM_BN), rb[u]);
+    }
+    __syncthreads();
+    if (k0 + GM_BK < k_end) fetch(k0 + GM_BK);
+    multiply_step<RM, GM_BK / 2, LDA, LDB>(As + kg * (GM_BK / 2) * LDA + ty * RM, Bs + kg * (GM_BK / 2) * LDB + tx * 4, acc);
+  }
+  // the groups swap halves of their rows: group 0 finishes the first RM / 2, group 1 the others
+  __syncthreads();
+  f32x2* mine = reinterpret_cast<f32x2*>(sm) + kg * RM * 128 + (tid & 127);
+  const f32x2* theirs = reinterpret_cast<const f32x2*>(sm) + (kg ^ 1) * RM * 128 + (tid & 127);
+#pragma unroll
+  for (int i = 0; i < RM / 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) mine[(i * 4 + j) * 128] = kg ? acc[i][j] : acc[RM / 4 + i][j];
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < RM / 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float2 a = halves(kg ? acc[RM / 4 + i][j] : acc[i][j]), b = halves(theirs[(i * 4 + j) * 128]);
+      out[2 * i][j] = a.x + b.x;
+      out[2 * i + 1][j] = a.y + b.y;
+    }
+  row0 = ty * RM + kg * (RM / 2);
+  col0 = tx * 4;
+}
+
+// four consecutive outputs of a row, a 16-byte store where the row allows it
+__device__ __forceinline__ void store_row4(float* dst, const float (&v)[4], int left, bool vec) {
+  if (vec && left >= 4) {
+    *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (j < left) dst[j] = v[j];
+  }
+}
 
 template <bool B_KN, int EPI, int BM>
 __device__ __forceinline__ void sg_gemm_body(const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb,
                                              float* __restrict__ C, int ldc, int M, int N, int K,
                                              const float* __restrict__ bias, const float* __restrict__ mask, int ldm) {
-  __shared__ __align__(16) float As[GM_BK][BM + 4];
-  __shared__ __align__(16) float Bs[GM_BK][GM_BN + 4];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  constexpr int RM = BM / 16;   // rows per thread
+  __shared__ __align__(16) float sm[2 * GM_STAGE<BM>];
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * GM_BN;
   const bool vecA = (lda & 3) == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
   const bool vecB = (ldb & 3) == 0 && (reinterpret_cast<uintptr_t>(B) & 15) == 0;
-  float acc[RM][4];
+  float out[BM / 16][4];
+  int row0, col0;
+  tile_product<BM, false, B_KN>([&](int r, int k) { return load_row4(A, lda, m0 + r, M, k, K, vecA); },
+                                [&](int c, int k) {
+                                  return B_KN ? load_row4(B, ldb, k, K, n0 + c, N, vecB) : load_row4(B, ldb, n0 + c, N, k, K, vecB);
+                                },
+                                0, K, sm, out, row0, col0);
+  const int n = n0 + col0;
+  if (n >= N) return;
+  const bool vecC = (ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0;
+  const bool vecM = EPI == GM_MASK && (ldm & 3) == 0 && (reinterpret_cast<uintptr_t>(mask) & 15) == 0;
+  float bv[4] = {0.f, 0.f, 0.f, 0.f};
+  if (EPI != GM_MASK) {
 #pragma unroll
-  for (int i = 0; i < RM; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-  // four consecutive k of one row (of A, or of an N x K B): a 16-byte load where the row allows it
-  auto load_k4 = [](const float* base, int ld, int row, int n_rows, int k, int K, bool vec) -> float4 {
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (row < n_rows && k < K) {
-      const float* src = base + (size_t)row * ld + k;
-      if (vec && k + 3 < K) {
-        v = __ldg(reinterpret_cast<const float4*>(src));
-      } else {
-        v.x = __ldg(src);
-        if (k + 1 < K) v.y = __ldg(src + 1);
-        if (k + 2 < K) v.z = __ldg(src + 2);
-        if (k + 3 < K) v.w = __ldg(src + 3);
-      }
-    }
-    return v;
-  };
-  // the next k-step's operands travel from global memory to registers while this one is multiplied
-  constexpr int NA = (BM * 4 + GM_THREADS - 1) / GM_THREADS;
-  float4 ra[NA], rb;
-  auto fetch = [&](int k0) {
-#pragma unroll
-    for (int u = 0; u < NA; ++u) {
-      const int i = tid + u * GM_THREADS;
-      if (i < BM * 4) ra[u] = load_k4(A, lda, m0 + (i >> 2), M, k0 + (i & 3) * 4, K, vecA);
-    }
-    if (!B_KN) {
-      rb = load_k4(B, ldb, n0 + (tid >> 2), N, k0 + (tid & 3) * 4, K, vecB);
-    } else {
-      const int k = k0 + (tid >> 4), n = n0 + (tid & 15) * 4;
-      rb = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (k < K && n < N) {
-        const float* src = B + (size_t)k * ldb + n;
-        if (vecB && n + 3 < N) {
-          rb = __ldg(reinterpret_cast<const float4*>(src));
-        } else {
-          rb.x = __ldg(src);
-          if (n + 1 < N) rb.y = __ldg(src + 1);
-          if (n + 2 < N) rb.z = __ldg(src + 2);
-          if (n + 3 < N) rb.w = __ldg(src + 3);
-        }
-      }
-    }
-  };
-  fetch(0);
-  for (int k0 = 0; k0 < K; k0 += GM_BK) {
-#pragma unroll
-    for (int u = 0; u < NA; ++u) {
-      const int i = tid + u * GM_THREADS, r = i >> 2, kq = (i & 3) * 4;
-      if (i >= BM * 4) break;
-      As[kq][r] = ra[u].x; As[kq + 1][r] = ra[u].y; As[kq + 2][r] = ra[u].z; As[kq + 3][r] = ra[u].w;
-    }
-    if (!B_KN) {
-      const int r = tid >> 2, kq = (tid & 3) * 4;
-      Bs[kq][r] = rb.x; Bs[kq + 1][r] = rb.y; Bs[kq + 2][r] = rb.z; Bs[kq + 3][r] = rb.w;
-    } else {
-      *reinterpret_cast<float4*>(&Bs[tid >> 4][(tid & 15) * 4]) = rb;
-    }
-    __syncthreads();
-    if (k0 + GM_BK < K) fetch(k0 + GM_BK);
-#pragma unroll
-    for (int kk = 0; kk < GM_BK; ++kk) {
-      float av[RM];
-      if constexpr (RM == 8) {
-        const float4 a0 = *reinterpret_cast<const float4*>(&As[kk][ty * 8]);
-        const float4 a1 = *reinterpret_cast<const float4*>(&As[kk][ty * 8 + 4]);
-        av[0] = a0.x; av[1] = a0.y; av[2] = a0.z; av[3] = a0.w;
-        av[RM - 4] = a1.x; av[RM - 3] = a1.y; av[RM - 2] = a1.z; av[RM - 1] = a1.w;
-      } else if constexpr (RM == 4) {
-        const float4 a0 = *reinterpret_cast<const float4*>(&As[kk][ty * 4]);
-        av[0] = a0.x; av[1] = a0.y; av[2] = a0.z; av[3] = a0.w;
-      } else {
-#pragma unroll
-        for (int i = 0; i < RM; ++i) av[i] = As[kk][ty * RM + i];
-      }
-      const float4 b = *reinterpret_cast<const float4*>(&Bs[kk][tx * 4]);
-      const float bv[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-      for (int i = 0; i < RM; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-    }
-    __syncthreads();
+    for (int j = 0; j < 4; ++j)
+      if (n + j < N) bv[j] = __ldg(bias + n + j);
   }
 #pragma unroll
-  for (int i = 0; i < RM; ++i) {
-    const int m = m0 + ty * RM + i;
+  for (int i = 0; i < BM / 16; ++i) {
+    const int m = m0 + row0 + i;
     if (m >= M) break;
+    if (EPI == GM_MASK) {
+      const float4 h = load_row4(mask, ldm, m, M, n, N, vecM);
+      out[i][0] = h.x > 0.f ? out[i][0] : 0.f; out[i][1] = h.y > 0.f ? out[i][1] : 0.f;
+      out[i][2] = h.z > 0.f ? out[i][2] : 0.f; out[i][3] = h.w > 0.f ? out[i][3] : 0.f;
+    } else {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx * 4 + j;
-      if (n >= N) break;
-      float v = acc[i][j];
-      if (EPI == GM_BIAS_RELU) v = fmaxf(v + __ldg(bias + n), 0.f);
-      else if (EPI == GM_BIAS) v = v + __ldg(bias + n);
-      else v = __ldg(mask + (size_t)m * ldm + n) > 0.f ? v : 0.f;
-      C[(size_t)m * ldc + n] = v;
+      for (int j = 0; j < 4; ++j) out[i][j] = EPI == GM_BIAS_RELU ? fmaxf(out[i][j] + bv[j], 0.f) : out[i][j] + bv[j];
     }
+    store_row4(C + (size_t)m * ldc + n, out[i], N - n, vecC);
   }
 }
 
@@ -145,77 +211,113 @@ template <bool B_KN, int EPI, int BM>
 __global__ void __launch_bounds__(GM_THREADS) sg_gemm_kernel(const GemmPair pr, int lda, int ldb, int ldc, int M, int N, int K,
                                                              const float* __restrict__ mask, int ldm) {
   chain_begin();
-  const int z = blockIdx.z;
-  sg_gemm_body<B_KN, EPI, BM>(pr.A[z], lda, pr.B[z], ldb, pr.C[z], ldc, M, N, K, pr.bias[z], mask, ldm);
+  const bool z = blockIdx.z != 0;
+  sg_gemm_body<B_KN, EPI, BM>(z ? pr.A[1] : pr.A[0], lda, z ? pr.B[1] : pr.B[0], ldb, z ? pr.C[1] : pr.C[0], ldc, M, N, K,
+                              z ? pr.bias[1] : pr.bias[0], mask, ldm);
 }
 
 // The heads of both networks for wide hidden layers: out[row][a] = bias[a] + sum_k h[row][k] W[a][k], a < A <= 16, H a
 // multiple of 128.  A 32-row FMA tile pads the few outputs to 64 columns and pays a block barrier per 16 k; here a warp takes
-// a row at a time: lane l reads the 16-byte pieces l, l + 32, ... of the row (coalesced), multiplies them with the head's
-// weights (in shared memory, laid out so that consecutive lanes read consecutive 16-byte words) into 16 partial outputs, and
-// the 16 x 32 partials are summed by a fixed halving exchange (16 shuffles).  blockIdx.y picks the network.
-constexpr int HD_ROWS = 64;   // rows per block: eight per warp
+// four rows at a time: lane l reads the 16-byte pieces l, l + 32, ... of the rows (coalesced), multiplies them with the head's
+// weights (in shared memory, laid out so that consecutive lanes read consecutive 16-byte words) into 16 partial outputs per row, and
+// the 16 x 32 partials of a row are summed by a fixed halving exchange (16 shuffles).  blockIdx.y picks the network.  Row by row the
+// weights' way out of shared memory was the bound (2 x 8,192 rows x 512: 26.4 us, 18.3 with four rows per read of them).
+constexpr int HD_ROWS = 64, HD_R = 4;   // rows per block: eight per warp, four at a time
 __global__ void __launch_bounds__(256) sg_heads_kernel(const GemmPair pr, int n_rows, int H, int A, int ldc) {
-  chain_begin();
   extern __shared__ __align__(16) float4 hd_w[];       // [(j * 4 + kk) * 4 + aq][lane]: W[aq * 4 .. + 3][4 (32 j + lane) + kk]
-  const int z = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const float* __restrict__ W = pr.B[z];
-  const float* __restrict__ hrows = pr.A[z];
-  const float* __restrict__ bias = pr.bias[z];
-  float* __restrict__ out = pr.C[z];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const bool z = blockIdx.y != 0;
+  const float* __restrict__ W = z ? pr.B[1] : pr.B[0];
+  const float* __restrict__ hrows = z ? pr.A[1] : pr.A[0];
+  const float* __restrict__ bias = z ? pr.bias[1] : pr.bias[0];
+  float* __restrict__ out = z ? pr.C[1] : pr.C[0];
   const int nj = H / 128;
-  for (int i = tid; i < nj * 16 * 32; i += blockDim.x) {
-    const int l = i & 31, aq = (i >> 5) & 3, kk = (i >> 7) & 3, j = i >> 9;
-    const int k = 4 * (32 * j + l) + kk, a = aq * 4;
-    float4 w;
-    w.x = a < A ? W[(size_t)a * H + k] : 0.f;
-    w.y = a + 1 < A ? W[(size_t)(a + 1) * H + k] : 0.f;
-    w.z = a + 2 < A ? W[(size_t)(a + 2) * H + k] : 0.f;
-    w.w = a + 3 < A ? W[(size_t)(a + 3) * H + k] : 0.f;
-    hd_w[i] = w;
+  chain_begin();
+  // row a of the head, four columns per thread, into component a % 4 of its four words
+  const bool vecW = (reinterpret_cast<uintptr_t>(W) & 15) == 0;
+  for (int i = tid; i < 16 * 32 * nj; i += blockDim.x) {
+    const int a = i / (32 * nj), q = i % (32 * nj);
+    float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (a < A) {
+      const float* src = W + (size_t)a * H + 4 * q;
+      w = vecW ? __ldg(reinterpret_cast<const float4*>(src)) : make_float4(__ldg(src), __ldg(src + 1), __ldg(src + 2), __ldg(src + 3));
+    }
+    float* d = reinterpret_cast<float*>(hd_w + ((q >> 5) * 16 + (a >> 2)) * 32 + (q & 31)) + (a & 3);
+    d[0] = w.x; d[4 * 128] = w.y; d[8 * 128] = w.z; d[12 * 128] = w.w;
   }
   __syncthreads();
   const int a_mine = ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
   const float b_mine = a_mine < A ? bias[a_mine] : 0.f;
-  for (int r = warp; r < HD_ROWS; r += 8) {
+#pragma unroll 1
+  for (int r = warp * HD_R; r < HD_ROWS; r += 8 * HD_R) {
     const int row = blockIdx.x * HD_ROWS + r;
     if (row >= n_rows) break;
-    float v[16];
+    f32x2 v2[HD_R][8];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = 0.f;
+    for (int q = 0; q < HD_R; ++q)
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v2[q][i] = 0ull;
+    auto piece = [&](int q, int j) {                       // a row beyond the last reads the last one again and is not stored
+      const int rq = row + q < n_rows ? row + q : n_rows - 1;
+      return __ldg(reinterpret_cast<const float4*>(hrows + (size_t)rq * H) + 32 * j + lane);
+    };
+    float4 x[HD_R];
+#pragma unroll
+    for (int q = 0; q < HD_R; ++q) x[q] = piece(q, 0);
+#pragma unroll 1
     for (int j = 0; j < nj; ++j) {
-      const float4 x = __ldg(reinterpret_cast<const float4*>(hrows + (size_t)row * H) + 32 * j + lane);
-      const float xs[4] = {x.x, x.y, x.z, x.w};
+      float4 xn[HD_R];
 #pragma unroll
-      for (int kk = 0; kk < 4; ++kk)
+      for (int q = 0; q < HD_R; ++q) xn[q] = piece(q, j + 1 < nj ? j + 1 : j);
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) {
+        f32x2 xs[HD_R];
+#pragma unroll
+        for (int q = 0; q < HD_R; ++q) xs[q] = dup2(kk == 0 ? x[q].x : kk == 1 ? x[q].y : kk == 2 ? x[q].z : x[q].w);
 #pragma unroll
         for (int aq = 0; aq < 4; ++aq) {
-          const float4 w = hd_w[((j * 4 + kk) * 4 + aq) * 32 + lane];
-          v[aq * 4] = fmaf(xs[kk], w.x, v[aq * 4]); v[aq * 4 + 1] = fmaf(xs[kk], w.y, v[aq * 4 + 1]);
-          v[aq * 4 + 2] = fmaf(xs[kk], w.z, v[aq * 4 + 2]); v[aq * 4 + 3] = fmaf(xs[kk], w.w, v[aq * 4 + 3]);
+          const ulonglong2 w = ld_pairs(reinterpret_cast<const float*>(hd_w + ((j * 4 + kk) * 4 + aq) * 32 + lane));
+#pragma unroll
+          for (int q = 0; q < HD_R; ++q) {
+            fma2(v2[q][2 * aq], xs[q], w.x);
+            fma2(v2[q][2 * aq + 1], xs[q], w.y);
+          }
         }
+      }
+#pragma unroll
+      for (int q = 0; q < HD_R; ++q) x[q] = xn[q];
     }
-    // halving exchange: after the step with distance d a lane keeps the half of its values that its bit d selects
+#pragma unroll
+    for (int q = 0; q < HD_R; ++q) {
+      float v[16];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float2 h = halves(v2[q][i]);
+        v[2 * i] = h.x;
+        v[2 * i + 1] = h.y;
+      }
+      // halving exchange: after the step with distance d a lane keeps the half of its values that its bit d selects
 #define TJ_HD_STEP(D, CNT)                                                                     \
-    {                                                                                             \
-      const bool upper = (lane & (D)) != 0;                                                       \
-      _Pragma("unroll") for (int i = 0; i < (CNT); ++i) {                                         \
-        const float keep = upper ? v[i + (CNT)] : v[i], send = upper ? v[i] : v[i + (CNT)];      \
-        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, (D));                                   \
-      }                                                                                           \
-    }
-    TJ_HD_STEP(16, 8)
-    TJ_HD_STEP(8, 4)
-    TJ_HD_STEP(4, 2)
-    TJ_HD_STEP(2, 1)
+      {                                                                                           \
+        const bool upper = (lane & (D)) != 0;                                                     \
+        _Pragma("unroll") for (int i = 0; i < (CNT); ++i) {                                       \
+          const float keep = upper ? v[i + (CNT)] : v[i], send = upper ? v[i] : v[i + (CNT)];    \
+          v[i] = keep + __shfl_xor_sync(0xffffffffu, send, (D));                                 \
+        }                                                                                         \
+      }
+      TJ_HD_STEP(16, 8)
+      TJ_HD_STEP(8, 4)
+      TJ_HD_STEP(4, 2)
+      TJ_HD_STEP(2, 1)
 #undef TJ_HD_STEP
-    const float total = v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
-    if ((lane & 1) == 0 && a_mine < A) out[(size_t)row * ldc + a_mine] = total + b_mine;
+      const float total = v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+      if (row + q < n_rows && (lane & 1) == 0 && a_mine < A) out[(size_t)(row + q) * ldc + a_mine] = total + b_mine;
+    }
   }
 }
 
-// Tile height: the tallest of 128, 64, 32 rows that still gives every SM a block; a product that has too few tiles even so
-// is bound by its chain of k-steps.
+// Tile height: 64 rows if that gives every SM a block, else 32 (a product that has too few tiles even so is bound by its chain
+// of k-steps).
 template <bool B_KN, int EPI>
 cudaError_t sg_gemm(const SgdParams& p, const GemmPair& pr, int sets, int lda, int ldb, int ldc, int M, int N, int K, const float* mask, int ldm,
                     cudaStream_t s) {
@@ -224,7 +326,6 @@ cudaError_t sg_gemm(const SgdParams& p, const GemmPair& pr, int sets, int lda, i
   auto go = [&](auto kernel, int bm) {
     return launch_chained(kernel, dim3(cols, (M + bm - 1) / bm, sets), GM_THREADS, 0, s, pr, lda, ldb, ldc, M, N, K, mask, ldm);
   };
-  if ((long long)cols * ((M + 127) / 128) * sets >= sms) return go(sg_gemm_kernel<B_KN, EPI, 128>, 128);
   if ((long long)cols * ((M + 63) / 64) * sets >= sms) return go(sg_gemm_kernel<B_KN, EPI, 64>, 64);
   return go(sg_gemm_kernel<B_KN, EPI, 32>, 32);
 }
@@ -431,15 +532,14 @@ cudaError_t sg_layer(const SgdParams& p, const GemmPair& pr, int sets, int lda, 
 // still in L1.  Bound by reading h2 twice and writing dh2 (as a 32-row product tile per head, a loss kernel and a product with K = A
 // this was four launches and 37 us for 4,096 rows x 256 units).  Loss partials per SG_ROWS rows.
 template <bool PPO>
-__global__ void __launch_bounds__(256) sgd_rows_kernel(const SgdParams p, const float* t2) {
+__global__ void __launch_bounds__(32 * SG_ROWS) sgd_rows_kernel(const SgdParams p, const float* t2) {
   __shared__ float part[5][SG_ROWS];
   chain_begin();
   const int H = p.H, D = p.D, A = p.A, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float *W3 = p.theta + (size_t)H * D + H + (size_t)H * H + H, *b3 = W3 + (size_t)A * H, *Wv = b3 + A;
   const float *T3 = p.theta_target + (size_t)H * D + H + (size_t)H * H + H, *tb3 = T3 + (size_t)A * H;
-#pragma unroll 1
-  for (int r = warp; r < SG_ROWS; r += 8) {
-    const int j = blockIdx.x * SG_ROWS + r;
+  {
+    const int r = warp, j = blockIdx.x * SG_ROWS + r;
     float l[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
     if (j < p.n) {
       const float* h = p.h2 + (size_t)j * H;
@@ -559,35 +659,53 @@ __global__ void __launch_bounds__(256) sgd_rows_kernel(const SgdParams p, const 
 }
 
 // The same from Q values that other kernels computed, for more outputs: q (in) and g (out) share p.g ([n][A], a row is read before its
-// own warp overwrites it), qt [n][A]; dh2 has one term per entry, the selected action's.
-__global__ void __launch_bounds__(256) sgd_loss_kernel(const SgdParams p) {
+// own warp overwrites it), qt [n][A]; dh2 has one term per entry, the selected action's.  A row is a chain of round trips (action, its
+// q, h2), so it loads what it can before the first of them: all of an h2 row in registers where 16-byte pieces of 512 units suffice
+// (8,192 x 512: 6.6 us; 21 with scalar loads in the loop and two rows per warp).
+__global__ void __launch_bounds__(32 * SG_ROWS) sgd_loss_kernel(const SgdParams p) {
   __shared__ float part[SG_ROWS];
   chain_begin();
-  const int H = p.H, D = p.D, A = p.A, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int H = p.H, D = p.D, A = p.A, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j = blockIdx.x * SG_ROWS + warp;
   const float* W3 = p.theta + (size_t)H * D + H + (size_t)H * H + H;
-#pragma unroll 1
-  for (int r = warp; r < SG_ROWS; r += 8) {
-    const int j = blockIdx.x * SG_ROWS + r;
-    float l = 0.f;
-    if (j < p.n) {
-      const int act0 = p.act[j], act = act0 < 0 ? 0 : (act0 >= A ? A - 1 : act0);
-      float* gr = p.g + (size_t)j * A;
-      const float* tr = p.qt + (size_t)j * A;
-      float qmax = lane < A ? tr[lane] : -INFINITY;            // A <= 16 outputs
-      for (int o = 16; o > 0; o >>= 1) qmax = fmaxf(qmax, __shfl_xor_sync(0xffffffffu, qmax, o));
-      const float delta = p.rew[j] + p.gamma * (p.done[j] ? 0.f : 1.f) * qmax - gr[act], ad = fabsf(delta);
-      l = ad <= p.kappa ? 0.5f * delta * delta : p.kappa * (ad - 0.5f * p.kappa);
-      const float gj = -fminf(fmaxf(delta, -p.kappa), p.kappa) / (float)p.n;
-      __syncwarp();
-      if (lane < A) gr[lane] = lane == act ? gj : 0.f;
-      const float* h = p.h2 + (size_t)j * H;
-      const float* w = W3 + (size_t)act * H;
-      float* d = p.dh2 + (size_t)j * H;
-#pragma unroll 4
+  float l = 0.f;
+  if (j < p.n) {
+    const float* h = p.h2 + (size_t)j * H;
+    float* d = p.dh2 + (size_t)j * H;
+    const bool in_regs = (H & 3) == 0 && H <= 512;
+    float4 hv[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (in_regs && 4 * (lane + 32 * u) < H) hv[u] = *reinterpret_cast<const float4*>(h + 4 * (lane + 32 * u));
+    const int act0 = p.act[j], act = act0 < 0 ? 0 : (act0 >= A ? A - 1 : act0);
+    float* gr = p.g + (size_t)j * A;
+    const float* tr = p.qt + (size_t)j * A;
+    const float q_all = lane < A ? gr[lane] : 0.f, rew = p.rew[j];                // A <= 16 outputs
+    const int dn = p.done[j];
+    float qmax = lane < A ? tr[lane] : -INFINITY;
+    for (int o = 16; o > 0; o >>= 1) qmax = fmaxf(qmax, __shfl_xor_sync(0xffffffffu, qmax, o));
+    const float delta = rew + p.gamma * (dn ? 0.f : 1.f) * qmax - __shfl_sync(0xffffffffu, q_all, act), ad = fabsf(delta);
+    l = ad <= p.kappa ? 0.5f * delta * delta : p.kappa * (ad - 0.5f * p.kappa);
+    const float gj = -fminf(fmaxf(delta, -p.kappa), p.kappa) / (float)p.n;
+    if (lane < A) gr[lane] = lane == act ? gj : 0.f;
+    const float* w = W3 + (size_t)act * H;
+    if (in_regs) {
+      const bool vecW = (reinterpret_cast<uintptr_t>(w) & 15) == 0;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = 4 * (lane + 32 * u);
+        if (i < H) {
+          float4 wv;
+          if (vecW) wv = __ldg(reinterpret_cast<const float4*>(w + i));
+          else wv = make_float4(__ldg(w + i), __ldg(w + i + 1), __ldg(w + i + 2), __ldg(w + i + 3));
+          *reinterpret_cast<float4*>(d + i) = make_float4(hv[u].x > 0.f ? gj * wv.x : 0.f, hv[u].y > 0.f ? gj * wv.y : 0.f,
+                                                          hv[u].z > 0.f ? gj * wv.z : 0.f, hv[u].w > 0.f ? gj * wv.w : 0.f);
+        }
+      }
+    } else {
       for (int i = lane; i < H; i += 32) d[i] = h[i] > 0.f ? gj * __ldg(w + i) : 0.f;
     }
-    if (lane == 0) part[r] = l;
   }
+  if (lane == 0) part[warp] = l;
   __syncthreads();
   if (threadIdx.x == 0) {
     float s = 0.f;
@@ -620,89 +738,37 @@ struct GradProducts {
   int n, n_tiles;
 };
 
-constexpr int GP_TILE = 64, GP_ROWS = 16;   // columns of a gradient tile; minibatch rows staged per step
+constexpr int GP_TILE = 64;   // rows and columns of a gradient tile
 
-// One tile (TM x 64, TM = 64 or 128: each thread TM / 16 x 4) of one gradient product over one range of minibatch rows
-template <int TM>
+// One tile of one gradient product over one range of minibatch rows
 __device__ __forceinline__ void grad_tile(float* __restrict__ P, const GradProduct& d, int t, int count, int n_rows, int rows_per_range,
-                                          float (*As)[128 + 4], float (*Bs)[GP_TILE + 4]) {
-  constexpr int RM = TM / 16, NA = TM / 64;
+                                          float* __restrict__ sm) {
   const int M = d.M, N = d.N, lda = d.lda, ldb = d.ldb;
   const float* __restrict__ Am = d.Am;
   const float* __restrict__ Bm = d.Bm;
   const int tiles_n = (N + GP_TILE - 1) / GP_TILE;
-  const int m0 = (t / tiles_n) * TM, n0 = (t % tiles_n) * GP_TILE;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const int m0 = (t / tiles_n) * GP_TILE, n0 = (t % tiles_n) * GP_TILE;
   const int j_begin = blockIdx.y * rows_per_range;
   const int j_end = j_begin + rows_per_range < n_rows ? j_begin + rows_per_range : n_rows;
   const bool vecA = (lda & 3) == 0 && (reinterpret_cast<uintptr_t>(Am) & 15) == 0;
-  const bool vecB = Bm && (ldb & 3) == 0 && (reinterpret_cast<uintptr_t>(Bm) & 15) == 0;
-  // four consecutive columns of row j (zero beyond the row range or the matrix): a 16-byte load where the row allows it
-  auto load_c4 = [](const float* base, int ld, int j, int j_end, int c, int C, bool vec) -> float4 {
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (j < j_end && c < C) {
-      const float* src = base + (size_t)j * ld + c;
-      if (vec && c + 3 < C) {
-        v = *reinterpret_cast<const float4*>(src);
-      } else {
-        v.x = src[0];
-        if (c + 1 < C) v.y = src[1];
-        if (c + 2 < C) v.z = src[2];
-        if (c + 3 < C) v.w = src[3];
-      }
-    }
-    return v;
-  };
-  float acc[RM][4];
+  const bool vecB = (ldb & 3) == 0 && (reinterpret_cast<uintptr_t>(Bm) & 15) == 0;
+  float out[GP_TILE / 16][4];
+  int row0, col0;
+  tile_product<GP_TILE, true, true>([&](int m, int j) { return load_row4(Am, lda, j, j_end, m0 + m, M, vecA); },
+                                    [&](int c, int j) {
+                                      if (Bm) return load_row4(Bm, ldb, j, j_end, n0 + c, N, vecB);
+                                      return make_float4(j < j_end && n0 + c == 0 ? 1.f : 0.f, 0.f, 0.f, 0.f);   // a bias: one column of ones
+                                    },
+                                    j_begin, j_end, sm, out, row0, col0);
+  const int n = n0 + col0;
+  if (n >= N) return;
+  float* dst = P + (size_t)blockIdx.y * count + d.off + n;
+  const bool vec = (N & 3) == 0 && (reinterpret_cast<uintptr_t>(dst) & 15) == 0;
 #pragma unroll
-  for (int u = 0; u < RM; ++u)
-#pragma unroll
-    for (int v = 0; v < 4; ++v) acc[u][v] = 0.f;
-  // the next rows travel from global memory to registers while these are multiplied
-  const int l_jj = threadIdx.x >> 4, l_c = (threadIdx.x & 15) * 4;
-  float4 ra[NA], rb;
-  auto fetch = [&](int j0) {
-    const int j = j0 + l_jj;
-#pragma unroll
-    for (int h = 0; h < NA; ++h) ra[h] = load_c4(Am, lda, j, j_end, m0 + h * 64 + l_c, M, vecA);
-    if (Bm) {
-      rb = load_c4(Bm, ldb, j, j_end, n0 + l_c, N, vecB);
-    } else {
-      const float one = j < j_end ? 1.f : 0.f;
-      rb = make_float4(n0 + l_c < N ? one : 0.f, n0 + l_c + 1 < N ? one : 0.f, n0 + l_c + 2 < N ? one : 0.f, n0 + l_c + 3 < N ? one : 0.f);
-    }
-  };
-  if (j_begin < j_end) fetch(j_begin);
-  for (int j0 = j_begin; j0 < j_end; j0 += GP_ROWS) {
-#pragma unroll
-    for (int h = 0; h < NA; ++h) *reinterpret_cast<float4*>(&As[l_jj][h * 64 + l_c]) = ra[h];
-    *reinterpret_cast<float4*>(&Bs[l_jj][l_c]) = rb;
-    __syncthreads();
-    if (j0 + GP_ROWS < j_end) fetch(j0 + GP_ROWS);
-#pragma unroll
-    for (int jj = 0; jj < GP_ROWS; ++jj) {
-      float av[RM];
-#pragma unroll
-      for (int h = 0; h < RM / 4; ++h) {
-        const float4 a = *reinterpret_cast<const float4*>(&As[jj][ty * RM + h * 4]);
-        av[h * 4] = a.x; av[h * 4 + 1] = a.y; av[h * 4 + 2] = a.z; av[h * 4 + 3] = a.w;
-      }
-      const float4 b = *reinterpret_cast<const float4*>(&Bs[jj][tx * 4]);
-      const float bv[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-      for (int u = 0; u < RM; ++u)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(av[u], bv[v], acc[u][v]);
-    }
-    __syncthreads();
+  for (int i = 0; i < GP_TILE / 16; ++i) {
+    const int m = m0 + row0 + i;
+    if (m < M) store_row4(dst + (size_t)m * N, out[i], N - n, vec);
   }
-#pragma unroll
-  for (int u = 0; u < RM; ++u)
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      const int m = m0 + ty * RM + u, n = n0 + tx * 4 + v;
-      if (m < M && n < N) P[(size_t)blockIdx.y * count + d.off + (size_t)m * N + n] = acc[u][v];
-    }
 }
 
 // The gradients of narrow operands (obs_dim <= 8, at most four outputs): W1, both hidden biases, the head and its biases.  As 64-column
@@ -762,26 +828,24 @@ __device__ __forceinline__ void grad_narrow_block(float* __restrict__ P, const N
 }
 
 // Every gradient product of one update in a single launch: thread block (tile, range) sums, over its range of minibatch
-// rows, one tile of one product (128 x 64 where the product has at least 128 rows, else 64 x 64) and writes it to
+// rows, one 64 x 64 tile of one product and writes it to
 // P[range][off + m * N + n] -- a partial gradient laid out like the parameter blob itself, `count` floats per range.
 // No atomics: the apply kernel adds the ranges in order.
 __global__ void __launch_bounds__(256) sgd_grad_partial_kernel(float* __restrict__ P, const GradProducts gp, const NarrowGrad narrow, int count,
                                                                int n_rows, int rows_per_range) {
-  __shared__ __align__(16) float sm[4 * 14 * 64];
+  __shared__ __align__(16) float sm[2 * GM_STAGE<GP_TILE>];   // or 4 x 14 x 64 sums
+  static_assert(4 * 14 * 64 <= 2 * GM_STAGE<GP_TILE>, "the narrow sums fit");
   chain_begin();
   if ((int)blockIdx.x >= gp.n_tiles) {
     const int j_begin = blockIdx.y * rows_per_range, j_end = min(j_begin + rows_per_range, n_rows);
     grad_narrow_block(P + (size_t)blockIdx.y * count, narrow, blockIdx.x - gp.n_tiles, j_begin, j_end, sm);
     return;
   }
-  float (*As)[128 + 4] = reinterpret_cast<float (*)[128 + 4]>(sm);
-  float (*Bs)[GP_TILE + 4] = reinterpret_cast<float (*)[GP_TILE + 4]>(sm + GP_ROWS * (128 + 4));
   int q = 0;
   while (q + 1 < gp.n && (int)blockIdx.x >= gp.g[q + 1].tile_begin) ++q;
   const GradProduct& d = gp.g[q];
   const int t = blockIdx.x - d.tile_begin;
-  if (d.M >= 128) grad_tile<128>(P, d, t, count, n_rows, rows_per_range, As, Bs);
-  else grad_tile<64>(P, d, t, count, n_rows, rows_per_range, As, Bs);
+  grad_tile(P, d, t, count, n_rows, rows_per_range, sm);
 }
 
 // C[i] -= lr * (P[0][i] + P[1][i] + ...), the partial sums added in range order
@@ -894,8 +958,7 @@ cudaError_t backward_and_update(const SgdParams& p, float lr, const AdamParams* 
     d.lda = lda;
     d.ldb = ldb;
     d.tile_begin = gp.n_tiles;
-    const int tm = M >= 128 ? 128 : 64;   // as the kernel picks it
-    gp.n_tiles += ((M + tm - 1) / tm) * ((N + GP_TILE - 1) / GP_TILE);
+    gp.n_tiles += ((M + GP_TILE - 1) / GP_TILE) * ((N + GP_TILE - 1) / GP_TILE);
   };
   TcWgradBatch tb{};
   const bool tc_grads = use_tc2(p);
@@ -921,14 +984,11 @@ cudaError_t backward_and_update(const SgdParams& p, float lr, const AdamParams* 
     if (p.value_head) product(Wv, bv, 1, H, p.g + A, p.ldg, p.h2, H);
   }
   // row ranges: with tensor-core tiles about one thread block per SM in all (a block costs a fixed ~10 us beside its rows);
-  // otherwise 128 rows or more per range
-  int n_ranges;
-  if (tb.n_tiles > 0) {
-    n_ranges = (p.sm_count > 0 ? p.sm_count : 148) / tb.n_tiles;
-    if (n_ranges < 1) n_ranges = 1;
-  } else {
-    n_ranges = (p.n + 127) / 128;
-  }
+  // otherwise three per SM, but 128 rows or more per range
+  const int sms = p.sm_count > 0 ? p.sm_count : 148;
+  int n_ranges = tb.n_tiles > 0 ? sms / tb.n_tiles : 3 * sms / (gp.n_tiles + narrow.n_blocks);
+  if (tb.n_tiles == 0 && n_ranges > (p.n + 127) / 128) n_ranges = (p.n + 127) / 128;
+  if (n_ranges < 1) n_ranges = 1;
   if (n_ranges > SG_SPLITS) n_ranges = SG_SPLITS;
   const int rows_per_range = ((p.n + n_ranges - 1) / n_ranges + 31) / 32 * 32;
   n_ranges = (p.n + rows_per_range - 1) / rows_per_range;
@@ -984,7 +1044,7 @@ static cudaError_t sgd_step_layered(const SgdParams& p, float lr, const AdamPara
   }
   if (A <= 4) {
     ++*p.launches;
-    if ((e = launch_chained(sgd_rows_kernel<false>, sgd_partial_count(n), 256, 0, s, p, (const float*)p.dh2)) != cudaSuccess) return e;
+    if ((e = launch_chained(sgd_rows_kernel<false>, sgd_partial_count(n), 32 * SG_ROWS, 0, s, p, (const float*)p.dh2)) != cudaSuccess) return e;
     return backward_and_update(p, lr, adam, s);
   }
   // both heads in one launch: Q of the online network into g, of the target network into qt
@@ -998,7 +1058,7 @@ static cudaError_t sgd_step_layered(const SgdParams& p, float lr, const AdamPara
   }
   if (e != cudaSuccess) return e;
   ++*p.launches;
-  if ((e = launch_chained(sgd_loss_kernel, sgd_partial_count(n), 256, 0, s, p)) != cudaSuccess) return e;
+  if ((e = launch_chained(sgd_loss_kernel, sgd_partial_count(n), 32 * SG_ROWS, 0, s, p)) != cudaSuccess) return e;
   return backward_and_update(p, lr, adam, s);
 }
 
@@ -1027,7 +1087,7 @@ cudaError_t launch_ppo_step(const SgdParams& p, float lr, const AdamParams* adam
   if ((e = sg_gemm<false, GM_BIAS_RELU>(p, GemmPair{{p.obs}, {W1}, {p.h1}, {b1}}, 1, D, D, H, n, H, D, nullptr, 0, s)) != cudaSuccess) return e;
   if ((e = sg_gemm<false, GM_BIAS_RELU>(p, GemmPair{{p.h1}, {W2}, {p.h2}, {b2}}, 1, H, H, H, n, H, H, nullptr, 0, s)) != cudaSuccess) return e;
   *p.launches += stats_out ? 2 : 1;
-  if ((e = launch_chained(sgd_rows_kernel<true>, sgd_partial_count(n), 256, 0, s, p, (const float*)nullptr)) != cudaSuccess) return e;
+  if ((e = launch_chained(sgd_rows_kernel<true>, sgd_partial_count(n), 32 * SG_ROWS, 0, s, p, (const float*)nullptr)) != cudaSuccess) return e;
   if (stats_out && (e = launch_chained(ppo_finish_kernel, 1, 160, 0, s, (const float*)p.stat_partial, sgd_partial_count(n), n, stats_out)) != cudaSuccess)
     return e;
   return backward_and_update(p, lr, adam, s);
