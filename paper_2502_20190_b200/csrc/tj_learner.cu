@@ -24,7 +24,8 @@ __global__ void transpose_pad_kernel(const float* __restrict__ src, float* __res
 // interval of blocks, or two where it wraps round the ring's end (p.n_lo blocks from 0, the rest from p.b_hi on).  The host
 // knows both from its own bookkeeping, and E[r] is arithmetic: no list of eligible blocks is built or read.
 //
-// draw_slots_kernel: draw j takes E[mulhi(x0, |E|)]; one thread per draw, bound by one launch's latency.
+// draw_slots_kernel: draw j takes E[mulhi(x0, |E|)]; one thread per draw, bound by one launch's latency (the arithmetic
+// reads no memory and runs before the wait for the kernel in front).
 __device__ __forceinline__ int eligible_slot(const SampleParams& p, uint32_t r) {
   const uint32_t i = r / (uint32_t)p.N, e = r % (uint32_t)p.N;
   const uint32_t block = i < (uint32_t)p.n_lo ? i : (uint32_t)p.b_hi + (i - (uint32_t)p.n_lo);
@@ -32,12 +33,12 @@ __device__ __forceinline__ int eligible_slot(const SampleParams& p, uint32_t r) 
 }
 
 __global__ void __launch_bounds__(256) draw_slots_kernel(const SampleParams p) {
-  chain_begin();
-  chain_next();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= p.B) return;
   const uint4 w = stream_words(p.seed, STREAM_SAMPLE, 0, (uint32_t)j, (unsigned long long)p.k);
   const int slot = eligible_slot(p, __umulhi(w.x, p.n_elig));
+  chain_begin();
+  chain_next();
+  if (j >= p.B) return;
   p.slots[j] = slot;
   if (p.idx_out) p.idx_out[j] = slot;
 }
@@ -49,14 +50,14 @@ __global__ void __launch_bounds__(256) draw_slots_kernel(const SampleParams p) {
 // handful of bins in use serialised in L2 (8,192 draws of 1,040 bytes: 10.4 us before, 4.9 us with the counts per block).
 template <int LPD, int UNR, bool VEC>
 __global__ void __launch_bounds__(256) gather_kernel(const SampleParams p) {
-  chain_begin();
-  chain_next();
   __shared__ unsigned int bins[33];
   __shared__ unsigned long long most;
   constexpr int DPW = 32 / LPD;                              // draws a warp covers at a time
   const int lane = threadIdx.x & 31, sub = lane % LPD, warp = threadIdx.x >> 5;
   for (int i = threadIdx.x; i < 33; i += blockDim.x) bins[i] = 0u;
   if (threadIdx.x == 0) most = 0ull;
+  chain_begin();
+  chain_next();
   __syncthreads();
   const int chunks = p.rec_words / 4, dq = p.D / 4;
   const int j0 = (blockIdx.x * (int)(blockDim.x >> 5) + warp) * (DPW * UNR) + lane / LPD;

@@ -580,6 +580,14 @@ __global__ void __launch_bounds__(FA_NT) sgd_fused_apply_kernel(float* __restric
   const int tid = threadIdx.x, lane = tid & 31, share = tid >> 5, q = blockIdx.x * 32 + lane;
   chain_begin();
   chain_next();
+  // this thread's parameter and moments are on their way while the partials are added
+  const int i = blockIdx.x * 128 + tid;
+  const bool mine = tid < 128 && i < count;
+  float theta_i = 0.f, m_i = 0.f, v_i = 0.f;
+  if (mine) {
+    theta_i = theta[i];
+    if (ADAM) { m_i = ap.m[i]; v_i = ap.v[i]; }
+  }
   float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
   if (4 * q < count) {
 #pragma unroll 8
@@ -591,20 +599,19 @@ __global__ void __launch_bounds__(FA_NT) sgd_fused_apply_kernel(float* __restric
   sums[share][lane] = s;
   __syncthreads();
   if (tid < 128) {
-    const int i = blockIdx.x * 128 + tid;
-    if (i < count) {
+    if (mine) {
       const float* col = reinterpret_cast<const float*>(&sums[0][0]) + tid;
       float g = 0.f;
 #pragma unroll
       for (int k = 0; k < FA_SHARES; ++k) g += col[k * 128];
       if (ADAM) {
-        const float mi = fmaf(ap.beta1, ap.m[i], (1.f - ap.beta1) * g);
-        const float vi = fmaf(ap.beta2, ap.v[i], (1.f - ap.beta2) * g * g);
+        const float mi = fmaf(ap.beta1, m_i, (1.f - ap.beta1) * g);
+        const float vi = fmaf(ap.beta2, v_i, (1.f - ap.beta2) * g * g);
         ap.m[i] = mi;
         ap.v[i] = vi;
-        theta[i] -= lr * (mi / ap.c1) / (sqrtf(vi / ap.c2) + ap.eps);
+        theta[i] = theta_i - lr * (mi / ap.c1) / (sqrtf(vi / ap.c2) + ap.eps);
       } else {
-        theta[i] -= lr * g;
+        theta[i] = theta_i - lr * g;
       }
     }
   } else if (blockIdx.x == 0 && loss_out && share >= 4 && share - 4 < n_terms) {
