@@ -479,7 +479,7 @@ int tj_actor_step(tj_ctx* x, int32_t n_steps, float* dbg_logits) {
       t.b1 = W + x->wl.off_b1; t.b2 = W + x->wl.off_b2; t.b3 = W + x->wl.off_b3;
       t.out = x->logits_buf; t.error = &x->dstats->error;
       if (x->use_tc_fused) {
-        // one kernel per step: network, selection, A s on the tensor cores, env epilogue, insert
+        // one kernel per step (the pipelined one: per call): network, selection, A s on the tensor cores, env epilogue, insert
         t.out = dbg_logits ? dbg_logits + (size_t)i * x->N * x->A : nullptr;
         TcEnvParams& ev = t.env;
         ev.fused = 1; ev.A = x->A; ev.max_ep = x->max_ep; ev.rec_words = x->rec_words; ev.version = (int)x->version;
@@ -492,9 +492,12 @@ int tj_actor_step(tj_ctx* x, int32_t n_steps, float* dbg_logits) {
         if (x->use_tc_pipelined) {
           t.wtc = x->wtc_pipe[x->active];
           ev.z_scratch = x->z_scratch;
-          ev.slot0 = ev.cursor % (unsigned long long)c.replay_capacity;
+          ev.n_blocks = (uint32_t)(c.replay_capacity / x->N);
+          ev.block0 = (uint32_t)(ev.cursor / (uint64_t)x->N % ev.n_blocks);
+          ev.n_steps = n_steps;
           ev.lgA16 = x->lgA16; ev.lgB_t = x->lgB_t; ev.z_to_t = x->z_to_t;
           e = launch_actor_tc_pipelined(t, x->sm_count, x->stream);
+          break;                           // every step of the call
         } else {
           e = launch_tc_mlp(t, x->sm_count, x->stream);
         }

@@ -220,7 +220,8 @@ struct TcEnvParams {
   float noise_std, done_norm;
   DevStats* stats;
   float* z_scratch;                  // pipelined actor: per thread block two tiles of z, [2][32][128][4] floats
-  unsigned long long slot0;          // pipelined actor: cursor mod C, the ring slot of env 0 in this step
+  uint32_t block0, n_blocks;         // pipelined actor: ring block of the first step, blocks (of n records) in the ring
+  int n_steps;                       // pipelined actor: steps per launch (t and out belong to the first)
   const uint16_t* lgA16;             // pipelined actor: scaled env matrix as FP16 high / low chunks
   const float* lgB_t;                // pipelined actor: B [A][D] times 2 log2(e)
   float z_to_t;                      // pipelined actor: accumulator of the scaled product -> 2 log2(e) * z

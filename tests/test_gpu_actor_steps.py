@@ -1,0 +1,32 @@
+"""Several steps in one launch of the pipelined actor against one launch per step: a block with one tile, blocks with one and two, blocks
+with several, a ring that wraps inside the call and one that a call writes more than once.  Bit for bit."""
+import numpy as np
+import pytest
+
+import test_gpu_two_stream
+from parity_util import blob_for, fields_for
+
+pytestmark = pytest.mark.gpu
+env = test_gpu_two_stream.env
+
+
+@pytest.mark.parametrize("H,N,blocks,calls", [(128, 1, 5, (3, 4)), (512, 100, 4, (2, 7)), (128, 128 * 150 + 5, 6, (5, 4)), (256, 128 * 400, 3, (2, 3))])
+def test_steps_of_a_call_equal_single_steps(env, H, N, blocks, calls):
+    torch, binding = env
+    f = fields_for(env_kind=2, n_envs=N, obs_dim=128, n_actions=7, hidden=H, epsilon=0.2, seed=91, weight_dtype=1, replay_capacity=N * blocks,
+                   minibatch=1, staleness_bound=4, warmup=0, target_sync_interval=5, gamma=0.99, huber_delta=1.0, max_episode_steps=3,
+                   lg_done_norm=9.0)
+    got = []
+    for single in (False, True):
+        ctx = binding.Context(**f)
+        for i, n in enumerate(calls):
+            ctx.publish_weights(torch.from_numpy(blob_for(f, i + 1)).cuda())
+            for _ in range(n if single else 1):
+                ctx.actor_step(1 if single else n)
+        ring, ver = ctx.ring_view()
+        view, s = ctx.get_state(), ctx.stats()
+        got.append([a.view(torch.int32).cpu().numpy().copy() for a in (ring, ver, view["state"], view["ep_step"])] +
+                   [np.int64([s["episodes_finished"], s["produced"], s["device_error"]])])
+    assert got[0][-1][2] == 0 and got[0][-1][0] > 0
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
