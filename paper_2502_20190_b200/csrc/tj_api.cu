@@ -470,7 +470,8 @@ int tj_actor_step(tj_ctx* x, int32_t n_steps, float* dbg_logits) {
   p.dbg_logits = dbg_logits; p.stats = x->dstats;
   cudaError_t e = cudaSuccess;
   if (x->use_tc && c.env_kind == TJ_ENV_LINGAUSS) {
-    // network on the tensor cores, then the env/selection/insert kernel reads its outputs; one pair per step
+    // fused where the sizes allow it; else the network on the tensor cores and an env/selection/insert kernel that reads its
+    // outputs, one pair per step
     const float* W = x->wbuf[x->active];
     for (int i = 0; i < n_steps && e == cudaSuccess; ++i) {
       TcMlpParams t{};
@@ -479,29 +480,28 @@ int tj_actor_step(tj_ctx* x, int32_t n_steps, float* dbg_logits) {
       t.b1 = W + x->wl.off_b1; t.b2 = W + x->wl.off_b2; t.b3 = W + x->wl.off_b3;
       t.out = x->logits_buf; t.error = &x->dstats->error;
       if (x->use_tc_fused) {
-        // one kernel per step (the pipelined one: per call): network, selection, A s on the tensor cores, env epilogue, insert
-        t.out = dbg_logits ? dbg_logits + (size_t)i * x->N * x->A : nullptr;
+        // one kernel for all steps of the call: network, selection, A s on the tensor cores, env epilogue, insert
+        t.out = dbg_logits;
         TcEnvParams& ev = t.env;
         ev.fused = 1; ev.A = x->A; ev.max_ep = x->max_ep; ev.rec_words = x->rec_words; ev.version = (int)x->version;
         ev.state = x->state; ev.ep_step = x->ep_step; ev.ep_return = x->ep_return;
-        ev.seed = p.seed; ev.explore_thr = p.explore_thr; ev.t = (unsigned long long)(x->t + i);
-        ev.ring = x->ring; ev.C = c.replay_capacity; ev.cursor = x->cursor + (uint64_t)i * x->N; ev.block_ver = x->block_ver;
+        ev.seed = p.seed; ev.explore_thr = p.explore_thr; ev.t = (unsigned long long)x->t;
+        ev.n_steps = n_steps;
+        ev.ring = x->ring; ev.block_ver = x->block_ver;
+        ev.n_blocks = (uint32_t)(c.replay_capacity / x->N);
+        ev.block0 = (uint32_t)(x->cursor / (uint64_t)x->N % ev.n_blocks);
         ev.lgA_hi = x->lgA_hi; ev.lgA_lo = x->lgA_lo; ev.lgB = x->lgB;
         ev.noise_std = c.lg_noise_std; ev.done_norm = c.lg_done_norm; ev.stats = x->dstats;
         LaunchScope scope(x, TJ_K_ACTOR_FUSED, 1);
         if (x->use_tc_pipelined) {
           t.wtc = x->wtc_pipe[x->active];
           ev.z_scratch = x->z_scratch;
-          ev.n_blocks = (uint32_t)(c.replay_capacity / x->N);
-          ev.block0 = (uint32_t)(ev.cursor / (uint64_t)x->N % ev.n_blocks);
-          ev.n_steps = n_steps;
           ev.lgA16 = x->lgA16; ev.lgB_t = x->lgB_t; ev.z_to_t = x->z_to_t;
           e = launch_actor_tc_pipelined(t, x->sm_count, x->stream);
-          break;                           // every step of the call
         } else {
           e = launch_tc_mlp(t, x->sm_count, x->stream);
         }
-        continue;
+        break;
       }
       {
         LaunchScope scope(x, TJ_K_MLP_TENSOR, 1);

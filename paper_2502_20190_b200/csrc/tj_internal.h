@@ -212,16 +212,14 @@ struct TcEnvParams {
   uint2 seed;
   unsigned long long explore_thr, t;
   float* ring;
-  long long C;
-  unsigned long long cursor;
   int* block_ver;
+  uint32_t block0, n_blocks;         // ring block of the first step, blocks (of n records) in the ring
+  int n_steps;                       // steps per launch (t and the outputs belong to the first)
   const uint32_t *lgA_hi, *lgA_lo;   // env matrix, TF32 high / low parts, tiled
   const float* lgB;                  // [A][D]
   float noise_std, done_norm;
   DevStats* stats;
   float* z_scratch;                  // pipelined actor: per thread block two tiles of z, [2][32][128][4] floats
-  uint32_t block0, n_blocks;         // pipelined actor: ring block of the first step, blocks (of n records) in the ring
-  int n_steps;                       // pipelined actor: steps per launch (t and out belong to the first)
   const uint16_t* lgA16;             // pipelined actor: scaled env matrix as FP16 high / low chunks
   const float* lgB_t;                // pipelined actor: B [A][D] times 2 log2(e)
   float z_to_t;                      // pipelined actor: accumulator of the scaled product -> 2 log2(e) * z

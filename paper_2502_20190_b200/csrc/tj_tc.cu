@@ -64,6 +64,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
   TcSmem* ctl = reinterpret_cast<TcSmem*>(bias + 2 * H + TC_N3);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n_tiles = (p.n + TC_M - 1) / TC_M;
+  // this block's work: its tiles, in fused mode once per step (a tile stays with its block: no step waits for another block)
+  const int my_tiles = (n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x, n_work = my_tiles * (FUSED ? p.env.n_steps : 1);
   const int n_blocks = H > 256 ? 2 : 1, NB = H / n_blocks;           // output-neuron blocks per hidden layer
 
   if (tid == 0) {
@@ -103,7 +105,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
   if (warp == 0 && lane == 0) {
     // ------------------------------------------------------------------ producer
     uint32_t it = 0;
-    for (int tile = blockIdx.x; tile < n_tiles && !*abort_flag; tile += gridDim.x) {
+    for (int v = 0; v < n_work && !*abort_flag; ++v) {
       const uint8_t* src = reinterpret_cast<const uint8_t*>(p.wtc);
       for (int c = 0; c < c1 + c2 + c3; ++c, ++it) {
         const uint32_t bytes = c < c1 + c2 ? (uint32_t)NB * TC_KC * 2 : (uint32_t)TC_N3 * H * 2;
@@ -128,7 +130,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
     const uint32_t leader = elect_one();
     // ------------------------------------------------------------------ MMA issuer
     uint32_t it = 0, layer_count = 0;
-    for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+    for (int v = 0; v < n_work; ++v) {
       for (int layer = 0; layer < 3; ++layer, ++layer_count) {
         const int K = layer == 0 ? D : H;
         const int nb_count = layer == 2 ? 1 : n_blocks;
@@ -208,7 +210,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
     double ret_sum = 0.0;
     float4 keep[FUSED ? TC_KEEP : 1];   // this thread's half row of the FP32 state (fused mode)
     bool have_row = false;
-    for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+    const bool several = my_tiles > 1;  // the next piece of work is another tile, whose last step is done
+    uint32_t step = 0, block = FUSED ? p.env.block0 : 0;
+    int tile = blockIdx.x;
+    for (int v = 0; v < n_work; ++v) {
+      int next_tile = tile + (int)gridDim.x;
+      const bool wrap = next_tile >= n_tiles;
+      if (wrap) next_tile = blockIdx.x;
       const long long row = (long long)tile * TC_M + r;
       const bool live = row < p.n;
       // layer-1 A operand: this row of x, FP32 -> BF16, 8 elements (16 bytes) at a time.  In fused mode
@@ -218,11 +226,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
         const float* xr = p.x + (size_t)(live ? row : 0) * D;
         uint8_t* dst = abuf + ((size_t)(r >> 3) * (D / 8)) * 128 + (r & 7) * 16;
         const int g0 = hsel * (D / (8 * TC_SPLIT)), g1 = g0 + D / (8 * TC_SPLIT);
-        if (FUSED && !have_row) {      // first tile of this block; later tiles were fetched during the previous env epilogue
+        if (FUSED && !have_row) {      // first piece of work; later ones came from the previous env epilogue
 #pragma unroll
           for (int i = 0; i < TC_KEEP; ++i) {
             keep[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (live && i < D / (4 * TC_SPLIT)) keep[i] = __ldg(reinterpret_cast<const float4*>(xr + g0 * 8 + i * 4));
+            if (live && i < D / (4 * TC_SPLIT)) keep[i] = __ldcg(reinterpret_cast<const float4*>(xr + g0 * 8 + i * 4));
           }
         }
 #pragma unroll
@@ -286,14 +294,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
 #pragma unroll
           for (int j = 0; j < 16; ++j) qv[j] = __uint_as_float(v[j]) + bias[2 * H + j];
           if (live && p.out && hsel == 0) {
-            float* o = p.out + (size_t)row * p.Aout;
+            float* o = p.out + ((size_t)step * p.n + (size_t)row) * p.Aout;
 #pragma unroll
             for (int j = 0; j < 16; ++j)
               if (j < p.Aout) o[j] = qv[j];
           }
           if (FUSED) {
             // epsilon-greedy on this row: explore iff x0 < threshold, else the first maximum
-            const uint4 w = stream_words(p.env.seed, STREAM_ACTION, 0, (uint32_t)row, p.env.t);
+            const uint4 w = stream_words(p.env.seed, STREAM_ACTION, 0, (uint32_t)row, p.env.t + step);
             int best = 0;
             float qb = qv[0];
 #pragma unroll
@@ -305,8 +313,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
       }
       if (FUSED) {
         const TcEnvParams& ev = p.env;
-        const unsigned long long slot = (ev.cursor + (unsigned long long)(live ? row : 0)) % (unsigned long long)ev.C;
-        float* rec = ev.ring + slot * ev.rec_words;
+        float* rec = ev.ring + ((unsigned long long)block * (uint32_t)p.n + (unsigned long long)(live ? row : 0)) * ev.rec_words;
         // the FP32 state row once more: record's observation, and TF32 high / low parts as the A operand
         {
           uint8_t* dst_hi = abuf + ((size_t)(r >> 3) * (D / 4)) * 128 + (r & 7) * 16;
@@ -334,14 +341,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
           for (int gi = 0; gi < TC_KEEP; ++gi)
             if (gi < D / (4 * TC_SPLIT)) *reinterpret_cast<float4*>(rec + (hsel * (D / (4 * TC_SPLIT)) + gi) * 4) = keep[gi];
         }
-        {
-          const long long nrow = (long long)(tile + (int)gridDim.x) * TC_M + r;
-          have_row = true;
+        have_row = true;
+        if (several) {
+          const long long nrow = (long long)next_tile * TC_M + r;
 #pragma unroll
           for (int i = 0; i < TC_KEEP; ++i) {
             keep[i] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (nrow < p.n && i < D / (4 * TC_SPLIT))
-              keep[i] = __ldg(reinterpret_cast<const float4*>(p.x + (size_t)nrow * D + hsel * (D / TC_SPLIT) + i * 4));
+              keep[i] = __ldcg(reinterpret_cast<const float4*>(p.x + (size_t)nrow * D + hsel * (D / TC_SPLIT) + i * 4));
           }
         }
         if (!tc_wait_warp(&ctl->acc_full, layer_count & 1, abort_flag)) goto done;
@@ -359,7 +366,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
           float sn[16];
 #pragma unroll
           for (int b4 = 0; b4 < 4; ++b4) {
-            const uint4 w = stream_words(ev.seed, STREAM_NOISE, (uint32_t)(c0 / 4 + b4), (uint32_t)row, ev.t);
+            const uint4 w = stream_words(ev.seed, STREAM_NOISE, (uint32_t)(c0 / 4 + b4), (uint32_t)row, ev.t + step);
             const float2 z01 = box_muller_fast(w.x, w.y), z23 = box_muller_fast(w.z, w.w);
             const float4 bb = __ldg(reinterpret_cast<const float4*>(Ba + c0 + 4 * b4));
             sn[4 * b4 + 0] = tanh_fast(__uint_as_float(v[4 * b4 + 0]) + bb.x) + ev.noise_std * z01.x;
@@ -394,18 +401,25 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
           float ep_ret = ret0 + rew;
           const int done = (sqrtf(sq) > ev.done_norm || ep >= ev.max_ep) ? 1 : 0;
           float* st = ev.state + (size_t)row * D;
-          const int b_begin = hsel * (D / (4 * TC_SPLIT)), b_end = b_begin + D / (4 * TC_SPLIT);
+          const int b_begin = hsel * (D / (4 * TC_SPLIT));
           if (done) {
             ep_ret = 0.f;
             ep = 0;
-            for (int b4 = b_begin; b4 < b_end; ++b4) {
-              const uint4 w = stream_words(ev.seed, STREAM_RESET, (uint32_t)b4, (uint32_t)row, ev.t);
-              *reinterpret_cast<float4*>(st + 4 * b4) = make_float4(uniform_range(w.x, -0.1f, 0.2f), uniform_range(w.y, -0.1f, 0.2f),
-                                                                    uniform_range(w.z, -0.1f, 0.2f), uniform_range(w.w, -0.1f, 0.2f));
+          }
+#pragma unroll
+          for (int i = 0; i < TC_KEEP; ++i) {
+            if (i >= D / (4 * TC_SPLIT)) break;
+            const int b4 = b_begin + i;
+            float4 o;
+            if (done) {
+              const uint4 w = stream_words(ev.seed, STREAM_RESET, (uint32_t)b4, (uint32_t)row, ev.t + step);
+              o = make_float4(uniform_range(w.x, -0.1f, 0.2f), uniform_range(w.y, -0.1f, 0.2f), uniform_range(w.z, -0.1f, 0.2f),
+                              uniform_range(w.w, -0.1f, 0.2f));
+            } else {
+              o = *reinterpret_cast<const float4*>(sb + 4 * b4);
             }
-          } else {
-            for (int b4 = b_begin; b4 < b_end; ++b4)
-              *reinterpret_cast<float4*>(st + 4 * b4) = *reinterpret_cast<const float4*>(sb + 4 * b4);
+            *reinterpret_cast<float4*>(st + 4 * b4) = o;
+            if (!several) keep[i] = o;                 // this row again in the next step
           }
           if (hsel == 0) {
             *reinterpret_cast<float4*>(rec + 2 * D) =
@@ -422,7 +436,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
         mbar_arrive(&ctl->rows_done);
         if (!tc_wait_warp(&ctl->rows_done, tiles_done & 1, abort_flag)) goto done;
         ++tiles_done;
+        if (wrap) {
+          ++step;
+          if (++block == ev.n_blocks) block = 0;
+        }
       }
+      tile = next_tile;
     }
     if (FUSED) {
       // episode statistics: one atomic pair per warp
@@ -436,8 +455,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
         atomicAdd(&p.env.stats->episodes, n);
         atomicAdd(&p.env.stats->return_sum, rs);
       }
-      if (blockIdx.x == 0 && tid == 64)
-        p.env.block_ver[(p.env.cursor % (unsigned long long)p.env.C) / (unsigned long long)p.n] = p.env.version;
+      if (blockIdx.x == 0 && tid == 64) {
+        uint32_t b = p.env.block0;
+        for (int i = 0; i < p.env.n_steps; ++i) {
+          p.env.block_ver[b] = p.env.version;
+          if (++b == p.env.n_blocks) b = 0;
+        }
+      }
     }
   }
 done:

@@ -1,4 +1,4 @@
-"""Several steps in one launch of the pipelined actor against one launch per step: a block with one tile, blocks with one and two, blocks
+"""Several steps in one launch of the tensor-core actors (128 state components: pipelined; others: serial) against one launch per step: a block with one tile, blocks with one and two, blocks
 with several, a ring that wraps inside the call and one that a call writes more than once.  Bit for bit."""
 import numpy as np
 import pytest
@@ -10,10 +10,12 @@ pytestmark = pytest.mark.gpu
 env = test_gpu_two_stream.env
 
 
-@pytest.mark.parametrize("H,N,blocks,calls", [(128, 1, 5, (3, 4)), (512, 100, 4, (2, 7)), (128, 128 * 150 + 5, 6, (5, 4)), (256, 128 * 400, 3, (2, 3))])
-def test_steps_of_a_call_equal_single_steps(env, H, N, blocks, calls):
+@pytest.mark.parametrize("D,H,N,blocks,calls", [(128, 128, 1, 5, (3, 4)), (128, 512, 100, 4, (2, 7)), (128, 128, 128 * 150 + 5, 6, (5, 4)),
+                                                (128, 256, 128 * 400, 3, (2, 3)), (32, 64, 1, 5, (3, 4)), (64, 512, 200, 4, (2, 7)),
+                                                (64, 128, 128 * 150 + 5, 6, (5, 4)), (96, 96, 128 * 400, 3, (2, 3))])
+def test_steps_of_a_call_equal_single_steps(env, D, H, N, blocks, calls):
     torch, binding = env
-    f = fields_for(env_kind=2, n_envs=N, obs_dim=128, n_actions=7, hidden=H, epsilon=0.2, seed=91, weight_dtype=1, replay_capacity=N * blocks,
+    f = fields_for(env_kind=2, n_envs=N, obs_dim=D, n_actions=7, hidden=H, epsilon=0.2, seed=91, weight_dtype=1, replay_capacity=N * blocks,
                    minibatch=1, staleness_bound=4, warmup=0, target_sync_interval=5, gamma=0.99, huber_delta=1.0, max_episode_steps=3,
                    lg_done_norm=9.0)
     got = []
