@@ -225,6 +225,14 @@ struct TcEnvParams {
   float z_to_t;                      // pipelined actor: accumulator of the scaled product -> 2 log2(e) * z
 };
 
+// one network's inputs, parameters and outputs
+struct TcNetwork {
+  const float* x;          // [n][D] FP32 rows
+  const uint16_t* wtc;     // BF16 weight chunks in streaming order
+  const float *b1, *b2, *b3;
+  float* out;              // [n][Aout] (nullable in fused mode)
+};
+
 struct TcMlpParams {
   const float* x;          // [n][D] FP32 rows
   int n, D, H, Aout;
@@ -232,6 +240,7 @@ struct TcMlpParams {
   const float *b1, *b2, *b3;
   float* out;              // [n][Aout] (nullable in fused mode)
   unsigned long long* error;
+  TcNetwork second;        // network only: another one of the same shape in the same launch, if its x is not null
   TcEnvParams env;
 };
 

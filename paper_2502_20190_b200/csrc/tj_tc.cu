@@ -57,6 +57,10 @@ struct TcSmem {
 template <bool FUSED>
 __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpParams p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
+  const bool one = FUSED || blockIdx.y == 0;
+  // member by member: chosen as a whole struct, nvcc 12.9 kept x of the first network for both
+  const TcNetwork net{one ? p.x : p.second.x,   one ? p.wtc : p.second.wtc, one ? p.b1 : p.second.b1,
+                      one ? p.b2 : p.second.b2, one ? p.b3 : p.second.b3,   one ? p.out : p.second.out};
   const int D = p.D, H = p.H;
   uint8_t* abuf = smem_raw;                                          // [128][Kmax] bf16, core-matrix layout
   uint8_t* ring = abuf + tc_abuf_bytes(D, H, FUSED);                 // TC_STAGES x TC_STAGE_BYTES
@@ -89,9 +93,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
   chain_begin();
   for (int i = tid; i < 2 * H + TC_N3; i += TC_THREADS) {
     float v;
-    if (i < H) v = p.b1[i];
-    else if (i < 2 * H) v = p.b2[i - H];
-    else v = (i - 2 * H) < p.Aout ? p.b3[i - 2 * H] : 0.f;
+    if (i < H) v = net.b1[i];
+    else if (i < 2 * H) v = net.b2[i - H];
+    else v = (i - 2 * H) < p.Aout ? net.b3[i - 2 * H] : 0.f;
     bias[i] = v;
   }
   __syncthreads();
@@ -106,7 +110,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
     // ------------------------------------------------------------------ producer
     uint32_t it = 0;
     for (int v = 0; v < n_work && !*abort_flag; ++v) {
-      const uint8_t* src = reinterpret_cast<const uint8_t*>(p.wtc);
+      const uint8_t* src = reinterpret_cast<const uint8_t*>(net.wtc);
       for (int c = 0; c < c1 + c2 + c3; ++c, ++it) {
         const uint32_t bytes = c < c1 + c2 ? (uint32_t)NB * TC_KC * 2 : (uint32_t)TC_N3 * H * 2;
         const int s = it % TC_STAGES;
@@ -223,7 +227,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
       // (D <= 128) the thread keeps its half row in registers: it is the record's observation and the TF32
       // operand later in the tile, so the state is read from memory once.
       {
-        const float* xr = p.x + (size_t)(live ? row : 0) * D;
+        const float* xr = net.x + (size_t)(live ? row : 0) * D;
         uint8_t* dst = abuf + ((size_t)(r >> 3) * (D / 8)) * 128 + (r & 7) * 16;
         const int g0 = hsel * (D / (8 * TC_SPLIT)), g1 = g0 + D / (8 * TC_SPLIT);
         if (FUSED && !have_row) {      // first piece of work; later ones came from the previous env epilogue
@@ -293,8 +297,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
           float qv[16];
 #pragma unroll
           for (int j = 0; j < 16; ++j) qv[j] = __uint_as_float(v[j]) + bias[2 * H + j];
-          if (live && p.out && hsel == 0) {
-            float* o = p.out + ((size_t)step * p.n + (size_t)row) * p.Aout;
+          if (live && net.out && hsel == 0) {
+            float* o = net.out + ((size_t)step * p.n + (size_t)row) * p.Aout;
 #pragma unroll
             for (int j = 0; j < 16; ++j)
               if (j < p.Aout) o[j] = qv[j];
@@ -348,7 +352,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
           for (int i = 0; i < TC_KEEP; ++i) {
             keep[i] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (nrow < p.n && i < D / (4 * TC_SPLIT))
-              keep[i] = __ldcg(reinterpret_cast<const float4*>(p.x + (size_t)nrow * D + hsel * (D / TC_SPLIT) + i * 4));
+              keep[i] = __ldcg(reinterpret_cast<const float4*>(net.x + (size_t)nrow * D + hsel * (D / TC_SPLIT) + i * 4));
           }
         }
         if (!tc_wait_warp(&ctl->acc_full, layer_count & 1, abort_flag)) goto done;
@@ -523,7 +527,8 @@ cudaError_t launch_tc_mlp(const TcMlpParams& p, int sm_count, cudaStream_t s) {
                       sizeof(TcSmem) + 64;
   if (smem > 227 * 1024) return cudaErrorInvalidConfiguration;
   const int n_tiles = (p.n + TC_M - 1) / TC_M;
-  const int grid = n_tiles < sm_count ? n_tiles : sm_count;
+  const int nets = !fused && p.second.x ? 2 : 1, most = sm_count / nets;
+  const dim3 grid(n_tiles < most ? n_tiles : most, nets);
   return launch_chained(fused ? mlp_bf16_tc_kernel<true> : mlp_bf16_tc_kernel<false>, grid, TC_THREADS, smem, s, p);
 }
 
