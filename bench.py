@@ -34,7 +34,7 @@ from paper_2502_20190_b200 import synth  # noqa: E402
 # dram__bytes (read + write) per env-step of the fused tensor-core actor launch, from one ncu capture of the kernel as it
 # stands (a smaller number of envs, scaled: traffic grows with the number of envs).  None once the kernel has changed
 # since the counters were taken.
-NCU_DRAM_BYTES_PER_ENV_STEP = {"cfg5": 1990.0}   # 226.3 MB per launch of 113,664 envs
+NCU_DRAM_BYTES_PER_ENV_STEP = {"cfg5": 1990.0}   # 226.3 MB per step of 113,664 envs
 L2_FLUSH_BYTES = 256 << 20
 # passes of the path per bench step: about 50 ms of GPU time per step
 PATTERNS_PER_STEP = {"cfg1": 512, "cfg2": 256, "cfg3": 128, "cfg4": 8, "cfg5": 64}
@@ -388,15 +388,16 @@ def run_ours(args):
     tensor_peak = peaks["bf16_tflops_sustained"] if sustained else peaks["bf16_tflops"]
     tensor_peak_name = ("cuBLAS bf16 sustained (timed region %.2f s >= 1 s)" if sustained else "cuBLAS bf16 burst (timed region %.2f s < 1 s)") % timed_s
     if dom == 0 and w["weight_dtype"] == synth.W_BF16:
-        # fused tensor-core actor: one launch = one env step for all N envs; MLP flops only, actor launches only
+        # fused tensor-core actor: one launch = actor_steps env steps for all N envs; MLP flops only, actor launches only
         us = 1e3 * kms[0] / kcnt[0]
-        achieved = mlp_flops * N / (us * 1e-6) / 1e12
-        roof = {"kernel": "actor_tc_pipelined_kernel (fused tcgen05 actor step: MLP + selection + A s + env step + insert)",
+        units = N * r.actor_steps
+        achieved = mlp_flops * units / (us * 1e-6) / 1e12
+        roof = {"kernel": "actor_tc_pipelined_kernel (fused tcgen05 actor steps: MLP + selection + A s + env step + insert)",
                 "bound": "tensor", "achieved": achieved, "peak": tensor_peak, "unit": "TFLOP/s",
                 "peak_source": tensor_peak_name + ", of " + peaks["source"], "us_per_launch": us,
-                "units_per_launch": N, "flop_per_unit": mlp_flops,
-                "hbm_view": {"bytes_per_unit": nbytes, "achieved_gbs": nbytes * N / (us * 1e-6) / 1e9,
-                             "frac_of_measured": nbytes * N / (us * 1e-6) / 1e9 / peaks["hbm_gbs"]}}
+                "units_per_launch": units, "flop_per_unit": mlp_flops,
+                "hbm_view": {"bytes_per_unit": nbytes, "achieved_gbs": nbytes * units / (us * 1e-6) / 1e9,
+                             "frac_of_measured": nbytes * units / (us * 1e-6) / 1e9 / peaks["hbm_gbs"]}}
     elif dom == 0 and w["weight_dtype"] == synth.W_FP32_TC:
         # split-operand tensor-core actor: one launch = actor_steps env steps; algorithmic MLP flops (the hidden x hidden
         # layer costs three tensor-core products per algorithmic product, so the pipe does about 3x this work)
@@ -414,7 +415,7 @@ def run_ours(args):
         us = 1e3 * kms[0] / kcnt[0]
         units = N * r.actor_steps
         achieved = flops * units / (us * 1e-6) / 1e12
-        roof = {"kernel": "actor_small_env_kernel (FP32 MLP + selection + env step + insert)", "bound": "alu",
+        roof = {"kernel": "actor_fma_kernel (FP32 MLP + selection + env step + insert)", "bound": "alu",
                 "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
                 "peak_source": "FP32 FMA loop on every SM, measured in this run (tj_calibrate_fp32)", "us_per_launch": us,
                 "units_per_launch": units, "flop_per_unit": flops,
@@ -422,7 +423,7 @@ def run_ours(args):
                              "frac_of_measured": nbytes * units / (us * 1e-6) / 1e9 / peaks["hbm_gbs"]}}
     elif dom == 1:
         us = 1e3 * kms[1] / kcnt[1]
-        rows = N if kcnt[1] and not kcnt[0] and not r.on_policy and kcnt[2] else w["minibatch"]
+        rows = N if kcnt[1] and not kcnt[0] and not r.on_policy and kcnt[2] else 2 * w["minibatch"]   # the learner's launch holds both networks
         achieved = mlp_flops * rows / (us * 1e-6) / 1e12
         roof = {"kernel": "mlp_bf16_tc_kernel (tcgen05 MLP forward)", "bound": "tensor", "achieved": achieved,
                 "peak": tensor_peak, "unit": "TFLOP/s", "peak_source": tensor_peak_name + ", of " + peaks["source"],
@@ -442,7 +443,7 @@ def run_ours(args):
         us = 1e3 * kms[dom] / (kcnt[dom] // 2 or 1)                 # the class counts the loss reduction launch as well
         if fp32_peak is None:
             fp32_peak = r.ctx.calibrate_fp32()
-        roof = {"kernel": "td_kernel (FP32 online + target forward, TD target, Huber) + loss reduction", "bound": "alu",
+        roof = {"kernel": "FP32 TD kernel (FP32 online + target forward, TD target, Huber) + loss reduction", "bound": "alu",
                 "achieved": 2 * mlp_flops * w["minibatch"] / (us * 1e-6) / 1e12, "peak": fp32_peak, "unit": "TFLOP/s",
                 "peak_source": "FP32 FMA loop on every SM, measured in this run (tj_calibrate_fp32)", "us_per_launch": us,
                 "units_per_launch": w["minibatch"], "flop_per_unit": 2 * mlp_flops}
@@ -456,8 +457,8 @@ def run_ours(args):
                 "bytes_per_unit": cb}
     roof["frac"] = roof["achieved"] / roof["peak"] if roof["peak"] else None
     per_env = NCU_DRAM_BYTES_PER_ENV_STEP.get(name) if (dom == 0 and w["weight_dtype"] == synth.W_BF16) else None
-    roof["traffic"] = per_env * N if per_env else None
-    roof["traffic_note"] = "bytes per fused actor launch (N env-steps), ncu capture at fewer envs scaled by N" if per_env else None
+    roof["traffic"] = per_env * N * r.actor_steps if per_env else None
+    roof["traffic_note"] = "bytes per fused actor launch (actor_steps x N env-steps), ncu capture at fewer envs scaled by N" if per_env else None
     if clocks and clocks.get("sm_mhz"):
         roof["sm_mhz_median_under_load"] = clocks["sm_mhz"]
     h2d, d2h = r.e2e_bytes()
