@@ -21,7 +21,6 @@
 
 #include "tj_fma.cuh"
 #include "tj_internal.h"
-#include "tj_mlp.cuh"
 #include "tj_tc.cuh"
 
 namespace tj {
