@@ -668,8 +668,12 @@ int tj_td_error(tj_ctx* x, const tj_batch* b, float* td_out, float* huber_out, f
     learner_launched(x);
     return TJ_OK;
   }
-  LaunchScope scope(x, TJ_K_TD, loss_mean_out ? 2 : 1, true, true);
-  e = launch_td(p, x->sm_count, x->lstream);
+  LaunchScope scope(x, TJ_K_TD, 0, true, true);
+  TdParams q = p;
+  q.layers = b->n <= x->sgd_rows ? x->sgd_scratch : nullptr;      // the update's h1, h2, dh1, dh2: same stream
+  int launches = 0;
+  e = launch_td(q, x->sm_count, x->lstream, &launches);
+  x->hs.kernel_launches += launches;
   if (e != cudaSuccess) return cuda_fail(x, e, "TD error");
   learner_launched(x);
   return TJ_OK;

@@ -115,6 +115,7 @@ struct TdParams {
   float* huber_out;
   float* loss_out;
   float* partial;  // scratch: one float per thread block
+  float* layers;   // scratch: four [n][H] activations, or null
   unsigned long long* error;  // device error word of the context (a bounded wait that ran out)
 };
 
@@ -269,8 +270,9 @@ cudaError_t launch_publish(const PublishParams& p, cudaStream_t s);
 cudaError_t launch_actor(int env_kind, const ActorParams& p, int sm_count, cudaStream_t s);
 cudaError_t launch_actor_fma(int env_kind, const ActorParams& p, int sm_count, cudaStream_t s);   // CartPole / Acrobot on the FP32 pipes
 cudaError_t launch_sample_gather(const SampleParams& p, cudaStream_t s);
-cudaError_t launch_td(const TdParams& p, int sm_count, cudaStream_t s);
+cudaError_t launch_td(const TdParams& p, int sm_count, cudaStream_t s, int* launches = nullptr);
 cudaError_t launch_td_fma(const TdParams& p, int sm_count, int* grid_out, cudaStream_t s);
+cudaError_t launch_td_layers(const TdParams& p, int sm_count, int* grid_out, cudaStream_t s);   // three launches
 int td_grid(int n);
 constexpr int SG_SPLITS = 32;     // at most this many row ranges per gradient product (partial sums go through scratch)
 // tensor-core products of the update (csrc/tj_sgd_tc.cu): C = epilogue(A B^T), B split and laid out once per update

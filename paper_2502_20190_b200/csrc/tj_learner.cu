@@ -311,10 +311,19 @@ cudaError_t launch_td_tile(const TdParams& p, cudaStream_t s, int* grid_out) {
   return cudaErrorInvalidConfiguration;
 }
 
-cudaError_t launch_td(const TdParams& p, int sm_count, cudaStream_t s) {
+// Parameters of both networks in shared memory where they fit; else, up to four outputs, layer by layer where the caller has room for
+// the activations (4,096 rows, hidden 256: 69 us by 32-row tiles that read W2 through L2,
+// 43 as layers; 300 rows: 66 and 15); else those tiles.
+cudaError_t launch_td(const TdParams& p, int sm_count, cudaStream_t s, int* launches) {
   int grid = 0;
   cudaError_t err = launch_td_fma(p, sm_count, &grid, s);
-  if (err == cudaSuccess && grid == 0)     // more outputs or parameters than that kernel holds
+  int n_launches = 1;
+  if (err == cudaSuccess && grid == 0 && p.layers && p.A <= 4) {
+    err = launch_td_layers(p, sm_count, &grid, s);
+    n_launches = 3;
+  }
+  if (launches) *launches = n_launches + (p.loss_out ? 1 : 0);
+  if (err == cudaSuccess && grid == 0)
     err = p.H >= 192 ? launch_td_tile<32, 128, 8, 8>(p, s, &grid) : launch_td_tile<kTdTile, kTdThreads, 4, 4>(p, s, &grid);
   if (err != cudaSuccess) return err;
   if (p.loss_out) {

@@ -658,6 +658,53 @@ __global__ void __launch_bounds__(32 * SG_ROWS) sgd_rows_kernel(const SgdParams 
   }
 }
 
+// TD error from both networks' second layers for at most four outputs, a warp per row; W3 transposed to [H][4] as publish lays it out
+__global__ void __launch_bounds__(32 * SG_ROWS) td_rows_kernel(const TdParams p, const float* __restrict__ h2, const float* __restrict__ t2) {
+  __shared__ float part[SG_ROWS];
+  chain_begin();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j = blockIdx.x * SG_ROWS + warp;
+  float l = 0.f;
+  if (j < p.n) {
+    const int act0 = p.act[j], act = act0 < 0 ? 0 : (act0 >= p.A ? p.A - 1 : act0), dn = p.done[j];
+    const float rew = p.rew[j];
+    const float4* W = reinterpret_cast<const float4*>(p.Wonline + p.off_W3t);
+    const float4* T = reinterpret_cast<const float4*>(p.Wtarget + p.off_W3t);
+    float q[4] = {0.f, 0.f, 0.f, 0.f}, qt[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+    for (int i = lane; i < p.H; i += 32) {
+      const float x = h2[(size_t)j * p.H + i], y = t2[(size_t)j * p.H + i];
+      const float4 w = __ldg(W + i), v = __ldg(T + i);
+      q[0] = fmaf(x, w.x, q[0]); q[1] = fmaf(x, w.y, q[1]); q[2] = fmaf(x, w.z, q[2]); q[3] = fmaf(x, w.w, q[3]);
+      qt[0] = fmaf(y, v.x, qt[0]); qt[1] = fmaf(y, v.y, qt[1]); qt[2] = fmaf(y, v.z, qt[2]); qt[3] = fmaf(y, v.w, qt[3]);
+    }
+    float qs = 0.f, qmax = -INFINITY;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      for (int o = 16; o > 0; o >>= 1) {
+        q[a] += __shfl_xor_sync(0xffffffffu, q[a], o);
+        qt[a] += __shfl_xor_sync(0xffffffffu, qt[a], o);
+      }
+      if (a < p.A) {
+        if (a == act) qs = q[a] + __ldg(p.Wonline + p.off_b3 + a);
+        qmax = fmaxf(qmax, qt[a] + __ldg(p.Wtarget + p.off_b3 + a));
+      }
+    }
+    const float delta = rew + p.gamma * (dn ? 0.f : 1.f) * qmax - qs, ad = fabsf(delta);
+    l = ad <= p.kappa ? 0.5f * delta * delta : p.kappa * (ad - 0.5f * p.kappa);
+    if (lane == 0) {
+      if (p.td_out) p.td_out[j] = delta;
+      if (p.huber_out) p.huber_out[j] = l;
+    }
+  }
+  if (lane == 0) part[warp] = l;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float s = 0.f;
+    for (int r = 0; r < SG_ROWS; ++r) s += part[r];
+    p.partial[blockIdx.x] = s;
+  }
+}
+
 // The same from Q values that other kernels computed, for more outputs: q (in) and g (out) share p.g ([n][A], a row is read before its
 // own warp overwrites it), qt [n][A]; dh2 has one term per entry, the selected action's.  A row is a chain of round trips (action, its
 // q, h2), so it loads what it can before the first of them: all of an h2 row in registers where 16-byte pieces of 512 units suffice
@@ -1072,6 +1119,23 @@ cudaError_t launch_sgd_step(const SgdParams& p, float lr, const AdamParams* adam
     ++*p.launches;
     e = launch_td_finish(p.partial, sgd_partial_count(p.n), p.n, loss_out, s);
   }
+  return e;
+}
+
+cudaError_t launch_td_layers(const TdParams& t, int sm_count, int* grid_out, cudaStream_t s) {
+  int launches = 0;
+  SgdParams p{};
+  p.sm_count = sm_count;
+  p.launches = &launches;
+  const size_t nH = (size_t)t.n * t.H;
+  float *h1 = t.layers, *h2 = h1 + nH, *t1 = h2 + nH, *t2 = t1 + nH;
+  const float *W = t.Wonline, *T = t.Wtarget;
+  const GemmPair l1{{t.obs, t.next_obs}, {W + t.off_W1t, T + t.off_W1t}, {h1, t1}, {W + t.off_b1, T + t.off_b1}};
+  const GemmPair l2{{h1, t1}, {W + t.off_W2t, T + t.off_W2t}, {h2, t2}, {W + t.off_b2, T + t.off_b2}};
+  cudaError_t e = sg_gemm<true, GM_BIAS_RELU>(p, l1, 2, t.D, t.Hp, t.H, t.n, t.H, t.D, nullptr, 0, s);
+  if (e == cudaSuccess) e = sg_gemm<true, GM_BIAS_RELU>(p, l2, 2, t.H, t.Hp, t.H, t.n, t.H, t.H, nullptr, 0, s);
+  *grid_out = sgd_partial_count(t.n);
+  if (e == cudaSuccess) e = launch_chained(td_rows_kernel, *grid_out, 32 * SG_ROWS, 0, s, t, (const float*)h2, (const float*)t2);
   return e;
 }
 

@@ -1,7 +1,8 @@
 """The layer-by-layer update at the edges of its tiles: heads of up to four outputs (a warp per row) and of more, each tile height of
-the hidden layers, narrow gradients whose last 64-neuron block is ragged, and fewer units than outputs."""
+the hidden layers, narrow gradients whose last 64-neuron block is ragged, and fewer units than outputs; the TD error by the same layers."""
 import pytest
 
+import test_gpu_parity
 import test_gpu_ppo
 import test_gpu_sgd
 
@@ -18,3 +19,8 @@ def test_sgd_step(env, kind, D, A, H, B):
 @pytest.mark.parametrize("kind,D,A,H,N,T,B", [(1, 6, 3, 129, 40, 10, 257), (0, 4, 2, 256, 300, 10, 2999), (0, 4, 2, 200, 20, 4, 40)])
 def test_ppo_step(env, kind, D, A, H, N, T, B):
     test_gpu_ppo.test_ppo_step_matches_oracle(env, kind, D, A, H, N, T, B, 0)
+
+
+@pytest.mark.parametrize("kind,D,A,H,B", [(1, 6, 3, 161, 33), (0, 4, 2, 256, 4097), (1, 6, 3, 256, 15), (2, 12, 4, 333, 300), (0, 4, 2, 768, 130)])
+def test_td_error(env, kind, D, A, H, B):
+    test_gpu_parity.test_td_error_parity(env, kind, D, A, H, B)
