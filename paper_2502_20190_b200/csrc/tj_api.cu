@@ -615,6 +615,7 @@ TdParams td_params(const tj_ctx* x, const tj_batch* b, float* td_out, float* hub
   p.gamma = x->cfg.gamma; p.kappa = x->cfg.huber_delta;
   p.td_out = td_out; p.huber_out = huber_out; p.loss_out = loss_mean_out; p.partial = partial;
   p.error = &x->dstats->error;
+  p.layers = b->n <= x->sgd_rows ? x->sgd_scratch : nullptr;      // the update's h1, h2, dh1, dh2: same stream
   return p;
 }
 }  // namespace
@@ -669,10 +670,8 @@ int tj_td_error(tj_ctx* x, const tj_batch* b, float* td_out, float* huber_out, f
     return TJ_OK;
   }
   LaunchScope scope(x, TJ_K_TD, 0, true, true);
-  TdParams q = p;
-  q.layers = b->n <= x->sgd_rows ? x->sgd_scratch : nullptr;      // the update's h1, h2, dh1, dh2: same stream
   int launches = 0;
-  e = launch_td(q, x->sm_count, x->lstream, &launches);
+  e = launch_td(p, x->sm_count, x->lstream, &launches);
   x->hs.kernel_launches += launches;
   if (e != cudaSuccess) return cuda_fail(x, e, "TD error");
   learner_launched(x);
@@ -690,8 +689,10 @@ int tj_td_error_static(tj_ctx* x, const tj_batch* b, float* td_out, float* huber
   }
   const TdParams p = td_params(x, b, td_out, huber_out, loss_mean_out, nullptr);
   bool too_large = false;
-  LaunchScope scope(x, TJ_K_TD, loss_mean_out ? 2 : 1, /*may_create=*/false, true);
-  cudaError_t e = launch_td_static(p, x->cfg.device, x->sm_count, x->lstream, &too_large);
+  int launches = 0;
+  LaunchScope scope(x, TJ_K_TD, 0, /*may_create=*/false, true);
+  cudaError_t e = launch_td_static(p, x->cfg.device, x->sm_count, x->lstream, &launches, &too_large);
+  x->hs.kernel_launches += launches;
   if (too_large) return fail(x, TJ_ERR_INVALID_ARG, "tj_td_error_static: batch too large for the library's scratch");
   if (e == cudaErrorInvalidDevice) return fail(x, TJ_ERR_INVALID_ARG, "tj_td_error_static: the context's device must be the current device");
   if (e != cudaSuccess) return cuda_fail(x, e, "TD error (library scratch)");

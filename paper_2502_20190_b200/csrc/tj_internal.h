@@ -274,9 +274,11 @@ cudaError_t launch_td(const TdParams& p, int sm_count, cudaStream_t s, int* laun
 cudaError_t launch_td_fma(const TdParams& p, int sm_count, int* grid_out, cudaStream_t s);
 cudaError_t launch_td_layers(const TdParams& p, int sm_count, int* grid_out, cudaStream_t s);   // three launches
 int td_grid(int n);
+inline int td_tile_rows(int H) { return H >= 192 ? 32 : 16; }   // rows of one loss partial of the FP32 TD error of a wide network
 constexpr int SG_SPLITS = 32;     // at most this many row ranges per gradient product (partial sums go through scratch)
 // tensor-core products of the update (csrc/tj_sgd_tc.cu): C = epilogue(A B^T), B split and laid out once per update
-enum { GM_BIAS_RELU = 0, GM_BIAS = 1, GM_MASK = 2 };   // relu(acc + bias[n]) | acc + bias[n] | acc where mask[m][n] > 0, else 0
+// relu(acc + bias[n]) | acc + bias[n] | acc where mask[m][n] > 0, else 0 | relu(acc) of sums that start with bias[n], k in order (FMA tiles only)
+enum { GM_BIAS_RELU = 0, GM_BIAS = 1, GM_MASK = 2, GM_CHAIN_RELU = 3 };
 struct TcGemm {
   const float* A; int lda;      // M x K row-major, 16-byte rows
   const float* Bpack;           // B (N x K) as launch_pack_tf32_operands wrote it
@@ -314,7 +316,7 @@ cudaError_t launch_sgd_step(const SgdParams& p, float lr, const AdamParams* adam
 cudaError_t launch_ppo_step(const SgdParams& p, float lr, const AdamParams* adam, float* stats_out /* device [5], nullable */,
                             cudaStream_t s);
 int td_static_max_rows();
-cudaError_t launch_td_static(const TdParams& p, int device, int sm_count, cudaStream_t s, bool* too_large);
+cudaError_t launch_td_static(const TdParams& p, int device, int sm_count, cudaStream_t s, int* launches, bool* too_large);
 cudaError_t launch_gae(const float* rew, const float* val, const uint8_t* done, int T, int N, float gamma, float lambda,
                        float* adv, float* ret, cudaStream_t s);
 int shuffle_half_bits(long long R);

@@ -311,9 +311,10 @@ cudaError_t launch_td_tile(const TdParams& p, cudaStream_t s, int* grid_out) {
   return cudaErrorInvalidConfiguration;
 }
 
-// Parameters of both networks in shared memory where they fit; else, up to four outputs, layer by layer where the caller has room for
-// the activations (4,096 rows, hidden 256: 69 us by 32-row tiles that read W2 through L2,
-// 43 as layers; 300 rows: 66 and 15); else those tiles.
+// Parameters of both networks in shared memory where they fit; else, up to four outputs, layer by layer where the context's update
+// scratch holds the activations (whole calls, hidden 256: 4,096 rows 64 us by 32-row tiles that read W2 through L2, 47 as layers; 300
+// rows 63 and 18); else those tiles.  All of them sum in the same order (tj_mlp.cuh), the layers' loss partials over the tiles' rows too:
+// the route depends on the configured minibatch, the bits do not.
 cudaError_t launch_td(const TdParams& p, int sm_count, cudaStream_t s, int* launches) {
   int grid = 0;
   cudaError_t err = launch_td_fma(p, sm_count, &grid, s);
@@ -324,7 +325,7 @@ cudaError_t launch_td(const TdParams& p, int sm_count, cudaStream_t s, int* laun
   }
   if (launches) *launches = n_launches + (p.loss_out ? 1 : 0);
   if (err == cudaSuccess && grid == 0)
-    err = p.H >= 192 ? launch_td_tile<32, 128, 8, 8>(p, s, &grid) : launch_td_tile<kTdTile, kTdThreads, 4, 4>(p, s, &grid);
+    err = td_tile_rows(p.H) == 32 ? launch_td_tile<32, 128, 8, 8>(p, s, &grid) : launch_td_tile<kTdTile, kTdThreads, 4, 4>(p, s, &grid);
   if (err != cudaSuccess) return err;
   if (p.loss_out) {
     err = launch_td_finish(p.partial, grid, p.n, p.loss_out, s);
@@ -339,7 +340,7 @@ static __device__ __align__(256) float g_td_static_partial[kStaticTdPartials];
 
 int td_static_max_rows() { return 65536; }
 
-cudaError_t launch_td_static(const TdParams& p_in, int device, int sm_count, cudaStream_t s, bool* too_large) {
+cudaError_t launch_td_static(const TdParams& p_in, int device, int sm_count, cudaStream_t s, int* launches, bool* too_large) {
   *too_large = p_in.n > td_static_max_rows() || td_grid(p_in.n) > kStaticTdPartials;
   if (*too_large) return cudaSuccess;
   // In host code the array's name is only a stand-in; the device address has to be asked for, once per device, with
@@ -364,7 +365,7 @@ cudaError_t launch_td_static(const TdParams& p_in, int device, int sm_count, cud
   }
   TdParams p = p_in;
   p.partial = scratch;
-  return launch_td(p, sm_count, s);
+  return launch_td(p, sm_count, s, launches);
 }
 
 cudaError_t launch_td_finish(const float* partial, int n_partial, int n, float* loss_out, cudaStream_t s) {

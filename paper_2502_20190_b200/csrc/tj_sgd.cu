@@ -6,6 +6,7 @@
 //   backward  dh2 = g W3[a] (h2 > 0), dh1 = (W2^T dh2) (h1 > 0)
 //   update    W3[a] -= lr sum_j g_j h2_j, W2 -= lr dh2^T h1, W1 -= lr dh1^T x, biases likewise
 // Every sum runs in a fixed order (rows ascending), so a step is reproducible bit for bit.
+#include "tj_async.cuh"
 #include "tj_internal.h"
 #include "tj_fma.cuh"
 #include "tj_tc.cuh"
@@ -35,10 +36,14 @@ __device__ __forceinline__ void multiply_step(const float* As, const float* Bs, 
   f32x2 av[2][RM / 2];
   float4 bq[2];
   auto load = [&](int k, f32x2 (&a)[RM / 2], float4& b) {
+    if constexpr (RM == 2) {
+      a[0] = *reinterpret_cast<const f32x2*>(As + k * LDA);
+    } else {
 #pragma unroll
-    for (int i = 0; i < RM / 4; ++i) {
-      const ulonglong2 v = ld_pairs(As + k * LDA + i * 4);
-      a[i * 2] = v.x; a[i * 2 + 1] = v.y;
+      for (int i = 0; i < RM / 4; ++i) {
+        const ulonglong2 v = ld_pairs(As + k * LDA + i * 4);
+        a[i * 2] = v.x; a[i * 2 + 1] = v.y;
+      }
     }
     b = *reinterpret_cast<const float4*>(Bs + k * LDB);
   };
@@ -75,16 +80,21 @@ __device__ __forceinline__ float4 load_row4(const float* base, int ld, int row, 
 // One BM x 64 tile over k in [k_begin, k_end).  load_a(r, k) gives A[r][k .. k+3] (A_KM: A[r .. r+3][k]) with r counted from the tile's
 // first row, load_b likewise (B_KN: four columns of row k).  This thread's share of the result is out[RM / 2][4]: rows `row0` .. and
 // columns `col0` .. of the tile.
-template <int BM, bool A_KM, bool B_KN, class LoadA, class LoadB>
-__device__ __forceinline__ void tile_product(LoadA load_a, LoadB load_b, int k_begin, int k_end, float* sm, float (&out)[BM / 16][4], int& row0,
-                                             int& col0) {
-  constexpr int RM = BM / 8, LDA = BM + 4, LDB = GM_BN + 4, NA = BM * GM_BK / 4 / GM_THREADS, NB = GM_BN * GM_BK / 4 / GM_THREADS;
+// CHAIN: the fixed rounding order of tj_fma.cuh instead, acc = first; acc = fma(A, B, acc) for k = 0, 1, 2, ...  The two groups then
+// take half of the rows each over the whole of every step (a third more operand loads per FMA).
+template <int BM, bool A_KM, bool B_KN, bool CHAIN, class LoadA, class LoadB>
+__device__ __forceinline__ void tile_product(LoadA load_a, LoadB load_b, int k_begin, int k_end, float* sm, const float (&first)[4],
+                                             float (&out)[BM / 16][4], int& row0, int& col0) {
+  constexpr int RM = CHAIN ? BM / 16 : BM / 8, LDA = BM + 4, LDB = GM_BN + 4, NA = BM * GM_BK / 4 / GM_THREADS,
+                NB = GM_BN * GM_BK / 4 / GM_THREADS;
   const int tid = threadIdx.x, kg = tid >> 7, ty = (tid & 127) >> 4, tx = tid & 15;
+  row0 = ty * (BM / 8) + kg * (BM / 16);
+  col0 = tx * 4;
   f32x2 acc[RM / 2][4];
 #pragma unroll
   for (int i = 0; i < RM / 2; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+    for (int j = 0; j < 4; ++j) acc[i][j] = CHAIN ? dup2(first[j]) : 0ull;
   // the next step's operands travel from global memory to registers while this one is multiplied.  Piece i of a row-major operand:
   // four k of a row, four pieces (64 bytes) of eight rows per warp; of a k-major one: four columns of row k
   auto piece_r = [](int i, int rows) { return (i >> 2) % rows; };
@@ -130,7 +140,19 @@ __device__ __forceinline__ void tile_product(LoadA load_a, LoadB load_b, int k_b
     }
     __syncthreads();
     if (k0 + GM_BK < k_end) fetch(k0 + GM_BK);
-    multiply_step<RM, GM_BK / 2, LDA, LDB>(As + kg * (GM_BK / 2) * LDA + ty * RM, Bs + kg * (GM_BK / 2) * LDB + tx * 4, acc);
+    if constexpr (CHAIN) multiply_step<RM, GM_BK, LDA, LDB>(As + row0, Bs + tx * 4, acc);
+    else multiply_step<RM, GM_BK / 2, LDA, LDB>(As + kg * (GM_BK / 2) * LDA + ty * RM, Bs + kg * (GM_BK / 2) * LDB + tx * 4, acc);
+  }
+  if constexpr (CHAIN) {
+#pragma unroll
+    for (int i = 0; i < RM / 2; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float2 v = halves(acc[i][j]);
+        out[2 * i][j] = v.x;
+        out[2 * i + 1][j] = v.y;
+      }
+    return;
   }
   // the groups swap halves of their rows: group 0 finishes the first RM / 2, group 1 the others
   __syncthreads();
@@ -149,8 +171,6 @@ __device__ __forceinline__ void tile_product(LoadA load_a, LoadB load_b, int k_b
       out[2 * i][j] = a.x + b.x;
       out[2 * i + 1][j] = a.y + b.y;
     }
-  row0 = ty * RM + kg * (RM / 2);
-  col0 = tx * 4;
 }
 
 // four consecutive outputs of a row, a 16-byte store where the row allows it
@@ -172,23 +192,25 @@ __device__ __forceinline__ void sg_gemm_body(const float* __restrict__ A, int ld
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * GM_BN;
   const bool vecA = (lda & 3) == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
   const bool vecB = (ldb & 3) == 0 && (reinterpret_cast<uintptr_t>(B) & 15) == 0;
+  float bv[4] = {0.f, 0.f, 0.f, 0.f};
+  auto load_bias = [&](int c) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (c + j < N) bv[j] = __ldg(bias + c + j);
+  };
+  if (EPI == GM_CHAIN_RELU) load_bias(n0 + (int)(threadIdx.x & 15) * 4);
   float out[BM / 16][4];
   int row0, col0;
-  tile_product<BM, false, B_KN>([&](int r, int k) { return load_row4(A, lda, m0 + r, M, k, K, vecA); },
+  tile_product<BM, false, B_KN, EPI == GM_CHAIN_RELU>([&](int r, int k) { return load_row4(A, lda, m0 + r, M, k, K, vecA); },
                                 [&](int c, int k) {
                                   return B_KN ? load_row4(B, ldb, k, K, n0 + c, N, vecB) : load_row4(B, ldb, n0 + c, N, k, K, vecB);
                                 },
-                                0, K, sm, out, row0, col0);
+                                0, K, sm, bv, out, row0, col0);
   const int n = n0 + col0;
   if (n >= N) return;
   const bool vecC = (ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0;
   const bool vecM = EPI == GM_MASK && (ldm & 3) == 0 && (reinterpret_cast<uintptr_t>(mask) & 15) == 0;
-  float bv[4] = {0.f, 0.f, 0.f, 0.f};
-  if (EPI != GM_MASK) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      if (n + j < N) bv[j] = __ldg(bias + n + j);
-  }
+  if (EPI == GM_BIAS_RELU || EPI == GM_BIAS) load_bias(n);
 #pragma unroll
   for (int i = 0; i < BM / 16; ++i) {
     const int m = m0 + row0 + i;
@@ -199,7 +221,8 @@ __device__ __forceinline__ void sg_gemm_body(const float* __restrict__ A, int ld
       out[i][2] = h.z > 0.f ? out[i][2] : 0.f; out[i][3] = h.w > 0.f ? out[i][3] : 0.f;
     } else {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) out[i][j] = EPI == GM_BIAS_RELU ? fmaxf(out[i][j] + bv[j], 0.f) : out[i][j] + bv[j];
+      for (int j = 0; j < 4; ++j)
+        out[i][j] = EPI == GM_CHAIN_RELU ? relu1(out[i][j]) : (EPI == GM_BIAS_RELU ? fmaxf(out[i][j] + bv[j], 0.f) : out[i][j] + bv[j]);
     }
     store_row4(C + (size_t)m * ldc + n, out[i], N - n, vecC);
   }
@@ -658,49 +681,77 @@ __global__ void __launch_bounds__(32 * SG_ROWS) sgd_rows_kernel(const SgdParams 
   }
 }
 
-// TD error from both networks' second layers for at most four outputs, a warp per row; W3 transposed to [H][4] as publish lays it out
-__global__ void __launch_bounds__(32 * SG_ROWS) td_rows_kernel(const TdParams p, const float* __restrict__ h2, const float* __restrict__ t2) {
-  __shared__ float part[SG_ROWS];
+// TD error from both networks' second layers for at most four outputs, every sum in the order of td_kernel: lane a of a group of four
+// sums output a of one (network, row) over k = 0, 1, 2, ..., with the block's rows of both layers and the heads' rows in shared memory;
+// the loss partials cover the rows of one of td_kernel's tiles, added in row order.
+struct TrLayout { int ldh, h, w3, q, hub, total; };       // row stride; offsets, floats: rows [2][rows], heads [2][4], outputs [2][rows][4]
+__host__ __device__ inline TrLayout tr_layout(int H, int rows) {
+  TrLayout L;
+  L.ldh = 4 * (((H + 3) / 4) | 1);
+  L.h = 0;
+  L.w3 = 2 * rows * L.ldh;
+  L.q = L.w3 + 8 * L.ldh;
+  L.hub = L.q + 8 * rows;
+  L.total = L.hub + rows;
+  return L;
+}
+constexpr int TR_NT = 256;
+__global__ void __launch_bounds__(TR_NT) td_rows_kernel(const TdParams p, const float* __restrict__ h2, const float* __restrict__ t2, int rows) {
+  extern __shared__ __align__(16) float tr_sm[];
   chain_begin();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j = blockIdx.x * SG_ROWS + warp;
-  float l = 0.f;
-  if (j < p.n) {
-    const int act0 = p.act[j], act = act0 < 0 ? 0 : (act0 >= p.A ? p.A - 1 : act0), dn = p.done[j];
-    const float rew = p.rew[j];
-    const float4* W = reinterpret_cast<const float4*>(p.Wonline + p.off_W3t);
-    const float4* T = reinterpret_cast<const float4*>(p.Wtarget + p.off_W3t);
-    float q[4] = {0.f, 0.f, 0.f, 0.f}, qt[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-    for (int i = lane; i < p.H; i += 32) {
-      const float x = h2[(size_t)j * p.H + i], y = t2[(size_t)j * p.H + i];
-      const float4 w = __ldg(W + i), v = __ldg(T + i);
-      q[0] = fmaf(x, w.x, q[0]); q[1] = fmaf(x, w.y, q[1]); q[2] = fmaf(x, w.z, q[2]); q[3] = fmaf(x, w.w, q[3]);
-      qt[0] = fmaf(y, v.x, qt[0]); qt[1] = fmaf(y, v.y, qt[1]); qt[2] = fmaf(y, v.z, qt[2]); qt[3] = fmaf(y, v.w, qt[3]);
-    }
-    float qs = 0.f, qmax = -INFINITY;
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      for (int o = 16; o > 0; o >>= 1) {
-        q[a] += __shfl_xor_sync(0xffffffffu, q[a], o);
-        qt[a] += __shfl_xor_sync(0xffffffffu, qt[a], o);
-      }
-      if (a < p.A) {
-        if (a == act) qs = q[a] + __ldg(p.Wonline + p.off_b3 + a);
-        qmax = fmaxf(qmax, qt[a] + __ldg(p.Wtarget + p.off_b3 + a));
-      }
-    }
-    const float delta = rew + p.gamma * (dn ? 0.f : 1.f) * qmax - qs, ad = fabsf(delta);
-    l = ad <= p.kappa ? 0.5f * delta * delta : p.kappa * (ad - 0.5f * p.kappa);
-    if (lane == 0) {
-      if (p.td_out) p.td_out[j] = delta;
-      if (p.huber_out) p.huber_out[j] = l;
+  const TrLayout L = tr_layout(p.H, rows);
+  float* sm = tr_sm;
+  const int tid = threadIdx.x, j0 = blockIdx.x * rows, here = min(rows, p.n - j0), H = p.H, Hq = 4 * ((H + 3) / 4);
+  int act = 0, done = 0;
+  float rew = 0.f;
+  if (tid < here) { act = p.act[j0 + tid]; rew = p.rew[j0 + tid]; done = p.done[j0 + tid]; }
+  // a warp per row: its units, then zeros up to a whole word, every copy of the block in flight at once (4,096 x 256: 10 us as a loop of
+  // loads, 6 so; 2,048 x 200: 19 and 6).  Rows beyond the last are computed from what lies there and not used
+  const bool vec = (H & 3) == 0 && (reinterpret_cast<uintptr_t>(h2) & 15) == 0 && (reinterpret_cast<uintptr_t>(t2) & 15) == 0;
+  for (int s = tid >> 5; s < 2 * rows; s += TR_NT / 32) {
+    const int net = s >= rows ? 1 : 0, r = s - net * rows, lane = tid & 31;
+    if (r >= here) continue;
+    const float* src = (net ? t2 : h2) + (size_t)(j0 + r) * H;
+    float* dst = sm + L.h + s * L.ldh;
+    if (vec) {
+      for (int k = 4 * lane; k < H; k += 128) cp_async16(dst + k, src + k);
+    } else {
+      for (int k = lane; k < H; k += 32) cp_async4(dst + k, src + k);
+      if (lane < Hq - H) dst[H + lane] = 0.f;
     }
   }
-  if (lane == 0) part[warp] = l;
+  cp_async_commit();
+#pragma unroll 2
+  for (int i = tid; i < 2 * Hq; i += TR_NT) {                    // W3 [H][4] as publish lays it out -> a row per output
+    const int net = i >= Hq ? 1 : 0, k = i - net * Hq;
+    float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (k < H) w = __ldg(reinterpret_cast<const float4*>((net ? p.Wtarget : p.Wonline) + p.off_W3t) + k);
+    float* d = sm + L.w3 + net * 4 * L.ldh + k;
+    d[0] = w.x; d[L.ldh] = w.y; d[2 * L.ldh] = w.z; d[3 * L.ldh] = w.w;
+  }
+  cp_async_wait<0>();
   __syncthreads();
-  if (threadIdx.x == 0) {
+  for (int g = tid; g < 8 * rows; g += TR_NT) {
+    const int a = g & 3, s = g >> 2, net = s >= rows ? 1 : 0;
+    sm[L.q + g] = fma_head(__ldg((net ? p.Wtarget : p.Wonline) + p.off_b3 + a), sm + L.w3 + (net * 4 + a) * L.ldh, sm + L.h + s * L.ldh, Hq / 4);
+  }
+  __syncthreads();
+  if (tid < here) {
+    act = act < 0 ? 0 : (act >= p.A ? p.A - 1 : act);
+    const float* qt = sm + L.q + 4 * (rows + tid);
+    float qmax = qt[0];
+    for (int i = 1; i < p.A; ++i) qmax = fmaxf(qmax, qt[i]);
+    const float y = rew + p.gamma * (done ? 0.f : 1.f) * qmax;
+    const float delta = y - sm[L.q + 4 * tid + act], ad = fabsf(delta);
+    const float l = ad <= p.kappa ? 0.5f * delta * delta : p.kappa * (ad - 0.5f * p.kappa);
+    if (p.td_out) p.td_out[j0 + tid] = delta;
+    if (p.huber_out) p.huber_out[j0 + tid] = l;
+    sm[L.hub + tid] = l;
+  }
+  __syncthreads();
+  if (tid == 0) {
     float s = 0.f;
-    for (int r = 0; r < SG_ROWS; ++r) s += part[r];
+    for (int r = 0; r < here; ++r) s += sm[L.hub + r];
     p.partial[blockIdx.x] = s;
   }
 }
@@ -799,14 +850,15 @@ __device__ __forceinline__ void grad_tile(float* __restrict__ P, const GradProdu
   const int j_end = j_begin + rows_per_range < n_rows ? j_begin + rows_per_range : n_rows;
   const bool vecA = (lda & 3) == 0 && (reinterpret_cast<uintptr_t>(Am) & 15) == 0;
   const bool vecB = (ldb & 3) == 0 && (reinterpret_cast<uintptr_t>(Bm) & 15) == 0;
+  const float none[4] = {0.f, 0.f, 0.f, 0.f};
   float out[GP_TILE / 16][4];
   int row0, col0;
-  tile_product<GP_TILE, true, true>([&](int m, int j) { return load_row4(Am, lda, j, j_end, m0 + m, M, vecA); },
+  tile_product<GP_TILE, true, true, false>([&](int m, int j) { return load_row4(Am, lda, j, j_end, m0 + m, M, vecA); },
                                     [&](int c, int j) {
                                       if (Bm) return load_row4(Bm, ldb, j, j_end, n0 + c, N, vecB);
                                       return make_float4(j < j_end && n0 + c == 0 ? 1.f : 0.f, 0.f, 0.f, 0.f);   // a bias: one column of ones
                                     },
-                                    j_begin, j_end, sm, out, row0, col0);
+                                    j_begin, j_end, sm, none, out, row0, col0);
   const int n = n0 + col0;
   if (n >= N) return;
   float* dst = P + (size_t)blockIdx.y * count + d.off + n;
@@ -1132,10 +1184,12 @@ cudaError_t launch_td_layers(const TdParams& t, int sm_count, int* grid_out, cud
   const float *W = t.Wonline, *T = t.Wtarget;
   const GemmPair l1{{t.obs, t.next_obs}, {W + t.off_W1t, T + t.off_W1t}, {h1, t1}, {W + t.off_b1, T + t.off_b1}};
   const GemmPair l2{{h1, t1}, {W + t.off_W2t, T + t.off_W2t}, {h2, t2}, {W + t.off_b2, T + t.off_b2}};
-  cudaError_t e = sg_gemm<true, GM_BIAS_RELU>(p, l1, 2, t.D, t.Hp, t.H, t.n, t.H, t.D, nullptr, 0, s);
-  if (e == cudaSuccess) e = sg_gemm<true, GM_BIAS_RELU>(p, l2, 2, t.H, t.Hp, t.H, t.n, t.H, t.H, nullptr, 0, s);
-  *grid_out = sgd_partial_count(t.n);
-  if (e == cudaSuccess) e = launch_chained(td_rows_kernel, *grid_out, 32 * SG_ROWS, 0, s, t, (const float*)h2, (const float*)t2);
+  cudaError_t e = sg_gemm<true, GM_CHAIN_RELU>(p, l1, 2, t.D, t.Hp, t.H, t.n, t.H, t.D, nullptr, 0, s);
+  if (e == cudaSuccess) e = sg_gemm<true, GM_CHAIN_RELU>(p, l2, 2, t.H, t.Hp, t.H, t.n, t.H, t.H, nullptr, 0, s);
+  const int rows = td_tile_rows(t.H);
+  *grid_out = (t.n + rows - 1) / rows;
+  if (e == cudaSuccess)
+    e = launch_chained(td_rows_kernel, *grid_out, TR_NT, (size_t)tr_layout(t.H, rows).total * sizeof(float), s, t, (const float*)h2, (const float*)t2, rows);
   return e;
 }
 

@@ -27,16 +27,6 @@ __host__ __device__ inline int fs_ld(int k) {
   return 4 * (q | 1);
 }
 
-__device__ __forceinline__ void cp_async16(float* dst, const float* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
 // One parameter matrix: rows x cols of the blob at float offset `src` to shared memory at `dst` (row stride ld), zeros up to
 // rows_pad x 4 ceil(cols / 4).
 struct FsLoad { int src, dst, ld, rows, cols, rows_pad; };
