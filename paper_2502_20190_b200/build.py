@@ -34,27 +34,31 @@ def build_calls(force: bool = False) -> str:
     return CALLS
 
 
-def build(force: bool = False, verbose: bool = False) -> str:
-    build_calls(force)
-    newest = max(os.path.getmtime(p) for p in _deps() if not p.endswith(".cpp"))
-    if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= newest:
-        return LIB
+def compile_library(out: str, bdir: str, more=()) -> str:
+    """All sources with the flags above and `more`, objects in `bdir`, linked to `out`."""
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
-    bdir = os.path.join(HERE, "_build")
     os.makedirs(bdir, exist_ok=True)
     objs, procs = [], []
     for src in SOURCES:
         obj = os.path.join(bdir, src.replace(".cu", ".o"))
         objs.append(obj)
-        cmd = [nvcc] + NVCC_FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-c", os.path.join(CSRC, src), "-o", obj]
+        cmd = [nvcc] + NVCC_FLAGS + list(more) + ["-c", os.path.join(CSRC, src), "-o", obj]
         procs.append((cmd, subprocess.Popen(cmd)))
     for cmd, pr in procs:
         if pr.wait() != 0:
             raise RuntimeError("nvcc failed: " + " ".join(cmd))
-    tmp = LIB + ".tmp.%d" % os.getpid()
+    tmp = out + ".tmp.%d" % os.getpid()
     subprocess.check_call([nvcc, "-shared", "-Wno-deprecated-gpu-targets", "-o", tmp] + objs)
-    os.replace(tmp, LIB)
-    return LIB
+    os.replace(tmp, out)
+    return out
+
+
+def build(force: bool = False, verbose: bool = False) -> str:
+    build_calls(force)
+    newest = max(os.path.getmtime(p) for p in _deps() if not p.endswith(".cpp"))
+    if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= newest:
+        return LIB
+    return compile_library(LIB, os.path.join(HERE, "_build"), ["-Xptxas", "-v"] if verbose else [])
 
 
 if __name__ == "__main__":

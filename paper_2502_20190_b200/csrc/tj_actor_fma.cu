@@ -132,31 +132,38 @@ struct AfHidden {
   FmaTile t;
 };
 
-// The hidden layer.  Chunks of the ring are queued by thread 0 two ahead of their use, into the slot of the chunk before last.
+// The hidden layer.  Chunks of the ring are queued by thread 0 two ahead of their use, into the slot of the chunk before last.  A wait
+// that runs out is flagged and the thread goes on, in this and later steps, with meaningless numbers and without further waits;
+// thread 0, which waits for every chunk it queues, first lets the queued ones arrive and queues no more.
 template <int EPT, int NPT, int SRC>
-__device__ __forceinline__ void af_hidden(const AfHidden& a) {
+__device__ __forceinline__ void af_hidden(const AfHidden& a, bool& ok) {
   FmaAcc<EPT, NPT> acc;
   if (a.computes) fma_bias<EPT, NPT>(acc, a.b, a.t);
   if (SRC == AF_RING) {
     if ((int)(threadIdx.x >> 5) < a.warps) {
       uint64_t* empty = a.full + AF_SLOTS;
-      bool ok = true;                               // a wait that runs out is flagged; the thread goes on with meaningless numbers
+      const bool ok_before = ok;
       uint32_t g = a.g0;
 #pragma unroll 1
       for (int c = 0; c < a.n_chunks; ++c, ++g) {
         const uint32_t sl = g % AF_SLOTS;
-        if (threadIdx.x == 0 && (c + 2 < a.n_chunks || a.more)) {
+        const bool live = ok;
+        uint32_t queued = g + (c + 1 < a.n_chunks || a.more ? 2 : 1);         // chunks queued so far
+        if (threadIdx.x == 0 && ok && (c + 2 < a.n_chunks || a.more)) {
           const uint32_t n = g + 2;
-          if (n >= AF_SLOTS) ok = ok && mbar_wait_bounded(empty + n % AF_SLOTS, ((n / AF_SLOTS) - 1) & 1);
+          if (n >= AF_SLOTS) ok = mbar_wait_bounded(empty + n % AF_SLOTS, ((n / AF_SLOTS) - 1) & 1);
+          queued += ok ? 1 : 0;
           if (ok) af_queue_chunk(const_cast<float*>(a.w), a.src, a.full, n, (uint32_t)(c + 2 < a.n_chunks ? c + 2 : c + 2 - a.n_chunks), a.kc, a.H, a.Hp);
         }
         __syncwarp();
         ok = ok && mbar_wait_bounded(a.full + sl, (g / AF_SLOTS) & 1);
+        if (threadIdx.x == 0 && live && !ok)
+          for (uint32_t n = g; n < queued; ++n) mbar_settle(a.full + n % AF_SLOTS, (n / AF_SLOTS) & 1);
         if (a.computes) fma_accumulate<EPT, NPT, 4>(acc, a.w + sl * (a.kc * a.Hp), a.Hp, a.h1 + c * a.kc * a.E, a.E, min(a.kc, a.H - c * a.kc), a.t);
         __syncwarp();
         if ((threadIdx.x & 31) == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(empty + sl)) : "memory");
       }
-      if (!ok) atomicExch(a.error, 1ull);
+      if (ok_before && !ok) atomicExch(a.error, 1ull);
     }
   } else if (a.computes) {
     fma_accumulate<EPT, NPT, (EPT * NPT > 8 ? 4 : 8)>(acc, a.w, a.Hp, a.h1, a.E, a.H, a.t);
@@ -253,6 +260,10 @@ __global__ void __launch_bounds__(af_most(EPT, NPT), 1) actor_fma_kernel(const A
     if (ok && !mbar_wait_bounded(b, parity)) {
       ok = false;
       atomicExch(&p.stats->error, 1ull);
+      if (tid == 0) {                                         // the copies queued so far have to arrive before the block leaves
+        mbar_settle(bar, 0);
+        if (SRC == AF_SMEM) mbar_settle(bar + 1, 0);
+      }
     }
   };
   wait(bar, 0);
@@ -263,7 +274,7 @@ __global__ void __launch_bounds__(af_most(EPT, NPT), 1) actor_fma_kernel(const A
   __syncthreads();
 
   const int n_chunks = (p.H + q.kc - 1) / q.kc;
-  if (SRC == AF_RING && tid == 0)
+  if (SRC == AF_RING && tid == 0 && ok)
     for (uint32_t g = 0; g < 2; ++g) af_queue_chunk(sm + q.w2, p.W + p.off_W2t, full, g, g, q.kc, p.H, p.Hp);
   long long slot = q.slot0;                                   // ring slot of env 0 in this step
   int blk = q.blk0, pos = q.pos0, seg = q.seg0;
@@ -278,7 +289,7 @@ __global__ void __launch_bounds__(af_most(EPT, NPT), 1) actor_fma_kernel(const A
     hd.E = E; hd.H = p.H; hd.Hp = p.Hp; hd.ldh = q.ldh; hd.kc = q.kc; hd.overlap = q.overlap; hd.warps = cw; hd.n_chunks = n_chunks;
     hd.g0 = (uint32_t)(it * n_chunks); hd.more = it + 1 < n_iters;
     hd.t = t; hd.computes = computes;
-    af_hidden<EPT, NPT, SRC>(hd);
+    af_hidden<EPT, NPT, SRC>(hd, ok);
     __syncthreads();
     draw(it + 1);
     if (head_warp) {

@@ -47,12 +47,25 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
+// Polls before a wait gives up.  A build with 0 makes every bounded wait run out at once: how the tests reach what follows then.
+#ifndef TJ_WAIT_POLLS
+#define TJ_WAIT_POLLS (1 << 22)
+#endif
+
 // Waits for the phase with the given parity; gives up after a fixed number of polls and reports false.
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity) {
 #pragma unroll 1
-  for (int i = 0; i < (1 << 22); ++i)
+  for (int i = 0; i < TJ_WAIT_POLLS; ++i)
     if (mbar_try_wait(bar, parity)) return true;
   return false;
+}
+
+// The wait of a block that gives up for what it still has in flight (bulk copies, matrix instructions): none of it may arrive after
+// the block has handed its shared memory to another.  Bounded as well, but whatever TJ_WAIT_POLLS says.
+__device__ __forceinline__ void mbar_settle(uint64_t* bar, uint32_t parity) {
+#pragma unroll 1
+  for (int i = 0; i < (1 << 22); ++i)
+    if (mbar_try_wait(bar, parity)) return;
 }
 
 // per-thread asynchronous copies of 16 (both addresses aligned) or 4 bytes, waited for by groups

@@ -109,11 +109,13 @@ __global__ void __launch_bounds__(256) gather_kernel(const SampleParams p) {
 
 // TD error on a tile of TE samples: online forward on obs, target forward on next_obs.
 // STAGE as in the actor kernel (stage_mlp_weights); the staging buffer is filled twice (online, then target parameters).
-// A staging wait that ran out: latch the context's error word and leave defined outputs (NaN) for this block's rows and
-// its partial sum, so that neither the caller nor the loss reduction reads what an earlier call left there.
-__device__ __forceinline__ void td_give_up(const TdParams& p, int n_here, int j0) {
+// A staging wait that ran out, for the whole block: latch the context's error word and leave defined outputs (NaN) for this block's rows
+// and its partial sum, so that neither the caller nor the loss reduction reads what an earlier call left there; the staged
+// parameters have to arrive before the block leaves.
+__device__ __forceinline__ void td_give_up(const TdParams& p, int n_here, int j0, uint64_t* bar, uint32_t parity) {
   const float nan = __int_as_float(0x7FC00000);
   if (threadIdx.x == 0) {
+    mbar_settle(bar, parity);
     if (p.error) atomicExch(p.error, 3ull);
     p.partial[blockIdx.x] = nan;
   }
@@ -148,8 +150,7 @@ __global__ void __launch_bounds__(NT) td_kernel(const TdParams p) {
     const int el = i / D, k = i % D;
     xs[k * TE + el] = el < n_here ? p.obs[(size_t)(j0 + el) * D + k] : 0.f;
   }
-  if (STAGE > 0 && !mbar_wait_bounded(&wbar, 0)) { td_give_up(p, n_here, j0); return; }
-  __syncthreads();
+  if (!__syncthreads_and(STAGE == 0 || mbar_wait_bounded(&wbar, 0))) { td_give_up(p, n_here, j0, &wbar, 0); return; }
   mlp_forward_tile<TE, NT, EPT, (STAGE > 0), (STAGE == 2), NPT>(mw, D, p.H, p.Hp, p.A, p.Ap, xs, h1, h2, out);
   if (tid < n_here) {
     int a = p.act[j0 + tid];
@@ -162,8 +163,7 @@ __global__ void __launch_bounds__(NT) td_kernel(const TdParams p) {
     const int el = i / D, k = i % D;
     xs[k * TE + el] = el < n_here ? p.next_obs[(size_t)(j0 + el) * D + k] : 0.f;
   }
-  if (STAGE > 0 && !mbar_wait_bounded(&wbar, 1)) { td_give_up(p, n_here, j0); return; }
-  __syncthreads();
+  if (!__syncthreads_and(STAGE == 0 || mbar_wait_bounded(&wbar, 1))) { td_give_up(p, n_here, j0, &wbar, 1); return; }
   mlp_forward_tile<TE, NT, EPT, (STAGE > 0), (STAGE == 2), NPT>(mw, D, p.H, p.Hp, p.A, p.Ap, xs, h1, h2, out);
   if (tid < TE) {
     float h = 0.f;

@@ -422,6 +422,7 @@ __global__ void __launch_bounds__(TG_THREADS, 2) sg_gemm_tc_kernel(const float* 
   const uint32_t idesc = make_idesc_tf32(TG_N);
   constexpr uint32_t SBO = (TG_K / 4) * 128u;     // eight rows further: one row group of K/4 core matrices
   bool ok = true;
+  int issued = 0;                                 // steps whose products the tensor core has been given
   // one step: registers -> split -> stage i & 1, the tensor core's products on it, the load of step i + TG_PF.  Returns
   // false (for every thread alike) when a wait ran out.
   auto step = [&](int i, float4 (&fa)[2], float4 (&fb)[2]) -> bool {
@@ -455,6 +456,7 @@ __global__ void __launch_bounds__(TG_THREADS, 2) sg_gemm_tc_kernel(const float* 
       }
       umma_commit(&done[s], 1u);
     }
+    issued = i + 1;
     if (i + TG_PF < nk) fetch((i + TG_PF) * TG_K, fa, fb);
     return true;
   };
@@ -508,6 +510,7 @@ __global__ void __launch_bounds__(TG_THREADS, 2) sg_gemm_tc_kernel(const float* 
     }
   } else if (tid == 0) {
     atomicExch(error, 3ull);
+    for (int i = issued > 2 ? issued - 2 : 0; i < issued; ++i) mbar_settle(&done[i & 1], (uint32_t)((i >> 1) & 1));
   }
   tc_fence_before();
   __syncthreads();

@@ -297,11 +297,6 @@ __device__ __forceinline__ void grad_narrow(const FsLayout& L, const float* sm, 
   }
 }
 
-// a wait for the parameters that ran out: flag it; the update is not valid
-__device__ __forceinline__ void fused_give_up(const SgdParams& p) {
-  if (threadIdx.x == 0) atomicExch(p.error, 3ull);
-}
-
 template <int R, bool PPO>
 __global__ void __launch_bounds__(FS_NT, 1) sgd_fused_kernel(const SgdParams p, const FsLayout L, int stride) {
   extern __shared__ __align__(128) float fs_sm[];
@@ -399,6 +394,7 @@ __global__ void __launch_bounds__(FS_NT, 1) sgd_fused_kernel(const SgdParams p, 
     }
   if (tid == 0) sm[L.one] = 1.f;
   const int n_chunks = (p.n + R - 1) / R;
+  bool ok = true;                                  // a wait that runs out: the thread goes on with meaningless numbers
   FsOut out{p.grad_partial + (size_t)blockIdx.x * stride, false};
   float part0 = 0.f, part1 = 0.f, part2 = 0.f, part3 = 0.f, part4 = 0.f;     // thread 0: the block's loss terms
   for (int chunk = blockIdx.x; chunk < n_chunks; chunk += gridDim.x, out.add = true) {
@@ -426,12 +422,12 @@ __global__ void __launch_bounds__(FS_NT, 1) sgd_fused_kernel(const SgdParams p, 
       }
     }
     __syncthreads();
-    if (L.bulk && !mbar_wait_bounded(bar, 0)) { fused_give_up(p); return; }
+    if (L.bulk) ok = ok && mbar_wait_bounded(bar, 0);
     if (!PPO) {
-      if (L.bulk && !mbar_wait_bounded(bar + 1, 0)) { fused_give_up(p); return; }
+      if (L.bulk) ok = ok && mbar_wait_bounded(bar + 1, 0);
       dense_rows<R>(sm + L.T2, L.ldH, sm + L.tb2, sm + L.d1, L.ldH, sm + L.d2, L.ldH, G, G, t, sm + L.red);
     }
-    if (L.bulk && !mbar_wait_bounded(bar + 2, 0)) { fused_give_up(p); return; }
+    if (L.bulk) ok = ok && mbar_wait_bounded(bar + 2, 0);
     dense_rows<R>(sm + L.W2, L.ldH, sm + L.b2, sm + L.h1, L.ldH, sm + L.h2, L.ldH, G, G, t, sm + L.red);
     // heads: eight lanes per (network, row)
     for (int slot = tid >> 3; slot < (PPO ? R : 2 * R); slot += FS_NT / 8) {
@@ -556,6 +552,14 @@ __global__ void __launch_bounds__(FS_NT, 1) sgd_fused_kernel(const SgdParams p, 
     float* pp = p.partial + (size_t)blockIdx.x * 5;
     pp[0] = part0;
     if (PPO) { pp[1] = part1; pp[2] = part2; pp[3] = part3; pp[4] = part4; }
+  }
+  if (!ok) {
+    atomicExch(p.error, 3ull);
+    if (tid == 0) {                                // thread 0 waits for every copy: if it was served, all have arrived
+      mbar_settle(bar, 0);
+      if (!PPO) mbar_settle(bar + 1, 0);
+      mbar_settle(bar + 2, 0);
+    }
   }
 }
 

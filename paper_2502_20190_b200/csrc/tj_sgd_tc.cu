@@ -14,7 +14,8 @@
 //     B slot are there, and commits free both; nobody else in its warp polls;
 //   the workers then drain the accumulator (bias + ReLU, or the backward pass's ReLU mask) to global memory.
 // Two problems (the online and the target network's layer) can share a launch: blockIdx.z picks the set.
-// Every wait is bounded; a timeout latches the error word, waits for the copies in flight and frees the tensor memory.
+// Every wait is bounded; a timeout latches the error word, waits for the copies and matrix instructions in flight and frees the
+// tensor memory.
 #include "tj_internal.h"
 #include "tj_tc.cuh"
 
@@ -34,8 +35,8 @@ constexpr int T2_B_SLOT = 2 * T2_B_PART;
 constexpr uint32_t T2_SBO = (T2_K / 4) * 128u;             // eight rows further: one row group of K/4 core matrices
 
 struct T2Ctl {
-  uint64_t a_ready[T2_ASTAGES], a_free[T2_ASTAGES], b_full[T2_BSLOTS], b_empty[T2_BSLOTS], acc_full;
-  uint32_t tmem_base;
+  uint64_t a_ready[T2_ASTAGES], a_free[T2_ASTAGES], b_full[T2_BSLOTS], b_empty[T2_BSLOTS], acc_full, settled;
+  uint32_t tmem_base, copies;                              // copies: bulk copies queued so far
   int abort_flag;
 };
 constexpr int T2_SMEM_BYTES = T2_ASTAGES * T2_A_STAGE + T2_BSLOTS * T2_B_SLOT + T2_STG_BYTES + (int)sizeof(T2Ctl) + 1024;
@@ -73,6 +74,8 @@ __global__ void __launch_bounds__(T2_THREADS, 1) sg_gemm_tc2_kernel(const TcGemm
     for (int i = 0; i < T2_ASTAGES; ++i) { mbar_init(&ctl->a_ready[i], T2_WORKERS / 32); mbar_init(&ctl->a_free[i], 1); }
     for (int i = 0; i < T2_BSLOTS; ++i) { mbar_init(&ctl->b_full[i], 1); mbar_init(&ctl->b_empty[i], 1); }
     mbar_init(&ctl->acc_full, 1);
+    mbar_init(&ctl->settled, 1);
+    ctl->copies = 0;
     ctl->abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -164,18 +167,14 @@ __global__ void __launch_bounds__(T2_THREADS, 1) sg_gemm_tc2_kernel(const TcGemm
   } else {
     if (lane == 0) {
       const uint8_t* src = reinterpret_cast<const uint8_t*>(g.Bpack) + (size_t)blockIdx.x * nk * T2_B_SLOT;
-      int issued = 0;
-      for (int i = 0; i < nk; ++i, ++issued) {
+      for (int i = 0; i < nk; ++i) {
         const int sl = i % T2_BSLOTS;
         if (i >= T2_BSLOTS && !tc_wait(&ctl->b_empty[sl], (uint32_t)(((i / T2_BSLOTS) - 1) & 1), abort_flag)) break;
         mbar_expect_tx(&ctl->b_full[sl], (uint32_t)T2_B_SLOT);
         const int c = i + rot < nk ? i + rot : i + rot - nk;
         bulk_copy_g2s(b_slots + (size_t)sl * T2_B_SLOT, src + (size_t)c * T2_B_SLOT, (uint32_t)T2_B_SLOT, &ctl->b_full[sl]);
+        ctl->copies = (uint32_t)i + 1u;
       }
-      // after a timeout elsewhere the last copies may still be on their way: they must land before the block leaves
-      if (*abort_flag)
-        for (int i = issued > T2_BSLOTS ? issued - T2_BSLOTS : 0; i < issued; ++i)
-          if (!tc_wait(&ctl->b_full[i % T2_BSLOTS], (uint32_t)((i / T2_BSLOTS) & 1), abort_flag)) break;
     }
     __syncwarp();
   }
@@ -217,8 +216,9 @@ __global__ void __launch_bounds__(T2_THREADS, 1) sg_gemm_tc2_kernel(const TcGemm
         }
       }
     }
-  } else if (!good && tid == 0) {
-    atomicExch(error, 3ull);
+  } else if (!good) {
+    if (tid == 0) atomicExch(error, 3ull);
+    tc_settle(&ctl->settled, warp == T2_WORKERS / 32, ctl->b_full, T2_BSLOTS, ctl->copies);
   }
   tc_fence_before();
   __syncthreads();
@@ -241,7 +241,7 @@ constexpr int WG_STAGES = 3;
 constexpr int WG_A_PART = T2_M * T2_K * 4, WG_B_PART = T2_N * T2_K * 4;          // 8 KB, 16 KB
 constexpr int WG_STAGE = 2 * WG_A_PART + 2 * WG_B_PART;                          // A_hi | A_lo | B_hi | B_lo: 48 KB
 struct WgCtl {
-  uint64_t ready[WG_STAGES], free_[WG_STAGES], acc_full;
+  uint64_t ready[WG_STAGES], free_[WG_STAGES], acc_full, settled;
   uint32_t tmem_base;
   int abort_flag;
   float bias_part[T2_WORKERS];     // per loader thread: its feature's sum over the row groups it read
@@ -269,6 +269,7 @@ __global__ void __launch_bounds__(T2_THREADS, 1) sg_wgrad_tc_kernel(const TcWgra
   if (tid == 0) {
     for (int i = 0; i < WG_STAGES; ++i) { mbar_init(&ctl->ready[i], T2_WORKERS / 32); mbar_init(&ctl->free_[i], 1); }
     mbar_init(&ctl->acc_full, 1);
+    mbar_init(&ctl->settled, 1);
     ctl->abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -420,8 +421,9 @@ __global__ void __launch_bounds__(T2_THREADS, 1) sg_wgrad_tc_kernel(const TcWgra
     // bias gradient: feature f was read by threads f (row groups 0 and 2 of every chunk) and f + 128 (groups 1 and 3)
     if (with_bias && tid < T2_M && m0 + tid < g.M)
       P[(size_t)blockIdx.y * count + g.bias_off + m0 + tid] = ctl->bias_part[tid] + ctl->bias_part[tid + T2_M];
-  } else if (!good && tid == 0) {
-    atomicExch(error, 3ull);
+  } else if (!good) {
+    if (tid == 0) atomicExch(error, 3ull);
+    tc_settle(&ctl->settled, warp == T2_WORKERS / 32, nullptr, 1, 0);     // no bulk copies here
   }
   tc_fence_before();
   __syncthreads();

@@ -16,7 +16,8 @@
 //   then exactly the FP32 kernel's selection, env step, record / segment write and reset.
 // The FP32 work per step (layer 1 with its split, drain, env step: about 14,000 warp instructions a tile) and the MMAs (6,100 cycles at
 // hidden 256) are of one size; what a step takes beyond them is latency.
-// Every wait is bounded; a timeout latches the context's error word and the block leaves after freeing its tensor memory.
+// Every wait is bounded; a timeout latches the context's error word and the block leaves after its copies and matrix instructions in
+// flight are over and its tensor memory is free.
 #include <cuda_fp16.h>
 
 #include "tj_fma.cuh"
@@ -69,8 +70,8 @@ constexpr int S2_A_SLOT = 2 * S2_A_PART;  // high part, low part
 struct S2Ctl {
   uint64_t full[SA_SLOTS], empty[SA_SLOTS];
   uint64_t a_ready[S2_A_SLOTS], a_free[S2_A_SLOTS];
-  uint64_t acc_full[2];
-  uint32_t tmem_base;
+  uint64_t acc_full[2], settled;
+  uint32_t tmem_base, copies;             // copies: bulk copies queued so far
   int abort_flag, range_flag;
 };
 
@@ -155,6 +156,8 @@ struct S2Smem {
       for (int s = 0; s < S2_A_SLOTS; ++s) { mbar_init(&ctl->a_ready[s], 4 * TPR); mbar_init(&ctl->a_free[s], 1); }
       mbar_init(&ctl->acc_full[0], 1);
       mbar_init(&ctl->acc_full[1], 1);
+      mbar_init(&ctl->settled, 1);
+      ctl->copies = 0;
       ctl->abort_flag = ctl->range_flag = 0;
     }
     __syncthreads();
@@ -170,6 +173,10 @@ struct S2Smem {
   __device__ __forceinline__ void tear_down(uint32_t tmem) const {
     tc_fence_before();
     __syncthreads();
+    if (ctl->abort_flag) {                                    // the issuing warp is the last but one
+      tc_settle(&ctl->settled, (int)(threadIdx.x >> 5) == NT / 32 - 2, ctl->full, SA_SLOTS, ctl->copies);
+      __syncthreads();
+    }
     if (threadIdx.x < 32) {
       __syncwarp();
       tc_fence_after();
@@ -251,11 +258,8 @@ struct S2Smem {
       if (c >= SA_SLOTS && !tc_wait(&ctl->empty[s], ((c / SA_SLOTS) - 1) & 1, abort_flag)) break;
       mbar_expect_tx(&ctl->full[s], CHUNK_BYTES);
       bulk_copy_g2s(w_ring + s * CHUNK_BYTES, reinterpret_cast<const uint8_t*>(parts) + (size_t)in_pass * CHUNK_BYTES, CHUNK_BYTES, &ctl->full[s]);
+      ctl->copies = c + 1;
     }
-    // after a timeout the last copies may still be on their way: they must land before the block gives its shared memory back
-    if (*abort_flag)
-      for (uint32_t i = c > SA_SLOTS ? c - SA_SLOTS : 0; i < c; ++i)
-        if (!mbar_wait_bounded(&ctl->full[i % SA_SLOTS], (i / SA_SLOTS) & 1)) break;
   }
 };
 

@@ -17,7 +17,8 @@
 // high and low parts; A s then runs on the tensor cores as three TF32 products (hi*hi + lo*hi + hi*lo, FP32
 // accumulation, error ~2^-21 relative per term), and the epilogue threads finish the step: + B[a], tanh, Philox
 // noise, reward, done, record, reset, new state.
-// Every wait is bounded: on a timeout the block raises an abort flag, records an error, frees its TMEM and leaves.
+// Every wait is bounded: on a timeout the block raises an abort flag, records an error, waits for its copies and matrix instructions in
+// flight, frees its TMEM and leaves.
 #include "tj_internal.h"
 #include "tj_tc.cuh"
 
@@ -48,9 +49,9 @@ __host__ __device__ inline size_t tc_abuf_bytes(int D, int H, bool fused) {
 }
 
 struct TcSmem {
-  uint64_t full[TC_STAGES], empty[TC_STAGES], a_ready, acc_full, rows_done, pair_sync;
+  uint64_t full[TC_STAGES], empty[TC_STAGES], a_ready, acc_full, rows_done, pair_sync, settled;
   float sq[TC_SPLIT][TC_M];
-  uint32_t tmem_base;
+  uint32_t tmem_base, copies;       // copies: bulk copies queued so far
   int abort_flag;
 };
 
@@ -78,6 +79,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
     mbar_init(&ctl->acc_full, 1);
     mbar_init(&ctl->rows_done, TC_EPI_THREADS);
     mbar_init(&ctl->pair_sync, TC_EPI_THREADS);
+    mbar_init(&ctl->settled, 1);
+    ctl->copies = 0;
     ctl->abort_flag = 0;
   }
   __syncthreads();
@@ -117,6 +120,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
         if (!tc_wait(&ctl->empty[s], ((it / TC_STAGES) & 1) ^ 1, abort_flag)) goto done;
         mbar_expect_tx(&ctl->full[s], bytes);
         bulk_copy_g2s(ring + (size_t)s * TC_STAGE_BYTES, src, bytes, &ctl->full[s]);
+        ctl->copies = it + 1;
         src += bytes;
       }
       if (FUSED) {
@@ -127,6 +131,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
           if (!tc_wait(&ctl->empty[s], ((it / TC_STAGES) & 1) ^ 1, abort_flag)) goto done;
           mbar_expect_tx(&ctl->full[s], bytes);
           bulk_copy_g2s(ring + (size_t)s * TC_STAGE_BYTES, esrc, bytes, &ctl->full[s]);
+          ctl->copies = it + 1;
         }
       }
     }
@@ -470,7 +475,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
   }
 done:
   __syncthreads();
-  if (tid == 0 && ctl->abort_flag) atomicExch(p.error, 2ull);
+  if (ctl->abort_flag) {
+    if (tid == 0) atomicExch(p.error, 2ull);
+    tc_settle(&ctl->settled, warp == 1, ctl->full, TC_STAGES, ctl->copies);
+    __syncthreads();
+  }
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();

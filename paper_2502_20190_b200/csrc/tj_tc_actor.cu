@@ -25,7 +25,8 @@
 // Code size counts here: five roles execute five different programs at once, and with everything unrolled the kernel no longer fitted
 // the instruction cache -- the issuing lane, which runs each line of its program once or a few times per tile, then took 446 cycles per
 // MMA of the z product (64 on the tensor pipe) fetching instructions from L2.  So loops are unrolled only as far as their latency asks.
-// Every wait is bounded: on a timeout the block raises an abort flag, records an error, frees its TMEM and leaves.
+// Every wait is bounded: on a timeout the block raises an abort flag, records an error, waits for its copies and matrix instructions in
+// flight, frees its TMEM and leaves.
 #include <cuda_fp16.h>
 
 #include "tj_internal.h"
@@ -62,8 +63,9 @@ struct PaSmem {
   uint64_t env_taken;      // env -> MMA: head outputs are in registers
   uint64_t z_stored;       // network -> env: z of the tile is in the scratch tile
   uint64_t act_ready;      // env: the rows' actions are in shared memory
+  uint64_t settled;        // after a timeout: the matrix instructions are over
   int act[2][PA_M];        // by tile parity
-  uint32_t tmem_base;
+  uint32_t tmem_base, copies;   // copies: bulk copies queued so far
   int abort_flag;
 };
 
@@ -99,6 +101,8 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
     mbar_init(&ctl->env_taken, PA_ENV_WARPS);
     mbar_init(&ctl->z_stored, PA_NET_WARPS);
     mbar_init(&ctl->act_ready, 4);
+    mbar_init(&ctl->settled, 1);
+    ctl->copies = 0;
     ctl->abort_flag = 0;
   }
   __syncthreads();
@@ -142,6 +146,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
           if (!tc_wait(&ctl->empty[s], ((it / PA_STAGES) & 1) ^ 1, abort_flag)) goto done;
           mbar_expect_tx(&ctl->full[s], bytes);
           bulk_copy_g2s_keep(ring + (size_t)s * PA_STAGE_BYTES, src, bytes, &ctl->full[s], keep_policy);
+          ctl->copies = it + 1;
         }
       }
     } else if (warp == 1) {
@@ -527,7 +532,11 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
   }
 done:
   __syncthreads();
-  if (tid == 0 && ctl->abort_flag) atomicExch(p.error, 2ull);
+  if (ctl->abort_flag) {
+    if (tid == 0) atomicExch(p.error, 2ull);
+    tc_settle(&ctl->settled, warp == 1, ctl->full, PA_STAGES, ctl->copies);
+    __syncthreads();
+  }
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();

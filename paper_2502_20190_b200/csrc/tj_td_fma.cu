@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(TF_NT, 1) td_fma_kernel(const TdParams p, cons
       const float out = fma_head(sm[q.w + n * q.s_w + p.off_b3 + a], sm + q.w3 + n * q.s_w3 + a * q.ldh, sm + q.h2 + n * q.s_h2 + r * q.ldh, p.Hp / 4);
       if (g < 2 * E) sm[q.q + 4 * g + a] = out;
     }
-    __syncthreads();
+    ok = __syncthreads_and(ok);                               // whichever thread's wait ran out, none of the block's rows is valid
     if (tid < 64) {
       float h = 0.f;
       if (tid < here) {
@@ -121,7 +121,11 @@ __global__ void __launch_bounds__(TF_NT, 1) td_fma_kernel(const TdParams p, cons
   }
   if (tid == 0) {
     p.partial[blockIdx.x] = sum;
-    if (!ok && p.error) atomicExch(p.error, 3ull);
+    if (!ok) {
+      if (p.error) atomicExch(p.error, 3ull);
+      mbar_settle(bar, 0);
+      mbar_settle(bar + 1, 0);
+    }
   }
 }
 
