@@ -12,7 +12,6 @@ from __future__ import annotations
 
 import ctypes as C
 import importlib.util
-import operator
 import os
 
 import numpy as np
@@ -318,7 +317,6 @@ class Context:
         if st != TJ_OK:
             raise TjError(st, tj_last_error())
         self._addr = self.h.value                      # what the extension module's calls take
-        self._blobs = self._ptrs = None                # parameter blobs of the last update, already checked
         self._segments = {}                            # views of the segment slots
         self._one = torch.empty(1, dtype=torch.float32, device=self.device)
         c = self.cfg
@@ -342,7 +340,7 @@ class Context:
     def close(self):
         if getattr(self, "h", None):
             tj_destroy(self.h)
-            self.h = self._addr = self._blobs = None
+            self.h = self._addr = None
             self._segments = {}
 
     def __del__(self):
@@ -352,19 +350,16 @@ class Context:
             pass
 
     def _check(self, st, ok=(TJ_OK,)):
-        if st and st not in ok:
+        if st not in ok:
             raise TjError(st, tj_last_error(self.h))
         return st
 
     def _blob_ptrs(self, blobs):
-        """Addresses of parameter blobs (float32, contiguous, of one size); those of the last call need no second look."""
-        ptrs = tuple([x.data_ptr() for x in blobs])
-        if self._blobs is None or ptrs != self._ptrs or len(blobs) != len(self._blobs) or not all(map(operator.is_, blobs, self._blobs)):
-            f32, n = self.torch.float32, blobs[0].numel()
-            for x in blobs:
-                assert x.dtype == f32 and x.is_contiguous() and x.numel() == n
-            self._blobs, self._ptrs = blobs, ptrs
-        return ptrs
+        """Addresses of parameter blobs: float32, contiguous, all of one size."""
+        f32, n = self.torch.float32, blobs[0].numel()
+        for x in blobs:
+            assert x.dtype == f32 and x.is_contiguous() and x.numel() == n
+        return [x.data_ptr() for x in blobs]
 
     def _view(self, ptr, shape, dtype):
         """torch view of a workspace address."""
@@ -432,13 +427,14 @@ class Context:
         """theta (updated in place) and theta_target: float32 device tensors in the publish layout; returns the loss tensor"""
         t, tt = self._blob_ptrs((theta, theta_target))
         loss = self._one.new_empty(1)
-        self._check(_calls.sgd_step(self._addr, batch["c"], lr, t, tt, loss.data_ptr()))
+        self._check(_calls.sgd_step(self._addr, batch["c"], float(lr), t, tt, loss.data_ptr()))
         return loss
 
     def adam_step(self, batch, lr, theta, theta_target, m, v, t, beta1=0.9, beta2=0.999, eps=1e-8):
         p, pt, pm, pv = self._blob_ptrs((theta, theta_target, m, v))
         loss = self._one.new_empty(1)
-        self._check(_calls.adam_step(self._addr, batch["c"], lr, beta1, beta2, eps, t, p, pt, pm, pv, loss.data_ptr()))
+        self._check(_calls.adam_step(self._addr, batch["c"], float(lr), float(beta1), float(beta2), float(eps), int(t), p, pt, pm, pv,
+                                     loss.data_ptr()))
         return loss
 
     def ppo_step(self, obs, act, logp_old, adv, ret, lr, theta, m, v, t, clip_eps=0.2, c_v=0.5, c_e=0.01, beta1=0.9,
@@ -446,13 +442,13 @@ class Context:
         """obs [n][D], act (int32), logp_old, adv, ret [n]: contiguous device tensors (views of a segment are fine);
         returns the 5 statistics tensor (loss, policy, value, entropy, clip fraction)"""
         n = act.numel()
-        for x_ in (obs, act, logp_old, adv, ret):
+        for x_ in (obs, act, logp_old, adv, ret, theta, m, v):
             assert x_.is_contiguous()
         assert obs.numel() == n * self.D and act.dtype == self.torch.int32
-        p, pm, pv = self._blob_ptrs((theta, m, v))
         stats = self._one.new_empty(5)
-        self._check(_calls.ppo_step(self._addr, n, obs.data_ptr(), act.data_ptr(), logp_old.data_ptr(), adv.data_ptr(), ret.data_ptr(), lr,
-                                    beta1, beta2, eps, t, clip_eps, c_v, c_e, p, pm, pv, stats.data_ptr()))
+        self._check(_calls.ppo_step(self._addr, n, obs.data_ptr(), act.data_ptr(), logp_old.data_ptr(), adv.data_ptr(), ret.data_ptr(),
+                                    float(lr), float(beta1), float(beta2), float(eps), int(t), float(clip_eps), float(c_v), float(c_e),
+                                    theta.data_ptr(), m.data_ptr(), v.data_ptr(), stats.data_ptr()))
         return stats
 
     def gae(self, rew, val, done, gamma, lam, adv=None, ret=None):
@@ -487,7 +483,7 @@ class Context:
         assert x.is_cuda and x.dtype == self.torch.float32 and x.is_contiguous()
         if out is None:
             out = self.torch.empty_like(x)
-        self._check(_calls.normalize(self._addr, x.data_ptr(), x.numel(), eps, out.data_ptr()))
+        self._check(_calls.normalize(self._addr, x.data_ptr(), x.numel(), float(eps), out.data_ptr()))
         return out
 
     def alloc_minibatch(self, n):
@@ -502,7 +498,7 @@ class Context:
     def segment_minibatch(self, seg, adv, ret, shuffle_id, first, mb):
         """Rows at positions first .. first + n - 1 of shuffle `shuffle_id` of the segment, copied into the minibatch arrays."""
         assert adv.is_contiguous() and ret.is_contiguous() and adv.numel() == seg["T"] * seg["N"] == ret.numel()
-        self._check(_calls.segment_minibatch(self._addr, seg["c"], adv.data_ptr(), ret.data_ptr(), shuffle_id, first, mb["c"]))
+        self._check(_calls.segment_minibatch(self._addr, seg["c"], adv.data_ptr(), ret.data_ptr(), int(shuffle_id), int(first), mb["c"]))
         return mb
 
     def segment_check(self, seg, allow=(TJ_OK, TJ_ERR_STALE_SEGMENT)):

@@ -1,0 +1,84 @@
+"""The per-iteration calls of the binding on the CPU: what Context hands to the library, and the extension module on its own."""
+import gc
+import weakref
+
+import pytest
+import torch
+
+from paper_2502_20190_b200 import binding as b
+
+
+class _Recorder:
+    """Stands in for the extension module: every call is kept and succeeds."""
+
+    def __init__(self):
+        self.calls = []
+
+    def __getattr__(self, name):
+        def call(*args):
+            self.calls.append((name, args))
+            return (0, 1) if name == "publish_weights" else 0
+        return call
+
+
+@pytest.fixture
+def ctx(monkeypatch):
+    rec = _Recorder()
+    monkeypatch.setattr(b, "_calls", rec)
+    c = b.Context.__new__(b.Context)
+    c.torch, c.device, c.h, c._addr, c._segments = torch, torch.device("cpu"), None, 4096, {}
+    c._one, c.D, c.A, c.rec = torch.empty(1), 4, 2, rec
+    return c
+
+
+def _blobs(n, count):
+    return [torch.zeros(n) for _ in range(count)]
+
+
+def test_updates_hold_no_parameters(ctx):
+    batch = dict(c=b.TjBatch())
+    theta, target, m, v = _blobs(10, 4)
+    refs = [weakref.ref(x) for x in (theta, target, m, v)]
+    ctx.adam_step(batch, 1e-3, theta, target, m, v, 1)
+    ctx.sgd_step(batch, 1e-3, theta, target)
+    act = torch.zeros(3, dtype=torch.int32)
+    ctx.ppo_step(torch.zeros(3, 4), act, *_blobs(3, 3), 1e-3, theta, m, v, 1)
+    del theta, target, m, v
+    gc.collect()
+    assert [r() for r in refs] == [None] * 4
+
+
+def test_updates_look_at_their_blobs_on_every_call(ctx):
+    batch = dict(c=b.TjBatch())
+    theta, target, m, v = _blobs(10, 4)
+    ctx.adam_step(batch, 1e-3, theta, target, m, v, 1)
+    target.resize_(4)                                 # the same tensor at the same address, smaller
+    for call in (lambda: ctx.adam_step(batch, 1e-3, theta, target, m, v, 1), lambda: ctx.sgd_step(batch, 1e-3, theta, target)):
+        with pytest.raises(AssertionError):
+            call()
+    wide = torch.zeros(10, 2)[:, 0]                   # right size, not contiguous
+    with pytest.raises(AssertionError):
+        ctx.sgd_step(batch, 1e-3, theta, wide)
+    with pytest.raises(AssertionError):
+        ctx.sgd_step(batch, 1e-3, theta, theta.double())
+
+
+def test_numbers_are_taken_as_int_and_float_take_them(ctx):
+    theta, target, m, v = _blobs(10, 4)
+    ctx.adam_step(dict(c=b.TjBatch()), torch.tensor(0.5), theta, target, m, v, 3.0, beta1="0.5", eps=1)
+    name, args = ctx.rec.calls[-1]
+    assert name == "adam_step" and args[2:7] == (0.5, 0.5, 0.999, 1.0, 3) and all(type(a) is float for a in args[2:6]) and type(args[6]) is int
+    act = torch.zeros(3, dtype=torch.int32)
+    ctx.ppo_step(torch.zeros(3, 4), act, *_blobs(3, 3), 1, theta, m, v, torch.tensor(7))
+    assert ctx.rec.calls[-1][1][7:15] == (1.0, 0.9, 0.999, 1e-8, 7, 0.2, 0.5, 0.01) and type(ctx.rec.calls[-1][1][11]) is int
+    seg = dict(T=2, N=3, c=b.TjSegment())
+    ctx.segment_minibatch(seg, torch.zeros(2, 3), torch.zeros(2, 3), 2.0, 4.0, dict(c=b.TjPpoMinibatch()))
+    assert ctx.rec.calls[-1][1][4:6] == (2, 4) and all(type(a) is int for a in ctx.rec.calls[-1][1][4:6])
+    ctx.sgd_step(dict(c=b.TjBatch()), 1, theta, target)
+    assert ctx.rec.calls[-1][1][2] == 1.0
+
+
+def test_a_status_outside_the_allowed_ones_raises(ctx):
+    with pytest.raises(b.TjError):
+        ctx._check(b.TJ_OK, (b.TJ_ERR_TIMEOUT,))
+    assert ctx._check(b.TJ_ERR_TIMEOUT, (b.TJ_ERR_TIMEOUT,)) == b.TJ_ERR_TIMEOUT
