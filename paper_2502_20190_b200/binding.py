@@ -168,8 +168,9 @@ def tj_wait(h, which: int, timeout_ms: int):
 
 
 def tj_publish_weights(h, blob_ptr: int, nbytes: int, on_device: int):
-    load_library()
-    return _calls.publish_weights(getattr(h, "value", h), blob_ptr or None, nbytes, on_device)
+    v = C.c_int64()
+    st = load_library().tj_publish_weights(h, blob_ptr, nbytes, on_device, C.byref(v))
+    return st, v.value
 
 
 def tj_actor_step(h, n_steps: int, dbg_logits_ptr: int = 0):

@@ -1,4 +1,5 @@
 """The per-iteration calls of the binding on the CPU: what Context hands to the library, and the extension module on its own."""
+import ctypes as C
 import gc
 import weakref
 
@@ -6,6 +7,7 @@ import pytest
 import torch
 
 from paper_2502_20190_b200 import binding as b
+from paper_2502_20190_b200 import build as tjbuild
 
 
 class _Recorder:
@@ -82,3 +84,16 @@ def test_a_status_outside_the_allowed_ones_raises(ctx):
     with pytest.raises(b.TjError):
         ctx._check(b.TJ_OK, (b.TJ_ERR_TIMEOUT,))
     assert ctx._check(b.TJ_ERR_TIMEOUT, (b.TJ_ERR_TIMEOUT,)) == b.TJ_ERR_TIMEOUT
+
+
+@pytest.fixture(scope="module")
+def lib():
+    tjbuild.build()
+    return b.load_library()
+
+
+def test_publish_takes_every_form_of_pointer(lib):
+    host = (C.c_float * 3)()
+    for blob in (None, 0, C.addressof(host), host, C.c_void_p(C.addressof(host)), C.pointer(host), b"blob"):
+        for h in (None, C.c_void_p()):
+            assert b.tj_publish_weights(h, blob, 12, 0) == (b.TJ_ERR_INVALID_ARG, 0)
