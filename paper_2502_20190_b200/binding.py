@@ -2,7 +2,7 @@
 
 The module-level ``tj_*`` functions mirror the C ABI one to one through ctypes; the calls that a training loop
 makes every iteration go through a small extension module (``csrc/tj_python.cpp``), which marshals them in a
-tenth of the time.  ``Context`` is a
+tenth of the time (through ctypes too where the module has not been built for the interpreter).  ``Context`` is a
 convenience wrapper that allocates the workspace and the output arrays with torch
 (device memory and the stream are torch's; every computation runs in the library's
 CUDA kernels).  There is no CPU fallback: without the compiled library or without a
@@ -81,10 +81,30 @@ _FAST = ("tj_actor_step", "tj_replay_sample", "tj_td_error", "tj_publish_weights
          "tj_normalize", "tj_segment_minibatch")
 
 
+class _CtypesCalls:
+    """The extension module's calls through ctypes, for an interpreter that the module has not been built for."""
+
+    def __init__(self, lib):
+        for name in _FAST:
+            if name not in ("tj_publish_weights", "tj_ppo_step"):
+                setattr(self, name[3:], self._plain(getattr(lib, name)))
+        self._ppo_step = lib.tj_ppo_step
+
+    @staticmethod
+    def _plain(f):
+        return lambda *args: f(*[C.byref(a) if isinstance(a, C.Structure) else a for a in args])
+
+    def publish_weights(self, h, blob_ptr, nbytes, on_device):
+        return tj_publish_weights(h, blob_ptr, nbytes, on_device)
+
+    def ppo_step(self, h, *args):                  # the batch's six fields come first
+        return self._ppo_step(h, C.byref(TjPpoBatch(*args[:6])), *args[6:])
+
+
 def _load_calls(lib):
-    """The extension module with the per-iteration calls, bound to this library's functions; raises when it is not built."""
+    """The per-iteration calls, bound to this library's functions: the extension module, or ctypes where it has not been built."""
     if not os.path.exists(_build.CALLS):
-        raise RuntimeError("%s is missing: build it with `python -m paper_2502_20190_b200.build`" % os.path.basename(_build.CALLS))
+        return _CtypesCalls(lib)
     spec = importlib.util.spec_from_file_location("_tjcall", _build.CALLS)
     m = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(m)

@@ -97,3 +97,28 @@ def test_publish_takes_every_form_of_pointer(lib):
     for blob in (None, 0, C.addressof(host), host, C.c_void_p(C.addressof(host)), C.pointer(host), b"blob"):
         for h in (None, C.c_void_p()):
             assert b.tj_publish_weights(h, blob, 12, 0) == (b.TJ_ERR_INVALID_ARG, 0)
+
+
+# arguments of each call with a null context; every one of them is refused by the library itself
+NULL_CALLS = {
+    "actor_step": (None, 1, None),
+    "replay_sample": (None, -1, None, b.TjBatch()),
+    "td_error": (None, b.TjBatch(), None, None, None),
+    "publish_weights": (None, None, 12, 0),
+    "sgd_step": (None, b.TjBatch(), 0.5, None, None, None),
+    "adam_step": (None, b.TjBatch(), 0.5, 0.9, 0.99, 1e-8, 1, None, None, None, None, None),
+    "ppo_step": (None, 3, None, None, None, None, None, 0.5, 0.9, 0.99, 1e-8, 1, 0.2, 0.5, 0.01, None, None, None, None),
+    "gae": (None, None, None, None, 2, 3, 0.9, 0.9, None, None),
+    "normalize": (None, None, 3, 1e-8, None),
+    "segment_minibatch": (None, b.TjSegment(), None, None, 7, 0, b.TjPpoMinibatch()),
+}
+REFUSED = {name: (b.TJ_ERR_INVALID_ARG, 0) if name == "publish_weights" else b.TJ_ERR_INVALID_ARG for name in NULL_CALLS}
+
+
+def test_the_library_loads_without_the_extension_module(lib, monkeypatch, tmp_path):
+    monkeypatch.setattr(b, "_lib", None)
+    monkeypatch.setattr(b, "_calls", None)
+    monkeypatch.setattr(tjbuild, "CALLS", str(tmp_path / "_tjcall.none.so"))
+    b.load_library()
+    for name, args in NULL_CALLS.items():
+        assert getattr(b._calls, name)(*args) == REFUSED[name], name
