@@ -19,29 +19,29 @@ decltype(&tj_gae) f_gae;
 decltype(&tj_normalize) f_normalize;
 decltype(&tj_segment_minibatch) f_segment_minibatch;
 
+bool ready = false;   // init() has handed over every function
+
 // arguments in order, converted as they are asked for; `bad` stays set after the first failure
 struct Args {
   PyObject* const* a;
   Py_ssize_t n, i = 0;
   bool bad = false;
-  Args(PyObject* const* args, Py_ssize_t count, Py_ssize_t want) : a(args), n(count) {
-    if (n != want) {
+  Args(PyObject* const* args, Py_ssize_t count, Py_ssize_t want, bool needs_init = true) : a(args), n(count) {
+    if (needs_init && !ready) {
+      PyErr_SetString(PyExc_RuntimeError, "init() has not been called with the library's functions");
+      bad = true;
+    } else if (n != want) {
       PyErr_Format(PyExc_TypeError, "expected %zd arguments, got %zd", want, n);
       bad = true;
     }
   }
-  long long integer() {
-    if (bad) return 0;
-    const long long v = PyLong_AsLongLong(a[i++]);
-    if (v == -1 && PyErr_Occurred()) bad = true;
-    return v;
-  }
-  unsigned long long word() {                 // modulo 2^64, as ctypes takes it
+  unsigned long long word() {                 // an integer modulo 2^64, as ctypes takes it; the caller narrows it
     if (bad) return 0;
     const unsigned long long v = PyLong_AsUnsignedLongLongMask(a[i++]);
     if (v == (unsigned long long)-1 && PyErr_Occurred()) bad = true;
     return v;
   }
+  long long integer() { return (long long)word(); }
   double real() {
     if (bad) return 0.0;
     const double v = PyFloat_AsDouble(a[i++]);
@@ -75,7 +75,8 @@ struct Args {
 };
 
 PyObject* init(PyObject*, PyObject* const* args, Py_ssize_t n) {
-  Args a(args, n, 10);
+  Args a(args, n, 10, false);
+  ready = false;
   f_actor_step = reinterpret_cast<decltype(f_actor_step)>(a.pointer<void>());
   f_replay_sample = reinterpret_cast<decltype(f_replay_sample)>(a.pointer<void>());
   f_td_error = reinterpret_cast<decltype(f_td_error)>(a.pointer<void>());
@@ -87,6 +88,12 @@ PyObject* init(PyObject*, PyObject* const* args, Py_ssize_t n) {
   f_normalize = reinterpret_cast<decltype(f_normalize)>(a.pointer<void>());
   f_segment_minibatch = reinterpret_cast<decltype(f_segment_minibatch)>(a.pointer<void>());
   if (a.bad) return nullptr;
+  if (!f_actor_step || !f_replay_sample || !f_td_error || !f_publish_weights || !f_sgd_step || !f_adam_step || !f_ppo_step || !f_gae ||
+      !f_normalize || !f_segment_minibatch) {
+    PyErr_SetString(PyExc_ValueError, "a null function");
+    return nullptr;
+  }
+  ready = true;
   Py_RETURN_NONE;
 }
 

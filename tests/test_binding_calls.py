@@ -1,6 +1,8 @@
 """The per-iteration calls of the binding on the CPU: what Context hands to the library, and the extension module on its own."""
 import ctypes as C
 import gc
+import subprocess
+import sys
 import weakref
 
 import pytest
@@ -23,8 +25,14 @@ class _Recorder:
         return call
 
 
+@pytest.fixture(scope="module")
+def lib():
+    tjbuild.build()
+    return b.load_library()
+
+
 @pytest.fixture
-def ctx(monkeypatch):
+def ctx(monkeypatch, lib):
     rec = _Recorder()
     monkeypatch.setattr(b, "_calls", rec)
     c = b.Context.__new__(b.Context)
@@ -86,12 +94,6 @@ def test_a_status_outside_the_allowed_ones_raises(ctx):
     assert ctx._check(b.TJ_ERR_TIMEOUT, (b.TJ_ERR_TIMEOUT,)) == b.TJ_ERR_TIMEOUT
 
 
-@pytest.fixture(scope="module")
-def lib():
-    tjbuild.build()
-    return b.load_library()
-
-
 def test_publish_takes_every_form_of_pointer(lib):
     host = (C.c_float * 3)()
     for blob in (None, 0, C.addressof(host), host, C.c_void_p(C.addressof(host)), C.pointer(host), b"blob"):
@@ -122,3 +124,74 @@ def test_the_library_loads_without_the_extension_module(lib, monkeypatch, tmp_pa
     b.load_library()
     for name, args in NULL_CALLS.items():
         assert getattr(b._calls, name)(*args) == REFUSED[name], name
+
+
+# ---- the extension module on its own
+def test_module_refuses_calls_before_a_complete_init(lib):
+    prog = """if True:
+        import importlib.util, sys
+        spec = importlib.util.spec_from_file_location("_tjcall", sys.argv[1])
+        m = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(m)
+        def raises(kind, f, *args):
+            try:
+                f(*args)
+            except kind:
+                return
+            raise SystemExit("no " + kind.__name__)
+        raises(RuntimeError, m.actor_step, None, 1, None)
+        raises(ValueError, m.init, *[None] * 10)
+        raises(TypeError, m.init, *[4096] * 9)
+        raises(TypeError, m.init, *([4096] * 9 + ["x"]))
+        raises(RuntimeError, m.gae, None, None, None, None, 1, 1, 0.5, 0.5, None, None)
+    """
+    r = subprocess.run([sys.executable, "-c", prog, tjbuild.CALLS], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0, (r.returncode, r.stdout, r.stderr)
+
+
+@pytest.mark.parametrize("name", list(NULL_CALLS))
+def test_module_arguments(lib, name):
+    call, args = getattr(b._calls, name), list(NULL_CALLS[name])
+    assert type(b._calls).__name__ == "module"
+    assert call(*args) == REFUSED[name]                # a closed context: the library's own status, no crash
+    for n in (0, len(args) - 1, len(args) + 1):
+        with pytest.raises(TypeError, match="arguments"):
+            call(*(args + [None])[:n])
+    for i, a in enumerate(args):
+        if isinstance(a, C.Structure):
+            for other in (C.create_string_buffer(C.sizeof(a) + 1), C.c_int32(), 5, None):
+                with pytest.raises(TypeError):
+                    call(*args[:i], other, *args[i + 1:])
+            continue
+        for wrong in ("x", 1.5, object()):
+            if isinstance(a, float) and wrong == 1.5:
+                continue
+            with pytest.raises(TypeError):             # nothing after the argument that failed is looked at
+                call(*args[:i], wrong, *args[i + 1:])
+        if isinstance(a, int):                         # integers are taken modulo 2^64 and narrowed, as by ctypes
+            for big in (2 ** 63, 2 ** 70, -2 ** 65):
+                assert call(*args[:i], big, *args[i + 1:]) == REFUSED[name]
+
+
+class _Fails:
+    def __init__(self, seen):
+        self.seen = seen
+
+    def __float__(self):
+        self.seen.append("float")
+        raise ZeroDivisionError("float")
+
+    def __index__(self):
+        self.seen.append("index")
+        raise KeyError("index")
+
+
+def test_module_passes_an_exception_on(lib):
+    seen = []
+    with pytest.raises(ZeroDivisionError):
+        b._calls.sgd_step(None, b.TjBatch(), _Fails(seen), None, None, None)
+    with pytest.raises(ZeroDivisionError):             # the first failure ends the call
+        b._calls.adam_step(None, b.TjBatch(), 0.5, _Fails(seen), _Fails(seen), 1e-8, _Fails(seen), None, None, None, None, None)
+    with pytest.raises(KeyError):
+        b._calls.actor_step(None, _Fails(seen), None)
+    assert seen == ["float", "float", "index"]
