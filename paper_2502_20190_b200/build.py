@@ -27,9 +27,7 @@ def build_calls(force: bool = False) -> str:
     srcs = [os.path.join(CSRC, "tj_python.cpp"), os.path.join(HERE, "..", "include", "tj.h")]
     if force or not os.path.exists(CALLS) or os.path.getmtime(CALLS) < max(os.path.getmtime(p) for p in srcs):
         tmp = CALLS + ".tmp.%d" % os.getpid()
-        cuda = os.path.join(os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"))), "include")
-        subprocess.check_call(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-I", cuda, srcs[0],
-                               "-o", tmp])
+        subprocess.check_call(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], srcs[0], "-o", tmp])
         os.replace(tmp, CALLS)
     return CALLS
 
