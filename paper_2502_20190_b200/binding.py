@@ -497,7 +497,8 @@ class Context:
                 obs=self._view(seg.obs, (T, N, D), torch.float32), act=self._view(seg.act, (T, N), torch.int32),
                 rew=self._view(seg.rew, (T, N), torch.float32), done=self._view(seg.done, (T, N), torch.uint8),
                 logp=self._view(seg.logp, (T, N), torch.float32), val=self._view(seg.val, (T + 1, N), torch.float32))
-        return st, dict(T=seg.T, N=seg.N, version=seg.version, c=seg, **views)
+        # as tensors of the caller's own: what is done to one in place (its shape, requires_grad) stays with it
+        return st, dict(T=seg.T, N=seg.N, version=seg.version, c=seg, **{k: v.detach() for k, v in views.items()})
 
     def normalize(self, x, eps=1e-8, out=None):
         """(x - mean) / (std + eps) over all entries of a float32 device tensor, in the library's kernels."""

@@ -101,6 +101,19 @@ def test_publish_takes_every_form_of_pointer(lib):
             assert b.tj_publish_weights(h, blob, 12, 0) == (b.TJ_ERR_INVALID_ARG, 0)
 
 
+def test_a_segment_comes_as_tensors_of_its_own(ctx, monkeypatch):
+    ws = ctx.workspace = torch.zeros(4096, dtype=torch.uint8)
+    seg, base = b.TjSegment(2, 3, 1), ws.data_ptr()
+    seg.obs, seg.act, seg.rew, seg.done, seg.logp, seg.val = (base + 256 * i for i in range(6))
+    monkeypatch.setattr(b, "tj_segment_acquire", lambda h: (b.TJ_OK, seg))
+    first = ctx.segment_acquire()[1]
+    first["obs"].requires_grad_()                      # what a caller does to its tensors stays with them
+    first["rew"].unsqueeze_(0)
+    second = ctx.segment_acquire()[1]
+    assert not second["obs"].requires_grad and second["rew"].shape == (2, 3)
+    assert all(second[k].data_ptr() == getattr(seg, k) for k in ("obs", "act", "rew", "done", "logp", "val"))
+
+
 # arguments of each call with a null context; every one of them is refused by the library itself
 NULL_CALLS = {
     "actor_step": (None, 1, None),
