@@ -274,13 +274,15 @@ int tj_td_error_static(tj_ctx *ctx, const tj_batch *batch, float *td_out, float 
  * as three TF32 products of high / low operand parts with FP32 accumulation: up to 3 * 2^-22 per product instead of 2^-24.
  * In a BF16 context theta is the FP32 master copy: the update and its loss are FP32 all the same, the rounding to BF16
  * happens at tj_publish_weights (so this loss differs from tj_td_error's, which uses the published BF16 copy, by that
- * rounding).  TJ_ERR_UNSUPPORTED for segment mode and the categorical policy. */
+ * rounding).  Should a kernel's bounded wait run out, theta stays as it was, the loss is NaN and device_error is latched
+ * (tj_stats).  TJ_ERR_UNSUPPORTED for segment mode and the categorical policy. */
 int tj_sgd_step(tj_ctx *ctx, const tj_batch *batch, float lr, float *theta, const float *theta_target, float *loss_mean_out);
 
 /* The same gradient through Adam (the optimiser of Table 2; Kingma & Ba 2015), step counter t >= 1:
  *   m <- beta1 m + (1 - beta1) g;  v <- beta2 v + (1 - beta2) g^2;
  *   theta <- theta - lr * (m / (1 - beta1^t)) / (sqrt(v / (1 - beta2^t)) + eps)
- * m, v: device FP32 moment blobs in the layout of theta, owned and zero-initialised by the caller, updated in place.
+ * m, v: device FP32 moment blobs in the layout of theta, owned and zero-initialised by the caller, updated in place (after a
+ * bounded wait that ran out they stay as they were, like theta).
  * Other arguments, limits and statuses as tj_sgd_step. */
 int tj_adam_step(tj_ctx *ctx, const tj_batch *batch, float lr, float beta1, float beta2, float eps, int64_t t, float *theta,
                  const float *theta_target, float *m, float *v, float *loss_mean_out);
@@ -294,7 +296,8 @@ int tj_adam_step(tj_ctx *ctx, const tj_batch *batch, float lr, float beta1, floa
  * segment (tj_segment_acquire) and of tj_gae's outputs can be passed as they lie: obs [n][obs_dim], the others [n].
  * stats_out (nullable, device, 5 floats): L, mean policy term, mean 0.5 (V - R)^2, mean entropy, fraction of rows where
  * the clipped term is the minimum -- all before the update.  batch.n <= the configured minibatch (4096 if none).
- * BF16 contexts: theta is the FP32 master copy, as for tj_sgd_step.
+ * BF16 contexts: theta is the FP32 master copy, as for tj_sgd_step.  A bounded wait that runs out: as for tj_adam_step, the
+ * statistics are NaN.
  * TJ_ERR_UNSUPPORTED unless the context is in segment mode with the categorical policy. */
 typedef struct {
   int32_t n;

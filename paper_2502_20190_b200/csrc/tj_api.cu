@@ -235,6 +235,32 @@ uint64_t explore_threshold(float eps) {
   return (uint64_t)std::floor(e * 4294967296.0);
 }
 
+// h1, h2, dh1, dh2 [rows][H] | g [rows][17] | qt [rows][16] | loss partials | PPO statistic partials | W2^T [H][H] | number of the last
+// failed update | gradient partial sums
+void lay_out_update_scratch(const tj_ctx* x, tj::SgdParams& p) {
+  const size_t rows = ((size_t)x->sgd_rows + 15) / 16 * 16, RH = rows * (size_t)x->H;
+  p.h1 = x->sgd_scratch; p.h2 = p.h1 + RH; p.dh1 = p.h2 + RH; p.dh2 = p.dh1 + RH;
+  p.g = p.dh2 + RH;
+  p.qt = p.g + rows * 17;
+  p.partial = p.qt + rows * 16;
+  p.stat_partial = p.partial + sgd_partial_floats(x->sgd_rows);
+  p.w2t = p.stat_partial + 5 * (rows / 16) + 8;
+  p.w2t += (4 - ((reinterpret_cast<uintptr_t>(p.w2t) / sizeof(float)) & 3)) & 3;   // 16-byte rows for the vector loads
+  p.grad_partial = p.w2t + (size_t)x->H * x->H;
+  p.grad_partial += (4 - ((reinterpret_cast<uintptr_t>(p.grad_partial) / sizeof(float)) & 3)) & 3;
+  p.watch.failed = reinterpret_cast<unsigned*>(p.grad_partial);
+  p.watch.error = &x->dstats->error;
+  p.watch.number = x->updates;
+  p.grad_partial += 4;
+  {
+    // after the partial gradients: split weight copies for the tensor-core products, 128-byte aligned for the bulk copies
+    float* w = p.grad_partial + sgd_grad_partial_floats(x->sgd_rows, x->D, x->H);
+    w += (32 - ((reinterpret_cast<uintptr_t>(w) / sizeof(float)) & 31)) & 31;
+    p.wpack = w;
+    p.sm_count = x->sm_count;
+  }
+}
+
 }  // namespace
 
 extern "C" {
@@ -290,6 +316,11 @@ int tj_create(const tj_config* cfg, void* workspace, size_t bytes, void* cuda_st
     return (int)TJ_ERR_CUDA;
   };
   if ((e = cudaMemsetAsync(x->dstats, 0, sizeof(DevStats), x->stream)) != cudaSuccess) return bail(e, "memset stats");
+  if (x->sgd_scratch) {
+    tj::SgdParams p{};
+    lay_out_update_scratch(x, p);
+    if ((e = cudaMemsetAsync(p.watch.failed, 0, sizeof(*p.watch.failed), x->stream)) != cudaSuccess) return bail(e, "memset update scratch");
+  }
   if (cfg->replay_capacity > 0) {
     if ((e = cudaMemsetAsync(x->block_ver, 0, sizeof(int) * x->h_block_ver.size(), x->stream)) != cudaSuccess)
       return bail(e, "memset block versions");
@@ -701,27 +732,6 @@ int tj_td_error_static(tj_ctx* x, const tj_batch* b, float* td_out, float* huber
 }
 
 namespace {
-// h1, h2, dh1, dh2 [rows][H] | g [rows][17] | qt [rows][16] | loss partials | PPO statistic partials | W2^T [H][H] | gradient partial sums
-void lay_out_update_scratch(const tj_ctx* x, tj::SgdParams& p) {
-  const size_t rows = ((size_t)x->sgd_rows + 15) / 16 * 16, RH = rows * (size_t)x->H;
-  p.h1 = x->sgd_scratch; p.h2 = p.h1 + RH; p.dh1 = p.h2 + RH; p.dh2 = p.dh1 + RH;
-  p.g = p.dh2 + RH;
-  p.qt = p.g + rows * 17;
-  p.partial = p.qt + rows * 16;
-  p.stat_partial = p.partial + sgd_partial_floats(x->sgd_rows);
-  p.w2t = p.stat_partial + 5 * (rows / 16) + 8;
-  p.w2t += (4 - ((reinterpret_cast<uintptr_t>(p.w2t) / sizeof(float)) & 3)) & 3;   // 16-byte rows for the vector loads
-  p.grad_partial = p.w2t + (size_t)x->H * x->H;
-  p.grad_partial += (4 - ((reinterpret_cast<uintptr_t>(p.grad_partial) / sizeof(float)) & 3)) & 3;
-  {
-    // after the partial gradients: split weight copies for the tensor-core products, 128-byte aligned for the bulk copies
-    float* w = p.grad_partial + sgd_grad_partial_floats(x->sgd_rows, x->D, x->H);
-    w += (32 - ((reinterpret_cast<uintptr_t>(w) / sizeof(float)) & 31)) & 31;
-    p.wpack = w;
-    p.sm_count = x->sm_count;
-  }
-}
-
 int learner_update(tj_ctx* x, const tj_batch* b, float lr, float* theta, const float* theta_target, const tj::AdamParams* adam,
                    float* loss_mean_out) {
   if (!b || !b->obs || !b->act || !b->rew || !b->next_obs || !b->done) return fail(x, TJ_ERR_INVALID_ARG, "batch arrays must not be null");
@@ -736,9 +746,9 @@ int learner_update(tj_ctx* x, const tj_batch* b, float lr, float* theta, const f
   p.theta = theta; p.theta_target = theta_target;
   p.obs = b->obs; p.act = b->act; p.rew = b->rew; p.next_obs = b->next_obs; p.done = b->done;
   p.gamma = x->cfg.gamma; p.kappa = x->cfg.huber_delta;
+  if (++x->updates == 0) x->updates = 1;
   lay_out_update_scratch(x, p);
   p.ldg = x->A; p.value_head = 0;
-  p.error = &x->dstats->error;
   int launches = 0;
   p.launches = &launches;
   LaunchScope scope(x, TJ_K_SGD, 0, true, true);
@@ -788,9 +798,9 @@ int tj_ppo_step(tj_ctx* x, const tj_ppo_batch* b, float lr, float beta1, float b
   p.theta = theta; p.theta_target = nullptr;
   p.obs = b->obs; p.act = b->act; p.logp_old = b->logp_old; p.adv = b->adv; p.ret = b->ret;
   p.clip_eps = clip_eps; p.c_v = c_v; p.c_e = c_e;
+  if (++x->updates == 0) x->updates = 1;
   lay_out_update_scratch(x, p);
   p.ldg = x->A + 1; p.value_head = 1;
-  p.error = &x->dstats->error;
   tj::AdamParams a{};
   a.m = m; a.v = v; a.beta1 = beta1; a.beta2 = beta2; a.eps = eps;
   a.c1 = (float)(1.0 - std::pow((double)beta1, (double)t));

@@ -119,6 +119,24 @@ struct TdParams {
   unsigned long long* error;  // device error word of the context (a bounded wait that ran out)
 };
 
+// Where the kernels of a parameter update report a bounded wait that ran out: the context's error word, and the number of the update in a
+// word that its last kernel looks at before it writes parameters and moments.
+struct UpdateWatch {
+  unsigned long long* error;
+  unsigned *failed, number;
+};
+
+#ifdef __CUDACC__
+__device__ __forceinline__ void update_failed(const UpdateWatch& w) {
+  atomicExch(w.error, 3ull);
+  atomicExch(w.failed, w.number);
+}
+// For a kernel behind those of the update: whether all of their waits were served, the same answer for the whole block (a block barrier).
+// Thread 0 alone has asked, early.
+__device__ __forceinline__ unsigned update_ask(const unsigned* failed, unsigned number) { return threadIdx.x == 0 ? __ldcg(failed) : ~number; }
+__device__ __forceinline__ bool update_valid(unsigned number, unsigned asked) { return __syncthreads_and(asked != number); }
+#endif
+
 struct SgdParams {
   int n, D, H, A;
   float* theta;                // online parameters, publish layout, updated in place
@@ -145,7 +163,7 @@ struct SgdParams {
   const float* ret;
   float clip_eps, c_v, c_e;
   float* stat_partial;         // scratch: five partial sums per 16 rows (loss, policy, value, entropy, clipped rows)
-  unsigned long long* error;   // device error word of the context (a bounded wait that ran out)
+  UpdateWatch watch;           // watch.failed: scratch too, zero at first
   int* launches;               // host: raised by the kernels an update launches
 };
 
@@ -261,7 +279,7 @@ cudaError_t launch_pack_pipelined_env(const float* A, const float* B, float scal
 cudaError_t launch_td_from_q(const float* q_online, const float* q_target, int n, int A, const int* act, const float* rew,
                              const int* done, float gamma, float kappa, float* td_out, float* huber_out, float* partial,
                              cudaStream_t s);
-cudaError_t launch_td_finish(const float* partial, int n_partial, int n, float* loss_out, cudaStream_t s);
+cudaError_t launch_td_finish(const float* partial, int n_partial, int n, float* loss_out, cudaStream_t s, const UpdateWatch& watch = {});
 
 // launchers (each returns the cudaGetLastError() of its launches)
 cudaError_t launch_init_env(int env_kind, int N, int S_d, uint2 seed, float* state, int* ep_step, float* ep_return,
@@ -296,11 +314,11 @@ struct TcWgradBatch { TcWgrad g[4]; int n; int n_tiles; };
 bool tc_wgrad_ok(int N, int rows);
 int tc_wgrad_tiles(int M, int N);
 cudaError_t launch_wgrad_tc(const TcWgradBatch& batch, float* P, int count, int n_rows, int rows_per_range, int n_ranges,
-                            unsigned long long* error, cudaStream_t s);
+                            const UpdateWatch& watch, cudaStream_t s);
 bool tc_gemm2_ok(const float* A, int lda, int M, int N, int K);
 size_t tc_pack_floats(int N, int K);
 cudaError_t launch_pack_tf32_operands(const TcPackJobs& jobs, cudaStream_t s);
-cudaError_t launch_gemm_tc2(const TcGemmBatch& batch, int epi, unsigned long long* error, cudaStream_t s);
+cudaError_t launch_gemm_tc2(const TcGemmBatch& batch, int epi, const UpdateWatch& watch, cudaStream_t s);
 // small networks: forward, backward and gradients fused (csrc/tj_sgd_small.cu)
 constexpr int SGD_FUSED_MAX_PARTS = 256;   // at most this many blocks, each with a partial gradient of its own
 bool sgd_fused_ok(int D, int H, int A, int value_head);
@@ -405,6 +423,7 @@ struct tj_ctx {
   bool has_target;
   int64_t t, k;
   uint64_t cursor;
+  uint32_t updates;     // number of the last parameter update (never 0)
   std::vector<int32_t> h_block_ver;
   std::vector<SegSlot> seg;
   int64_t next_consume;

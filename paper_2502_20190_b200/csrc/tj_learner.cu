@@ -190,21 +190,23 @@ __global__ void __launch_bounds__(NT) td_kernel(const TdParams p) {
 
 // Fixed-order sum of the per-block partial losses: thread i adds partials i, i + 256, ... (independent loads), then a tree.  One block,
 // bound by one memory latency (a warp that added them in index order, one shuffle each, took 6-8 us for 512 partials).
-__global__ void __launch_bounds__(256) td_finish_kernel(const float* __restrict__ partial, int n_partial, int n, float* __restrict__ loss_out) {
+__global__ void __launch_bounds__(256) td_finish_kernel(const float* __restrict__ partial, int n_partial, int n, float* __restrict__ loss_out,
+                                                        const UpdateWatch watch) {
   __shared__ float ws[8];
   chain_begin();
   chain_next();
+  const unsigned asked = watch.failed ? update_ask(watch.failed, watch.number) : ~watch.number;    // the loss of a TD error has no update
   float s = 0.f;
 #pragma unroll 4
   for (int i = threadIdx.x; i < n_partial; i += 256) s += __ldcg(partial + i);
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = s;
-  __syncthreads();
+  const bool valid = update_valid(watch.number, asked);
   if (threadIdx.x == 0) {
     s = 0.f;
 #pragma unroll
     for (int w = 0; w < 8; ++w) s += ws[w];
-    *loss_out = s / (float)n;
+    *loss_out = valid ? s / (float)n : __int_as_float(0x7FC00000);
   }
 }
 
@@ -368,8 +370,8 @@ cudaError_t launch_td_static(const TdParams& p_in, int device, int sm_count, cud
   return launch_td(p, sm_count, s, launches);
 }
 
-cudaError_t launch_td_finish(const float* partial, int n_partial, int n, float* loss_out, cudaStream_t s) {
-  return launch_chained(td_finish_kernel, 1, 256, 0, s, partial, n_partial, n, loss_out);
+cudaError_t launch_td_finish(const float* partial, int n_partial, int n, float* loss_out, cudaStream_t s, const UpdateWatch& watch) {
+  return launch_chained(td_finish_kernel, 1, 256, 0, s, partial, n_partial, n, loss_out, watch);
 }
 
 cudaError_t launch_gae(const float* rew, const float* val, const uint8_t* done, int T, int N, float gamma, float lambda,

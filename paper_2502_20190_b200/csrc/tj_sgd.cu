@@ -370,7 +370,7 @@ template <int EPI>
 __global__ void __launch_bounds__(TG_THREADS, 2) sg_gemm_tc_kernel(const float* __restrict__ A, int lda, const float* __restrict__ B,
                                                                    int ldb, float* __restrict__ C, int ldc, int M, int N, int K,
                                                                    const float* __restrict__ bias, const float* __restrict__ mask,
-                                                                   int ldm, unsigned long long* __restrict__ error) {
+                                                                   int ldm, const UpdateWatch watch) {
   extern __shared__ uint8_t tg_raw[];
   uint8_t* stage0 = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(tg_raw) + 1023) & ~(uintptr_t)1023);
   __shared__ __align__(8) uint64_t done[2];
@@ -509,7 +509,7 @@ __global__ void __launch_bounds__(TG_THREADS, 2) sg_gemm_tc_kernel(const float* 
       }
     }
   } else if (tid == 0) {
-    atomicExch(error, 3ull);
+    update_failed(watch);
     for (int i = issued > 2 ? issued - 2 : 0; i < issued; ++i) mbar_settle(&done[i & 1], (uint32_t)((i >> 1) & 1));
   }
   tc_fence_before();
@@ -547,7 +547,7 @@ cudaError_t sg_layer(const SgdParams& p, const GemmPair& pr, int sets, int lda, 
   for (int z = 0; z < sets; ++z) {
     ++*p.launches;
     const cudaError_t e = launch_chained(sg_gemm_tc_kernel<EPI>, dim3((N + TG_N - 1) / TG_N, (M + TG_M - 1) / TG_M), TG_THREADS, TG_SMEM_BYTES, s, pr.A[z],
-                                         lda, pr.B[z], ldb, pr.C[z], ldc, M, N, K, pr.bias[z], mask, ldm, p.error);
+                                         lda, pr.B[z], ldb, pr.C[z], ldc, M, N, K, pr.bias[z], mask, ldm, p.watch);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -950,28 +950,31 @@ __global__ void __launch_bounds__(256) sgd_grad_partial_kernel(float* __restrict
   grad_tile(P, d, t, count, n_rows, rows_per_range, sm);
 }
 
-// C[i] -= lr * (P[0][i] + P[1][i] + ...), the partial sums added in range order
-__global__ void sgd_apply_kernel(float* __restrict__ Cm, const float* __restrict__ P, int count, int n_ranges, float lr) {
+// C[i] -= lr * (P[0][i] + P[1][i] + ...), the partial sums added in range order; nothing after a wait of the update that ran out
+__global__ void sgd_apply_kernel(float* __restrict__ Cm, const float* __restrict__ P, int count, int n_ranges, float lr, const UpdateWatch watch) {
   chain_begin();
   chain_next();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= count) return;
+  const unsigned asked = update_ask(watch.failed, watch.number);
   float s = 0.f;
-  for (int z = 0; z < n_ranges; ++z) s += P[(size_t)z * count + i];
-  Cm[i] -= lr * s;
+  if (i < count)
+    for (int z = 0; z < n_ranges; ++z) s += P[(size_t)z * count + i];
+  if (update_valid(watch.number, asked) && i < count) Cm[i] -= lr * s;
 }
 
 // the same gradient through Adam (Table 2's optimiser): m <- b1 m + (1-b1) g, v <- b2 v + (1-b2) g^2,
 // theta <- theta - lr (m / c1) / (sqrt(v / c2) + eps) with the bias corrections c1 = 1 - b1^t, c2 = 1 - b2^t from the host
 __global__ void sgd_apply_adam_kernel(float* __restrict__ Cm, float* __restrict__ m, float* __restrict__ v,
                                       const float* __restrict__ P, int count, int n_ranges, float lr, float beta1, float beta2,
-                                      float eps, float c1, float c2) {
+                                      float eps, float c1, float c2, const UpdateWatch watch) {
   chain_begin();
   chain_next();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= count) return;
+  const unsigned asked = update_ask(watch.failed, watch.number);
   float g = 0.f;
-  for (int z = 0; z < n_ranges; ++z) g += P[(size_t)z * count + i];
+  if (i < count)
+    for (int z = 0; z < n_ranges; ++z) g += P[(size_t)z * count + i];
+  if (!update_valid(watch.number, asked) || i >= count) return;
   const float mi = fmaf(beta1, m[i], (1.f - beta1) * g);
   const float vi = fmaf(beta2, v[i], (1.f - beta2) * g * g);
   m[i] = mi;
@@ -1002,7 +1005,7 @@ size_t sgd_scratch_floats(int max_rows, int D, int H) {
   // h1, h2, dh1, dh2, g [rows][<= 16 actions + value], qt [rows][<= 16], loss partials, PPO's five per 16 rows, partial gradients of the whole
   // parameter blob (at most 16 actions and a value head); W2 transposed
   // + split copies of W1 (x 2 networks), W2 (x 2) and W2^T for the tensor-core products
-  return 4 * rows * (size_t)H + rows * 33 + sgd_partial_floats(max_rows) + 5 * (rows / SG_ROWS) + 64 + (size_t)H * H +
+  return 4 * rows * (size_t)H + rows * 33 + sgd_partial_floats(max_rows) + 5 * (rows / SG_ROWS) + 64 + (size_t)H * H + 4 /* UpdateWatch */ +
          sgd_grad_partial_floats(max_rows, D, H) + 2 * tc_pack_floats(H, D) + 3 * tc_pack_floats(H, H) + 64;
 }
 
@@ -1028,7 +1031,7 @@ cudaError_t backward_and_update(const SgdParams& p, float lr, const AdamParams* 
     b.g[0] = TcGemm{p.dh2, H, p.wpack + 2 * tc_pack_floats(H, D) + 2 * tc_pack_floats(H, H), p.dh1, H, p.n, H, H, nullptr, p.h1, H};
     b.n = 1;
     ++*p.launches;
-    e = launch_gemm_tc2(b, GM_MASK, p.error, s);
+    e = launch_gemm_tc2(b, GM_MASK, p.watch, s);
   } else if (!p.value_head && H >= 128 && tc_gemm_ok(p.dh2, H, p.w2t, H, p.n, H, H)) {
     // the tensor-core product wants both operands K-major: dh1 = dh2 (W2^T)^T with W2^T written out first
     ++*p.launches;
@@ -1096,15 +1099,15 @@ cudaError_t backward_and_update(const SgdParams& p, float lr, const AdamParams* 
   n_ranges = (p.n + rows_per_range - 1) / rows_per_range;
   const int count = (int)((p.value_head ? bv + 1 : b3 + A) - p.theta);
   *p.launches += (tb.n ? 1 : 0) + (gp.n_tiles + narrow.n_blocks > 0 ? 1 : 0) + 1;
-  if (tb.n && (e = launch_wgrad_tc(tb, p.grad_partial, count, p.n, rows_per_range, n_ranges, p.error, s)) != cudaSuccess) return e;
+  if (tb.n && (e = launch_wgrad_tc(tb, p.grad_partial, count, p.n, rows_per_range, n_ranges, p.watch, s)) != cudaSuccess) return e;
   if (gp.n_tiles + narrow.n_blocks > 0 &&
       (e = launch_chained(sgd_grad_partial_kernel, dim3(gp.n_tiles + narrow.n_blocks, n_ranges), 256, 0, s, p.grad_partial, gp, narrow, count, p.n,
                           rows_per_range)) != cudaSuccess)
     return e;
   if (adam)
     return launch_chained(sgd_apply_adam_kernel, (count + 255) / 256, 256, 0, s, p.theta, adam->m, adam->v, p.grad_partial, count, n_ranges, lr,
-                          adam->beta1, adam->beta2, adam->eps, adam->c1, adam->c2);
-  return launch_chained(sgd_apply_kernel, (count + 255) / 256, 256, 0, s, p.theta, p.grad_partial, count, n_ranges, lr);
+                          adam->beta1, adam->beta2, adam->eps, adam->c1, adam->c2, p.watch);
+  return launch_chained(sgd_apply_kernel, (count + 255) / 256, 256, 0, s, p.theta, p.grad_partial, count, n_ranges, lr, p.watch);
 }
 }  // namespace
 
@@ -1132,12 +1135,12 @@ static cudaError_t sgd_step_layered(const SgdParams& p, float lr, const AdamPara
     l1.g[0] = TcGemm{p.obs, D, pk_W1, p.h1, H, n, H, D, b1, nullptr, 0};
     l1.g[1] = TcGemm{p.next_obs, D, pk_T1, p.dh1, H, n, H, D, tb1, nullptr, 0};
     l1.n = 2;
-    if ((e = launch_gemm_tc2(l1, GM_BIAS_RELU, p.error, s)) != cudaSuccess) return e;
+    if ((e = launch_gemm_tc2(l1, GM_BIAS_RELU, p.watch, s)) != cudaSuccess) return e;
     TcGemmBatch l2{};
     l2.g[0] = TcGemm{p.h1, H, pk_W2, p.h2, H, n, H, H, b2, nullptr, 0};
     l2.g[1] = TcGemm{p.dh1, H, pk_T2, p.dh2, H, n, H, H, tb2, nullptr, 0};
     l2.n = 2;
-    if ((e = launch_gemm_tc2(l2, GM_BIAS_RELU, p.error, s)) != cudaSuccess) return e;
+    if ((e = launch_gemm_tc2(l2, GM_BIAS_RELU, p.watch, s)) != cudaSuccess) return e;
     *p.launches += 3;
   } else {
     const GemmPair l1{{p.obs, p.next_obs}, {W1, T1}, {p.h1, p.dh1}, {b1, tb1}}, l2{{p.h1, p.dh1}, {W2, T2}, {p.h2, p.dh2}, {b2, tb2}};
@@ -1172,7 +1175,7 @@ cudaError_t launch_sgd_step(const SgdParams& p, float lr, const AdamParams* adam
   cudaError_t e = sgd_step_layered(p, lr, adam, s);
   if (e == cudaSuccess && loss_out) {
     ++*p.launches;
-    e = launch_td_finish(p.partial, sgd_partial_count(p.n), p.n, loss_out, s);
+    e = launch_td_finish(p.partial, sgd_partial_count(p.n), p.n, loss_out, s, p.watch);
   }
   return e;
 }

@@ -554,7 +554,7 @@ __global__ void __launch_bounds__(FS_NT, 1) sgd_fused_kernel(const SgdParams p, 
     if (PPO) { pp[1] = part1; pp[2] = part2; pp[3] = part3; pp[4] = part4; }
   }
   if (!ok) {
-    atomicExch(p.error, 3ull);
+    update_failed(p.watch);
     if (tid == 0) {                                // thread 0 waits for every copy: if it was served, all have arrived
       mbar_settle(bar, 0);
       if (!PPO) mbar_settle(bar + 1, 0);
@@ -566,54 +566,65 @@ __global__ void __launch_bounds__(FS_NT, 1) sgd_fused_kernel(const SgdParams p, 
 // theta from the sums of the blocks' partial gradients: a block takes 128 parameters, sixteen warps a share of the partials each
 // (sixteen bytes per lane and partial), added in a fixed order; block 0 also adds up the loss terms
 constexpr int FA_SHARES = 16, FA_NT = 32 * FA_SHARES;
+//
+// The parameters are 96 bytes on purpose: with 24 more the kernel's first look at the last of them missed the constant cache once more
+// and the launch took 4.75 us instead of 4.0 (hidden 64, 1,024 rows).
+struct FaParams {
+  float *theta, *m, *v;
+  const float *P, *loss_parts;
+  float* loss_out;
+  float lr, beta1, beta2, eps, c1, c2;
+  int stride, count, n_parts, n_terms, n_rows;
+  unsigned number;                                 // of the update; the number of the last one that failed lies in front of P
+};
+static_assert(sizeof(FaParams) <= 96, "a fourth constant line");
 template <bool ADAM>
-__global__ void __launch_bounds__(FA_NT) sgd_fused_apply_kernel(float* __restrict__ theta, const AdamParams ap, const float* __restrict__ P, int stride,
-                                                              int count, int n_parts, float lr, const float* __restrict__ loss_parts, int n_terms,
-                                                              int n_rows, float* __restrict__ loss_out) {
+__global__ void __launch_bounds__(FA_NT) sgd_fused_apply_kernel(const FaParams p) {
   __shared__ float4 sums[FA_SHARES][32];
   const int tid = threadIdx.x, lane = tid & 31, share = tid >> 5, q = blockIdx.x * 32 + lane;
   chain_begin();
   chain_next();
   // this thread's parameter and moments are on their way while the partials are added
   const int i = blockIdx.x * 128 + tid;
-  const bool mine = tid < 128 && i < count;
+  const bool mine = tid < 128 && i < p.count;
+  const unsigned asked = update_ask(reinterpret_cast<const unsigned*>(p.P) - 4, p.number);
   float theta_i = 0.f, m_i = 0.f, v_i = 0.f;
   if (mine) {
-    theta_i = theta[i];
-    if (ADAM) { m_i = ap.m[i]; v_i = ap.v[i]; }
+    theta_i = p.theta[i];
+    if (ADAM) { m_i = p.m[i]; v_i = p.v[i]; }
   }
   float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (4 * q < count) {
+  if (4 * q < p.count) {
 #pragma unroll 8
-    for (int b = share; b < n_parts; b += FA_SHARES) {
-      const float4 v = __ldcg(reinterpret_cast<const float4*>(P + (size_t)b * stride) + q);
+    for (int b = share; b < p.n_parts; b += FA_SHARES) {
+      const float4 v = __ldcg(reinterpret_cast<const float4*>(p.P + (size_t)b * p.stride) + q);
       s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
     }
   }
   sums[share][lane] = s;
-  __syncthreads();
+  const bool valid = update_valid(p.number, asked);   // and the sums are there
   if (tid < 128) {
-    if (mine) {
+    if (mine && valid) {                           // else parameters and moments stay as they were
       const float* col = reinterpret_cast<const float*>(&sums[0][0]) + tid;
       float g = 0.f;
 #pragma unroll
       for (int k = 0; k < FA_SHARES; ++k) g += col[k * 128];
       if (ADAM) {
-        const float mi = fmaf(ap.beta1, m_i, (1.f - ap.beta1) * g);
-        const float vi = fmaf(ap.beta2, v_i, (1.f - ap.beta2) * g * g);
-        ap.m[i] = mi;
-        ap.v[i] = vi;
-        theta[i] = theta_i - lr * (mi / ap.c1) / (sqrtf(vi / ap.c2) + ap.eps);
+        const float mi = fmaf(p.beta1, m_i, (1.f - p.beta1) * g);
+        const float vi = fmaf(p.beta2, v_i, (1.f - p.beta2) * g * g);
+        p.m[i] = mi;
+        p.v[i] = vi;
+        p.theta[i] = theta_i - p.lr * (mi / p.c1) / (sqrtf(vi / p.c2) + p.eps);
       } else {
-        theta[i] = theta_i - lr * g;
+        p.theta[i] = theta_i - p.lr * g;
       }
     }
-  } else if (blockIdx.x == 0 && loss_out && share >= 4 && share - 4 < n_terms) {
+  } else if (blockIdx.x == 0 && p.loss_out && share >= 4 && share - 4 < p.n_terms) {
     const int k = share - 4;
     float t = 0.f;
-    for (int b = lane; b < n_parts; b += 32) t += loss_parts[(size_t)b * 5 + k];
+    for (int b = lane; b < p.n_parts; b += 32) t += p.loss_parts[(size_t)b * 5 + k];
     for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (lane == 0) loss_out[k] = t / (float)n_rows;
+    if (lane == 0) p.loss_out[k] = valid ? t / (float)p.n_rows : __int_as_float(0x7FC00000);
   }
 }
 
@@ -655,8 +666,10 @@ cudaError_t launch_sgd_fused(const SgdParams& p, float lr, const AdamParams* ada
       : R == 16 ? launch_fused<16, false>(p, stride, grid, s) : launch_fused<32, false>(p, stride, grid, s);
   }
   if (e != cudaSuccess) return e;
-  return launch_chained(adam ? sgd_fused_apply_kernel<true> : sgd_fused_apply_kernel<false>, (count + 127) / 128, FA_NT, 0, s, p.theta,
-                        adam ? *adam : AdamParams{}, p.grad_partial, stride, count, grid, lr, p.partial, p.value_head ? 5 : 1, p.n, loss_out);
+  FaParams a{p.theta, nullptr, nullptr, p.grad_partial, p.partial, loss_out};
+  if (adam) { a.m = adam->m; a.v = adam->v; a.beta1 = adam->beta1; a.beta2 = adam->beta2; a.eps = adam->eps; a.c1 = adam->c1; a.c2 = adam->c2; }
+  a.lr = lr; a.stride = stride; a.count = count; a.n_parts = grid; a.n_terms = p.value_head ? 5 : 1; a.n_rows = p.n; a.number = p.watch.number;
+  return launch_chained(adam ? sgd_fused_apply_kernel<true> : sgd_fused_apply_kernel<false>, (count + 127) / 128, FA_NT, 0, s, a);
 }
 
 }  // namespace tj

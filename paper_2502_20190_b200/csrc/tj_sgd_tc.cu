@@ -56,7 +56,7 @@ __device__ __forceinline__ float4 staged_piece(const float* stg, int lane, int i
   return *reinterpret_cast<const float4*>(stg + ((lane >> 3) + 4 * i) * T2_STG_LD + (lane & 7) * 4);
 }
 
-__global__ void __launch_bounds__(T2_THREADS, 1) sg_gemm_tc2_kernel(const TcGemmBatch batch, int epi, unsigned long long* __restrict__ error) {
+__global__ void __launch_bounds__(T2_THREADS, 1) sg_gemm_tc2_kernel(const TcGemmBatch batch, int epi, const UpdateWatch watch) {
   extern __shared__ uint8_t t2_raw[];
   uint8_t* a_stages = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(t2_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* b_slots = a_stages + T2_ASTAGES * T2_A_STAGE;
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(T2_THREADS, 1) sg_gemm_tc2_kernel(const TcGemm
       }
     }
   } else if (!good) {
-    if (tid == 0) atomicExch(error, 3ull);
+    if (tid == 0) update_failed(watch);
     tc_settle(&ctl->settled, warp == T2_WORKERS / 32, ctl->b_full, T2_BSLOTS, ctl->copies);
   }
   tc_fence_before();
@@ -249,7 +249,7 @@ struct WgCtl {
 constexpr int WG_SMEM_BYTES = WG_STAGES * WG_STAGE + T2_STG_BYTES + (int)sizeof(WgCtl) + 1024;
 
 __global__ void __launch_bounds__(T2_THREADS, 1) sg_wgrad_tc_kernel(const TcWgradBatch batch, float* __restrict__ P, int count, int n_rows,
-                                                                    int rows_per_range, unsigned long long* __restrict__ error) {
+                                                                    int rows_per_range, const UpdateWatch watch) {
   extern __shared__ uint8_t wg_raw[];
   uint8_t* stages = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(wg_raw) + 1023) & ~(uintptr_t)1023);
   float* stg_all = reinterpret_cast<float*>(stages + WG_STAGES * WG_STAGE);
@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(T2_THREADS, 1) sg_wgrad_tc_kernel(const TcWgra
     if (with_bias && tid < T2_M && m0 + tid < g.M)
       P[(size_t)blockIdx.y * count + g.bias_off + m0 + tid] = ctl->bias_part[tid] + ctl->bias_part[tid + T2_M];
   } else if (!good) {
-    if (tid == 0) atomicExch(error, 3ull);
+    if (tid == 0) update_failed(watch);
     tc_settle(&ctl->settled, warp == T2_WORKERS / 32, nullptr, 1, 0);     // no bulk copies here
   }
   tc_fence_before();
@@ -479,12 +479,12 @@ cudaError_t launch_pack_tf32_operands(const TcPackJobs& jobs, cudaStream_t s) {
   return launch_chained(sg_pack_tf32_kernel, dim3((most / 4 + 255) / 256, jobs.n), 256, 0, s, jobs);
 }
 
-cudaError_t launch_gemm_tc2(const TcGemmBatch& batch, int epi, unsigned long long* error, cudaStream_t s) {
+cudaError_t launch_gemm_tc2(const TcGemmBatch& batch, int epi, const UpdateWatch& watch, cudaStream_t s) {
   if (batch.n <= 0) return cudaSuccess;
   const TcGemm& g0 = batch.g[0];
   for (int i = 1; i < batch.n; ++i)
     if (batch.g[i].M != g0.M || batch.g[i].N != g0.N) return cudaErrorInvalidValue;   // one grid for all problems of a launch
-  return launch_chained(sg_gemm_tc2_kernel, dim3(g0.N / T2_N, (g0.M + T2_M - 1) / T2_M, batch.n), T2_THREADS, T2_SMEM_BYTES, s, batch, epi, error);
+  return launch_chained(sg_gemm_tc2_kernel, dim3(g0.N / T2_N, (g0.M + T2_M - 1) / T2_M, batch.n), T2_THREADS, T2_SMEM_BYTES, s, batch, epi, watch);
 }
 
 bool tc_wgrad_ok(int N, int rows) { return N % 128 == 0 && rows >= 1024; }
@@ -492,9 +492,9 @@ bool tc_wgrad_ok(int N, int rows) { return N % 128 == 0 && rows >= 1024; }
 int tc_wgrad_tiles(int M, int N) { return ((M + T2_M - 1) / T2_M) * (N / (N % T2_N == 0 ? T2_N : 128)); }
 
 cudaError_t launch_wgrad_tc(const TcWgradBatch& batch, float* P, int count, int n_rows, int rows_per_range, int n_ranges,
-                            unsigned long long* error, cudaStream_t s) {
+                            const UpdateWatch& watch, cudaStream_t s) {
   if (batch.n <= 0 || batch.n_tiles <= 0) return cudaSuccess;
-  return launch_chained(sg_wgrad_tc_kernel, dim3(batch.n_tiles, n_ranges), T2_THREADS, WG_SMEM_BYTES, s, batch, P, count, n_rows, rows_per_range, error);
+  return launch_chained(sg_wgrad_tc_kernel, dim3(batch.n_tiles, n_ranges), T2_THREADS, WG_SMEM_BYTES, s, batch, P, count, n_rows, rows_per_range, watch);
 }
 
 }  // namespace tj

@@ -58,6 +58,32 @@ def case_actor(H, N, steps):
     assert ctx.stats()["produced"] == 2 * steps * N
 
 
+def _unchanged(torch, ctx, blobs, update):
+    kept = [b.clone() for b in blobs]
+    loss = update()
+    _latched(torch, ctx, 3)
+    assert bool(torch.isnan(loss).all())
+    for a, b in zip(kept, blobs):
+        assert torch.equal(a, b)
+
+
+def case_update(adam, kind, D, A, H, n):
+    torch, binding, ctx, theta = _context(kind, D, A, H, n)
+    b, target, m, v = _batch(torch, ctx, n), theta.clone(), torch.full_like(theta, 1e-3), torch.full_like(theta, 1e-6)
+    if adam:
+        _unchanged(torch, ctx, (theta, m, v), lambda: ctx.adam_step(b, 1e-2, theta, target, m, v, 3))
+    else:
+        _unchanged(torch, ctx, (theta,), lambda: ctx.sgd_step(b, 1e-2, theta, target))
+
+
+def case_ppo(n):
+    torch, binding, ctx, theta = _context(policy_kind=1, epsilon=0.0, replay_capacity=0, rollout_len=8, n_segments=2, B=n)
+    x = [torch.rand(n, device="cuda") for _ in range(3)]
+    obs, act = torch.randn((n, 4), device="cuda"), torch.zeros(n, dtype=torch.int32, device="cuda")
+    m, v = torch.full_like(theta, 1e-3), torch.full_like(theta, 1e-6)
+    _unchanged(torch, ctx, (theta, m, v), lambda: ctx.ppo_step(obs, act, *x, 1e-2, theta, m, v, 3))
+
+
 CASES = {
     "td, both networks in shared memory": (case_td, 64, 300, 300),
     "td, both networks in shared memory, several tiles": (case_td, 24, 9000, 300),
@@ -67,6 +93,11 @@ CASES = {
     "actor, two blocks per SM": (case_actor, 64, 6000, 2),
     "actor, hidden matrix through the ring": (case_actor, 256, 500, 3),
     "actor, largest ring": (case_actor, 768, 90, 2),
+    "update, fused, SGD": (case_update, False, 0, 4, 2, 64, 300),
+    "update, fused, Adam, several chunks of rows per block": (case_update, True, 1, 6, 3, 128, 9000),
+    "update, fused, PPO": (case_ppo, 700),
+    "update, tensor-core products, SGD": (case_update, False, 2, 32, 7, 512, 3100),
+    "update, tensor-core products, Adam": (case_update, True, 2, 32, 7, 512, 3100),
 }
 
 
