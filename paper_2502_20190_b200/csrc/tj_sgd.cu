@@ -1047,8 +1047,6 @@ cudaError_t backward_and_update(const SgdParams& p, float lr, const AdamParams* 
   float* b2 = W2 + (size_t)H * H;
   float* W3 = b2 + H;
   float* b3 = W3 + (size_t)A * H;
-  float* Wv = b3 + A;
-  float* bv = Wv + H;
   // the backward pass has read W2 and the heads; now the parameters may change: all products in one or two launches, then
   // one pass over the whole blob.  Products whose input width is a multiple of 128 go to the tensor cores (with their bias
   // gradient), the others to the FMA tiles.
@@ -1085,8 +1083,7 @@ cudaError_t backward_and_update(const SgdParams& p, float lr, const AdamParams* 
   } else {
     product(W1, b1, H, D, p.dh1, H, p.obs, D);
     product(W2, b2, H, H, p.dh2, H, p.h1, H);
-    product(W3, b3, A, H, p.g, p.ldg, p.h2, H);
-    if (p.value_head) product(Wv, bv, 1, H, p.g + A, p.ldg, p.h2, H);
+    product(W3, b3, A, H, p.g, p.ldg, p.h2, H);    // no value head here: it comes with CartPole and Acrobot only
   }
   // row ranges: with tensor-core tiles about one thread block per SM in all (a block costs a fixed ~10 us beside its rows);
   // otherwise three per SM, but 128 rows or more per range
@@ -1097,7 +1094,7 @@ cudaError_t backward_and_update(const SgdParams& p, float lr, const AdamParams* 
   if (n_ranges > SG_SPLITS) n_ranges = SG_SPLITS;
   const int rows_per_range = ((p.n + n_ranges - 1) / n_ranges + 31) / 32 * 32;
   n_ranges = (p.n + rows_per_range - 1) / rows_per_range;
-  const int count = (int)((p.value_head ? bv + 1 : b3 + A) - p.theta);
+  const int count = (int)(b3 + A - p.theta) + (p.value_head ? H + 1 : 0);
   *p.launches += (tb.n ? 1 : 0) + (gp.n_tiles + narrow.n_blocks > 0 ? 1 : 0) + 1;
   if (tb.n && (e = launch_wgrad_tc(tb, p.grad_partial, count, p.n, rows_per_range, n_ranges, p.watch, s)) != cudaSuccess) return e;
   if (gp.n_tiles + narrow.n_blocks > 0 &&
