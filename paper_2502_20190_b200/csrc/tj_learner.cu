@@ -107,8 +107,6 @@ __global__ void __launch_bounds__(256) gather_kernel(const SampleParams p) {
   }
 }
 
-// TD error on a tile of TE samples: online forward on obs, target forward on next_obs.
-// STAGE as in the actor kernel (stage_mlp_weights); the staging buffer is filled twice (online, then target parameters).
 // A staging wait that ran out, for the whole block: latch the context's error word and leave defined outputs (NaN) for this block's rows
 // and its partial sum, so that neither the caller nor the loss reduction reads what an earlier call left there; the staged
 // parameters have to arrive before the block leaves.
@@ -125,6 +123,8 @@ __device__ __forceinline__ void td_give_up(const TdParams& p, int n_here, int j0
   }
 }
 
+// TD error on a tile of TE samples: online forward on obs, target forward on next_obs.  STAGE: what of the parameters lies in shared
+// memory (stage_mlp_weights); the staging buffer is filled twice (online, then target parameters).
 template <int TE, int NT, int EPT, int NPT, int STAGE>
 __global__ void __launch_bounds__(NT) td_kernel(const TdParams p) {
   extern __shared__ __align__(128) float smem[];

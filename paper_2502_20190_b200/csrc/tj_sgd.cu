@@ -529,8 +529,11 @@ __global__ void __launch_bounds__(256) sg_transpose_kernel(const float* __restri
     if (c0 + i < n && r0 + tx < n) dst[(size_t)(c0 + i) * n + r0 + tx] = tile[tx][i];
 }
 
-// shapes the tensor-core product takes: 16-byte rows on both operands and enough 128 x 128 tiles to occupy most SMs (with
-// fewer, the 128 x 64 FMA tiles spread the work over more blocks and finish sooner)
+// Shapes the tensor-core product takes: 16-byte rows on both operands and enough 128 x 128 tiles to occupy most SMs (with
+// fewer, the FMA tiles spread the work over more blocks and finish sooner).  The 96 were measured against 128 x 64 FMA tiles; against
+// the present ones the line lies higher.  Whole tj_sgd_step, us, on the tensor cores / FMA tiles: 32 inputs, hidden 384: 96 tiles
+// 203 / 177, 192 336 / 322, 384 657 / 618, 768 1,117 / 1,217; 4 inputs, hidden 256: 64 tiles 123 / 86, 128 150 / 147, 256 253 / 270,
+// 512 520 / 559; 32 inputs, hidden 700: 384 tiles 961 / 1,002.
 static bool tc_gemm_ok(const float* A, int lda, const float* B, int ldb, int M, int N, int K) {
   const long long tiles = (long long)((M + TG_M - 1) / TG_M) * ((N + TG_N - 1) / TG_N);
   return (K & 3) == 0 && (lda & 3) == 0 && (ldb & 3) == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0 &&
