@@ -212,7 +212,7 @@ cudaError_t launch_actor(int env_kind, const ActorParams& p, int sm_count, cudaS
   const bool ext = p.logits_in != nullptr;
   const size_t smem = actor_smem_floats(TE, p.D, ext ? 0 : p.Hp, ext ? 0 : p.Ap) * sizeof(float);
   if (smem > kSmemMax) return cudaErrorInvalidConfiguration;
-  return launch_chained(actor_lingauss_kernel<TE, NT>, (p.N + TE - 1) / TE, NT, smem, s, p);
+  return launch_chained<1024>(actor_lingauss_kernel<TE, NT>, (p.N + TE - 1) / TE, NT, smem, s, p);
 }
 
 }  // namespace tj

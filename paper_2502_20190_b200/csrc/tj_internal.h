@@ -15,10 +15,15 @@ namespace tj {
 // kernel before it in the stream has called chain_next() or left (tj_async.cuh), and each waits in chain_begin() until that
 // kernel has finished, so set-up and launch latency overlap the tail of the one before.  Every kernel launched this way
 // calls chain_begin() before it touches global memory.
-template <typename... P, typename... A>
+//
+// The limit of a kernel's dynamic shared memory belongs to the kernel on the device, not to a launch: it is shared by every context and
+// thread, and one that set it to its own launch's size could lower it between another's setting and launch.  So every launch
+// above 48 KB sets the same value, all that a block may have; a kernel that also has static shared memory (STATIC_SMEM bytes at
+// most) leaves that much.
+template <size_t STATIC_SMEM = 0, typename... P, typename... A>
 cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
   if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(227 * 1024 - STATIC_SMEM));
     if (e != cudaSuccess) return e;
   }
   cudaLaunchConfig_t cfg{};

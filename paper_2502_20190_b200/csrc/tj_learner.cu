@@ -293,7 +293,7 @@ int td_grid(int n) { return (n + kTdTile - 1) / kTdTile; }
 
 template <int TE, int NT, int EPT, int NPT, int STAGE>
 cudaError_t launch_td_stage(const TdParams& p, size_t smem, int grid, cudaStream_t s) {
-  return launch_chained(td_kernel<TE, NT, EPT, NPT, STAGE>, grid, NT, smem, s, p);
+  return launch_chained<1024>(td_kernel<TE, NT, EPT, NPT, STAGE>, grid, NT, smem, s, p);
 }
 
 // tile: 16 rows x 128 threads with 4 x 4 register tiles; wide layers (hidden >= 192) 32 rows x 128 threads, 8 x 8

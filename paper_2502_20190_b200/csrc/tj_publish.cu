@@ -196,9 +196,7 @@ cudaError_t launch_publish(const PublishParams& p, cudaStream_t s) {
   const int rest = 2 * L.Hp + L.H * L.Ap + L.Ap + (p.tc ? 16 * L.H : 0), n_rest = (rest + NT - 1) / NT;
   const size_t tile_bytes = (size_t)32 * (KT + 1) * sizeof(float);
   if (!split) return launch_chained(publish_kernel<256, false>, n1 + n2 + n_rest, 256, tile_bytes, s, p);
-  const size_t smem = tile_bytes * ((n2 + 7) / 8);
-  const cudaError_t e = cudaFuncSetAttribute(publish_kernel<1024, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
+  const size_t smem = tile_bytes * ((n2 + 7) / 8);       // 33 KB at most (hidden 256)
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute at[2];
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;

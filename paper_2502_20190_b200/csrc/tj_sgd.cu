@@ -549,7 +549,7 @@ cudaError_t sg_layer(const SgdParams& p, const GemmPair& pr, int sets, int lda, 
   if (!tc) return sg_gemm<false, EPI>(p, pr, sets, lda, ldb, ldc, M, N, K, mask, ldm, s);
   for (int z = 0; z < sets; ++z) {
     ++*p.launches;
-    const cudaError_t e = launch_chained(sg_gemm_tc_kernel<EPI>, dim3((N + TG_N - 1) / TG_N, (M + TG_M - 1) / TG_M), TG_THREADS, TG_SMEM_BYTES, s, pr.A[z],
+    const cudaError_t e = launch_chained<1024>(sg_gemm_tc_kernel<EPI>, dim3((N + TG_N - 1) / TG_N, (M + TG_M - 1) / TG_M), TG_THREADS, TG_SMEM_BYTES, s, pr.A[z],
                                          lda, pr.B[z], ldb, pr.C[z], ldc, M, N, K, pr.bias[z], mask, ldm, p.watch);
     if (e != cudaSuccess) return e;
   }
