@@ -62,7 +62,8 @@ typedef enum {
 
 enum { TJ_ENV_CARTPOLE = 0, TJ_ENV_ACROBOT = 1, TJ_ENV_LINGAUSS = 2 };
 enum { TJ_POLICY_EPS_GREEDY = 0, TJ_POLICY_CATEGORICAL = 1 };
-enum { TJ_W_FP32 = 0,      /* FP32 FMA in one fixed rounding order: outputs (and actions) reproducible bit for bit */
+enum { TJ_W_FP32 = 0,      /* FP32 FMA: network outputs, actions and TD errors in one fixed rounding order (bias, then k = 0, 1, 2, ...),
+                              whichever kernel a size takes; updates in an order of their own, reproducible bit for bit */
        TJ_W_BF16 = 1,      /* weight matrices rounded to bfloat16, tensor cores, FP32 accumulation: 2e-2 */
        TJ_W_FP32_TC = 2 }; /* FP32 weights; the actor's hidden x hidden layer on the tensor cores as three products of split
                               operands (the role a 3 x TF32 product plays, here with FP16 parts at twice that rate; about

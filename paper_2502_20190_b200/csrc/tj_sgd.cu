@@ -5,7 +5,7 @@
 //             delta = r + gamma (1 - done) q' - q, g = -clip(delta, -kappa, kappa) / n  (= dL/dq)
 //   backward  dh2 = g W3[a] (h2 > 0), dh1 = (W2^T dh2) (h1 > 0)
 //   update    W3[a] -= lr sum_j g_j h2_j, W2 -= lr dh2^T h1, W1 -= lr dh1^T x, biases likewise
-// Every sum runs in a fixed order (rows ascending), so a step is reproducible bit for bit.
+// Every sum runs in a fixed order that depends on the shapes alone, so a step is reproducible bit for bit.
 #include "tj_async.cuh"
 #include "tj_internal.h"
 #include "tj_fma.cuh"
@@ -18,9 +18,9 @@ namespace {
 constexpr int SG_ROWS = 16;       // minibatch rows per loss partial
 
 // ---------------------------------------------------------------------------------------------------------------------
-// Wide networks and large minibatches: the layers as tiled FP32 matrix products (a weight element is reused for 128 rows
-// instead of 16).  C[m][n] = epi(sum_k A[m][k] Bop[k][n]): A row-major M x K.  B_KN false: B is N x K row-major (a weight
-// matrix as the forward pass uses it, Bop = B^T); true: B is K x N row-major (the same matrix in the backward pass).
+// Wide networks and large minibatches: the layers as tiled FP32 matrix products.  C[m][n] = epi(sum_k A[m][k] Bop[k][n]): A row-major
+// M x K.  B_KN false: B is N x K row-major (a weight matrix as the forward pass uses it, Bop = B^T); true: B is K x N row-major (the
+// same matrix in the backward pass).
 // 64 x 64 tile per block (32 rows where that leaves SMs idle), 32 k per step in one of two stages.  Two groups of 128 threads take
 // alternate halves of each step, a thread 8 x 4 outputs (4 x 4 in the 32-row tile) with two rows per instruction, and add their sums
 // at the end: a fixed order.  An update has few tiles per SM, so what bounds a tile is latency: one group of four warps with

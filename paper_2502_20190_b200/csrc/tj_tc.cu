@@ -5,7 +5,7 @@
 // One thread block owns a tile of 128 rows (one row per TMEM lane) and walks tiles persistently.  Roles:
 //   warp 0, one lane   producer: streams pre-tiled BF16 weight chunks from global/L2 into a shared-memory ring with
 //                      bulk async copies (mbarrier complete_tx)
-//   warp 1, one lane   issues tcgen05.mma (M = 128, N <= 256, K = 16) over the ring; tcgen05.commit frees ring
+//   warp 1             issues tcgen05.mma (M = 128, N <= 256, K = 16; one elected lane) over the ring; tcgen05.commit frees ring
 //                      slots and signals "accumulator full"
 //   warps 2-9          (256 threads, TC_SPLIT = 2 per row, each owning half of the columns) convert the FP32 input rows to BF16 into the A-operand buffer;
 //                      after each layer read the accumulator from TMEM (tcgen05.ld), add the bias, apply ReLU,

@@ -5,7 +5,7 @@
 // its block, so no step waits for another block, and the weights' ring, the pipeline and the launch are set up once (four steps of
 // 20,000 envs, hidden 512: 206 us as four launches, 171 as one).  Roles:
 //   warp 0, one lane    producer: streams 32 KB operand chunks (weights, the env matrix) from L2 into a ring of two slots
-//   warp 1, one lane    MMA issuer (tcgen05.mma, M = 128, N = 128 per hidden block)
+//   warp 1              MMA issuer, its loop warp-uniform, one elected lane at the instruction (tcgen05.mma, M = 128, N = 128 per hidden block)
 //   warps 4-19          network warps (four threads per row): per 128-neuron block of a hidden layer: accumulator -> bias, ReLU, BF16
 //                       -> next layer's operand; z -> a scratch tile in global memory
 //   warps 20-27         env warps: the next tile's state rows as BF16 (layer-1 operand) and, with the record's observation, as FP16
@@ -303,7 +303,6 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
     const int ew = warp - PA_ENV0;                 // 0..7; the first four also read the head outputs (one TMEM quarter each)
     const int e_r4 = lane >> 3, e_kq = lane & 7;   // four rows x eight 16-byte pieces per warp instruction, four pieces per lane and row
     uint32_t tiles = 0;
-    // FP16 high / low parts of a tile's scaled rows -> U (A operand of z = A s); the FP32 row is the record's observation
     // BF16 rows of a tile -> X (layer-1 A operand)
     auto convert_x = [&](int tile) {
 #pragma unroll 1
@@ -326,6 +325,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
       fence_async_smem();
       mbar_arrive_warp(&ctl->x_ready);
     };
+    // FP16 high / low parts of a tile's scaled rows -> U (A operand of z = A s); the FP32 row is the record's observation
     auto convert_u = [&](int tile, uint32_t block) {
 #pragma unroll 1
       for (int g = 0; g < 4; ++g) {
