@@ -276,7 +276,8 @@ int tj_td_error_static(tj_ctx *ctx, const tj_batch *batch, float *td_out, float 
  * In a BF16 context theta is the FP32 master copy: the update and its loss are FP32 all the same, the rounding to BF16
  * happens at tj_publish_weights (so this loss differs from tj_td_error's, which uses the published BF16 copy, by that
  * rounding).  Should a kernel's bounded wait run out, theta stays as it was, the loss is NaN and device_error is latched
- * (tj_stats).  TJ_ERR_UNSUPPORTED for segment mode and the categorical policy. */
+ * (tj_stats); the next call is an update of its own again, a replay of a captured one that failed stays without effect.
+ * TJ_ERR_UNSUPPORTED for segment mode and the categorical policy. */
 int tj_sgd_step(tj_ctx *ctx, const tj_batch *batch, float lr, float *theta, const float *theta_target, float *loss_mean_out);
 
 /* The same gradient through Adam (the optimiser of Table 2; Kingma & Ba 2015), step counter t >= 1:
