@@ -88,38 +88,30 @@ __device__ __forceinline__ f32x2 pair2(float a, float b) {
   return d;
 }
 
-// 8 NB hidden units from n0 of layer 1 in the canonical order (bias, then inputs in index order; weights and biases come scaled by
-// SA_H_SCALE, a power of two, which leaves every rounding where it was), ReLU, split -> NB 16-byte row segments of each part of the A
-// operand; returns the largest scaled activation.  All units are computed before the first store: a store orders the loads after it.
-template <int D, int H, int NB>
-__device__ __forceinline__ float s2_layer1(const float* w1, const float* b1, const f32x2 (&x)[D], int n0, uint8_t* hi_dst, float vmax) {
-  f32x2 acc[4 * NB];
+// Eight hidden units of layer 1 for ROWS rows, eight apart, in the canonical order (bias, then inputs in index order; weights and biases
+// come scaled by SA_H_SCALE, a power of two, which leaves every rounding where it was), ReLU, split -> a 16-byte row segment of each part
+// of the A operand per row; returns the largest scaled activation.
+template <int D, int ROWS>
+__device__ __forceinline__ float s2_layer1(const f32x2 (&w)[D][4], const f32x2 (&b)[4], const f32x2 (&x)[ROWS][D], uint8_t* hi_dst, float vmax) {
 #pragma unroll
-  for (int i = 0; i < 2 * NB; ++i) {
-    const ulonglong2 b = ld_pairs(b1 + n0 + 4 * i);
-    acc[2 * i] = b.x; acc[2 * i + 1] = b.y;
-  }
+  for (int r = 0; r < ROWS; ++r) {
+    f32x2 acc[4] = {b[0], b[1], b[2], b[3]};
 #pragma unroll
-  for (int k = 0; k < D; ++k)
+    for (int k = 0; k < D; ++k)
 #pragma unroll
-    for (int i = 0; i < 2 * NB; ++i) {
-      const ulonglong2 w = ld_pairs(w1 + k * H + n0 + 4 * i);
-      fma2(acc[2 * i], w.x, x[k]); fma2(acc[2 * i + 1], w.y, x[k]);
+      for (int i = 0; i < 4; ++i) fma2(acc[i], w[k][i], x[r][k]);
+    uint32_t hi[4], lo[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float2 a = halves(acc[i]);
+      const float v0 = fmaxf(a.x, 0.f), v1 = fmaxf(a.y, 0.f);
+      vmax = fmaxf(vmax, fmaxf(a.x, a.y));
+      const float h0 = __uint_as_float(__float_as_uint(v0) & 0xFFFFE000u), h1 = __uint_as_float(__float_as_uint(v1) & 0xFFFFE000u);
+      hi[i] = pack_f16x2(h0, h1);
+      lo[i] = pack_f16x2(v0 - h0, v1 - h1);
     }
-  uint32_t hi[4 * NB], lo[4 * NB];
-#pragma unroll
-  for (int i = 0; i < 4 * NB; ++i) {
-    const float2 a = halves(acc[i]);
-    const float v0 = fmaxf(a.x, 0.f), v1 = fmaxf(a.y, 0.f);
-    vmax = fmaxf(vmax, fmaxf(a.x, a.y));
-    const float h0 = __uint_as_float(__float_as_uint(v0) & 0xFFFFE000u), h1 = __uint_as_float(__float_as_uint(v1) & 0xFFFFE000u);
-    hi[i] = pack_f16x2(h0, h1);
-    lo[i] = pack_f16x2(v0 - h0, v1 - h1);
-  }
-#pragma unroll
-  for (int b = 0; b < NB; ++b) {
-    *reinterpret_cast<uint4*>(hi_dst + b * 128) = make_uint4(hi[4 * b], hi[4 * b + 1], hi[4 * b + 2], hi[4 * b + 3]);
-    *reinterpret_cast<uint4*>(hi_dst + S2_A_PART + b * 128) = make_uint4(lo[4 * b], lo[4 * b + 1], lo[4 * b + 2], lo[4 * b + 3]);
+    *reinterpret_cast<uint4*>(hi_dst + r * ((SA_KC / 8) * 128)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+    *reinterpret_cast<uint4*>(hi_dst + S2_A_PART + r * ((SA_KC / 8) * 128)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
   }
   return vmax;
 }
@@ -132,8 +124,9 @@ struct S2Smem {
   static constexpr int AS = S2_A_SLOTS / GROUPS, NT = 128 * TPR * GROUPS + 64;   // A slots of a tile in flight; threads
   static constexpr uint32_t ACC_COLS = H <= 128 ? 128 : 256;
   uint8_t *a_ring, *w_ring;
-  float *w1, *b1, *b2;    // [D][H] and [H], scaled; [H]
-  float* w3;              // TPR 1: [4][H / 2] pairs (column c, column c + H / 2); 2: [H][4]
+  float *w1, *b1;         // [D][H] and [H], scaled
+  float* hw;              // per pair of hidden units: second-layer biases, head weights of outputs 0, 1, 2, two floats each
+  float* hw3;             // per pair: those of output 3
   float* b3;              // [4]
   float* part;            // TPR 2: head sums [tile in flight][pass parity][half][TE][4]
   S2Ctl* ctl;
@@ -141,7 +134,7 @@ struct S2Smem {
     a_ring = base;
     w_ring = a_ring + S2_A_SLOTS * S2_A_SLOT;
     w1 = reinterpret_cast<float*>(w_ring + SA_SLOTS * CHUNK_BYTES);
-    b1 = w1 + D * H; b2 = b1 + H; w3 = b2 + H; b3 = w3 + 4 * H; part = b3 + 4;
+    b1 = w1 + D * H; hw = b1 + H; hw3 = hw + 4 * H; b3 = hw3 + H; part = b3 + 4;
     ctl = reinterpret_cast<S2Ctl*>(part + (TPR == 2 ? GROUPS * 2 * 2 * SA_TE * 4 : 0));
   }
   static size_t bytes() {
@@ -195,13 +188,9 @@ struct S2Smem {
 #pragma unroll
       for (int k = 0; k < D; ++k) w1[k * H + i] = SA_H_SCALE * wk[k];
       b1[i] = SA_H_SCALE * c1;
-      b2[i] = c2;
-      if (TPR == 2) {
-        reinterpret_cast<float4*>(w3)[i] = w;
-      } else {
-        float* d = w3 + 2 * (i % (H / 2)) + i / (H / 2);
-        d[0] = w.x; d[H] = w.y; d[2 * H] = w.z; d[3 * H] = w.w;
-      }
+      float* d = hw + 8 * (i >> 1) + (i & 1);
+      d[0] = c2; d[2] = w.x; d[4] = w.y; d[6] = w.z;
+      hw3[i] = w.w;
     }
     if (threadIdx.x >= NT - 4) {
       const int a = threadIdx.x - (NT - 4);
@@ -281,83 +270,98 @@ struct S2Worker {
     t_row = tmem + (uint32_t)g * M::ACC_COLS + ((uint32_t)((warp & 3) * 32) << 16);
     inv_scale = inv;
   }
-  // network outputs of one observation
+  // network outputs of one observation.  What a thread keeps in registers decides what the layers read from shared memory, whose read path
+  // returns a word per lane and cycle, broadcast or not: layer 1 with a thread per environment read every weight for every environment,
+  // 320 16-byte words a thread and pass, and the drain 256, two thirds of the cycles of the read path.  So
+  //   layer 1: a lane takes eight hidden units of four (TPR 2: two) rows of its warp, eight apart, whose observations come by shuffle;
+  //   drain: fragments of 8 columns x 16 rows (a lane holds two neighbouring columns of four rows), so a weight read serves four rows.
   __device__ __forceinline__ void forward(const float (&obs)[6], int Aout, float (&out)[4]) {
+    constexpr int ROWS = 4 / TPR;
     volatile int* abort_flag = &m.ctl->abort_flag;
+    const int lane = threadIdx.x & 31, first = (row & ~31) + (TPR == 2 ? half * 16 : 0);   // first row of this warp's share
     tc_fence_before();                                        // this thread's accumulator reads of the previous pass are complete
-    f32x2 x[D];
+    f32x2 x[ROWS][D];
 #pragma unroll
-    for (int k = 0; k < D; ++k) x[k] = dup2(obs[k]);
+    for (int r = 0; r < ROWS; ++r)
+#pragma unroll
+      for (int k = 0; k < D; ++k) x[r][k] = dup2(__shfl_sync(0xffffffffu, obs[k], (first & 31) + 8 * r + (lane & 7)));
+    const float *w1 = m.w1 + (lane >> 3) * 8, *b1 = m.b1 + (lane >> 3) * 8;
+    uint8_t* dst = m.a_ring + (first >> 3) * ((SA_KC / 8) * 128) + (lane & 7) * 16 + (lane >> 3) * 128;
 #pragma unroll 1
     for (int kc = 0; kc < M::NKC; ++kc, ++ac) {
       const uint32_t as = (uint32_t)g * M::AS + ac % M::AS;
-      if (ac >= M::AS) ok = ok && tc_wait_elect(&m.ctl->a_free[as], ((ac / M::AS) - 1) & 1, abort_flag);
-      uint8_t* dst = m.a_ring + as * S2_A_SLOT + (row >> 3) * ((SA_KC / 8) * 128) + (row & 7) * 16 + half * 256;
+      f32x2 w[D][4], b[4];
 #pragma unroll
-      for (int b = 0; b < 4 / TPR; b += 2) vmax = s2_layer1<D, H, 2>(m.w1, m.b1, x, kc * SA_KC + half * 16 + 8 * b, dst + 128 * b, vmax);
+      for (int i = 0; i < 2; ++i) {
+        const ulonglong2 bb = ld_pairs(b1 + kc * SA_KC + 4 * i);
+        b[2 * i] = bb.x; b[2 * i + 1] = bb.y;
+#pragma unroll
+        for (int k = 0; k < D; ++k) {
+          const ulonglong2 ww = ld_pairs(w1 + k * H + kc * SA_KC + 4 * i);
+          w[k][2 * i] = ww.x; w[k][2 * i + 1] = ww.y;
+        }
+      }
+      if (ac >= M::AS) ok = ok && tc_wait_elect(&m.ctl->a_free[as], ((ac / M::AS) - 1) & 1, abort_flag);
+      vmax = s2_layer1<D, ROWS>(w, b, x, dst + as * S2_A_SLOT, vmax);
       fence_async_smem();
       mbar_arrive_warp(&m.ctl->a_ready[as]);
     }
     ok = ok && tc_wait_elect(&m.ctl->acc_full[g], pass & 1, abort_flag);
     tc_fence_after();
-    const float* b2 = m.b2;
-    const float* w3 = m.w3;
-    if (TPR == 1) {
-      // h2 = relu(acc / scale + b2); the sums over the two halves of the columns side by side, each in column order
-      // (fetching the next columns ahead took 17 % longer: the registers for it spill)
-      f32x2 s[4] = {0ull, 0ull, 0ull, 0ull};
+    // h2 = relu(acc / scale + b2) and the head's sums; s[i][a]: row lane / 4 + 8 i of the warp's 32, output a, even and odd columns apart
+    f32x2 s[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int a = 0; a < 4; ++a) s[i][a] = 0ull;
+    const f32x2 inv2 = dup2(inv_scale);
+    const int c_begin = half * (H / 2), c_end = TPR == 2 ? c_begin + H / 2 : H;
 #pragma unroll 1
-      for (int c0 = 0; c0 < H / 2; c0 += 16) {
-        uint32_t u[16], v[16];
-        tmem_ld16(t_row + (uint32_t)c0, u);
-        tmem_ld16(t_row + (uint32_t)(c0 + H / 2), v);
-        tmem_ld_wait();
-#pragma unroll
-          for (int i = 0; i < 16; i += 4) {
-            const float4 ba = *reinterpret_cast<const float4*>(b2 + c0 + i), bb = *reinterpret_cast<const float4*>(b2 + c0 + i + H / 2);
-            const float b_lo[4] = {ba.x, ba.y, ba.z, ba.w}, b_hi[4] = {bb.x, bb.y, bb.z, bb.w};
-            f32x2 h[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-              h[j] = pair2(fmaxf(fmaf(__uint_as_float(u[i + j]), inv_scale, b_lo[j]), 0.f), fmaxf(fmaf(__uint_as_float(v[i + j]), inv_scale, b_hi[j]), 0.f));
-#pragma unroll
-            for (int a = 0; a < 4; ++a) {
-              if (a == 3 && Aout <= 3) break;
-              const ulonglong2 wa = ld_pairs(w3 + a * H + 2 * (c0 + i)), wb = ld_pairs(w3 + a * H + 2 * (c0 + i) + 4);
-              fma2(s[a], wa.x, h[0]); fma2(s[a], wa.y, h[1]); fma2(s[a], wb.x, h[2]); fma2(s[a], wb.y, h[3]);
-            }
-          }
-        }
-#pragma unroll
-      for (int a = 0; a < 4; ++a) { const float2 t = halves(s[a]); out[a] = (m.b3[a] + t.x) + t.y; }
-    } else {
-      f32x2 s01 = 0ull, s23 = 0ull;
-      const int c_begin = half * (H / 2);
+    for (int c0 = c_begin; c0 < c_end; c0 += 32) {
       uint32_t u[2][16];
-      tmem_ld16(t_row + (uint32_t)c_begin, u[0]);
-#pragma unroll 1
-      for (int c1 = c_begin; c1 < c_begin + H / 2; c1 += 32)
+      tmem_ld_16x32(t_row + (uint32_t)c0, u[0]);
+      tmem_ld_16x32(t_row + (16u << 16) + (uint32_t)c0, u[1]);
+      const float *hw = m.hw + 4 * c0 + 8 * (lane & 3), *hw3 = m.hw3 + c0 + 2 * (lane & 3);
+      tmem_ld_wait();
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int c0 = c1 + 16 * q;
-          tmem_ld_wait();
-          if (c0 + 16 < c_begin + H / 2) tmem_ld16(t_row + (uint32_t)(c0 + 16), u[q ^ 1]);
+      for (int j = 0; j < 4; ++j) {
+        const ulonglong2 p01 = ld_pairs(hw + 32 * j), p23 = ld_pairs(hw + 32 * j + 4);
+        f32x2 w3 = 0ull;
+        if (Aout > 3) w3 = *reinterpret_cast<const unsigned long long*>(hw3 + 8 * j);
 #pragma unroll
-          for (int i = 0; i < 16; i += 4) {
-            const float4 ba = *reinterpret_cast<const float4*>(b2 + c0 + i);
-            const float bv[4] = {ba.x, ba.y, ba.z, ba.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const f32x2 h = dup2(fmaxf(fmaf(__uint_as_float(u[q][i + j]), inv_scale, bv[j]), 0.f));
-              const ulonglong2 w = ld_pairs(w3 + 4 * (c0 + i + j));
-              fma2(s01, w.x, h);
-              fma2(s23, w.y, h);
-            }
-          }
+        for (int i = 0; i < 4; ++i) {
+          const uint32_t* v = &u[i >> 1][4 * j + 2 * (i & 1)];
+          f32x2 h = p01.x;
+          fma2(h, pair2(__uint_as_float(v[0]), __uint_as_float(v[1])), inv2);
+          const float2 t = halves(h);
+          h = pair2(fmaxf(t.x, 0.f), fmaxf(t.y, 0.f));
+          fma2(s[i][0], p01.y, h);
+          fma2(s[i][1], p23.x, h);
+          fma2(s[i][2], p23.y, h);
+          if (Aout > 3) fma2(s[i][3], w3, h);
         }
-      const float2 a = halves(s01), b = halves(s23);
+      }
+    }
+    // the four lanes of a row meet: lane 4 r + i keeps row r + 8 i, then hands it to that row's lane
+    const bool up2 = lane & 2, up1 = lane & 1;
+    float sum[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      if (a == 3 && Aout <= 3) break;
+      float t[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) { const float2 e = halves(s[i][a]); t[i] = e.x + e.y; }
+      const float k0 = (up2 ? t[2] : t[0]) + __shfl_xor_sync(0xffffffffu, up2 ? t[0] : t[2], 2);
+      const float k1 = (up2 ? t[3] : t[1]) + __shfl_xor_sync(0xffffffffu, up2 ? t[1] : t[3], 2);
+      const float k = (up1 ? k1 : k0) + __shfl_xor_sync(0xffffffffu, up1 ? k0 : k1, 1);
+      sum[a] = __shfl_sync(0xffffffffu, k, 4 * (lane & 7) + (lane >> 3));
+    }
+    if (TPR == 1) {
+#pragma unroll
+      for (int a = 0; a < 4; ++a) out[a] = m.b3[a] + sum[a];
+    } else {
       float4* px = reinterpret_cast<float4*>(m.part) + (size_t)(2 * g + (pass & 1)) * 2 * SA_TE;
-      px[half * SA_TE + row] = make_float4(a.x, a.y, b.x, b.y);
+      px[half * SA_TE + row] = make_float4(sum[0], sum[1], sum[2], sum[3]);
       asm volatile("bar.sync %0, 256;" ::"r"(1 + g) : "memory");
       const float4 l = px[row], h = px[SA_TE + row];
       const float* b3 = m.b3;
