@@ -92,6 +92,18 @@ __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.laun
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
 }
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// arrival at the barrier at this block's address `bar` in block `rank` of the cluster.  It counts and hands no data over: what the waiting
+// block's products read of this block is in this block's own shared memory, behind fence_async_smem()
+__device__ __forceinline__ void mbar_arrive_cluster(uint64_t* bar, uint32_t rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr(bar)), "r"(rank));
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(a) : "memory");
+}
 // a float at this block's shared-memory address `p` in block `rank` of the cluster
 __device__ __forceinline__ float cluster_load_f32(const float* p, uint32_t rank) {
   uint32_t a;

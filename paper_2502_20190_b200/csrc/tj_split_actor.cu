@@ -9,10 +9,11 @@
 // warps, one MMA-issuing warp, one copy warp; per step and tile:
 //   workers: layer 1 in the fixed FMA order of the FP32 path, ReLU, split -> FP16 A operand, 32 hidden units (one K chunk of
 //     the next layer) at a time, each chunk handed to the issuing lane through its own mbarrier;
-//   copy lane: streams W2's parts in 32-column chunks (bulk copies, four ring slots, the stream running on across steps);
-//   issuing lane: per K chunk, issues W_hi x (h_hi, h_lo) and W_lo x h_hi (M = 128, N = H) as soon as that chunk of h1 exists, so
-//     the tensor pipe works underneath layer 1;
-//   workers: accumulator -> + b2, ReLU, head sums in column order -> outputs;
+//   copy lane: streams W2's parts in 32-column chunks (bulk copies, four ring slots, the stream running on across steps), or, for a pair
+//     of blocks, brings its half of both parts once;
+//   issuing lane: per K chunk, issues W_hi x (h_hi, h_lo) and W_lo x h_hi (M = 128 or a pair's 256, N = H) as soon as that chunk of h1
+//     exists, so the tensor pipe works underneath layer 1;
+//   workers: accumulator -> + b2, ReLU, head sums -> outputs;
 //   then exactly the FP32 kernel's selection, env step, record / segment write and reset.
 // The FP32 work per step (layer 1 with its split, drain, env step: about 14,000 warp instructions a tile) and the MMAs (6,100 cycles at
 // hidden 256) are of one size; what a step takes beyond them is latency.
@@ -55,22 +56,27 @@ __device__ __forceinline__ void sa_observe(float4 s, float* obs) {
 // The actor.  A thread owns an environment for the whole call: observation, layer 1, head sums, selection and environment step stay
 // in its registers, so the workers meet nobody but the issuing lane.  TPR threads per environment:
 //   1  two groups of four warps, each on a tile of its own: while one tile's MMAs run, the other tile's threads drain, step and
-//      compute layer 1 (calls with more tiles than SMs);
-//   2  eight warps on one tile: each thread takes half the neurons and half the columns of the drain, the two exchange their head
+//      compute layer 1 (calls with more tiles than SMs).  Two blocks of a cluster share every product (cta_group::2, 256 rows): each holds half
+//      of W2's rows, which then stay in shared memory for the whole call instead of passing through it once per tile and step, and a product
+//      reads 64 of the 128 bytes per cycle instead of 96;
+//   2  eight warps on one tile: each thread takes half the rows of layer 1 and half the columns of the drain, the two exchange their head
 //      sums once per step and both step the environment (one tile per SM: the chain of one step is the bound).
-// With two tiles in flight shared memory is the bound: the MMAs read 96 of its 128 bytes per cycle while they run (40 % of the time) and
-// the broadcast weights and the A operand take another 53 %.  65,536 CartPole envs, hidden 256, 128 steps: 3.71 ms (one tile at a time
-// 5.16; two threads per env and two tiles, 18 warps: 4.19).
+// 65,536 CartPole envs, hidden 256, 128 steps: 3.69 ms with a block per tile whose threads computed layer 1 and the head each for its own
+// env, 2.80 with layer 1 and the drain as in S2Worker::forward, 2.53 as pairs.  A step of two tiles is then 18,000 cycles, 12,300 of them
+// MMAs: what bounds it is the chain layer 1 (5,500; a fence and an arrival per chunk) -> MMA of the last chunk (2,000 with its signals) ->
+// drain (4,000) -> environment (3,000) of four warps per tile.  More of them do not fit: eight warps per tile (one thread of two steps the
+// environment) spill at 96 registers, 2.73 ms.  The next columns fetched ahead in the drain: 2.62.  Arrivals of the second block through a
+// relaying warp: 4.26; with cluster-scope release semantics: 3.25.
 // Layer 1 hands 32 hidden units (one K chunk) at a time to the issuing lane through a ring of A-operand slots.
 constexpr int S2_NT = 320;                // eight worker warps on one tile, the issuing warp, the copy warp
-constexpr int S2_A_SLOTS = 8;             // A-operand slots of a block, 16 KB each: four per group, or eight for the one tile
+constexpr int S2_A_SLOTS = 8;             // most A-operand slots of a block, 16 KB each
 constexpr int S2_A_PART = SA_TE * SA_KC * 2;
 constexpr int S2_A_SLOT = 2 * S2_A_PART;  // high part, low part
 
 struct S2Ctl {
   uint64_t full[SA_SLOTS], empty[SA_SLOTS];
   uint64_t a_ready[S2_A_SLOTS], a_free[S2_A_SLOTS];
-  uint64_t acc_full[2], settled;
+  uint64_t acc_full[2], settled, w_ready;  // w_ready: a pair's halves of W2 are in shared memory
   uint32_t tmem_base, copies;             // copies: bulk copies queued so far
   int abort_flag, range_flag;
 };
@@ -93,6 +99,7 @@ __device__ __forceinline__ f32x2 pair2(float a, float b) {
 // of the A operand per row; returns the largest scaled activation.
 template <int D, int ROWS>
 __device__ __forceinline__ float s2_layer1(const f32x2 (&w)[D][4], const f32x2 (&b)[4], const f32x2 (&x)[ROWS][D], uint8_t* hi_dst, float vmax) {
+  const f32x2 minus1 = dup2(-1.f);
 #pragma unroll
   for (int r = 0; r < ROWS; ++r) {
     f32x2 acc[4] = {b[0], b[1], b[2], b[3]};
@@ -103,12 +110,14 @@ __device__ __forceinline__ float s2_layer1(const f32x2 (&w)[D][4], const f32x2 (
     uint32_t hi[4], lo[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
+      // the high part is the value cut to 11 bits, so the remainder has the value's sign and both conversions clamp: no maximum of its own
       const float2 a = halves(acc[i]);
-      const float v0 = fmaxf(a.x, 0.f), v1 = fmaxf(a.y, 0.f);
-      vmax = fmaxf(vmax, fmaxf(a.x, a.y));
-      const float h0 = __uint_as_float(__float_as_uint(v0) & 0xFFFFE000u), h1 = __uint_as_float(__float_as_uint(v1) & 0xFFFFE000u);
-      hi[i] = pack_f16x2(h0, h1);
-      lo[i] = pack_f16x2(v0 - h0, v1 - h1);
+      vmax = max3(vmax, a.x, a.y);
+      f32x2 rest = acc[i];
+      fma2(rest, pair2(__uint_as_float(__float_as_uint(a.x) & 0xFFFFE000u), __uint_as_float(__float_as_uint(a.y) & 0xFFFFE000u)), minus1);
+      const float2 d = halves(rest);
+      hi[i] = pack_f16x2_rz_relu(a.x, a.y);
+      lo[i] = pack_f16x2_relu(d.x, d.y);
     }
     *reinterpret_cast<uint4*>(hi_dst + r * ((SA_KC / 8) * 128)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
     *reinterpret_cast<uint4*>(hi_dst + S2_A_PART + r * ((SA_KC / 8) * 128)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
@@ -119,9 +128,15 @@ __device__ __forceinline__ float s2_layer1(const f32x2 (&w)[D][4], const f32x2 (
 // where everything lies in shared memory
 template <int D, int H, int TPR, int GROUPS>
 struct S2Smem {
+  static constexpr bool PAIR = GROUPS == 2;                   // two blocks share every product
   static constexpr uint32_t CHUNK_BYTES = H * SA_KC * 2;      // one chunk of one part of W2
+  static constexpr uint32_t W_CHUNK = PAIR ? CHUNK_BYTES / 2 : CHUNK_BYTES;      // what of it lies in this block
   static constexpr int NKC = H / SA_KC, NSTREAM = 2 * NKC;
-  static constexpr int AS = S2_A_SLOTS / GROUPS, NT = 128 * TPR * GROUPS + 64;   // A slots of a tile in flight; threads
+  static constexpr int W_SLOTS = PAIR ? NSTREAM : SA_SLOTS;
+  // A slots: one ring that the groups' passes go through in turn; threads.  A worker waits only for the chunks whose slots it takes over, so
+  // the one two rounds of the ring back must be known to be used up: the ring holds more than half of two passes' chunks
+  static constexpr int AS = PAIR && H > 192 ? 5 : S2_A_SLOTS, NT = 128 * TPR * GROUPS + 64;
+  static_assert(2 * AS > NKC || GROUPS == 1, "the phase of a slot's barrier is unambiguous");
   static constexpr uint32_t ACC_COLS = H <= 128 ? 128 : 256;
   uint8_t *a_ring, *w_ring;
   float *w1, *b1;         // [D][H] and [H], scaled
@@ -132,13 +147,13 @@ struct S2Smem {
   S2Ctl* ctl;
   __device__ __forceinline__ explicit S2Smem(uint8_t* base) {
     a_ring = base;
-    w_ring = a_ring + S2_A_SLOTS * S2_A_SLOT;
-    w1 = reinterpret_cast<float*>(w_ring + SA_SLOTS * CHUNK_BYTES);
+    w_ring = a_ring + AS * S2_A_SLOT;
+    w1 = reinterpret_cast<float*>(w_ring + W_SLOTS * W_CHUNK);
     b1 = w1 + D * H; hw = b1 + H; hw3 = hw + 4 * H; b3 = hw3 + H; part = b3 + 4;
     ctl = reinterpret_cast<S2Ctl*>(part + (TPR == 2 ? GROUPS * 2 * 2 * SA_TE * 4 : 0));
   }
   static size_t bytes() {
-    return (size_t)S2_A_SLOTS * S2_A_SLOT + (size_t)SA_SLOTS * CHUNK_BYTES +
+    return (size_t)AS * S2_A_SLOT + (size_t)W_SLOTS * W_CHUNK +
            ((size_t)(D + 6) * H + 4 + (TPR == 2 ? GROUPS * 2 * 2 * SA_TE * 4 : 0)) * sizeof(float) + sizeof(S2Ctl) + 64;
   }
 
@@ -146,34 +161,53 @@ struct S2Smem {
   __device__ __forceinline__ uint32_t set_up() const {
     if (threadIdx.x == 0) {
       for (int s = 0; s < SA_SLOTS; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
-      for (int s = 0; s < S2_A_SLOTS; ++s) { mbar_init(&ctl->a_ready[s], 4 * TPR); mbar_init(&ctl->a_free[s], 1); }
+      for (int s = 0; s < S2_A_SLOTS; ++s) { mbar_init(&ctl->a_ready[s], 4 * TPR * (PAIR ? 2 : 1)); mbar_init(&ctl->a_free[s], 1); }
       mbar_init(&ctl->acc_full[0], 1);
       mbar_init(&ctl->acc_full[1], 1);
       mbar_init(&ctl->settled, 1);
+      mbar_init(&ctl->w_ready, 2);
       ctl->copies = 0;
       ctl->abort_flag = ctl->range_flag = 0;
     }
     __syncthreads();
     if (threadIdx.x < 32) {
-      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&ctl->tmem_base)), "r"(GROUPS * ACC_COLS) : "memory");
-      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+      if (PAIR) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&ctl->tmem_base)), "r"(GROUPS * ACC_COLS) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+      } else {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&ctl->tmem_base)), "r"(GROUPS * ACC_COLS) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+      }
     }
     tc_fence_before();
-    __syncthreads();
+    if (PAIR) cluster_sync_all();                             // the other block's barriers are set up too
+    else __syncthreads();
     tc_fence_after();
     return ctl->tmem_base;
   }
   __device__ __forceinline__ void tear_down(uint32_t tmem) const {
     tc_fence_before();
     __syncthreads();
-    if (ctl->abort_flag) {                                    // the issuing warp is the last but one
-      tc_settle(&ctl->settled, (int)(threadIdx.x >> 5) == NT / 32 - 2, ctl->full, SA_SLOTS, ctl->copies);
+    const bool issuing_warp = (int)(threadIdx.x >> 5) == NT / 32 - 2;     // the last but one
+    if (PAIR) {
+      // neither block leaves before the products that read both blocks' operands are over and the last arrival has reached the first one
+      if (ctl->abort_flag) {
+        if (issuing_warp && cluster_rank() == 0) {
+          umma_commit_pair(&ctl->settled, elect_one());
+          mbar_settle(&ctl->settled, 0);
+        }
+        if (threadIdx.x == 0 && ctl->copies) mbar_settle(&ctl->full[0], 0);
+      }
+      cluster_sync_all();
+    } else if (ctl->abort_flag) {
+      tc_settle(&ctl->settled, issuing_warp, ctl->full, SA_SLOTS, ctl->copies);
       __syncthreads();
     }
     if (threadIdx.x < 32) {
       __syncwarp();
       tc_fence_after();
-      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(GROUPS * ACC_COLS) : "memory");
+      if (PAIR) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(GROUPS * ACC_COLS) : "memory");
+      else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(GROUPS * ACC_COLS) : "memory");
     }
   }
   // the parameters around the hidden matrix, from the packed FP32 layout P describes
@@ -197,6 +231,49 @@ struct S2Smem {
       b3[a] = a < Aout ? __ldg(W + p.off_b3 + a) : 0.f;
     }
   }
+  // Issuing warp of a pair's first block: the products of n_pass passes over each of `tiles` tiles of 256 rows, the groups' passes in turn
+  __device__ __forceinline__ void issue_pair(uint32_t tmem, int tiles, int n_pass) const {
+    volatile int* abort_flag = &ctl->abort_flag;
+    const uint32_t leader = elect_one();
+    const uint32_t idesc = make_idesc_f16_m256(H);
+    const uint32_t a0 = desc_lo(smem_addr(a_ring), 128u), w0 = desc_lo(smem_addr(w_ring), 128u);
+    const uint32_t hiword = desc_hi((uint32_t)(SA_KC / 8) * 128u);            // A slots and W2 chunks: 32 columns wide
+    uint32_t as = 0, round = 0;                               // slot of the ring, rounds of it
+    bool alive = tc_wait_warp(&ctl->w_ready, 0, abort_flag);
+    for (int r = 0; r * GROUPS < tiles && alive; ++r)
+      for (int i = 0; i < n_pass && alive; ++i)
+#pragma unroll
+        for (int g = 0; g < GROUPS; ++g) {
+          if (!alive || r * GROUPS + g >= tiles) break;
+          const uint32_t acc = tmem + (uint32_t)g * ACC_COLS;
+#pragma unroll 1
+          for (int kc = 0; kc < NKC; ++kc) {
+            if (!tc_wait_warp(&ctl->a_ready[as], round & 1, abort_flag)) { alive = false; break; }
+            tc_fence_after();
+            const uint32_t a_hi = a0 + as * (S2_A_SLOT / 16), a_lo = a_hi + S2_A_PART / 16, b = w0 + 2 * kc * (W_CHUNK / 16);
+#pragma unroll
+            for (int j = 0; j < SA_KC / 16; ++j) {
+              umma_ss_pair(acc, a_hi + 16u * j, hiword, b + 16u * j, hiword, idesc, (kc | j) != 0, leader);
+              umma_ss_pair(acc, a_lo + 16u * j, hiword, b + 16u * j, hiword, idesc, 1u, leader);
+            }
+#pragma unroll
+            for (int j = 0; j < SA_KC / 16; ++j)
+              umma_ss_pair(acc, a_hi + 16u * j, hiword, b + W_CHUNK / 16 + 16u * j, hiword, idesc, 1u, leader);
+            umma_commit_both(&ctl->a_free[as], leader);
+            if (++as == AS) { as = 0; ++round; }
+          }
+          if (alive) umma_commit_both(&ctl->acc_full[g], leader);
+        }
+  }
+  // Copy lane of a block of a pair: its half of W2's rows, both parts, once
+  __device__ __forceinline__ void copy_half(const uint16_t* parts) const {
+    mbar_expect_tx(&ctl->full[0], NSTREAM * W_CHUNK);
+    for (uint32_t c = 0; c < NSTREAM; ++c)
+      bulk_copy_g2s(w_ring + c * W_CHUNK, reinterpret_cast<const uint8_t*>(parts) + (size_t)c * CHUNK_BYTES + cluster_rank() * W_CHUNK, W_CHUNK,
+                    &ctl->full[0]);
+    ctl->copies = NSTREAM;
+    if (tc_wait(&ctl->full[0], 0, &ctl->abort_flag)) mbar_arrive_cluster(&ctl->w_ready, 0);
+  }
   // Issuing warp: the MMAs of n_pass passes over each of `tiles` tiles, the groups' passes in turn
   __device__ __forceinline__ void issue(uint32_t tmem, int tiles, int n_pass) const {
     volatile int* abort_flag = &ctl->abort_flag;
@@ -204,7 +281,7 @@ struct S2Smem {
     const uint32_t idesc = make_idesc_f16(H);
     const uint32_t a0 = desc_lo(smem_addr(a_ring), 128u), w0 = desc_lo(smem_addr(w_ring), 128u);
     const uint32_t hiword = desc_hi((uint32_t)(SA_KC / 8) * 128u);            // A slots and W2 chunks: 32 columns wide
-    uint32_t wc = 0, ac[2] = {0, 0};
+    uint32_t wc = 0, ac = 0;
     bool alive = true;
     for (int r = 0; r * GROUPS < tiles && alive; ++r)
       for (int i = 0; i < n_pass && alive; ++i)
@@ -213,9 +290,9 @@ struct S2Smem {
           if (!alive || r * GROUPS + g >= tiles) break;
           const uint32_t acc = tmem + (uint32_t)g * ACC_COLS;
 #pragma unroll 1
-          for (int kc = 0; kc < NKC; ++kc, ++ac[g]) {
-            const uint32_t as = (uint32_t)g * AS + ac[g] % AS;
-            if (!tc_wait_warp(&ctl->a_ready[as], (ac[g] / AS) & 1, abort_flag)) { alive = false; break; }
+          for (int kc = 0; kc < NKC; ++kc, ++ac) {
+            const uint32_t as = ac % AS;
+            if (!tc_wait_warp(&ctl->a_ready[as], (ac / AS) & 1, abort_flag)) { alive = false; break; }
             tc_fence_after();
             const uint32_t a_hi = a0 + as * (S2_A_SLOT / 16), a_lo = a_hi + S2_A_PART / 16;
 #pragma unroll
@@ -259,7 +336,7 @@ struct S2Worker {
   using M = S2Smem<D, H, TPR, GROUPS>;
   const M& m;
   int g, half, row;                                           // tile in flight, half of the columns, row of the tile = TMEM lane
-  uint32_t t_row, ac = 0, pass = 0;
+  uint32_t t_row, pass = 0;
   float inv_scale, vmax = 0.f;                                // 1 / (activation scale x weight scale); largest scaled activation
   bool ok = true;
   __device__ __forceinline__ S2Worker(const M& mm, uint32_t tmem, float inv) : m(mm) {
@@ -275,7 +352,8 @@ struct S2Worker {
   // 320 16-byte words a thread and pass, and the drain 256, two thirds of the cycles of the read path.  So
   //   layer 1: a lane takes eight hidden units of four (TPR 2: two) rows of its warp, eight apart, whose observations come by shuffle;
   //   drain: fragments of 8 columns x 16 rows (a lane holds two neighbouring columns of four rows), so a weight read serves four rows.
-  __device__ __forceinline__ void forward(const float (&obs)[6], int Aout, float (&out)[4]) {
+  // `chunk`: number of this pass's first chunk in the ring's order.
+  __device__ __forceinline__ void forward(const float (&obs)[6], int Aout, uint32_t chunk, float (&out)[4]) {
     constexpr int ROWS = 4 / TPR;
     volatile int* abort_flag = &m.ctl->abort_flag;
     const int lane = threadIdx.x & 31, first = (row & ~31) + (TPR == 2 ? half * 16 : 0);   // first row of this warp's share
@@ -288,8 +366,8 @@ struct S2Worker {
     const float *w1 = m.w1 + (lane >> 3) * 8, *b1 = m.b1 + (lane >> 3) * 8;
     uint8_t* dst = m.a_ring + (first >> 3) * ((SA_KC / 8) * 128) + (lane & 7) * 16 + (lane >> 3) * 128;
 #pragma unroll 1
-    for (int kc = 0; kc < M::NKC; ++kc, ++ac) {
-      const uint32_t as = (uint32_t)g * M::AS + ac % M::AS;
+    for (int kc = 0; kc < M::NKC; ++kc, ++chunk) {
+      const uint32_t as = chunk % M::AS;
       f32x2 w[D][4], b[4];
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
@@ -301,10 +379,15 @@ struct S2Worker {
           w[k][2 * i] = ww.x; w[k][2 * i + 1] = ww.y;
         }
       }
-      if (ac >= M::AS) ok = ok && tc_wait_elect(&m.ctl->a_free[as], ((ac / M::AS) - 1) & 1, abort_flag);
+      if (chunk >= M::AS) ok = ok && tc_wait_elect(&m.ctl->a_free[as], ((chunk / M::AS) - 1) & 1, abort_flag);
       vmax = s2_layer1<D, ROWS>(w, b, x, dst + as * S2_A_SLOT, vmax);
       fence_async_smem();
-      mbar_arrive_warp(&m.ctl->a_ready[as]);
+      if (M::PAIR) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(&m.ctl->a_ready[as], 0);
+      } else {
+        mbar_arrive_warp(&m.ctl->a_ready[as]);
+      }
     }
     ok = ok && tc_wait_elect(&m.ctl->acc_full[g], pass & 1, abort_flag);
     tc_fence_after();
@@ -377,20 +460,30 @@ __global__ void __launch_bounds__(128 * TPR * GROUPS + 64, 1) actor_split_tc_ker
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   constexpr int D = ENV == TJ_ENV_CARTPOLE ? 4 : 6;
   constexpr int WW = 4 * TPR * GROUPS;                        // worker warps, then the issuing warp and the copy warp
-  const S2Smem<D, H, TPR, GROUPS> m(smem_raw);
+  using M = S2Smem<D, H, TPR, GROUPS>;
+  const M m(smem_raw);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int n_tiles = (p.N + SA_TE - 1) / SA_TE;
+  // a pair of blocks walks tiles of 256 envs, each block its 128 of them
+  constexpr int BLOCKS = GROUPS == 2 ? 2 : 1;
+  const int n_tiles = (p.N + SA_TE * BLOCKS - 1) / (SA_TE * BLOCKS), walker = (int)blockIdx.x / BLOCKS, walkers = (int)gridDim.x / BLOCKS;
   const bool on_policy = p.C == 0;
   const uint32_t tmem = m.set_up();
   chain_begin();
   m.stage(p, p.W, p.Aout);
-  const int my_tiles = ((int)blockIdx.x < n_tiles) ? (n_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+  const int my_tiles = walker < n_tiles ? (n_tiles - 1 - walker) / walkers + 1 : 0;
   __syncthreads();
   if (warp == WW + 1) {
-    if (lane == 0) m.copy(w2parts, (uint32_t)my_tiles * (uint32_t)pl.n_pass);
+    if (lane == 0) {
+      if constexpr (GROUPS == 2) m.copy_half(w2parts);
+      else m.copy(w2parts, (uint32_t)my_tiles * (uint32_t)pl.n_pass);
+    }
     __syncwarp();
   } else if (warp == WW) {
-    m.issue(tmem, my_tiles, pl.n_pass);
+    if constexpr (GROUPS == 2) {
+      if (cluster_rank() == 0) m.issue_pair(tmem, my_tiles, pl.n_pass);
+    } else {
+      m.issue(tmem, my_tiles, pl.n_pass);
+    }
   } else {
     S2Worker<D, H, TPR, GROUPS> wk(m, tmem, __ldg(w2scale + 1));
     const int g = wk.g, half = wk.half, row = wk.row;
@@ -399,8 +492,11 @@ __global__ void __launch_bounds__(128 * TPR * GROUPS + 64, 1) actor_split_tc_ker
     const bool first = half == 0;                             // of an environment's threads the one that writes what is written once
 #pragma unroll 1
     for (int tl = g; tl < my_tiles; tl += GROUPS) {
-      const int e = ((int)blockIdx.x + tl * (int)gridDim.x) * SA_TE + row;
+      const int e = ((walker + tl * walkers) * BLOCKS + (int)blockIdx.x % BLOCKS) * SA_TE + row;
       const bool owner = e < p.N;
+      // the passes of the tiles in flight alternate: this tile's first chunk, and from one of its passes to the next
+      uint32_t chunk = (uint32_t)((tl - g) * pl.n_pass + g) * M::NKC;
+      const uint32_t next_pass = (uint32_t)min(GROUPS, my_tiles - (tl - g)) * M::NKC;
       float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
       int ep = 0;
       float ep_ret = 0.f;
@@ -418,7 +514,8 @@ __global__ void __launch_bounds__(128 * TPR * GROUPS + 64, 1) actor_split_tc_ker
         const unsigned long long t = (unsigned long long)p.t0 + step;
         float out[4];
         const uint4 w = stream_words(p.seed, STREAM_ACTION, 0, (uint32_t)e, t);
-        wk.forward(obs, p.Aout, out);
+        wk.forward(obs, p.Aout, chunk, out);
+        chunk += next_pass;
         auto logit = [&](int i) { return i == 0 ? out[0] : (i == 1 ? out[1] : (i == 2 ? out[2] : out[3])); };
         if (p.dbg_logits && owner && first) {
           float* dl = p.dbg_logits + ((size_t)step * p.N + e) * p.A;
@@ -480,7 +577,8 @@ __global__ void __launch_bounds__(128 * TPR * GROUPS + 64, 1) actor_split_tc_ker
         }
         if (on_policy) {
           if (++pos == p.T) {                                 // bootstrap value of the state each env is now in
-            wk.forward(obs, p.Aout, out);
+            wk.forward(obs, p.Aout, chunk, out);
+            chunk += next_pass;
             if (owner && first) p.seg_val[((size_t)seg * (p.T + 1) + p.T) * p.N + e] = logit(p.A);
             pos = 0;
             seg = seg + 1 == p.G ? 0 : seg + 1;
@@ -558,7 +656,7 @@ __global__ void __launch_bounds__(S2_NT, 1) td_split_tc_kernel(const TdParams p,
         done = p.done[j];
       }
     }
-    wk.forward(obs, p.A, out);
+    wk.forward(obs, p.A, 0u, out);
     if (!(wk.vmax <= 65504.f)) m.ctl->range_flag = 1;
     if (row_thread && net == 1) {
       float q = out[0];
@@ -591,12 +689,32 @@ __global__ void __launch_bounds__(S2_NT, 1) td_split_tc_kernel(const TdParams p,
   }
 }
 
+// launch_chained for a kernel of block pairs
+template <typename... P, typename... A>
+cudaError_t launch_pairs(void (*kernel)(P...), int grid, int threads, size_t smem, cudaStream_t s, A&&... args) {
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+
 template <int ENV, int H>
 cudaError_t launch_split(const ActorParams& p, const S2Plan& pl, const uint16_t* w2parts, const float* w2scale, int grid, int groups, cudaStream_t s) {
   constexpr int D = ENV == TJ_ENV_CARTPOLE ? 4 : 6;
-#define TJ_SPLIT(T, G) launch_chained(actor_split_tc_kernel<ENV, H, T, G>, grid, S2Smem<D, H, T, G>::NT, S2Smem<D, H, T, G>::bytes(), s, p, pl, w2parts, w2scale)
-  return groups == 1 ? TJ_SPLIT(2, 1) : TJ_SPLIT(1, 2);
-#undef TJ_SPLIT
+  if (groups == 1)
+    return launch_chained(actor_split_tc_kernel<ENV, H, 2, 1>, grid, S2Smem<D, H, 2, 1>::NT, S2Smem<D, H, 2, 1>::bytes(), s, p, pl, w2parts, w2scale);
+  return launch_pairs(actor_split_tc_kernel<ENV, H, 1, 2>, grid, S2Smem<D, H, 1, 2>::NT, S2Smem<D, H, 1, 2>::bytes(), s, p, pl, w2parts, w2scale);
 }
 
 template <int ENV>
@@ -626,7 +744,8 @@ cudaError_t launch_actor_split(int env_kind, const ActorParams& p, const uint16_
   if (p.N <= 0) return cudaSuccess;
   if (!split_actor_supported(env_kind, p.D, p.H, p.Aout)) return cudaErrorInvalidConfiguration;
   const int n_tiles = (p.N + SA_TE - 1) / SA_TE;
-  const int grid = n_tiles < sm_count ? n_tiles : sm_count;
+  const int groups = n_tiles > sm_count && sm_count > 1 ? 2 : 1;    // more tiles than SMs: pairs of blocks with two tiles each in flight
+  const int grid = groups == 2 ? sm_count & ~1 : (n_tiles < sm_count ? n_tiles : sm_count);
   S2Plan pl{};
   pl.n_pass = p.n_steps;
   if (p.C > 0) {
@@ -638,7 +757,6 @@ cudaError_t launch_actor_split(int env_kind, const ActorParams& p, const uint16_
     pl.seg0 = (int)((p.t0 / p.T) % p.G);
     pl.n_pass += (pl.pos0 + p.n_steps) / p.T;
   }
-  const int groups = n_tiles > sm_count ? 2 : 1;             // a second tile per SM runs in the first one's gaps
   return env_kind == TJ_ENV_CARTPOLE ? launch_split_env<TJ_ENV_CARTPOLE>(p, pl, w2parts, w2scale, grid, groups, s)
                                      : launch_split_env<TJ_ENV_ACROBOT>(p, pl, w2parts, w2scale, grid, groups, s);
 }
@@ -647,22 +765,7 @@ int td_split_grid(int n) { return (n + SA_TE - 1) / SA_TE; }
 
 template <int D, int H>
 static cudaError_t launch_td_split_dh(const TdParams& p, const uint16_t* po, const float* so, const uint16_t* pt, const float* st, cudaStream_t s) {
-  const size_t smem = S2Smem<D, H, 2, 1>::bytes();
-  const cudaError_t e = cudaFuncSetAttribute(td_split_tc_kernel<D, H>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg{};
-  cudaLaunchAttribute at[2];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.gridDim = dim3(2 * td_split_grid(p.n));
-  cfg.blockDim = dim3(S2_NT);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cfg.attrs = at;
-  cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, td_split_tc_kernel<D, H>, p, po, so, pt, st);
+  return launch_pairs(td_split_tc_kernel<D, H>, 2 * td_split_grid(p.n), S2_NT, S2Smem<D, H, 2, 1>::bytes(), s, p, po, so, pt, st);
 }
 
 template <int D>
