@@ -58,9 +58,8 @@ __device__ __forceinline__ void load_matrix(float* sm, const float* blob, const 
 struct FsLayout {
   int ldD, ldH, Hp;
   int W2, W3, b2, b3, T2, T3, tb2, tb3, xs, xn, h1, h2, d1, d2, g, q, part, one, red, bar, total;
-  int G, T, KS;                                    // neuron quads; 4 x 4 output tiles of a hidden layer; shares of a contraction
+  int G, T, KS, KB;                                // neuron quads; 4 x 4 output tiles of a hidden layer; shares of a contraction, of the backward one
   int bulk;                                        // rows of the parameter blobs are whole 16-byte words
-  unsigned tx;                                     // bytes of one network's bulk copies
 };
 
 inline FsLayout fs_layout(int D, int H, int R, bool ppo) {
@@ -82,22 +81,26 @@ inline FsLayout fs_layout(int D, int H, int R, bool ppo) {
   L.g = take(R * 4); L.q = take(2 * R * 4); L.part = take(5 * R); L.one = take(4);
   L.G = L.Hp / 4;
   L.T = L.G * (R / 4);
-  L.KS = FS_NT / L.T;
+  const int nets = ppo ? 1 : 2;                    // the hidden layers of both networks run side by side
+  L.KS = FS_NT / (nets * L.T);
+  L.KB = FS_NT / L.T;
   L.KS = L.KS < 1 ? 1 : (L.KS > 4 ? 4 : L.KS);   // a whole update, us, with up to 2 / 4 / 8 / 16 shares:
                                                    // hidden 64, 256 rows 13.1 / 12.3 / 12.2 / 12.5, 1,024 rows 13.8 / 12.8 / 12.9 / 13.6;
                                                    // hidden 128, 256 rows 16.8 / 14.6 / 14.4 / 14.8
+  L.KB = L.KB < 1 ? 1 : (L.KB > 4 ? 4 : L.KB);
   if (L.KS > L.G) L.KS = L.G;
-  if (o + L.KS * L.T * 16 + 8 > 227 * 256) L.KS = 1;
-  L.red = L.KS > 1 ? take(L.KS * L.T * 16) : 0;    // only where a layer's contraction is split
+  if (L.KB > L.G) L.KB = L.G;
+  auto red = [&] { const int f = L.KS > 1 ? L.KS * nets * L.T * 16 : 0, b = L.KB > 1 ? L.KB * L.T * 16 : 0; return f > b ? f : b; };
+  if (o + red() + 8 > 227 * 256) L.KS = L.KB = 1;
+  L.red = take(red());                             // only where a layer's contraction is split
   L.bar = take(8);
   L.bulk = 0;
-  L.tx = 0;
   L.total = o;
   return L;
 }
 
 // this thread's part in a layer's product, the same for all hidden layers: output tile (row group rg, neuron group g), share
-struct FsTile { int T, KS, tile, share, rg, g; bool active; };
+struct FsTile { int T, KS, tile, share, rg, g; bool active; };   // T, tile: over all networks of the product
 
 // the partial sums of a split contraction: 4 x 4 values per tile and share; slot j of a tile is finished by share j mod KS
 template <typename F>
@@ -304,33 +307,40 @@ __global__ void __launch_bounds__(FS_NT, 1) sgd_fused_kernel(const SgdParams p, 
   extern __shared__ __align__(128) float fs_sm[];
   const int D = p.D, H = p.H, A = p.A, tid = threadIdx.x, G = L.G, Dq = (D + 3) / 4, Dp = 4 * Dq;
   float* sm = fs_sm;
-  uint64_t* bar = reinterpret_cast<uint64_t*>(sm + L.bar);   // [0]: small parameters; [1], [2]: the target's, the online W2
-  FsTile t;
-  t.T = L.T; t.KS = L.KS;
-  t.share = tid / L.T; t.tile = tid - t.share * L.T; t.g = t.tile / (R / 4); t.rg = t.tile % (R / 4);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(sm + L.bar);   // the parameters are here
+  FsTile t, tb;                                    // of the forward layers and of the backward one
+  t.T = (PPO ? 1 : 2) * L.T; t.KS = L.KS;
+  t.share = tid / t.T; t.tile = tid - t.share * t.T;
   t.active = t.share < L.KS;
-  if (L.bulk && tid < 3) mbar_init(bar + tid, 1);
+  const bool target = !PPO && t.tile >= L.T;               // this thread's network in the forward layers
+  t.g = (t.tile - (target ? L.T : 0)) / (R / 4); t.rg = t.tile % (R / 4);
+  tb.T = L.T; tb.KS = L.KB;
+  tb.share = tid / L.T; tb.tile = tid - tb.share * L.T; tb.g = tb.tile / (R / 4); tb.rg = tb.tile % (R / 4);
+  tb.active = tb.share < L.KB;
+  if (L.bulk && tid == 0) mbar_init(bar, FS_NT);
   __syncthreads();
   chain_begin();
   const int o_b1 = H * D, o_W2 = o_b1 + H, o_b2 = o_W2 + H * H, o_W3 = o_b2 + H, o_b3 = o_W3 + A * H;
   // every load of the prologue is in flight before the first result is used: a load that waits for another costs a round trip
   // to L2 (0.45 us), and four of them in a row were a third of the kernel
   if (L.bulk) {
-    // parameters by one bulk copy per row, issued by one thread per row (cp.async by all threads, with its index arithmetic per
-    // matrix, took 5 us at hidden 64)
-    if (tid == 0) {
-      mbar_expect_tx(bar, PPO ? L.tx : 2 * L.tx);
-      if (!PPO) mbar_expect_tx(bar + 1, (unsigned)(4 * H * H));
-      mbar_expect_tx(bar + 2, (unsigned)(4 * H * H));
-    }
-    __syncthreads();                               // the barriers expect the bytes before the first copy can arrive
+    // a thread copies one 16-byte column of every RP-th row of the hidden matrices, the first rows' threads the head and the biases too.
+    // (One bulk copy per row, issued by a thread per row, took 32 cycles each, one after the other: 4,400 cycles for two networks at
+    // hidden 64, a quarter of the kernel.)
+    const int RP = FS_NT / G, r0 = tid / G, c = 4 * (tid - r0 * G);
+    if (r0 < RP) {
 #pragma unroll 1
-    for (int net = PPO ? 0 : 1; net >= 0; --net) {
-      const float* blob = net ? p.theta_target : p.theta;
-      if (tid < H) bulk_copy_g2s(sm + (net ? L.T2 : L.W2) + tid * L.ldH, blob + o_W2 + tid * H, (unsigned)(4 * H), bar + 2 - net);
-      else if (tid >= 128 && tid < 128 + A) bulk_copy_g2s(sm + (net ? L.T3 : L.W3) + (tid - 128) * L.ldH, blob + o_W3 + (tid - 128) * H, (unsigned)(4 * H), bar);
-      else if (tid == 160) bulk_copy_g2s(sm + (net ? L.tb2 : L.b2), blob + o_b2, (unsigned)(4 * H), bar);
+      for (int net = PPO ? 0 : 1; net >= 0; --net) {
+        const float* blob = net ? p.theta_target : p.theta;
+        if (r0 < A) cp_async16(sm + (net ? L.T3 : L.W3) + r0 * L.ldH + c, blob + o_W3 + r0 * H + c);
+        else if (r0 == 4) cp_async16(sm + (net ? L.tb2 : L.b2) + c, blob + o_b2 + c);
+        const float* src = blob + o_W2 + r0 * H + c;
+        float* dst = sm + (net ? L.T2 : L.W2) + r0 * L.ldH + c;
+#pragma unroll 4
+        for (int r = r0; r < H; r += RP, src += RP * H, dst += RP * L.ldH) cp_async16(dst, src);
+      }
     }
+    cp_async_arrive(bar);
   } else {
 #pragma unroll 1
     for (int net = PPO ? 0 : 1; net >= 0; --net) {
@@ -425,12 +435,9 @@ __global__ void __launch_bounds__(FS_NT, 1) sgd_fused_kernel(const SgdParams p, 
     }
     __syncthreads();
     if (L.bulk) ok = ok && mbar_wait_bounded(bar, 0);
-    if (!PPO) {
-      if (L.bulk) ok = ok && mbar_wait_bounded(bar + 1, 0);
-      dense_rows<R>(sm + L.T2, L.ldH, sm + L.tb2, sm + L.d1, L.ldH, sm + L.d2, L.ldH, G, G, t, sm + L.red);
-    }
-    if (L.bulk) ok = ok && mbar_wait_bounded(bar + 2, 0);
-    dense_rows<R>(sm + L.W2, L.ldH, sm + L.b2, sm + L.h1, L.ldH, sm + L.h2, L.ldH, G, G, t, sm + L.red);
+    // both networks side by side: the target's activations lie in d1, d2
+    dense_rows<R>(sm + (target ? L.T2 : L.W2), L.ldH, sm + (target ? L.tb2 : L.b2), sm + (target ? L.d1 : L.h1), L.ldH, sm + (target ? L.d2 : L.h2),
+                  L.ldH, G, G, t, sm + L.red);
     // heads: eight lanes per (network, row)
     for (int slot = tid >> 3; slot < (PPO ? R : 2 * R); slot += FS_NT / 8) {
       const int net = PPO ? 0 : slot / R, r = PPO ? slot : slot % R, s = tid & 7;
@@ -543,7 +550,7 @@ __global__ void __launch_bounds__(FS_NT, 1) sgd_fused_kernel(const SgdParams p, 
       else if (PPO && a == A) out.one(off + A + H, s);
     }
     __syncthreads();
-    dense_back<R>(sm + L.W2, L.ldH, sm + L.d2, sm + L.h1, sm + L.d1, L.ldH, G, t, sm + L.red);
+    dense_back<R>(sm + L.W2, L.ldH, sm + L.d2, sm + L.h1, sm + L.d1, L.ldH, G, tb, sm + L.red);
     if (G * G <= FS_NT) grad_hidden<R, 1>(sm + L.d2, sm + L.h1, L.ldH, H, G, H * D + H, out);
     else grad_hidden<R, 2>(sm + L.d2, sm + L.h1, L.ldH, H, G, H * D + H, out);
     if (chunk + (int)gridDim.x < n_chunks) fetch_rows(chunk + gridDim.x);
@@ -557,11 +564,7 @@ __global__ void __launch_bounds__(FS_NT, 1) sgd_fused_kernel(const SgdParams p, 
   }
   if (!ok) {
     update_failed(p.watch);
-    if (tid == 0) {                                // thread 0 waits for every copy: if it was served, all have arrived
-      mbar_settle(bar, 0);
-      if (!PPO) mbar_settle(bar + 1, 0);
-      mbar_settle(bar + 2, 0);
-    }
+    if (L.bulk) mbar_settle(bar, 0);
   }
 }
 
@@ -641,7 +644,6 @@ cudaError_t launch_fused(const SgdParams& p, int stride, int grid, cudaStream_t 
   FsLayout L = fs_layout(p.D, p.H, R, PPO);
   // H a multiple of four makes every row and the start of W2, W3 and the hidden biases whole 16-byte words of the blob
   L.bulk = p.H % 4 == 0 && ((reinterpret_cast<uintptr_t>(p.theta) | reinterpret_cast<uintptr_t>(p.theta_target)) & 15) == 0;
-  L.tx = (unsigned)(4 * p.H * (p.A + 1));
   return launch_chained(sgd_fused_kernel<R, PPO>, grid, FS_NT, (size_t)L.total * sizeof(float), s, p, L, stride);
 }
 
