@@ -27,6 +27,8 @@
 // MMA of the z product (64 on the tensor pipe) fetching instructions from L2.  So loops are unrolled only as far as their latency asks.
 // Every wait is bounded: on a timeout the block raises an abort flag, records an error, waits for its copies and matrix instructions in
 // flight, frees its TMEM and leaves.
+#include <cstddef>
+
 #include <cuda_fp16.h>
 
 #include "tj_internal.h"
@@ -64,11 +66,30 @@ struct PaSmem {
   uint64_t z_stored;       // network -> env: z of the tile is in the scratch tile
   uint64_t act_ready;      // env: the rows' actions are in shared memory
   uint64_t settled;        // after a timeout: the matrix instructions are over
-  int act[2][PA_M];        // by tile parity
+  alignas(16) float bias[PA_NET_WARPS][32];   // per network warp: the biases of the columns it drains next
+  uint8_t act[2][PA_M];    // by tile parity
   uint32_t tmem_base, copies;   // copies: bulk copies queued so far
   int abort_flag;
 };
 
+static_assert(offsetof(PaSmem, bias) % 16 == 0 && sizeof(PaSmem) <= 227 * 1024 - PA_X_BYTES - PA_U_BYTES - PA_STAGES * PA_STAGE_BYTES - 64, "layout");
+
+// loads that stay where they are written: the compiler moves ordinary ones down to their uses
+__device__ __forceinline__ float4 load_f4_cg(const float* p) {
+  float4 v;
+  asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float4 load_f4_nc(const float* p) {
+  float4 v;
+  asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float load_f1(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+  return v;
+}
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const TcMlpParams p) {
@@ -247,9 +268,21 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
     const int r = q * 32 + lane;                  // row of the tile = TMEM lane
     const uint32_t t_lane = tmem + ((uint32_t)(q * 32) << 16);
     uint32_t tiles = 0, nfull0 = 0, nfull1 = 0;
+    // Biases go through a shared-memory row of this warp, loaded one use ahead: 28 KB of L1 hold little beside 227 KB of shared memory, so
+    // eight loads between accumulator and operand cost an L2 round trip in every drain
+    float* bias_row = ctl->bias[warp - 4];
+    int b = rot;                                  // neuron block of the next use that has one
+    float bias_next = __ldg(p.b1 + b * PA_NB + hsel * 32 + lane);
     for (; tiles < (uint32_t)n_work; ++tiles) {
       for (int u = 0; u <= 2 * n_hb; ++u) {
         const int buf = u & 1;
+        const int layer = u < n_hb ? 0 : 1, c0 = b * PA_NB + hsel * 32;   // first of this thread's 32 columns
+        if (u != n_hb) {
+          __syncwarp();
+          bias_row[lane] = bias_next;
+          b = b + 1 == n_hb ? 0 : b + 1;
+          bias_next = __ldg((u + 1 < n_hb || u == 2 * n_hb ? p.b1 : p.b2) + b * PA_NB + hsel * 32 + lane);
+        }
         if (!tc_wait_elect(buf ? &ctl->acc_full[1] : &ctl->acc_full[0], (buf ? nfull1++ : nfull0++) & 1, abort_flag)) goto done;
         tc_fence_after();
         const uint32_t t_acc = t_lane + (buf ? PA_COL_ACC1 : PA_COL_ACC0) + (uint32_t)(hsel * 32);
@@ -269,17 +302,13 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
           mbar_arrive_warp(&ctl->z_stored);
           continue;
         }
-        const int layer = u < n_hb ? 0 : 1;
-        const int b = ((layer == 0 ? u : u - n_hb - 1) + rot) % n_hb;   // neuron block of this use
-        const float* bias = layer == 0 ? p.b1 : p.b2;
-        const int c0 = b * PA_NB + hsel * 32;          // first of this thread's 32 columns
         uint32_t v[32], o[16];
         tmem_ld16(t_acc, v);
         tmem_ld16(t_acc + 16u, v + 16);
         tmem_ld_wait();
 #pragma unroll
         for (int j4 = 0; j4 < 8; ++j4) {
-          const float4 bb = __ldg(reinterpret_cast<const float4*>(bias + c0 + 4 * j4));
+          const float4 bb = *reinterpret_cast<const float4*>(bias_row + 4 * j4);
           o[2 * j4] = pack_bf16x2_relu(__uint_as_float(v[4 * j4]) + bb.x, __uint_as_float(v[4 * j4 + 1]) + bb.y);
           o[2 * j4 + 1] = pack_bf16x2_relu(__uint_as_float(v[4 * j4 + 2]) + bb.z, __uint_as_float(v[4 * j4 + 3]) + bb.w);
         }
@@ -303,23 +332,33 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
     const int ew = warp - PA_ENV0;                 // 0..7; the first four also read the head outputs (one TMEM quarter each)
     const int e_r4 = lane >> 3, e_kq = lane & 7;   // four rows x eight 16-byte pieces per warp instruction, four pieces per lane and row
     uint32_t tiles = 0;
+    // this lane's pieces of a tile's row groups g and g + 1, all in flight at once
+    auto load_rows = [&](int tile, int g, float4 (&v)[2][4]) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const long long row = (long long)tile * PA_M + ew * 16 + (g + h) * 4 + e_r4;
+        const float* xr = p.x + (size_t)(row < p.n ? row : 0) * D;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          v[h][i] = row < p.n ? __ldcg(reinterpret_cast<const float4*>(xr + (e_kq + 8 * i) * 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    };
     // BF16 rows of a tile -> X (layer-1 A operand)
     auto convert_x = [&](int tile) {
 #pragma unroll 1
-      for (int g = 0; g < 4; ++g) {
-        const int rr = ew * 16 + g * 4 + e_r4;
-        const long long row = (long long)tile * PA_M + rr;
-        const float* xr = p.x + (size_t)(row < p.n ? row : 0) * D;
-        float4 v[4];
+      for (int g = 0; g < 4; g += 2) {
+        float4 v[2][4];
+        load_rows(tile, g, v);
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-          v[i] = row < p.n ? __ldcg(reinterpret_cast<const float4*>(xr + (e_kq + 8 * i) * 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
-        uint8_t* dx = xbuf + ((size_t)(rr >> 3) * (D / 8)) * 128 + (rr & 7) * 16;
+        for (int h = 0; h < 2; ++h) {
+          const int rr = ew * 16 + (g + h) * 4 + e_r4;
+          uint8_t* dx = xbuf + ((size_t)(rr >> 3) * (D / 8)) * 128 + (rr & 7) * 16;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int k4 = e_kq + 8 * i;
-          *reinterpret_cast<uint2*>(dx + (size_t)(k4 >> 1) * 128 + (k4 & 1) * 8) =
-              make_uint2(pack_bf16x2(v[i].x, v[i].y), pack_bf16x2(v[i].z, v[i].w));
+          for (int i = 0; i < 4; ++i) {
+            const int k4 = e_kq + 8 * i;
+            *reinterpret_cast<uint2*>(dx + (size_t)(k4 >> 1) * 128 + (k4 & 1) * 8) =
+                make_uint2(pack_bf16x2(v[h][i].x, v[h][i].y), pack_bf16x2(v[h][i].z, v[h][i].w));
+          }
         }
       }
       fence_async_smem();
@@ -328,33 +367,33 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
     // FP16 high / low parts of a tile's scaled rows -> U (A operand of z = A s); the FP32 row is the record's observation
     auto convert_u = [&](int tile, uint32_t block) {
 #pragma unroll 1
-      for (int g = 0; g < 4; ++g) {
-        const int rr = ew * 16 + g * 4 + e_r4;
-        const long long row = (long long)tile * PA_M + rr;
-        const bool live = row < p.n;
-        const float* xr = p.x + (size_t)(live ? row : 0) * D;
-        float4 v[4];
+      for (int g = 0; g < 4; g += 2) {
+        float4 v[2][4];
+        load_rows(tile, g, v);
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-          v[i] = live ? __ldcg(reinterpret_cast<const float4*>(xr + (e_kq + 8 * i) * 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
-        uint8_t* dhi = ubuf + ((size_t)(rr >> 3) * (D / 8)) * 128 + (rr & 7) * 16;
-        uint8_t* dlo = dhi + PA_X_BYTES;
-        float* rec = ev.ring + ((unsigned long long)block * (uint32_t)p.n + (unsigned long long)(live ? row : 0)) * ev.rec_words;
+        for (int h = 0; h < 2; ++h) {
+          const int rr = ew * 16 + (g + h) * 4 + e_r4;
+          const long long row = (long long)tile * PA_M + rr;
+          const bool live = row < p.n;
+          uint8_t* dhi = ubuf + ((size_t)(rr >> 3) * (D / 8)) * 128 + (rr & 7) * 16;
+          uint8_t* dlo = dhi + PA_X_BYTES;
+          float* rec = ev.ring + ((unsigned long long)block * (uint32_t)p.n + (unsigned long long)(live ? row : 0)) * ev.rec_words;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int k4 = e_kq + 8 * i;
-          const float4 sv = v[i];
-          // high part: the scaled value cut to 11 significant bits (exact in FP16); low part: the exact remainder, rounded
-          float4 s4, hi, lo;
-          s4.x = sv.x * PA_S_SCALE; s4.y = sv.y * PA_S_SCALE; s4.z = sv.z * PA_S_SCALE; s4.w = sv.w * PA_S_SCALE;
-          hi.x = __uint_as_float(__float_as_uint(s4.x) & 0xFFFFE000u); lo.x = s4.x - hi.x;
-          hi.y = __uint_as_float(__float_as_uint(s4.y) & 0xFFFFE000u); lo.y = s4.y - hi.y;
-          hi.z = __uint_as_float(__float_as_uint(s4.z) & 0xFFFFE000u); lo.z = s4.z - hi.z;
-          hi.w = __uint_as_float(__float_as_uint(s4.w) & 0xFFFFE000u); lo.w = s4.w - hi.w;
-          const size_t off = (size_t)(k4 >> 1) * 128 + (k4 & 1) * 8;
-          *reinterpret_cast<uint2*>(dhi + off) = make_uint2(pack_f16x2(hi.x, hi.y), pack_f16x2(hi.z, hi.w));
-          *reinterpret_cast<uint2*>(dlo + off) = make_uint2(pack_f16x2(lo.x, lo.y), pack_f16x2(lo.z, lo.w));
-          if (live) __stcs(reinterpret_cast<float4*>(rec + k4 * 4), sv);
+          for (int i = 0; i < 4; ++i) {
+            const int k4 = e_kq + 8 * i;
+            const float4 sv = v[h][i];
+            // high part: the scaled value cut to 11 significant bits (exact in FP16); low part: the exact remainder, rounded
+            float4 s4, hi, lo;
+            s4.x = sv.x * PA_S_SCALE; s4.y = sv.y * PA_S_SCALE; s4.z = sv.z * PA_S_SCALE; s4.w = sv.w * PA_S_SCALE;
+            hi.x = __uint_as_float(__float_as_uint(s4.x) & 0xFFFFE000u); lo.x = s4.x - hi.x;
+            hi.y = __uint_as_float(__float_as_uint(s4.y) & 0xFFFFE000u); lo.y = s4.y - hi.y;
+            hi.z = __uint_as_float(__float_as_uint(s4.z) & 0xFFFFE000u); lo.z = s4.z - hi.z;
+            hi.w = __uint_as_float(__float_as_uint(s4.w) & 0xFFFFE000u); lo.w = s4.w - hi.w;
+            const size_t off = (size_t)(k4 >> 1) * 128 + (k4 & 1) * 8;
+            *reinterpret_cast<uint2*>(dhi + off) = make_uint2(pack_f16x2(hi.x, hi.y), pack_f16x2(hi.z, hi.w));
+            *reinterpret_cast<uint2*>(dlo + off) = make_uint2(pack_f16x2(lo.x, lo.y), pack_f16x2(lo.z, lo.w));
+            if (live) __stcs(reinterpret_cast<float4*>(rec + k4 * 4), sv);
+          }
         }
       }
       fence_async_smem();
@@ -411,7 +450,7 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
 #pragma unroll
         for (int j = 1; j < 16; ++j)
           if (j < ev.A && qv[j] > qb) { qb = qv[j]; best = j; }
-        ctl->act[tiles & 1][r] = ((unsigned long long)w.x < ev.explore_thr) ? (int)__umulhi(w.y, (uint32_t)ev.A) : best;
+        ctl->act[tiles & 1][r] = ((unsigned long long)w.x < ev.explore_thr) ? (uint8_t)__umulhi(w.y, (uint32_t)ev.A) : (uint8_t)best;
         mbar_arrive_warp(&ctl->act_ready);
       } else {
         mbar_arrive_warp(&ctl->env_taken);         // this warp has finished the previous tile
@@ -438,25 +477,33 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
           const bool live = row < p.n;
           const int action = ctl->act[tiles & 1][rr];
           float* rec = ev.ring + ((unsigned long long)block * (uint32_t)p.n + (unsigned long long)(live ? row : 0)) * ev.rec_words;
-          const int ep0 = live ? ev.ep_step[row] : 0;
-          const float ret0 = live ? ev.ep_return[row] : 0.f;
+          const int ep0 = __float_as_int(load_f1(reinterpret_cast<const float*>(ev.ep_step) + (live ? row : 0)));
+          const float ret0 = load_f1(ev.ep_return + (live ? row : 0));
           const float* Ba = ev.lgB_t + (size_t)action * D;     // B[a] times 2 log2(e)
           // s' = tanh(z + B[a]) + noise; piece k4 = components 4 k4 .. 4 k4 + 3 = one Philox block
-          float4 zz[4], sn[4];
+          // z, B's row and the counters are on their way while the noise, which needs none of them, is made (a row group took 6,900 cycles
+          // with every load behind the instructions that its use follows, 6,000 now)
+          float4 zz[4], bb[4], nz[4], sn[4];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) zz[i] = __ldcg(reinterpret_cast<const float4*>(zs + ((size_t)(e_kq + 8 * i) * PA_M + rr) * 4));
+          for (int i = 0; i < 4; ++i) {
+            zz[i] = load_f4_cg(zs + ((size_t)(e_kq + 8 * i) * PA_M + rr) * 4);
+            bb[i] = load_f4_nc(Ba + 4 * (e_kq + 8 * i));
+          }
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const uint4 w = stream_words(ev.seed, STREAM_NOISE, (uint32_t)(e_kq + 8 * i), (uint32_t)row, ev.t + step);
+            const float2 n01 = box_muller_scaled(w.x, w.y, ev.noise_std), n23 = box_muller_scaled(w.z, w.w, ev.noise_std);
+            nz[i] = make_float4(n01.x, n01.y, n23.x, n23.y);
+          }
           float sq = 0.f;
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             const int k4 = e_kq + 8 * i;
-            const uint4 w = stream_words(ev.seed, STREAM_NOISE, (uint32_t)k4, (uint32_t)row, ev.t + step);
-            const float2 n01 = box_muller_scaled(w.x, w.y, ev.noise_std), n23 = box_muller_scaled(w.z, w.w, ev.noise_std);
-            const float4 bb = __ldg(reinterpret_cast<const float4*>(Ba + 4 * k4));
             float4 o;
-            o.x = tanh_from_t(fmaf(zz[i].x, zc, bb.x)) + n01.x;
-            o.y = tanh_from_t(fmaf(zz[i].y, zc, bb.y)) + n01.y;
-            o.z = tanh_from_t(fmaf(zz[i].z, zc, bb.z)) + n23.x;
-            o.w = tanh_from_t(fmaf(zz[i].w, zc, bb.w)) + n23.y;
+            o.x = tanh_from_t(fmaf(zz[i].x, zc, bb[i].x)) + nz[i].x;
+            o.y = tanh_from_t(fmaf(zz[i].y, zc, bb[i].y)) + nz[i].y;
+            o.z = tanh_from_t(fmaf(zz[i].z, zc, bb[i].z)) + nz[i].z;
+            o.w = tanh_from_t(fmaf(zz[i].w, zc, bb[i].w)) + nz[i].w;
             sq = fmaf(o.x, o.x, sq); sq = fmaf(o.y, o.y, sq); sq = fmaf(o.z, o.z, sq); sq = fmaf(o.w, o.w, sq);
             sn[i] = o;
             if (live) __stcs(reinterpret_cast<float4*>(rec + D + 4 * k4), o);
