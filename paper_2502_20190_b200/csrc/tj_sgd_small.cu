@@ -282,20 +282,21 @@ __device__ __forceinline__ void grad_hidden(const float* d2, const float* h1, in
 }
 
 // W1, the biases of the hidden layers and the head, one sum per thread and turn: neuron n of a column -- an input (times d1), ones
-// (times d1, then d2), an output's gradient (times h2).  Lanes run along the neurons; the column's value is a broadcast.
+// (times d1, then d2), an output's gradient (times h2).  Lanes run along the neurons; the column's value is a broadcast.  The block's
+// threads from `first` on (a multiple of 128) share the columns.
 template <int R>
-__device__ __forceinline__ void grad_narrow(const FsLayout& L, const float* sm, int D, int H, int A, int vh, const FsOut& out) {
-  const int shift = H > 64 ? 7 : (H > 32 ? 6 : 5), n = threadIdx.x & ((1 << shift) - 1), n_cols = D + 2 + A + vh;
-  if (n >= H) return;
+__device__ __forceinline__ void grad_narrow(const FsLayout& L, const float* sm, int D, int H, int A, int vh, int first, const FsOut& out) {
+  const int shift = H > 64 ? 7 : (H > 32 ? 6 : 5), id = (int)threadIdx.x - first, n = id & ((1 << shift) - 1), n_cols = D + 2 + A + vh;
+  if (id < 0 || n >= H) return;
 #pragma unroll 1
-  for (int c = threadIdx.x >> shift; c < n_cols; c += FS_NT >> shift) {
+  for (int c = id >> shift; c < n_cols; c += (FS_NT - first) >> shift) {
     const int a = c - D - 2;
     const float* d = sm + (c <= D ? L.d1 : (a < 0 ? L.d2 : L.h2)) + n;
     const float* x = sm + (c < D ? L.xs + c : (a < 0 ? L.one : L.g + a));
     const int ldx = c < D ? L.ldD : (a < 0 ? 0 : 4);
     float s = 0.f;
-#pragma unroll 4
-    for (int r = 0; r < R; ++r) s = fmaf(d[r * L.ldH], x[r * ldx], s);
+#pragma unroll 8
+    for (int r = 0; r < R; ++r, d += L.ldH, x += ldx) s = fmaf(*d, *x, s);
     const int o_b1 = H * D, o_b2 = o_b1 + H + H * H, o_W3 = o_b2 + H;
     // the value head's row follows the action heads' rows and their biases
     out.one(c < D ? n * D + c : (a < 0 ? (a == -2 ? o_b1 : o_b2) + n : o_W3 + a * H + (a == A ? A : 0) + n), s);
@@ -408,7 +409,8 @@ __global__ void __launch_bounds__(FS_NT, 1) sgd_fused_kernel(const SgdParams p, 
   const int n_chunks = (p.n + R - 1) / R;
   bool ok = true;                                  // a wait that runs out: the thread goes on with meaningless numbers
   FsOut out{p.grad_partial + (size_t)blockIdx.x * stride, false};
-  float part0 = 0.f, part1 = 0.f, part2 = 0.f, part3 = 0.f, part4 = 0.f;     // thread 0: the block's loss terms
+  const int lane = tid & 31;
+  float part[5] = {0.f, 0.f, 0.f, 0.f, 0.f};       // the block's loss terms, in one of its warps
   for (int chunk = blockIdx.x; chunk < n_chunks; chunk += gridDim.x, out.add = true) {
     const int rows = min(R, p.n - chunk * R);
     if (tid < 8 * R && (tid & 7) < Dp) {
@@ -467,55 +469,64 @@ __global__ void __launch_bounds__(FS_NT, 1) sgd_fused_kernel(const SgdParams p, 
     // loss and its gradient at the outputs, one thread per row
     if (tid < R) {
       const int r = tid;
-      const float* qs = sm + L.q + r * 4;
+      // outputs in registers: an array indexed at run time is a shared-memory latency per access
+      const float4 q4 = *reinterpret_cast<const float4*>(sm + L.q + r * 4);
+      const float q[4] = {q4.x, q4.y, q4.z, q4.w};
+      auto pick = [](const float (&v)[4], int i) { return i == 0 ? v[0] : (i == 1 ? v[1] : (i == 2 ? v[2] : v[3])); };
       act = act < 0 ? 0 : (act >= A ? A - 1 : act);
-      float* gs = sm + L.g + r * 4;
-      float l[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-      *reinterpret_cast<float4*>(gs) = make_float4(0.f, 0.f, 0.f, 0.f);
+      float g[4] = {0.f, 0.f, 0.f, 0.f}, l[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
       if (r < rows) {
         if (PPO) {
-          float lmax = qs[0];
-#pragma unroll 1
-          for (int i = 1; i < A; ++i) lmax = fmaxf(lmax, qs[i]);
+          float lmax = q[0];
+#pragma unroll
+          for (int i = 1; i < 4; ++i)
+            if (i < A) lmax = fmaxf(lmax, q[i]);
           float Z = 0.f;
-#pragma unroll 1
-          for (int i = 0; i < A; ++i) Z += expf(qs[i] - lmax);
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (i < A) Z += expf(q[i] - lmax);
           const float logZ = lmax + logf(Z);
-          float ent = 0.f;
-#pragma unroll 1
-          for (int i = 0; i < A; ++i) {
-            const float lp = qs[i] - logZ;
-            ent -= expf(lp) * lp;
-          }
-          const float logp = qs[act] - logZ, ratio = expf(logp - rew);
+          float ent = 0.f, lp[4] = {0.f, 0.f, 0.f, 0.f}, pi[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (i < A) {
+              lp[i] = q[i] - logZ;
+              pi[i] = expf(lp[i]);
+              ent -= pi[i] * lp[i];
+            }
+          const float logp = pick(q, act) - logZ, ratio = expf(logp - rew);
           const float rc = fminf(fmaxf(ratio, 1.f - p.clip_eps), 1.f + p.clip_eps);
           const float t1 = ratio * adv, t2 = rc * adv;
           const bool unclipped = t1 <= t2;
-          const float dv = qs[A] - ret;
+          const float dv = pick(q, A) - ret;
           l[1] = -(unclipped ? t1 : t2);
           l[2] = 0.5f * dv * dv;
           l[3] = ent;
           l[4] = unclipped ? 0.f : 1.f;
           l[0] = l[1] + p.c_v * l[2] - p.c_e * l[3];
           const float g_logp = unclipped ? -adv * ratio : 0.f, inv_n = 1.f / (float)p.n;
-          gs[A] = p.c_v * dv * inv_n;
-#pragma unroll 1
-          for (int i = 0; i < A; ++i) {
-            const float lp = qs[i] - logZ, pi = expf(lp);
-            const float dlogp = (i == act ? 1.f : 0.f) - pi, dent = -pi * (lp + ent);
-            gs[i] = (g_logp * dlogp - p.c_e * dent) * inv_n;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float dlogp = (i == act ? 1.f : 0.f) - pi[i], dent = -pi[i] * (lp[i] + ent);
+            if (i < A) g[i] = (g_logp * dlogp - p.c_e * dent) * inv_n;
+            else if (i == A) g[i] = p.c_v * dv * inv_n;
           }
         } else {
-          const float* qt = sm + L.q + (R + r) * 4;
+          const float4 t4 = *reinterpret_cast<const float4*>(sm + L.q + (R + r) * 4);
+          const float qt[4] = {t4.x, t4.y, t4.z, t4.w};
           float qmax = qt[0];
-#pragma unroll 1
-          for (int i = 1; i < A; ++i) qmax = fmaxf(qmax, qt[i]);
+#pragma unroll
+          for (int i = 1; i < 4; ++i)
+            if (i < A) qmax = fmaxf(qmax, qt[i]);
           const float y = rew + p.gamma * (done ? 0.f : 1.f) * qmax;
-          const float delta = y - qs[act], ad = fabsf(delta);
+          const float delta = y - pick(q, act), ad = fabsf(delta);
           l[0] = ad <= p.kappa ? 0.5f * delta * delta : p.kappa * (ad - 0.5f * p.kappa);
-          gs[act] = -fminf(fmaxf(delta, -p.kappa), p.kappa) / (float)p.n;
+          const float ga = -fminf(fmaxf(delta, -p.kappa), p.kappa) / (float)p.n;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) g[i] = i == act ? ga : 0.f;
         }
       }
+      *reinterpret_cast<float4*>(sm + L.g + r * 4) = make_float4(g[0], g[1], g[2], g[3]);
 #pragma unroll
       for (int k = 0; k < (PPO ? 5 : 1); ++k) sm[L.part + k * R + r] = l[k];
     }
@@ -536,31 +547,44 @@ __global__ void __launch_bounds__(FS_NT, 1) sgd_fused_kernel(const SgdParams p, 
       d.x = h.x > 0.f ? d.x : 0.f; d.y = h.y > 0.f ? d.y : 0.f; d.z = h.z > 0.f ? d.z : 0.f; d.w = h.w > 0.f ? d.w : 0.f;
       *reinterpret_cast<float4*>(sm + L.d2 + r * L.ldH + 4 * q) = d;
     }
-    if (tid == 0) {
-      for (int r = 0; r < rows; ++r) {
-        part0 += sm[L.part + r];
-        if (PPO) { part1 += sm[L.part + R + r]; part2 += sm[L.part + 2 * R + r]; part3 += sm[L.part + 3 * R + r]; part4 += sm[L.part + 4 * R + r]; }
+    // the block's loss terms and the output biases' gradients (column sums of g), a warp each, lane r row r: added by one thread row after
+    // row they kept this phase at 2,070 cycles for 32 rows of PPO
+    if (tid >> 5 == FS_NT / 32 - 2) {
+      float v[5];
+#pragma unroll
+      for (int k = 0; k < (PPO ? 5 : 1); ++k) v[k] = lane < R ? sm[L.part + k * R + lane] : 0.f;
+#pragma unroll
+      for (int k = 0; k < (PPO ? 5 : 1); ++k) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+        part[k] += v[k];
       }
-    }
-    if (tid >= FS_NT - 4) {                        // output biases: column sums of g
-      const int a = tid - (FS_NT - 4), off = H * D + H + H * H + H + A * H;
-      float s = 0.f;
-      for (int r = 0; r < R; ++r) s += sm[L.g + r * 4 + a];
-      if (a < A) out.one(off + a, s);
-      else if (PPO && a == A) out.one(off + A + H, s);
+    } else if (tid >> 5 == FS_NT / 32 - 1) {
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (lane < R) v = *reinterpret_cast<const float4*>(sm + L.g + lane * 4);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        v.x += __shfl_xor_sync(0xffffffffu, v.x, o); v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+        v.z += __shfl_xor_sync(0xffffffffu, v.z, o); v.w += __shfl_xor_sync(0xffffffffu, v.w, o);
+      }
+      const int off = H * D + H + H * H + H + A * H;
+      const float s = lane == 0 ? v.x : (lane == 1 ? v.y : (lane == 2 ? v.z : v.w));
+      if (lane < A) out.one(off + lane, s);
+      else if (PPO && lane == A) out.one(off + A + H, s);
     }
     __syncthreads();
     dense_back<R>(sm + L.W2, L.ldH, sm + L.d2, sm + L.h1, sm + L.d1, L.ldH, G, tb, sm + L.red);
     if (G * G <= FS_NT) grad_hidden<R, 1>(sm + L.d2, sm + L.h1, L.ldH, H, G, H * D + H, out);
     else grad_hidden<R, 2>(sm + L.d2, sm + L.h1, L.ldH, H, G, H * D + H, out);
     if (chunk + (int)gridDim.x < n_chunks) fetch_rows(chunk + gridDim.x);
-    grad_narrow<R>(L, sm, D, H, A, PPO ? 1 : 0, out);
+    // where the hidden matrix's gradient leaves half of the threads idle (up to hidden 64), they do the narrow ones meanwhile
+    grad_narrow<R>(L, sm, D, H, A, PPO ? 1 : 0, G * G <= FS_NT / 2 ? FS_NT / 2 : 0, out);
     __syncthreads();
   }
-  if (tid == 0) {
+  if (tid == FS_NT - 64) {
     float* pp = p.partial + (size_t)blockIdx.x * 5;
-    pp[0] = part0;
-    if (PPO) { pp[1] = part1; pp[2] = part2; pp[3] = part3; pp[4] = part4; }
+#pragma unroll
+    for (int k = 0; k < (PPO ? 5 : 1); ++k) pp[k] = part[k];
   }
   if (!ok) {
     update_failed(p.watch);

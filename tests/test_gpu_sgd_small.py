@@ -19,3 +19,9 @@ def test_sgd_step(env, kind, D, A, H, B):
 @pytest.mark.parametrize("kind,D,A,H,N,T,B", [(1, 6, 3, 101, 40, 10, 257), (0, 4, 2, 128, 300, 10, 2999), (0, 4, 2, 30, 300, 16, 4800)])
 def test_ppo_step(env, kind, D, A, H, N, T, B):
     test_gpu_ppo.test_ppo_step_matches_oracle(env, kind, D, A, H, N, T, B, 0)
+
+
+# hidden 61-64: half of the threads do the narrow gradients beside the hidden matrix's; 8, 16 and 32 rows per block, three outputs and four
+@pytest.mark.parametrize("kind,D,A,H,N,T,B", [(0, 4, 2, 64, 100, 10, 1000), (1, 6, 3, 61, 300, 10, 2300), (1, 6, 3, 64, 300, 10, 2999)])
+def test_ppo_step_idle_half(env, kind, D, A, H, N, T, B):
+    test_gpu_ppo.test_ppo_step_matches_oracle(env, kind, D, A, H, N, T, B, 0)
