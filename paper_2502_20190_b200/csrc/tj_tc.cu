@@ -380,10 +380,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) mlp_bf16_tc_kernel(const TcMlpP
             const uint4 w = stream_words(ev.seed, STREAM_NOISE, (uint32_t)(c0 / 4 + b4), (uint32_t)row, ev.t + step);
             const float2 z01 = box_muller_fast(w.x, w.y), z23 = box_muller_fast(w.z, w.w);
             const float4 bb = __ldg(reinterpret_cast<const float4*>(Ba + c0 + 4 * b4));
-            sn[4 * b4 + 0] = tanh_fast(__uint_as_float(v[4 * b4 + 0]) + bb.x) + ev.noise_std * z01.x;
-            sn[4 * b4 + 1] = tanh_fast(__uint_as_float(v[4 * b4 + 1]) + bb.y) + ev.noise_std * z01.y;
-            sn[4 * b4 + 2] = tanh_fast(__uint_as_float(v[4 * b4 + 2]) + bb.z) + ev.noise_std * z23.x;
-            sn[4 * b4 + 3] = tanh_fast(__uint_as_float(v[4 * b4 + 3]) + bb.w) + ev.noise_std * z23.y;
+            sn[4 * b4 + 0] = tanh_from_t(2.88539008177792681472f * (__uint_as_float(v[4 * b4 + 0]) + bb.x)) + ev.noise_std * z01.x;
+            sn[4 * b4 + 1] = tanh_from_t(2.88539008177792681472f * (__uint_as_float(v[4 * b4 + 1]) + bb.y)) + ev.noise_std * z01.y;
+            sn[4 * b4 + 2] = tanh_from_t(2.88539008177792681472f * (__uint_as_float(v[4 * b4 + 2]) + bb.z)) + ev.noise_std * z23.x;
+            sn[4 * b4 + 3] = tanh_from_t(2.88539008177792681472f * (__uint_as_float(v[4 * b4 + 3]) + bb.w)) + ev.noise_std * z23.y;
           }
 #pragma unroll
           for (int j = 0; j < 16; ++j) sq = fmaf(sn[j], sn[j], sq);
