@@ -117,7 +117,7 @@ __device__ __forceinline__ void af_layer1(const float* b1, const float* W1t, con
   if (!computes) return;
   FmaAcc<EPT, NPT> acc;
   fma_bias<EPT, NPT>(acc, b1, t);
-  fma_accumulate<EPT, NPT, 1>(acc, W1t, Hp, xs, E, D, t);
+  fma_accumulate<EPT, NPT, (EPT * NPT > 16 ? 1 : 6)>(acc, W1t, Hp, xs, E, D, t);
   fma_store_kmajor(acc, h1, E, t);
 }
 
@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(af_most(EPT, NPT), 1) actor_fma_kernel(const A
     draw(it + 1);
     if (head_warp) {
       const float* b3 = sm + q.w + p.off_b3 - q.gap;
-      const float out = fma_head(b3[a], w3 + a * q.ldh, h2 + (el < E ? el : 0) * q.ldh, p.Hp / 4);
+      const float out = fma_head<(EPT * NPT > 16 ? 4 : 8)>(b3[a], w3 + a * q.ldh, h2 + (el < E ? el : 0) * q.ldh, p.Hp / 4);
       float l[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) l[i] = __shfl_sync(0xffffffffu, out, (lane & ~3) + i);

@@ -117,8 +117,9 @@ __device__ __forceinline__ void fma_store_rows(const FmaAcc<EPT, NPT>& acc, floa
 }
 
 // one output of the narrow head: acc = b; acc = fma(w[k], h[k], acc) over a row of h (both 16-byte aligned, zero padded to 4)
+template <int UNROLL>
 __device__ __forceinline__ float fma_head(float acc, const float* w, const float* h, int K4) {
-#pragma unroll 4
+#pragma unroll UNROLL
   for (int k = 0; k < K4; ++k) {
     const float4 a = *reinterpret_cast<const float4*>(w + 4 * k), b = *reinterpret_cast<const float4*>(h + 4 * k);
     acc = fmaf(a.x, b.x, acc);

@@ -739,7 +739,7 @@ __global__ void __launch_bounds__(TR_NT) td_rows_kernel(const TdParams p, const 
   __syncthreads();
   for (int g = tid; g < 8 * rows; g += TR_NT) {
     const int a = g & 3, s = g >> 2, net = s >= rows ? 1 : 0;
-    sm[L.q + g] = fma_head(__ldg((net ? p.Wtarget : p.Wonline) + p.off_b3 + a), sm + L.w3 + (net * 4 + a) * L.ldh, sm + L.h + s * L.ldh, Hq / 4);
+    sm[L.q + g] = fma_head<4>(__ldg((net ? p.Wtarget : p.Wonline) + p.off_b3 + a), sm + L.w3 + (net * 4 + a) * L.ldh, sm + L.h + s * L.ldh, Hq / 4);
   }
   __syncthreads();
   if (tid < here) {

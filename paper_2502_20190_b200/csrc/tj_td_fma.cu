@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(TF_NT, 1) td_fma_kernel(const TdParams p, cons
     // heads: lane a of a group of four sums output a of (network, row)
     for (int g = tid >> 2; g < (2 * E + 7) / 8 * 8; g += q.nt >> 2) {
       const int n = g >= E ? 1 : 0, r = g < 2 * E ? g - n * E : 0, a = lane & 3;
-      const float out = fma_head(sm[q.w + n * q.s_w + p.off_b3 + a], sm + q.w3 + n * q.s_w3 + a * q.ldh, sm + q.h2 + n * q.s_h2 + r * q.ldh, p.Hp / 4);
+      const float out = fma_head<4>(sm[q.w + n * q.s_w + p.off_b3 + a], sm + q.w3 + n * q.s_w3 + a * q.ldh, sm + q.h2 + n * q.s_h2 + r * q.ldh, p.Hp / 4);
       if (g < 2 * E) sm[q.q + 4 * g + a] = out;
     }
     ok = __syncthreads_and(ok);                               // whichever thread's wait ran out, none of the block's rows is valid
