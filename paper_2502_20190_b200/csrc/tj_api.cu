@@ -8,6 +8,8 @@
 #include <cstring>
 #include <new>
 
+#include <cuda.h>
+
 #include "tj_internal.h"
 
 using namespace tj;
@@ -419,6 +421,35 @@ int tj_set_profiling(tj_ctx* x, int32_t on) {
   return TJ_OK;
 }
 
+namespace {
+// Page-locked host memory as the publish kernel can read it, null where the blob has to be copied first: pageable memory, an allocation
+// that ends before the blob does, and large blobs.  A copy in front of the kernel costs its own start and the overlap of the kernel's
+// launch with the tail of the one before (publish and one actor step, copy / no copy: 18 KB 14.3 / 11.9 us, 70 KB 15.1 / 10.4,
+// 166 KB 22.4 / 14.2, 270 KB 34.2 / 22.6, 473 KB 52.7 / 45.0: the copy engine's rate gains on the kernel's).
+constexpr size_t kMappedBlobBytes = 512 * 1024;
+const float* mapped_blob(const void* blob, size_t nbytes) {
+  typedef CUresult (*Query)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+  static const Query query = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+    const cudaError_t e = cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &found);
+    if (e != cudaSuccess) cudaGetLastError();
+    return reinterpret_cast<Query>(e == cudaSuccess && found == cudaDriverEntryPointSuccess ? f : nullptr);
+  }();
+  if (!query || nbytes > kMappedBlobBytes) return nullptr;
+  unsigned type = 0;
+  CUdeviceptr on_device = 0, start = 0;
+  size_t size = 0;
+  CUpointer_attribute what[4] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_POINTER, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                 CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void* into[4] = {&type, &on_device, &start, &size};
+  const CUdeviceptr p = reinterpret_cast<CUdeviceptr>(blob);
+  if (query(4, what, into, p) != CUDA_SUCCESS || type != CU_MEMORYTYPE_HOST || !on_device) return nullptr;
+  if (p < start || p - start > size || size - (p - start) < nbytes || on_device % sizeof(float)) return nullptr;
+  return reinterpret_cast<const float*>(on_device);
+}
+}  // namespace
+
 int tj_publish_weights(tj_ctx* x, const void* blob, size_t nbytes, int32_t on_device, int64_t* version_out) {
   if (!x) return TJ_ERR_INVALID_ARG;
   if (!blob) return fail(x, TJ_ERR_INVALID_ARG, "blob is null");
@@ -428,9 +459,12 @@ int tj_publish_weights(tj_ctx* x, const void* blob, size_t nbytes, int32_t on_de
   learner_waits_for_actor(x);
   const float* src = static_cast<const float*>(blob);
   if (!on_device) {
-    if ((e = cudaMemcpyAsync(x->blob_stage, blob, nbytes, cudaMemcpyHostToDevice, x->lstream)) != cudaSuccess)
-      return cuda_fail(x, e, "publish: host to device copy");
-    src = x->blob_stage;
+    src = mapped_blob(blob, nbytes);
+    if (!src) {
+      if ((e = cudaMemcpyAsync(x->blob_stage, blob, nbytes, cudaMemcpyHostToDevice, x->lstream)) != cudaSuccess)
+        return cuda_fail(x, e, "publish: host to device copy");
+      src = x->blob_stage;
+    }
   }
   LaunchScope scope(x, TJ_K_PUBLISH, 1, true, true);
   const int next = x->active ^ 1, slot = x->version == 0 ? x->active : next;
