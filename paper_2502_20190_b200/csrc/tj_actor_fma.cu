@@ -41,28 +41,22 @@ __device__ __forceinline__ float4 reset4(uint2 seed, uint32_t block, uint32_t e,
                      uniform_range(w.w, lo, width));
 }
 
-// Acrobot's derivative with the three angles' sines spread over the four lanes of an environment (a = lane of the group): lane 0
-// takes th2, lane 1 th1 + th2, the others th1.  Same expressions as acrobot_deriv.
-__device__ __forceinline__ float4 acrobot_deriv4(float4 y, float torque, int lane) {
-  constexpr float m1 = 1.0f, m2 = 1.0f, l1 = 1.0f, lc1 = 0.5f, lc2 = 0.5f, I1 = 1.0f, I2 = 1.0f, g = 9.8f;
-  const float th1 = y.x, th2 = y.y, w1 = y.z, w2 = y.w;
+// Acrobot's angles with their sines spread over the four lanes of an environment: lane 0 takes th1, lane 1 th1 + th2, the others th2
+struct AcrobotAngles { float4 trig; float s12, c12; };       // trig = (cos th1, sin th1, cos th2, sin th2)
+__device__ __forceinline__ AcrobotAngles acrobot_angles4(float4 s, int lane) {
   const int a = lane & 3, base = lane & ~3;
-  float s, c;
-  sincosf(a == 0 ? th2 : (a == 1 ? th1 + th2 : th1), &s, &c);
-  const float s2 = __shfl_sync(0xffffffffu, s, base), c2 = __shfl_sync(0xffffffffu, c, base);
-  const float s12 = __shfl_sync(0xffffffffu, s, base + 1), s1 = __shfl_sync(0xffffffffu, s, base + 2);
-  const float d1 = m1 * lc1 * lc1 + m2 * (l1 * l1 + lc2 * lc2 + 2.0f * l1 * lc2 * c2) + I1 + I2;
-  const float d2 = m2 * (lc2 * lc2 + l1 * lc2 * c2) + I2;
-  const float phi2 = m2 * lc2 * g * s12;
-  const float phi1 = -m2 * l1 * lc2 * w2 * w2 * s2 - 2.0f * m2 * l1 * lc2 * w2 * w1 * s2 +
-                     (m1 * lc1 + m2 * l1) * g * s1 + phi2;
-  const float ddth2 = (torque + d2 / d1 * phi1 - m2 * l1 * lc2 * w1 * w1 * s2 - phi2) / (m2 * lc2 * lc2 + I2 - d2 * d2 / d1);
-  const float ddth1 = -(d2 * ddth2 + phi1) / d1;
-  return make_float4(w1, w2, ddth1, ddth2);
+  float sn, cs;
+  sincosf(a == 0 ? s.x : (a == 1 ? s.x + s.y : s.y), &sn, &cs);
+  AcrobotAngles r;
+  r.trig = make_float4(__shfl_sync(0xffffffffu, cs, base), __shfl_sync(0xffffffffu, sn, base), __shfl_sync(0xffffffffu, cs, base + 2),
+                       __shfl_sync(0xffffffffu, sn, base + 2));
+  r.s12 = __shfl_sync(0xffffffffu, sn, base + 1);
+  r.c12 = __shfl_sync(0xffffffffu, cs, base + 1);
+  return r;
 }
 
-// one RK4 step as in acrobot_step
-__device__ __forceinline__ StepResult acrobot_step4(float4 s, int act, int lane, float4& sn) {
+// one RK4 step as in acrobot_step; `at`: the angles of s on entry (the first stage's), of the new state on return (its observation and tip)
+__device__ __forceinline__ StepResult acrobot_step4(float4 s, AcrobotAngles& at, int act, int lane, float4& sn) {
   constexpr float dt = 0.2f, PI = 3.14159265358979323846f;
   const float torque = (float)(act - 1);
   float4 k1, acc, y = s;
@@ -70,7 +64,8 @@ __device__ __forceinline__ StepResult acrobot_step4(float4 s, int act, int lane,
   // stages 1 .. 4 in one copy of the derivative's code; the sums keep acrobot_step's order k1 + 2 k2 + 2 k3 + k4
 #pragma unroll 1
   for (int st = 0; st < 4; ++st) {
-    k1 = acrobot_deriv4(y, torque, lane);
+    if (st > 0) at = acrobot_angles4(y, lane);
+    k1 = acrobot_deriv(y, torque, at.trig.y, at.s12, at.trig.w, at.trig.z);
     if (st == 0) acc = k1;
     else if (st == 3) acc = make_float4(acc.x + k1.x, acc.y + k1.y, acc.z + k1.z, acc.w + k1.w);
     else acc = make_float4(acc.x + 2.0f * k1.x, acc.y + 2.0f * k1.y, acc.z + 2.0f * k1.z, acc.w + 2.0f * k1.w);
@@ -84,25 +79,16 @@ __device__ __forceinline__ StepResult acrobot_step4(float4 s, int act, int lane,
   sn.y = wrap_pi(y.y);
   sn.z = fminf(fmaxf(y.z, -4.0f * PI), 4.0f * PI);
   sn.w = fminf(fmaxf(y.w, -9.0f * PI), 9.0f * PI);
-  const float c = cosf((lane & 3) == 0 ? sn.x : sn.x + sn.y);
-  const float tip = -__shfl_sync(0xffffffffu, c, lane & ~3) - __shfl_sync(0xffffffffu, c, (lane & ~3) + 1);
+  at = acrobot_angles4(sn, lane);
+  const float tip = -at.trig.x - at.c12;
   StepResult r;
   r.terminated = tip > 1.0f;
   r.reward = r.terminated ? 0.0f : -1.0f;
   return r;
 }
 
-// (cos th1, sin th1, cos th2, sin th2) of a state, the two angles on two lanes
-__device__ __forceinline__ float4 acrobot_trig4(float4 s, int lane) {
-  float sn, cs;
-  sincosf((lane & 1) ? s.y : s.x, &sn, &cs);
-  const int base = lane & ~3;
-  return make_float4(__shfl_sync(0xffffffffu, cs, base), __shfl_sync(0xffffffffu, sn, base), __shfl_sync(0xffffffffu, cs, base + 1),
-                     __shfl_sync(0xffffffffu, sn, base + 1));
-}
-
-// one environment between steps; trig = (cos th1, sin th1, cos th2, sin th2) of an Acrobot state
-struct __align__(16) AfEnv { float4 s, trig; int ep; float ret; int episodes, pad; double ret_sum, pad2; };
+// one environment between steps; trig = (cos th1, sin th1, cos th2, sin th2) and s12 = sin(th1 + th2) of an Acrobot state
+struct __align__(16) AfEnv { float4 s, trig; int ep; float ret; int episodes; float s12; double ret_sum, pad2; };
 
 // One chunk of W2 (kc rows, chunk c of a step, number g of the stream) into slot g mod AF_SLOTS; the chunk that was there is used up
 __device__ __forceinline__ void af_queue_chunk(float* ring, const float* W2, uint64_t* full, uint32_t g, uint32_t c, int kc, int H, int Hp) {
@@ -241,13 +227,15 @@ __global__ void __launch_bounds__(af_most(EPT, NPT), 1) actor_fma_kernel(const A
   };
   draw(0);
   if (head_warp) {
-    float4 s = make_float4(0.f, 0.f, 0.f, 0.f), trig = s;
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    AcrobotAngles at{s, 0.f, 0.f};
     if (owner) s = reinterpret_cast<const float4*>(p.state)[e];
-    if (ENV == TJ_ENV_ACROBOT) trig = acrobot_trig4(s, lane);
-    put_obs(s, trig);
+    if (ENV == TJ_ENV_ACROBOT) at = acrobot_angles4(s, lane);
+    put_obs(s, at.trig);
     if (el < E && a == 0) {
       env->s = s;
-      env->trig = trig;
+      env->trig = at.trig;
+      env->s12 = at.s12;
       env->ep = owner ? p.ep_step[e] : 0;
       env->ret = owner ? p.ep_return[e] : 0.f;
       env->episodes = 0;
@@ -311,13 +299,13 @@ __global__ void __launch_bounds__(af_most(EPT, NPT), 1) actor_fma_kernel(const A
         float logp = 0.f;
         if (p.policy_kind == TJ_POLICY_EPS_GREEDY) act = select_eps_greedy(p.A, logit, w, p.explore_thr);
         else act = select_categorical(p.A, logit, u01(w.x), logp);
-        float4 sn, trig_n = trig;
+        float4 sn;
+        AcrobotAngles at{trig, ENV == TJ_ENV_ACROBOT ? env->s12 : 0.f, 0.f};   // of s, then of the new state
         StepResult r;
         if (ENV == TJ_ENV_CARTPOLE) {
           r = cartpole_step(s, act, sn);
         } else {
-          r = acrobot_step4(s, act, lane, sn);
-          trig_n = acrobot_trig4(sn, lane);
+          r = acrobot_step4(s, at, act, lane, sn);
         }
         const int done = (r.terminated || ep >= p.max_ep) ? 1 : 0;
         if (owner) {
@@ -341,8 +329,8 @@ __global__ void __launch_bounds__(af_most(EPT, NPT), 1) actor_fma_kernel(const A
             if (ENV == TJ_ENV_CARTPOLE) {
               if (a < 3) rec[a] = a == 0 ? s : (a == 1 ? sn : tail);
             } else {
-              rec[a] = a == 0 ? trig : (a == 1 ? make_float4(s.z, s.w, trig_n.x, trig_n.y)
-                                               : (a == 2 ? make_float4(trig_n.z, trig_n.w, sn.z, sn.w) : tail));
+              rec[a] = a == 0 ? trig : (a == 1 ? make_float4(s.z, s.w, at.trig.x, at.trig.y)
+                                               : (a == 2 ? make_float4(at.trig.z, at.trig.w, sn.z, sn.w) : tail));
             }
           }
         }
@@ -353,14 +341,14 @@ __global__ void __launch_bounds__(af_most(EPT, NPT), 1) actor_fma_kernel(const A
           next = ENV == TJ_ENV_CARTPOLE ? reset4(p.seed, 0, (uint32_t)e, t_now, -0.05f, 0.1f) : reset4(p.seed, 0, (uint32_t)e, t_now, -0.1f, 0.2f);
         }
         if (ENV == TJ_ENV_ACROBOT && __any_sync(0xffffffffu, done)) {
-          const float4 fresh = acrobot_trig4(next, lane);
-          if (done) trig_n = fresh;
+          const AcrobotAngles fresh = acrobot_angles4(next, lane);
+          if (done) at = fresh;
         }
-        put_obs(next, trig_n);
+        put_obs(next, at.trig);
         __syncwarp();                                         // the other lanes of the environment have read it
         if (el < E && a == 0) {
           env->s = next;
-          if (ENV == TJ_ENV_ACROBOT) env->trig = trig_n;
+          if (ENV == TJ_ENV_ACROBOT) { env->trig = at.trig; env->s12 = at.s12; }
           env->ep = done ? 0 : ep;
           env->ret = done ? 0.f : ret;
           if (done) { env->episodes += 1; env->ret_sum += (double)ret; }

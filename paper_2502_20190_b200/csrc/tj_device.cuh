@@ -73,19 +73,29 @@ __device__ __forceinline__ StepResult cartpole_step(float4 s, int a, float4& sn)
 
 // ------------------------------------------------------------------ Acrobot
 // Two-link pendulum (Sutton & Barto), torque on the second joint, angles from the downward vertical.
-__device__ __forceinline__ float4 acrobot_deriv(float4 y, float torque) {
+__device__ __forceinline__ float4 acrobot_deriv(float4 y, float torque, float s1, float s12, float s2, float c2) {
   constexpr float m1 = 1.0f, m2 = 1.0f, l1 = 1.0f, lc1 = 0.5f, lc2 = 0.5f, I1 = 1.0f, I2 = 1.0f, g = 9.8f;
-  const float th1 = y.x, th2 = y.y, w1 = y.z, w2 = y.w;
-  float s2, c2;
-  sincosf(th2, &s2, &c2);
+  const float w1 = y.z, w2 = y.w;
   const float d1 = m1 * lc1 * lc1 + m2 * (l1 * l1 + lc2 * lc2 + 2.0f * l1 * lc2 * c2) + I1 + I2;
   const float d2 = m2 * (lc2 * lc2 + l1 * lc2 * c2) + I2;
-  const float phi2 = m2 * lc2 * g * sinf(th1 + th2);
+  const float phi2 = m2 * lc2 * g * s12;
   const float phi1 = -m2 * l1 * lc2 * w2 * w2 * s2 - 2.0f * m2 * l1 * lc2 * w2 * w1 * s2 +
-                     (m1 * lc1 + m2 * l1) * g * sinf(th1) + phi2;
+                     (m1 * lc1 + m2 * l1) * g * s1 + phi2;
   const float ddth2 = (torque + d2 / d1 * phi1 - m2 * l1 * lc2 * w1 * w1 * s2 - phi2) / (m2 * lc2 * lc2 + I2 - d2 * d2 / d1);
   const float ddth1 = -(d2 * ddth2 + phi1) / d1;
   return make_float4(w1, w2, ddth1, ddth2);
+}
+__device__ __forceinline__ float4 acrobot_deriv(float4 y, float torque) {
+  float s2, c2;
+  sincosf(y.y, &s2, &c2);
+  return acrobot_deriv(y, torque, sinf(y.x), sinf(y.x + y.y), s2, c2);
+}
+// (cos th1, sin th1, cos th2, sin th2)
+__device__ __forceinline__ float4 acrobot_trig(float4 s) {
+  float4 t;
+  sincosf(s.x, &t.y, &t.x);
+  sincosf(s.y, &t.w, &t.z);
+  return t;
 }
 
 __device__ __forceinline__ float4 axpy4(float4 y, float h, float4 k) {
@@ -97,10 +107,11 @@ __device__ __forceinline__ float wrap_pi(float x) {
   return x - TWO_PI * floorf((x + PI) / TWO_PI);
 }
 
-__device__ __forceinline__ StepResult acrobot_step(float4 s, int a, float4& sn) {
+// trig, trig_n: acrobot_trig of the state before and after the step (the observation has both; the first stage and the tip's height use them)
+__device__ __forceinline__ StepResult acrobot_step(float4 s, float4 trig, int a, float4& sn, float4& trig_n) {
   constexpr float dt = 0.2f, PI = 3.14159265358979323846f;
   const float torque = (float)(a - 1);
-  const float4 k1 = acrobot_deriv(s, torque);
+  const float4 k1 = acrobot_deriv(s, torque, trig.y, sinf(s.x + s.y), trig.w, trig.z);
   const float4 k2 = acrobot_deriv(axpy4(s, 0.5f * dt, k1), torque);
   const float4 k3 = acrobot_deriv(axpy4(s, 0.5f * dt, k2), torque);
   const float4 k4 = acrobot_deriv(axpy4(s, dt, k3), torque);
@@ -113,7 +124,8 @@ __device__ __forceinline__ StepResult acrobot_step(float4 s, int a, float4& sn) 
   sn.y = wrap_pi(y.y);
   sn.z = fminf(fmaxf(y.z, -4.0f * PI), 4.0f * PI);
   sn.w = fminf(fmaxf(y.w, -9.0f * PI), 9.0f * PI);
-  const float tip = -cosf(sn.x) - cosf(sn.x + sn.y);
+  trig_n = acrobot_trig(sn);
+  const float tip = -trig_n.x - cosf(sn.x + sn.y);
   StepResult r;
   r.terminated = tip > 1.0f;
   r.reward = r.terminated ? 0.0f : -1.0f;

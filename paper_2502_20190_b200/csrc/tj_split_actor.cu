@@ -45,10 +45,8 @@ __device__ __forceinline__ void sa_observe(float4 s, float* obs) {
   if (ENV == TJ_ENV_CARTPOLE) {
     obs[0] = s.x; obs[1] = s.y; obs[2] = s.z; obs[3] = s.w; obs[4] = obs[5] = 0.f;
   } else {
-    float s1, c1, s2, c2;
-    sincosf(s.x, &s1, &c1);
-    sincosf(s.y, &s2, &c2);
-    obs[0] = c1; obs[1] = s1; obs[2] = c2; obs[3] = s2; obs[4] = s.z; obs[5] = s.w;
+    const float4 t = acrobot_trig(s);
+    obs[0] = t.x; obs[1] = t.y; obs[2] = t.z; obs[3] = t.w; obs[4] = s.z; obs[5] = s.w;
   }
 }
 
@@ -526,11 +524,18 @@ __global__ void __launch_bounds__(128 * TPR * GROUPS + 64, 1) actor_split_tc_ker
         if (p.policy_kind == TJ_POLICY_EPS_GREEDY) a = select_eps_greedy(p.A, logit, w, p.explore_thr);
         else a = select_categorical(p.A, logit, u01(w.x), logp);
         float4 sn;
-        const StepResult r = (ENV == TJ_ENV_CARTPOLE) ? cartpole_step(s, a, sn) : acrobot_step(s, a, sn);
+        float obs_n[6];
+        StepResult r;
+        if (ENV == TJ_ENV_CARTPOLE) {
+          r = cartpole_step(s, a, sn);
+          sa_observe<ENV>(sn, obs_n);
+        } else {
+          float4 trig_n;
+          r = acrobot_step(s, make_float4(obs[0], obs[1], obs[2], obs[3]), a, sn, trig_n);
+          obs_n[0] = trig_n.x; obs_n[1] = trig_n.y; obs_n[2] = trig_n.z; obs_n[3] = trig_n.w; obs_n[4] = sn.z; obs_n[5] = sn.w;
+        }
         ep += 1;
         const int done = (r.terminated || ep >= p.max_ep) ? 1 : 0;
-        float obs_n[6];
-        sa_observe<ENV>(sn, obs_n);
         if (owner) {
           if (on_policy) {
             const size_t i = ((size_t)seg * p.T + pos) * p.N + e;
