@@ -323,40 +323,8 @@ __global__ void __launch_bounds__(FS_NT, 1) sgd_fused_kernel(const SgdParams p, 
   chain_begin();
   const int o_b1 = H * D, o_W2 = o_b1 + H, o_b2 = o_W2 + H * H, o_W3 = o_b2 + H, o_b3 = o_W3 + A * H;
   // every load of the prologue is in flight before the first result is used: a load that waits for another costs a round trip
-  // to L2 (0.45 us), and four of them in a row were a third of the kernel
-  if (L.bulk) {
-    // a thread copies one 16-byte column of every RP-th row of the hidden matrices, the first rows' threads the head and the biases too.
-    // (One bulk copy per row, issued by a thread per row, took 32 cycles each, one after the other: 4,400 cycles for two networks at
-    // hidden 64, a quarter of the kernel.)
-    const int RP = FS_NT / G, r0 = tid / G, c = 4 * (tid - r0 * G);
-    if (r0 < RP) {
-#pragma unroll 1
-      for (int net = PPO ? 0 : 1; net >= 0; --net) {
-        const float* blob = net ? p.theta_target : p.theta;
-        if (r0 < A) cp_async16(sm + (net ? L.T3 : L.W3) + r0 * L.ldH + c, blob + o_W3 + r0 * H + c);
-        else if (r0 == 4) cp_async16(sm + (net ? L.tb2 : L.b2) + c, blob + o_b2 + c);
-        const float* src = blob + o_W2 + r0 * H + c;
-        float* dst = sm + (net ? L.T2 : L.W2) + r0 * L.ldH + c;
-#pragma unroll 4
-        for (int r = r0; r < H; r += RP, src += RP * H, dst += RP * L.ldH) cp_async16(dst, src);
-      }
-    }
-    cp_async_arrive(bar);
-  } else {
-#pragma unroll 1
-    for (int net = PPO ? 0 : 1; net >= 0; --net) {
-#pragma unroll 1
-      for (int m = 0; m < (PPO ? 4 : 3); ++m) {
-        FsLoad ld;
-        if (m == 0) ld = FsLoad{o_b2, net ? L.tb2 : L.b2, L.Hp, 1, H, 1};
-        else if (m == 1) ld = FsLoad{o_W3, net ? L.T3 : L.W3, L.ldH, A, H, PPO ? A : 4};
-        else if (m == 2) ld = FsLoad{o_W2, net ? L.T2 : L.W2, L.ldH, H, H, L.Hp};
-        else ld = FsLoad{o_b3 + A, L.W3 + A * L.ldH, L.ldH, 1, H, 4 - A};
-        load_matrix(sm, net ? p.theta_target : p.theta, ld);
-      }
-    }
-    cp_async_commit();
-  }
+  // to L2 (0.45 us), and four of them in a row were a third of the kernel.  What layer 1 needs goes first: the hidden matrices, which every
+  // block reads at the same time, hold up whatever is queued behind them.
   // layer 1: a thread owns neuron n for rows r0, r0 + dr, ...; its weights and biases of both networks go straight to registers
   const int shift = H > 64 ? 7 : (H > 32 ? 6 : 5), n = tid & ((1 << shift) - 1), r0 = tid >> shift, dr = FS_NT >> shift;
   float w1[8], t1[8], c1 = 0.f, e1 = 0.f, head_bias = 0.f, head_value = 0.f;
@@ -399,6 +367,39 @@ __global__ void __launch_bounds__(FS_NT, 1) sgd_fused_kernel(const SgdParams p, 
     }
   };
   fetch_rows(blockIdx.x);
+  if (L.bulk) {
+    // a thread copies one 16-byte column of every RP-th row of the hidden matrices, the first rows' threads the head and the biases too.
+    // (One bulk copy per row, issued by a thread per row, took 32 cycles each, one after the other: 4,400 cycles for two networks at
+    // hidden 64, a quarter of the kernel.)
+    const int RP = FS_NT / G, first = tid / G, c = 4 * (tid - first * G);
+    if (first < RP) {
+#pragma unroll 1
+      for (int net = PPO ? 0 : 1; net >= 0; --net) {
+        const float* blob = net ? p.theta_target : p.theta;
+        if (first < A) cp_async16(sm + (net ? L.T3 : L.W3) + first * L.ldH + c, blob + o_W3 + first * H + c);
+        else if (first == 4) cp_async16(sm + (net ? L.tb2 : L.b2) + c, blob + o_b2 + c);
+        const float* src = blob + o_W2 + first * H + c;
+        float* dst = sm + (net ? L.T2 : L.W2) + first * L.ldH + c;
+#pragma unroll 4
+        for (int r = first; r < H; r += RP, src += RP * H, dst += RP * L.ldH) cp_async16(dst, src);
+      }
+    }
+    cp_async_arrive(bar);
+  } else {
+#pragma unroll 1
+    for (int net = PPO ? 0 : 1; net >= 0; --net) {
+#pragma unroll 1
+      for (int m = 0; m < (PPO ? 4 : 3); ++m) {
+        FsLoad ld;
+        if (m == 0) ld = FsLoad{o_b2, net ? L.tb2 : L.b2, L.Hp, 1, H, 1};
+        else if (m == 1) ld = FsLoad{o_W3, net ? L.T3 : L.W3, L.ldH, A, H, PPO ? A : 4};
+        else if (m == 2) ld = FsLoad{o_W2, net ? L.T2 : L.W2, L.ldH, H, H, L.Hp};
+        else ld = FsLoad{o_b3 + A, L.W3 + A * L.ldH, L.ldH, 1, H, 4 - A};
+        load_matrix(sm, net ? p.theta_target : p.theta, ld);
+      }
+    }
+    cp_async_commit();
+  }
   if (tid < (PPO ? 4 : 8)) sm[(tid >> 2 ? L.tb3 : L.b3) + (tid & 3)] = head_bias;
   if (L.bulk && tid < H)
     for (int a = A; a < 4; ++a) {                  // zeros for the head's unused outputs (PPO's value head is output A)
