@@ -101,12 +101,25 @@ __device__ __forceinline__ uint32_t cluster_rank() {
   asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
-// arrival at the barrier at this block's address `bar` in block `rank` of the cluster.  It counts and hands no data over: what the waiting
-// block's products read of this block is in this block's own shared memory, behind fence_async_smem()
+// Arrival at the barrier at this block's address `bar` in block `rank` of the cluster, and the wait for arrivals from another block.  They
+// hand over what the arriving block has in its own shared memory (and, with the tcgen05 fences, its reads of tensor memory): a release and
+// an acquire at cluster scope, of shared memory alone.  The same without that restriction also waits for the record stores in flight
+// (65,536 CartPole envs, hidden 256, 128 steps: 3.25 ms; 2.58 like this).
 __device__ __forceinline__ void mbar_arrive_cluster(uint64_t* bar, uint32_t rank) {
   uint32_t a;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr(bar)), "r"(rank));
-  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(a) : "memory");
+  asm volatile("fence.release.sync_restrict::shared::cta.cluster;" ::: "memory");
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(a) : "memory");
+}
+__device__ __forceinline__ void cluster_acquire() { asm volatile("fence.acquire.sync_restrict::shared::cluster.cluster;" ::: "memory"); }
+__device__ __forceinline__ bool mbar_try_wait_relaxed(uint64_t* bar, uint32_t parity) {    // cluster_acquire() has to follow
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_addr(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
 }
 // a float at this block's shared-memory address `p` in block `rank` of the cluster
 __device__ __forceinline__ float cluster_load_f32(const float* p, uint32_t rank) {

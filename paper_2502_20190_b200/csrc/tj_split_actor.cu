@@ -188,13 +188,17 @@ struct S2Smem {
     __syncthreads();
     const bool issuing_warp = (int)(threadIdx.x >> 5) == NT / 32 - 2;     // the last but one
     if (PAIR) {
-      // neither block leaves before the products that read both blocks' operands are over and the last arrival has reached the first one
+      // Neither block leaves before the products that read both blocks' operands are over and the last arrival has reached the first one.
+      // Where one block gives up, the other follows: a warp whose wait ran out arrives no more, so the first block's issuing warp waits in
+      // vain and stops, and with it every completion that the second block waits for.  If nothing but the last waits is left, the other
+      // block's results are whole and its own; the error word is set by either.
       if (ctl->abort_flag) {
         if (issuing_warp && cluster_rank() == 0) {
           umma_commit_pair(&ctl->settled, elect_one());
           mbar_settle(&ctl->settled, 0);
         }
         if (threadIdx.x == 0 && ctl->copies) mbar_settle(&ctl->full[0], 0);
+        __syncwarp();                                         // a wait's lanes leave it one by one
       }
       cluster_sync_all();
     } else if (ctl->abort_flag) {
@@ -237,7 +241,7 @@ struct S2Smem {
     const uint32_t a0 = desc_lo(smem_addr(a_ring), 128u), w0 = desc_lo(smem_addr(w_ring), 128u);
     const uint32_t hiword = desc_hi((uint32_t)(SA_KC / 8) * 128u);            // A slots and W2 chunks: 32 columns wide
     uint32_t as = 0, round = 0;                               // slot of the ring, rounds of it
-    bool alive = tc_wait_warp(&ctl->w_ready, 0, abort_flag);
+    bool alive = tc_wait_warp<true>(&ctl->w_ready, 0, abort_flag);
     for (int r = 0; r * GROUPS < tiles && alive; ++r)
       for (int i = 0; i < n_pass && alive; ++i)
 #pragma unroll
@@ -246,7 +250,7 @@ struct S2Smem {
           const uint32_t acc = tmem + (uint32_t)g * ACC_COLS;
 #pragma unroll 1
           for (int kc = 0; kc < NKC; ++kc) {
-            if (!tc_wait_warp(&ctl->a_ready[as], round & 1, abort_flag)) { alive = false; break; }
+            if (!tc_wait_warp<true>(&ctl->a_ready[as], round & 1, abort_flag)) { alive = false; break; }
             tc_fence_after();
             const uint32_t a_hi = a0 + as * (S2_A_SLOT / 16), a_lo = a_hi + S2_A_PART / 16, b = w0 + 2 * kc * (W_CHUNK / 16);
 #pragma unroll
@@ -327,8 +331,8 @@ struct S2Smem {
   }
 };
 
-// A worker thread's side of the forward passes.  After a timeout the abort flag is up: the waits return at once and the thread runs to
-// its end on meaningless numbers, through the same barriers as the others.
+// A worker thread's side of the forward passes.  After a timeout the abort flag is up: the thread neither waits nor hands operands over any
+// more and runs to its end on meaningless numbers, through the same barriers as the others.
 template <int D, int H, int TPR, int GROUPS>
 struct S2Worker {
   using M = S2Smem<D, H, TPR, GROUPS>;
@@ -377,17 +381,17 @@ struct S2Worker {
           w[k][2 * i] = ww.x; w[k][2 * i + 1] = ww.y;
         }
       }
-      if (chunk >= M::AS) ok = ok && tc_wait_elect(&m.ctl->a_free[as], ((chunk / M::AS) - 1) & 1, abort_flag);
+      if (chunk >= M::AS) ok = ok && tc_wait_elect<M::PAIR>(&m.ctl->a_free[as], ((chunk / M::AS) - 1) & 1, abort_flag);
       vmax = s2_layer1<D, ROWS>(w, b, x, dst + as * S2_A_SLOT, vmax);
       fence_async_smem();
       if (M::PAIR) {
         __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(&m.ctl->a_ready[as], 0);
-      } else {
+        if (lane == 0 && ok) mbar_arrive_cluster(&m.ctl->a_ready[as], 0);
+      } else if (ok) {
         mbar_arrive_warp(&m.ctl->a_ready[as]);
       }
     }
-    ok = ok && tc_wait_elect(&m.ctl->acc_full[g], pass & 1, abort_flag);
+    ok = ok && tc_wait_elect<M::PAIR>(&m.ctl->acc_full[g], pass & 1, abort_flag);
     tc_fence_after();
     // h2 = relu(acc / scale + b2) and the head's sums; s[i][a]: row lane / 4 + 8 i of the warp's 32, output a, even and odd columns apart
     f32x2 s[4][4];

@@ -7,6 +7,35 @@ from parity_util import RTOL_FP32, blob_for, fields_for
 pytestmark = pytest.mark.gpu
 
 
+def _segment(f, N, T, state, ep):
+    import torch
+    from paper_2502_20190_b200 import binding
+    ctx = binding.Context(**dict(f, n_envs=N))
+    ctx.publish_weights(blob_for(f, 1))
+    ctx.set_state(state, ep)
+    ctx.actor_step(T)
+    seg = ctx.segment_acquire()[1]
+    return [seg[k].view(torch.uint8).clone() for k in ("obs", "act", "rew", "done", "logp", "val")], ctx
+
+
+@pytest.mark.parametrize("kind,D,A,H,tiles", [(0, 4, 2, 256, 301), (1, 6, 3, 192, 150)])
+def test_a_call_repeats_itself(kind, D, A, H, tiles):
+    """64 rollouts from the same states give the same segment bit for bit.  (What a block of a pair hands to the other -- operands in its shared
+    memory, accumulators it has read -- is ordered by release and acquire at cluster scope; this would show only a gross lack of it.)"""
+    import torch
+    N, T = tiles * 128 - 5, 8
+    f = fields_for(env_kind=kind, n_envs=N, obs_dim=D, n_actions=A, hidden=H, policy_kind=1, weight_dtype=2, seed=7, replay_capacity=0, rollout_len=T,
+                   n_segments=2, staleness_bound=4, gamma=0.99, gae_lambda=0.95, max_episode_steps=5)
+    gen = torch.Generator(device="cuda").manual_seed(2)
+    state = torch.rand((N, 4), generator=gen, device="cuda") - 0.5
+    ep = torch.zeros(N, dtype=torch.int32, device="cuda")
+    first, ctx = _segment(f, N, T, state, ep)
+    assert ctx.stats()["device_error"] == 0
+    for _ in range(63):
+        again, _ = _segment(f, N, T, state, ep)
+        assert all(torch.equal(a, b) for a, b in zip(first, again))
+
+
 @pytest.mark.parametrize("kind,D,A,H,tiles,more", [(0, 4, 2, 64, 148, 1), (1, 6, 3, 128, 149, 0), (0, 4, 2, 192, 150, 0), (1, 6, 3, 256, 298, 1)])
 def test_outputs_of_every_env_and_step(kind, D, A, H, tiles, more):
     import torch

@@ -2,7 +2,7 @@
 
 The library is built once more with waits that give up at their first look (TJ_WAIT_POLLS = 0), and each case runs in a process of its
 own on that build.  Only kernels whose other waits all end are run this way: the FP32 ones, whose threads go on to the same block
-barriers, and the update's TF32 products, whose issuing warp then issues nothing."""
+barriers, and the update's TF32 products and the split-operand actor's pairs of blocks, whose issuing warp then issues nothing."""
 import os
 import subprocess
 import sys
@@ -58,6 +58,15 @@ def case_actor(H, N, steps):
     assert ctx.stats()["produced"] == 2 * steps * N
 
 
+def case_split_pairs(kind, D, A, H, N):
+    """Neither block of a pair gets its half of the hidden matrix in time: both stop, wait for their copies and leave."""
+    torch, binding, ctx, _ = _context(kind, D, A, H, N=N, weight_dtype=2)
+    ctx.actor_step(2)
+    ctx.actor_step(2)
+    _latched(torch, ctx, 4)
+    assert ctx.stats()["produced"] == 4 * N
+
+
 def _unchanged(torch, ctx, blobs, update):
     kept = [b.clone() for b in blobs]
     loss = update()
@@ -93,6 +102,8 @@ CASES = {
     "actor, two blocks per SM": (case_actor, 64, 6000, 2),
     "actor, hidden matrix through the ring": (case_actor, 256, 500, 3),
     "actor, largest ring": (case_actor, 768, 90, 2),
+    "actor, pairs of blocks, split operands": (case_split_pairs, 1, 6, 3, 256, 148 * 128 + 1),
+    "actor, pairs of blocks, split operands, two tiles each": (case_split_pairs, 0, 4, 2, 64, 300 * 128),
     "update, fused, SGD": (case_update, False, 0, 4, 2, 64, 300),
     "update, fused, Adam, several chunks of rows per block": (case_update, True, 1, 6, 3, 128, 9000),
     "update, fused, PPO": (case_ppo, 700),
