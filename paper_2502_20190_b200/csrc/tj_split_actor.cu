@@ -57,14 +57,13 @@ __device__ __forceinline__ void sa_observe(float4 s, float* obs) {
 //      compute layer 1 (calls with more tiles than SMs).  Two blocks of a cluster share every product (cta_group::2, 256 rows): each holds half
 //      of W2's rows, which then stay in shared memory for the whole call instead of passing through it once per tile and step, and a product
 //      reads 64 of the 128 bytes per cycle instead of 96;
-//   2  eight warps on one tile: each thread takes half the rows of layer 1 and half the columns of the drain, the two exchange their head
-//      sums once per step and both step the environment (one tile per SM: the chain of one step is the bound).
-// 65,536 CartPole envs, hidden 256, 128 steps: 3.69 ms with a block per tile whose threads computed layer 1 and the head each for its own
-// env, 2.80 with layer 1 and the drain as in S2Worker::forward, 2.53 as pairs.  A step of two tiles is then 18,000 cycles, 12,300 of them
-// MMAs: what bounds it is the chain layer 1 (5,500; a fence and an arrival per chunk) -> MMA of the last chunk (2,000 with its signals) ->
-// drain (4,000) -> environment (3,000) of four warps per tile.  More of them do not fit: eight warps per tile (one thread of two steps the
-// environment) spill at 96 registers, 2.73 ms.  The next columns fetched ahead in the drain: 2.62.  Arrivals of the second block through a
-// relaying warp: 4.26; with cluster-scope release semantics: 3.25.
+//   2  eight warps on one tile: each thread takes half the rows of layer 1 and two of the outputs, the two exchange their outputs once per
+//      step and both step the environment (one tile per SM: the chain of one step is the bound).
+// 65,536 CartPole envs, hidden 256, 128 steps: 3.55 ms with a block per tile whose threads computed layer 1 each for its own env, 2.77 as
+// pairs.  A step of two tiles is then about 19,500 cycles, 12,300 of them MMAs: what bounds it is the chain layer 1 (5,500; a fence and an
+// arrival per chunk) -> MMA of the last chunk (2,000 with its signals) -> drain -> environment (3,000) of four warps per tile.  More of them
+// do not fit: eight warps per tile (one thread of two steps the environment) spill at 96 registers.  Arrivals of the second block through
+// a relaying warp: 4.26.
 // Layer 1 hands 32 hidden units (one K chunk) at a time to the issuing lane through a ring of A-operand slots.
 constexpr int S2_NT = 320;                // eight worker warps on one tile, the issuing warp, the copy warp
 constexpr int S2_A_SLOTS = 8;             // most A-operand slots of a block, 16 KB each
@@ -138,21 +137,22 @@ struct S2Smem {
   static constexpr uint32_t ACC_COLS = H <= 128 ? 128 : 256;
   uint8_t *a_ring, *w_ring;
   float *w1, *b1;         // [D][H] and [H], scaled
-  float* hw;              // per pair of hidden units: second-layer biases, head weights of outputs 0, 1, 2, two floats each
-  float* hw3;             // per pair: those of output 3
+  float* hw;              // second-layer biases and head weights as the drain reads them.  TPR 1, per column c < H / 2: biases, head weights of
+                          // outputs 0, 1, 2 of hidden units c and c + H / 2; TPR 2: [2][H] head weights of outputs 0, 1 and of outputs 2, 3
+  float* hw3;             // TPR 1: head weights of output 3 of units c and c + H / 2; TPR 2: [H] second-layer biases
   float* b3;              // [4]
-  float* part;            // TPR 2: head sums [tile in flight][pass parity][half][TE][4]
+  float* part;            // TPR 2: outputs [pass parity][pair of outputs][TE][2]
   S2Ctl* ctl;
   __device__ __forceinline__ explicit S2Smem(uint8_t* base) {
     a_ring = base;
     w_ring = a_ring + AS * S2_A_SLOT;
     w1 = reinterpret_cast<float*>(w_ring + W_SLOTS * W_CHUNK);
     b1 = w1 + D * H; hw = b1 + H; hw3 = hw + 4 * H; b3 = hw3 + H; part = b3 + 4;
-    ctl = reinterpret_cast<S2Ctl*>(part + (TPR == 2 ? GROUPS * 2 * 2 * SA_TE * 4 : 0));
+    ctl = reinterpret_cast<S2Ctl*>(part + (TPR == 2 ? GROUPS * 2 * 2 * SA_TE * 2 : 0));
   }
   static size_t bytes() {
     return (size_t)AS * S2_A_SLOT + (size_t)W_SLOTS * W_CHUNK +
-           ((size_t)(D + 6) * H + 4 + (TPR == 2 ? GROUPS * 2 * 2 * SA_TE * 4 : 0)) * sizeof(float) + sizeof(S2Ctl) + 64;
+           ((size_t)(D + 6) * H + 4 + (TPR == 2 ? GROUPS * 2 * 2 * SA_TE * 2 : 0)) * sizeof(float) + sizeof(S2Ctl) + 64;
   }
 
   // barriers and tensor memory; returns its base.  Ends with a block barrier.
@@ -224,9 +224,16 @@ struct S2Smem {
 #pragma unroll
       for (int k = 0; k < D; ++k) w1[k * H + i] = SA_H_SCALE * wk[k];
       b1[i] = SA_H_SCALE * c1;
-      float* d = hw + 8 * (i >> 1) + (i & 1);
-      d[0] = c2; d[2] = w.x; d[4] = w.y; d[6] = w.z;
-      hw3[i] = w.w;
+      if (TPR == 1) {
+        const int c = i % (H / 2), upper = i / (H / 2);
+        float* d = hw + 8 * c + upper;
+        d[0] = c2; d[2] = w.x; d[4] = w.y; d[6] = w.z;
+        hw3[2 * c + upper] = w.w;
+      } else {
+        reinterpret_cast<float2*>(hw)[i] = make_float2(w.x, w.y);
+        reinterpret_cast<float2*>(hw)[H + i] = make_float2(w.z, w.w);
+        hw3[i] = c2;
+      }
     }
     if (threadIdx.x >= NT - 4) {
       const int a = threadIdx.x - (NT - 4);
@@ -349,11 +356,17 @@ struct S2Worker {
     t_row = tmem + (uint32_t)g * M::ACC_COLS + ((uint32_t)((warp & 3) * 32) << 16);
     inv_scale = inv;
   }
-  // network outputs of one observation.  What a thread keeps in registers decides what the layers read from shared memory, whose read path
-  // returns a word per lane and cycle, broadcast or not: layer 1 with a thread per environment read every weight for every environment,
-  // 320 16-byte words a thread and pass, and the drain 256, two thirds of the cycles of the read path.  So
-  //   layer 1: a lane takes eight hidden units of four (TPR 2: two) rows of its warp, eight apart, whose observations come by shuffle;
-  //   drain: fragments of 8 columns x 16 rows (a lane holds two neighbouring columns of four rows), so a weight read serves four rows.
+  // Network outputs of one observation.  What a thread keeps in registers decides what the layers read from shared memory, whose read path
+  // returns a word per lane and cycle, broadcast or not.
+  //   Layer 1: a lane takes eight hidden units of four (TPR 2: two) rows of its warp, eight apart, whose observations come by shuffle, so a
+  //   weight read serves four rows.  (A thread per environment read every weight for every environment.)
+  //   Drain: an output is (b3 + sum over the lower half of the hidden units) + sum over the upper half, both in column order from zero, in
+  //   every form and for every width.  The order is part of the result: with another one of the same rounding error about one categorical
+  //   draw in 17 million falls the other way.  It leaves a weight read two rows at most: TPR 2 gives a lane one half of the columns of two
+  //   rows and two of the outputs (actor call of four steps, 16,384 Acrobot envs, hidden 256: 45.1 us; a row and all outputs per lane, 45.7;
+  //   four rows per weight read by sums of every fourth pair of columns, 43.2).  TPR 1, where every warp has a tile's rows to itself, has a
+  //   row per lane and both halves side by side in one instruction: 65,536 CartPole envs, 128 steps 2.77 ms; two rows and one half per
+  //   lane read half as much but issue more, 3.27; double-buffered loads of 8 columns take 6 % longer, blocks of 32 columns the same.
   // `chunk`: number of this pass's first chunk in the ring's order.
   __device__ __forceinline__ void forward(const float (&obs)[6], int Aout, uint32_t chunk, float (&out)[4]) {
     constexpr int ROWS = 4 / TPR;
@@ -393,64 +406,68 @@ struct S2Worker {
     }
     ok = ok && tc_wait_elect<M::PAIR>(&m.ctl->acc_full[g], pass & 1, abort_flag);
     tc_fence_after();
-    // h2 = relu(acc / scale + b2) and the head's sums; s[i][a]: row lane / 4 + 8 i of the warp's 32, output a, even and odd columns apart
-    f32x2 s[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int a = 0; a < 4; ++a) s[i][a] = 0ull;
-    const f32x2 inv2 = dup2(inv_scale);
-    const int c_begin = half * (H / 2), c_end = TPR == 2 ? c_begin + H / 2 : H;
+    // h2 = relu(acc / scale + b2) and the head's sums
+    if (TPR == 1) {
+      const f32x2 inv2 = dup2(inv_scale);
+      f32x2 s[4] = {0ull, 0ull, 0ull, 0ull};
 #pragma unroll 1
-    for (int c0 = c_begin; c0 < c_end; c0 += 32) {
-      uint32_t u[2][16];
-      tmem_ld_16x32(t_row + (uint32_t)c0, u[0]);
-      tmem_ld_16x32(t_row + (16u << 16) + (uint32_t)c0, u[1]);
-      const float *hw = m.hw + 4 * c0 + 8 * (lane & 3), *hw3 = m.hw3 + c0 + 2 * (lane & 3);
-      tmem_ld_wait();
+      for (int c0 = 0; c0 < H / 2; c0 += 16) {
+        uint32_t u[16], v[16];
+        tmem_ld16(t_row + (uint32_t)c0, u);
+        tmem_ld16(t_row + (uint32_t)(c0 + H / 2), v);
+        tmem_ld_wait();
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const ulonglong2 p01 = ld_pairs(hw + 32 * j), p23 = ld_pairs(hw + 32 * j + 4);
-        f32x2 w3 = 0ull;
-        if (Aout > 3) w3 = *reinterpret_cast<const unsigned long long*>(hw3 + 8 * j);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const uint32_t* v = &u[i >> 1][4 * j + 2 * (i & 1)];
+        for (int i = 0; i < 16; ++i) {
+          const ulonglong2 p01 = ld_pairs(m.hw + 8 * (c0 + i)), p23 = ld_pairs(m.hw + 8 * (c0 + i) + 4);
           f32x2 h = p01.x;
-          fma2(h, pair2(__uint_as_float(v[0]), __uint_as_float(v[1])), inv2);
+          fma2(h, pair2(__uint_as_float(u[i]), __uint_as_float(v[i])), inv2);
           const float2 t = halves(h);
           h = pair2(fmaxf(t.x, 0.f), fmaxf(t.y, 0.f));
-          fma2(s[i][0], p01.y, h);
-          fma2(s[i][1], p23.x, h);
-          fma2(s[i][2], p23.y, h);
-          if (Aout > 3) fma2(s[i][3], w3, h);
+          fma2(s[0], p01.y, h);
+          fma2(s[1], p23.x, h);
+          fma2(s[2], p23.y, h);
+          if (Aout > 3) fma2(s[3], *reinterpret_cast<const unsigned long long*>(m.hw3 + 2 * (c0 + i)), h);
         }
       }
-    }
-    // the four lanes of a row meet: lane 4 r + i keeps row r + 8 i, then hands it to that row's lane
-    const bool up2 = lane & 2, up1 = lane & 1;
-    float sum[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      if (a == 3 && Aout <= 3) break;
-      float t[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) { const float2 e = halves(s[i][a]); t[i] = e.x + e.y; }
-      const float k0 = (up2 ? t[2] : t[0]) + __shfl_xor_sync(0xffffffffu, up2 ? t[0] : t[2], 2);
-      const float k1 = (up2 ? t[3] : t[1]) + __shfl_xor_sync(0xffffffffu, up2 ? t[1] : t[3], 2);
-      const float k = (up1 ? k1 : k0) + __shfl_xor_sync(0xffffffffu, up1 ? k0 : k1, 1);
-      sum[a] = __shfl_sync(0xffffffffu, k, 4 * (lane & 7) + (lane >> 3));
-    }
-    if (TPR == 1) {
-#pragma unroll
-      for (int a = 0; a < 4; ++a) out[a] = m.b3[a] + sum[a];
+      for (int a = 0; a < 4; ++a) { const float2 t = halves(s[a]); out[a] = (m.b3[a] + t.x) + t.y; }
     } else {
-      float4* px = reinterpret_cast<float4*>(m.part) + (size_t)(2 * g + (pass & 1)) * 2 * SA_TE;
-      px[half * SA_TE + row] = make_float4(sum[0], sum[1], sum[2], sum[3]);
+      // lanes r and r + 16: rows r and r + 16 of the warp's 32, lower and upper half of the columns; this warp: outputs 2 half and 2 half + 1
+      const int upper = lane >> 4;
+      const float *w = m.hw + half * 2 * H + upper * H, *b2 = m.hw3 + upper * (H / 2);
+      float s[2][2] = {{0.f, 0.f}, {0.f, 0.f}};                // [row][output]
+#pragma unroll 1
+      for (int c0 = 0; c0 < H / 2; c0 += 16) {
+        uint32_t u[2][16];
+        tmem_ld16_halves<H / 2>(t_row + (uint32_t)c0, u[0]);
+        tmem_ld16_halves<H / 2>(t_row + (16u << 16) + (uint32_t)c0, u[1]);
+        tmem_ld_wait();
+#pragma unroll
+        for (int i = 0; i < 16; i += 4) {
+          const float4 b = *reinterpret_cast<const float4*>(b2 + c0 + i), wa = *reinterpret_cast<const float4*>(w + 2 * (c0 + i)),
+                       wb = *reinterpret_cast<const float4*>(w + 2 * (c0 + i) + 4);
+          const float bv[4] = {b.x, b.y, b.z, b.w}, w0[4] = {wa.x, wa.z, wb.x, wb.z}, w1[4] = {wa.y, wa.w, wb.y, wb.w};
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+              const float h = fmaxf(fmaf(__uint_as_float(u[r][i + j]), inv_scale, bv[j]), 0.f);
+              s[r][0] = fmaf(w0[j], h, s[r][0]);
+              s[r][1] = fmaf(w1[j], h, s[r][1]);
+            }
+        }
+      }
+      float o[2];
+#pragma unroll
+      for (int a = 0; a < 2; ++a) {                            // this lane's row: one half's sum is here, the other in the lane 16 away
+        const float own = upper ? s[1][a] : s[0][a], other = __shfl_xor_sync(0xffffffffu, upper ? s[0][a] : s[1][a], 16);
+        o[a] = (m.b3[2 * half + a] + (upper ? other : own)) + (upper ? own : other);
+      }
+      float2* px = reinterpret_cast<float2*>(m.part) + (size_t)(pass & 1) * 2 * SA_TE;
+      px[half * SA_TE + row] = make_float2(o[0], o[1]);
       asm volatile("bar.sync %0, 256;" ::"r"(1 + g) : "memory");
-      const float4 l = px[row], h = px[SA_TE + row];
-      const float* b3 = m.b3;
-      out[0] = (b3[0] + l.x) + h.x; out[1] = (b3[1] + l.y) + h.y; out[2] = (b3[2] + l.z) + h.z; out[3] = (b3[3] + l.w) + h.w;
+      const float2 o01 = px[row], o23 = px[SA_TE + row];
+      out[0] = o01.x; out[1] = o01.y; out[2] = o23.x; out[3] = o23.y;
     }
     ++pass;
   }
@@ -638,7 +655,7 @@ __global__ void __launch_bounds__(S2_NT, 1) td_split_tc_kernel(const TdParams p,
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int net = (int)(blockIdx.x & 1u), tile = (int)(blockIdx.x >> 1);   // the cluster is blocks 2 t and 2 t + 1
   const int j = tile * SA_TE + (tid & (SA_TE - 1));
-  float* qmax = m.part + 2 * SA_TE * 4;                       // the exchange area of the pass that never comes
+  float* qmax = m.part + 2 * SA_TE * 2;                       // the exchange area of the pass that never comes
   const uint32_t tmem = m.set_up();
   chain_begin();
   m.stage(p, net ? p.Wtarget : p.Wonline, p.A);
