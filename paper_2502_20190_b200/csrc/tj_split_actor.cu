@@ -59,8 +59,8 @@ __device__ __forceinline__ void sa_observe(float4 s, float* obs) {
 //      reads 64 of the 128 bytes per cycle instead of 96;
 //   2  eight warps on one tile: each thread takes half the rows of layer 1 and two of the outputs, the two exchange their outputs once per
 //      step and both step the environment (one tile per SM: the chain of one step is the bound).
-// 65,536 CartPole envs, hidden 256, 128 steps: 3.55 ms with a block per tile whose threads computed layer 1 each for its own env, 2.77 as
-// pairs.  A step of two tiles is then about 19,500 cycles, 12,300 of them MMAs: what bounds it is the chain layer 1 (5,500; a fence and an
+// 65,536 CartPole envs, hidden 256, 128 steps: 3.55 ms with a block per tile whose threads computed layer 1 each for its own env, 2.86 as
+// pairs.  A step of two tiles is then about 20,000 cycles, 12,300 of them MMAs: what bounds it is the chain layer 1 (5,500; a fence and an
 // arrival per chunk) -> MMA of the last chunk (2,000 with its signals) -> drain -> environment (3,000) of four warps per tile.  More of them
 // do not fit: eight warps per tile (one thread of two steps the environment) spill at 96 registers.  Arrivals of the second block through
 // a relaying warp: 4.26.
@@ -107,14 +107,18 @@ __device__ __forceinline__ float s2_layer1(const f32x2 (&w)[D][4], const f32x2 (
     uint32_t hi[4], lo[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      // the high part is the value cut to 11 bits, so the remainder has the value's sign and both conversions clamp: no maximum of its own
+      // The ReLU is a maximum, which takes a NaN to 0 as in the other weight modes (a clamping conversion hands it on).  The high part is the
+      // value cut to 11 bits, then converted: below 2^-14, where FP16 has fewer, rounding that is exact to 2^-25, a truncating conversion of
+      // the whole value to 2^-24.
       const float2 a = halves(acc[i]);
-      vmax = max3(vmax, a.x, a.y);
-      f32x2 rest = acc[i];
-      fma2(rest, pair2(__uint_as_float(__float_as_uint(a.x) & 0xFFFFE000u), __uint_as_float(__float_as_uint(a.y) & 0xFFFFE000u)), minus1);
+      const float v0 = fmaxf(a.x, 0.f), v1 = fmaxf(a.y, 0.f);
+      vmax = max3(vmax, v0, v1);
+      const float h0 = __uint_as_float(__float_as_uint(v0) & 0xFFFFE000u), h1 = __uint_as_float(__float_as_uint(v1) & 0xFFFFE000u);
+      f32x2 rest = pair2(v0, v1);
+      fma2(rest, pair2(h0, h1), minus1);
       const float2 d = halves(rest);
-      hi[i] = pack_f16x2_rz_relu(a.x, a.y);
-      lo[i] = pack_f16x2_relu(d.x, d.y);
+      hi[i] = pack_f16x2(h0, h1);
+      lo[i] = pack_f16x2(d.x, d.y);
     }
     *reinterpret_cast<uint4*>(hi_dst + r * ((SA_KC / 8) * 128)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
     *reinterpret_cast<uint4*>(hi_dst + S2_A_PART + r * ((SA_KC / 8) * 128)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
@@ -631,8 +635,8 @@ __global__ void __launch_bounds__(128 * TPR * GROUPS + 64, 1) actor_split_tc_ker
       n_episodes = 0;
       ret_sum = 0.0;
     }
-    // 65,504 is FP16's largest finite value (the comparison is written to catch a NaN too)
-    if (!(wk.vmax <= 65504.f)) m.ctl->range_flag = 1;
+    // 65,504 is FP16's largest finite value
+    if (wk.vmax > 65504.f) m.ctl->range_flag = 1;
   }
   m.tear_down(tmem);
   if (tid == 0) {
@@ -683,7 +687,7 @@ __global__ void __launch_bounds__(S2_NT, 1) td_split_tc_kernel(const TdParams p,
       }
     }
     wk.forward(obs, p.A, 0u, out);
-    if (!(wk.vmax <= 65504.f)) m.ctl->range_flag = 1;
+    if (wk.vmax > 65504.f) m.ctl->range_flag = 1;
     if (row_thread && net == 1) {
       float q = out[0];
       for (int i = 1; i < p.A; ++i) q = fmaxf(q, i == 1 ? out[1] : (i == 2 ? out[2] : out[3]));

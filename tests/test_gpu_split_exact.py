@@ -73,3 +73,36 @@ def test_head_sums_run_over_both_halves_in_column_order(kind, H, on_policy, N):
         want[:, a] = (b3[a] + half[0]) + half[1]
     assert np.array_equal(got.view(np.uint32), want.view(np.uint32))
     assert ctx.stats()["device_error"] == 0
+
+
+@pytest.mark.parametrize("N,H", [(5000, 64), (PAIRS, 128)])
+def test_small_activations_keep_their_rounding(N, H):
+    """Scaled activations around FP16's smallest normal number, 2^-14: the high part is the value cut to 11 bits and rounded to FP16, the low part
+    the rounded remainder; an output that takes one unit is the sum of the two."""
+    rng = np.random.default_rng(4)
+    b, unit_input = _blob(rng, 0, H, False)
+    for k in ("b2", "W3", "b3"):
+        b[k][:] = 0
+    b["W1"] = np.abs(b["W1"])
+    b["W3"][0, 0] = b["W3"][1, H - 1] = 1
+    state = np.exp2(rng.uniform(-24, -10, (N, 4))).astype(np.float32)
+    got, _ = _run(0, False, N, b, state)
+    for out, unit in ((0, 0), (1, H - 1)):
+        v = np.float32(16) * b["W1"][unit, unit_input[unit]] * state[:, unit_input[unit]]
+        cut = (v.view(np.uint32) & np.uint32(0xFFFFE000)).view(np.float32)
+        want = (cut.astype(np.float16).astype(np.float32) + (v - cut).astype(np.float16).astype(np.float32)) / np.float32(16)
+        assert (v < 2.0 ** -14).mean() > 0.2
+        assert np.array_equal(got[:, out].view(np.uint32), want.view(np.uint32))
+
+
+@pytest.mark.parametrize("N", [300, PAIRS])
+def test_a_nan_before_the_relu_is_zero_behind_it_as_in_the_fp32_mode(N):
+    rng = np.random.default_rng(6)
+    b, _ = _blob(rng, 0, 64, True)
+    b["W1"][5] = np.nan
+    b["b1"][40] = np.nan
+    state = (rng.integers(-4096, 4096, (N, 4)) / 4096).astype(np.float32)
+    (split, ctx), (fp32, _) = _run(0, True, N, b, state), _run(0, True, N, b, state, W=0)
+    assert np.isfinite(fp32).all()
+    assert np.allclose(split, fp32, rtol=1e-5, atol=1e-5 * float(np.sqrt(np.mean(fp32 ** 2))))
+    assert ctx.stats()["device_error"] == 0
