@@ -483,7 +483,8 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
           // s' = tanh(z + B[a]) + noise; piece k4 = components 4 k4 .. 4 k4 + 3 = one Philox block
           // z, B's row and the counters are on their way while the noise, which needs none of them, is made (a row group took 6,900 cycles
           // with every load behind the instructions that its use follows, 6,000 now)
-          float4 zz[4], bb[4], nz[4], sn[4];
+          float4 zz[4], bb[4], sn[4];
+          float3 n01[4], n23[4];
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             zz[i] = load_f4_cg(zs + ((size_t)(e_kq + 8 * i) * PA_M + rr) * 4);
@@ -492,18 +493,18 @@ __global__ void __launch_bounds__(PA_THREADS, 1) actor_tc_pipelined_kernel(const
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             const uint4 w = stream_words(ev.seed, STREAM_NOISE, (uint32_t)(e_kq + 8 * i), (uint32_t)row, ev.t + step);
-            const float2 n01 = box_muller_scaled(w.x, w.y, ev.noise_std), n23 = box_muller_scaled(w.z, w.w, ev.noise_std);
-            nz[i] = make_float4(n01.x, n01.y, n23.x, n23.y);
+            n01[i] = box_muller_scaled(w.x, w.y, ev.noise_std);
+            n23[i] = box_muller_scaled(w.z, w.w, ev.noise_std);
           }
           float sq = 0.f;
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             const int k4 = e_kq + 8 * i;
             float4 o;
-            o.x = tanh_from_t(fmaf(zz[i].x, zc, bb[i].x)) + nz[i].x;
-            o.y = tanh_from_t(fmaf(zz[i].y, zc, bb[i].y)) + nz[i].y;
-            o.z = tanh_from_t(fmaf(zz[i].z, zc, bb[i].z)) + nz[i].z;
-            o.w = tanh_from_t(fmaf(zz[i].w, zc, bb[i].w)) + nz[i].w;
+            o.x = fmaf(n01[i].x, n01[i].y, tanh_from_t(fmaf(zz[i].x, zc, bb[i].x)));
+            o.y = fmaf(n01[i].x, n01[i].z, tanh_from_t(fmaf(zz[i].y, zc, bb[i].y)));
+            o.z = fmaf(n23[i].x, n23[i].y, tanh_from_t(fmaf(zz[i].z, zc, bb[i].z)));
+            o.w = fmaf(n23[i].x, n23[i].z, tanh_from_t(fmaf(zz[i].w, zc, bb[i].w)));
             sq = fmaf(o.x, o.x, sq); sq = fmaf(o.y, o.y, sq); sq = fmaf(o.z, o.z, sq); sq = fmaf(o.w, o.w, sq);
             sn[i] = o;
             if (live) __stcs(reinterpret_cast<float4*>(rec + D + 4 * k4), o);
