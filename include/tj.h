@@ -203,8 +203,10 @@ int tj_destroy(tj_ctx *ctx);
  * when to send it; dependency I as an asynchronous exchange).  `blob` holds FP32
  *   [W1 HxD, b1 H, W2 HxH, b2 H, W3 AxH, b3 A (, Wv 1xH, bv 1 when policy_kind = categorical)]
  * row-major (out x in); nbytes must match exactly.  on_device = 0: host pointer, copied with an asynchronous
- * host-to-device copy on the stream (pageable memory is staged before the call returns) or, up to 512 KB of page-locked memory,
- * read by the publish itself (page-locked memory must stay unchanged until the stream has passed the publish); 1: device pointer (read on the stream).  The new parameters become version+1 (returned in version_out)
+ * host-to-device copy on the stream (pageable memory is staged before the call returns) or, up to 512 KB of
+ * page-locked memory, read by the publish itself.  Either way page-locked memory must stay allocated and unchanged
+ * until the stream has passed the whole publish, and a publish captured in a graph reads it at every replay.
+ * on_device = 1: device pointer (read on the stream).  The new parameters become version+1 (returned in version_out)
  * and are what the actor uses from its next call and what the learner's online forward uses.  The target
  * network takes the same parameters on the first publish and then on the first publish after
  * target_sync_interval further learner steps.  With TJ_W_BF16 the weight matrices are rounded to bfloat16

@@ -424,8 +424,10 @@ int tj_set_profiling(tj_ctx* x, int32_t on) {
 namespace {
 // Page-locked host memory as the publish kernel can read it, null where the blob has to be copied first: pageable memory, an allocation
 // that ends before the blob does, and large blobs.  A copy in front of the kernel costs its own start and the overlap of the kernel's
-// launch with the tail of the one before (publish and one actor step, copy / no copy: 18 KB 14.3 / 11.9 us, 70 KB 15.1 / 10.4,
-// 166 KB 22.4 / 14.2, 270 KB 34.2 / 22.6, 473 KB 52.7 / 45.0: the copy engine's rate gains on the kernel's).
+// launch with the tail of the one before (publish and one actor step of 256 envs, copy / no copy, us: 18 KB 15.0 / 9.5, 70 KB 17.0 / 12.2,
+// 270 KB 29.1 / 25.5, 473 KB 49.1 / 45.6, 513 KB 49.6 / 49.3: the copy engine's rate gains on the kernel's).  The kernel holds its SMs while
+// it reads, but beside an actor on another stream that costs less than the copy does (four steps of 4,096 CartPole envs, sample, TD error
+// and publish on two streams: hidden 128, 70 KB 54.4 / 49.7; 256, 270 KB 142.7 / 130.5; 354, 513 KB 275.2 / 257.9).
 constexpr size_t kMappedBlobBytes = 512 * 1024;
 const float* mapped_blob(const void* blob, size_t nbytes) {
   typedef CUresult (*Query)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
