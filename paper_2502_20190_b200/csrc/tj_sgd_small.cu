@@ -59,7 +59,7 @@ struct FsLayout {
   int ldD, ldH, Hp;
   int W2, W3, b2, b3, T2, T3, tb2, tb3, xs, xn, h1, h2, d1, d2, g, q, part, one, red, bar, total;
   int G, T, KS, KB;                                // neuron quads; 4 x 4 output tiles of a hidden layer; shares of a contraction, of the backward one
-  int bulk;                                        // rows of the parameter blobs are whole 16-byte words
+  int words16;                                     // rows of the parameter blobs are whole 16-byte words
 };
 
 inline FsLayout fs_layout(int D, int H, int R, bool ppo) {
@@ -94,7 +94,7 @@ inline FsLayout fs_layout(int D, int H, int R, bool ppo) {
   if (o + red() + 8 > 227 * 256) L.KS = L.KB = 1;
   L.red = take(red());                             // only where a layer's contraction is split
   L.bar = take(8);
-  L.bulk = 0;
+  L.words16 = 0;
   L.total = o;
   return L;
 }
@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(FS_NT, 1) sgd_fused_kernel(const SgdParams p, 
   tb.T = L.T; tb.KS = L.KB;
   tb.share = tid / L.T; tb.tile = tid - tb.share * L.T; tb.g = tb.tile / (R / 4); tb.rg = tb.tile % (R / 4);
   tb.active = tb.share < L.KB;
-  if (L.bulk && tid == 0) mbar_init(bar, FS_NT);
+  if (L.words16 && tid == 0) mbar_init(bar, FS_NT);
   __syncthreads();
   chain_begin();
   const int o_b1 = H * D, o_W2 = o_b1 + H, o_b2 = o_W2 + H * H, o_W3 = o_b2 + H, o_b3 = o_W3 + A * H;
@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(FS_NT, 1) sgd_fused_kernel(const SgdParams p, 
     if (a < A) head_bias = __ldg((tid >> 2 ? p.theta_target : p.theta) + o_b3 + a);
     else if (PPO && a == A) head_bias = __ldg(p.theta + o_b3 + A + H);
   }
-  if (PPO && L.bulk && tid < H) head_value = __ldg(p.theta + o_b3 + A + tid);
+  if (PPO && L.words16 && tid < H) head_value = __ldg(p.theta + o_b3 + A + tid);
   // a chunk's rows: element k of row r by thread 8 r + k, the row's scalars by thread r
   float x = 0.f, y = 0.f, rew = 0.f, adv = 0.f, ret = 0.f;
   int act = 0, done = 0;
@@ -367,7 +367,7 @@ __global__ void __launch_bounds__(FS_NT, 1) sgd_fused_kernel(const SgdParams p, 
     }
   };
   fetch_rows(blockIdx.x);
-  if (L.bulk) {
+  if (L.words16) {
     // a thread copies one 16-byte column of every RP-th row of the hidden matrices, the first rows' threads the head and the biases too.
     // (One bulk copy per row, issued by a thread per row, took 32 cycles each, one after the other: 4,400 cycles for two networks at
     // hidden 64, a quarter of the kernel.)
@@ -401,7 +401,7 @@ __global__ void __launch_bounds__(FS_NT, 1) sgd_fused_kernel(const SgdParams p, 
     cp_async_commit();
   }
   if (tid < (PPO ? 4 : 8)) sm[(tid >> 2 ? L.tb3 : L.b3) + (tid & 3)] = head_bias;
-  if (L.bulk && tid < H)
+  if (L.words16 && tid < H)
     for (int a = A; a < 4; ++a) {                  // zeros for the head's unused outputs (PPO's value head is output A)
       sm[L.W3 + a * L.ldH + tid] = PPO && a == A ? head_value : 0.f;
       if (!PPO) sm[L.T3 + a * L.ldH + tid] = 0.f;
@@ -418,7 +418,7 @@ __global__ void __launch_bounds__(FS_NT, 1) sgd_fused_kernel(const SgdParams p, 
       sm[L.xs + (tid >> 3) * L.ldD + (tid & 7)] = x;
       if (!PPO) sm[L.xn + (tid >> 3) * L.ldD + (tid & 7)] = y;
     }
-    if (!L.bulk) cp_async_wait<0>();
+    if (!L.words16) cp_async_wait<0>();
     __syncthreads();
     if (n < L.Hp) {
 #pragma unroll 1
@@ -437,7 +437,7 @@ __global__ void __launch_bounds__(FS_NT, 1) sgd_fused_kernel(const SgdParams p, 
       }
     }
     __syncthreads();
-    if (L.bulk) ok = ok && mbar_wait_bounded(bar, 0);
+    if (L.words16) ok = ok && mbar_wait_bounded(bar, 0);
     // both networks side by side: the target's activations lie in d1, d2
     dense_rows<R>(sm + (target ? L.T2 : L.W2), L.ldH, sm + (target ? L.tb2 : L.b2), sm + (target ? L.d1 : L.h1), L.ldH, sm + (target ? L.d2 : L.h2),
                   L.ldH, G, G, t, sm + L.red);
@@ -589,7 +589,7 @@ __global__ void __launch_bounds__(FS_NT, 1) sgd_fused_kernel(const SgdParams p, 
   }
   if (!ok) {
     update_failed(p.watch);
-    if (L.bulk) mbar_settle(bar, 0);
+    if (L.words16) mbar_settle(bar, 0);
   }
 }
 
@@ -668,7 +668,7 @@ template <int R, bool PPO>
 cudaError_t launch_fused(const SgdParams& p, int stride, int grid, cudaStream_t s) {
   FsLayout L = fs_layout(p.D, p.H, R, PPO);
   // H a multiple of four makes every row and the start of W2, W3 and the hidden biases whole 16-byte words of the blob
-  L.bulk = p.H % 4 == 0 && ((reinterpret_cast<uintptr_t>(p.theta) | reinterpret_cast<uintptr_t>(p.theta_target)) & 15) == 0;
+  L.words16 = p.H % 4 == 0 && ((reinterpret_cast<uintptr_t>(p.theta) | reinterpret_cast<uintptr_t>(p.theta_target)) & 15) == 0;
   return launch_chained(sgd_fused_kernel<R, PPO>, grid, FS_NT, (size_t)L.total * sizeof(float), s, p, L, stride);
 }
 

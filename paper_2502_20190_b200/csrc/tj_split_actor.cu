@@ -65,7 +65,7 @@ __device__ __forceinline__ void sa_observe(float4 s, float* obs) {
 // do not fit: eight warps per tile (one thread of two steps the environment) spill at 96 registers.  Arrivals of the second block through
 // a relaying warp: 4.26.
 // Layer 1 hands 32 hidden units (one K chunk) at a time to the issuing lane through a ring of A-operand slots.
-constexpr int S2_NT = 320;                // eight worker warps on one tile, the issuing warp, the copy warp
+constexpr int S2_NT = 320;                // eight worker warps (on one tile or on two), the issuing warp, the copy warp
 constexpr int S2_A_SLOTS = 8;             // most A-operand slots of a block, 16 KB each
 constexpr int S2_A_PART = SA_TE * SA_KC * 2;
 constexpr int S2_A_SLOT = 2 * S2_A_PART;  // high part, low part
@@ -127,17 +127,18 @@ __device__ __forceinline__ float s2_layer1(const f32x2 (&w)[D][4], const f32x2 (
 }
 
 // where everything lies in shared memory
-template <int D, int H, int TPR, int GROUPS>
+template <int D, int H, int TPR>
 struct S2Smem {
-  static constexpr bool PAIR = GROUPS == 2;                   // two blocks share every product
+  static constexpr bool PAIR = TPR == 1;                      // two blocks share every product
+  static constexpr int GROUPS = PAIR ? 2 : 1;                 // tiles in flight per block
   static constexpr uint32_t CHUNK_BYTES = H * SA_KC * 2;      // one chunk of one part of W2
   static constexpr uint32_t W_CHUNK = PAIR ? CHUNK_BYTES / 2 : CHUNK_BYTES;      // what of it lies in this block
   static constexpr int NKC = H / SA_KC, NSTREAM = 2 * NKC;
   static constexpr int W_SLOTS = PAIR ? NSTREAM : SA_SLOTS;
-  // A slots: one ring that the groups' passes go through in turn; threads.  A worker waits only for the chunks whose slots it takes over, so
+  // A slots: one ring that the groups' passes go through in turn.  A worker waits only for the chunks whose slots it takes over, so
   // the one two rounds of the ring back must be known to be used up: the ring holds more than half of two passes' chunks
-  static constexpr int AS = PAIR && H > 192 ? 5 : S2_A_SLOTS, NT = 128 * TPR * GROUPS + 64;
-  static_assert(2 * AS > NKC || GROUPS == 1, "the phase of a slot's barrier is unambiguous");
+  static constexpr int AS = PAIR && H > 192 ? 5 : S2_A_SLOTS;
+  static_assert(2 * AS > NKC || !PAIR, "the phase of a slot's barrier is unambiguous");
   static constexpr uint32_t ACC_COLS = H <= 128 ? 128 : 256;
   uint8_t *a_ring, *w_ring;
   float *w1, *b1;         // [D][H] and [H], scaled
@@ -152,11 +153,11 @@ struct S2Smem {
     w_ring = a_ring + AS * S2_A_SLOT;
     w1 = reinterpret_cast<float*>(w_ring + W_SLOTS * W_CHUNK);
     b1 = w1 + D * H; hw = b1 + H; hw3 = hw + 4 * H; b3 = hw3 + H; part = b3 + 4;
-    ctl = reinterpret_cast<S2Ctl*>(part + (TPR == 2 ? GROUPS * 2 * 2 * SA_TE * 2 : 0));
+    ctl = reinterpret_cast<S2Ctl*>(part + (TPR == 2 ? 2 * 2 * SA_TE * 2 : 0));
   }
   static size_t bytes() {
     return (size_t)AS * S2_A_SLOT + (size_t)W_SLOTS * W_CHUNK +
-           ((size_t)(D + 6) * H + 4 + (TPR == 2 ? GROUPS * 2 * 2 * SA_TE * 2 : 0)) * sizeof(float) + sizeof(S2Ctl) + 64;
+           ((size_t)(D + 6) * H + 4 + (TPR == 2 ? 2 * 2 * SA_TE * 2 : 0)) * sizeof(float) + sizeof(S2Ctl) + 64;
   }
 
   // barriers and tensor memory; returns its base.  Ends with a block barrier.
@@ -190,7 +191,7 @@ struct S2Smem {
   __device__ __forceinline__ void tear_down(uint32_t tmem) const {
     tc_fence_before();
     __syncthreads();
-    const bool issuing_warp = (int)(threadIdx.x >> 5) == NT / 32 - 2;     // the last but one
+    const bool issuing_warp = (int)(threadIdx.x >> 5) == S2_NT / 32 - 2;  // the last but one
     if (PAIR) {
       // Neither block leaves before the products that read both blocks' operands are over and the last arrival has reached the first one.
       // Where one block gives up, the other follows: a warp whose wait ran out arrives no more, so the first block's issuing warp waits in
@@ -219,7 +220,7 @@ struct S2Smem {
   // the parameters around the hidden matrix, from the packed FP32 layout P describes
   template <typename P>
   __device__ __forceinline__ void stage(const P& p, const float* W, int Aout) const {
-    for (int i = threadIdx.x; i < H; i += NT) {
+    for (int i = threadIdx.x; i < H; i += S2_NT) {
       float wk[D];
 #pragma unroll
       for (int k = 0; k < D; ++k) wk[k] = __ldg(W + p.off_W1t + k * H + i);
@@ -239,8 +240,8 @@ struct S2Smem {
         hw3[i] = c2;
       }
     }
-    if (threadIdx.x >= NT - 4) {
-      const int a = threadIdx.x - (NT - 4);
+    if (threadIdx.x >= S2_NT - 4) {
+      const int a = threadIdx.x - (S2_NT - 4);
       b3[a] = a < Aout ? __ldg(W + p.off_b3 + a) : 0.f;
     }
   }
@@ -287,8 +288,8 @@ struct S2Smem {
     ctl->copies = NSTREAM;
     if (tc_wait(&ctl->full[0], 0, &ctl->abort_flag)) mbar_arrive_cluster(&ctl->w_ready, 0);
   }
-  // Issuing warp: the MMAs of n_pass passes over each of `tiles` tiles, the groups' passes in turn
-  __device__ __forceinline__ void issue(uint32_t tmem, int tiles, int n_pass) const {
+  // Issuing warp of a block on its own: the MMAs of `passes` passes, one after the other
+  __device__ __forceinline__ void issue(uint32_t tmem, uint32_t passes) const {
     volatile int* abort_flag = &ctl->abort_flag;
     const uint32_t leader = elect_one();
     const uint32_t idesc = make_idesc_f16(H);
@@ -296,36 +297,31 @@ struct S2Smem {
     const uint32_t hiword = desc_hi((uint32_t)(SA_KC / 8) * 128u);            // A slots and W2 chunks: 32 columns wide
     uint32_t wc = 0, ac = 0;
     bool alive = true;
-    for (int r = 0; r * GROUPS < tiles && alive; ++r)
-      for (int i = 0; i < n_pass && alive; ++i)
-#pragma unroll
-        for (int g = 0; g < GROUPS; ++g) {
-          if (!alive || r * GROUPS + g >= tiles) break;
-          const uint32_t acc = tmem + (uint32_t)g * ACC_COLS;
+    for (uint32_t i = 0; i < passes && alive; ++i) {
 #pragma unroll 1
-          for (int kc = 0; kc < NKC; ++kc, ++ac) {
-            const uint32_t as = ac % AS;
-            if (!tc_wait_warp(&ctl->a_ready[as], (ac / AS) & 1, abort_flag)) { alive = false; break; }
-            tc_fence_after();
-            const uint32_t a_hi = a0 + as * (S2_A_SLOT / 16), a_lo = a_hi + S2_A_PART / 16;
+      for (int kc = 0; kc < NKC; ++kc, ++ac) {
+        const uint32_t as = ac % AS;
+        if (!tc_wait_warp(&ctl->a_ready[as], (ac / AS) & 1, abort_flag)) { alive = false; break; }
+        tc_fence_after();
+        const uint32_t a_hi = a0 + as * (S2_A_SLOT / 16), a_lo = a_hi + S2_A_PART / 16;
 #pragma unroll
-            for (int half = 0; half < 2; ++half, ++wc) {
-              const uint32_t s = wc % SA_SLOTS;
-              if (!tc_wait_warp(&ctl->full[s], (wc / SA_SLOTS) & 1, abort_flag)) { alive = false; break; }
-              tc_fence_after();
-              const uint32_t b = w0 + s * (CHUNK_BYTES / 16);
+        for (int half = 0; half < 2; ++half, ++wc) {
+          const uint32_t s = wc % SA_SLOTS;
+          if (!tc_wait_warp(&ctl->full[s], (wc / SA_SLOTS) & 1, abort_flag)) { alive = false; break; }
+          tc_fence_after();
+          const uint32_t b = w0 + s * (CHUNK_BYTES / 16);
 #pragma unroll
-              for (int j = 0; j < SA_KC / 16; ++j) {
-                umma_ss(acc, a_hi + 16u * j, hiword, b + 16u * j, hiword, idesc, (kc | half | j) != 0, leader);
-                if (half == 0) umma_ss(acc, a_lo + 16u * j, hiword, b + 16u * j, hiword, idesc, 1u, leader);
-              }
-              umma_commit(&ctl->empty[s], leader);
-            }
-            if (!alive) break;
-            umma_commit(&ctl->a_free[as], leader);
+          for (int j = 0; j < SA_KC / 16; ++j) {
+            umma_ss(tmem, a_hi + 16u * j, hiword, b + 16u * j, hiword, idesc, (kc | half | j) != 0, leader);
+            if (half == 0) umma_ss(tmem, a_lo + 16u * j, hiword, b + 16u * j, hiword, idesc, 1u, leader);
           }
-          umma_commit(&ctl->acc_full[g], leader);
+          umma_commit(&ctl->empty[s], leader);
         }
+        if (!alive) break;
+        umma_commit(&ctl->a_free[as], leader);
+      }
+      umma_commit(&ctl->acc_full[0], leader);
+    }
   }
   // Copy lane: W2's parts, chunk by chunk, `passes` times
   __device__ __forceinline__ void copy(const uint16_t* parts, uint32_t passes) const {
@@ -344,17 +340,17 @@ struct S2Smem {
 
 // A worker thread's side of the forward passes.  After a timeout the abort flag is up: the thread neither waits nor hands operands over any
 // more and runs to its end on meaningless numbers, through the same barriers as the others.
-template <int D, int H, int TPR, int GROUPS>
+template <int D, int H, int TPR>
 struct S2Worker {
-  using M = S2Smem<D, H, TPR, GROUPS>;
+  using M = S2Smem<D, H, TPR>;
   const M& m;
-  int g, half, row;                                           // tile in flight, half of the columns, row of the tile = TMEM lane
+  int g, half, row;                                           // tile in flight (TPR 2: 0), which thread of its env, row of the tile = TMEM lane
   uint32_t t_row, pass = 0;
   float inv_scale, vmax = 0.f;                                // 1 / (activation scale x weight scale); largest scaled activation
   bool ok = true;
   __device__ __forceinline__ S2Worker(const M& mm, uint32_t tmem, float inv) : m(mm) {
     const int warp = threadIdx.x >> 5;
-    g = warp / (4 * TPR);
+    g = TPR == 1 ? warp >> 2 : 0;
     half = TPR == 2 ? (warp >> 2) & 1 : 0;
     row = threadIdx.x & (SA_TE - 1);
     t_row = tmem + (uint32_t)g * M::ACC_COLS + ((uint32_t)((warp & 3) * 32) << 16);
@@ -469,7 +465,7 @@ struct S2Worker {
       }
       float2* px = reinterpret_cast<float2*>(m.part) + (size_t)(pass & 1) * 2 * SA_TE;
       px[half * SA_TE + row] = make_float2(o[0], o[1]);
-      asm volatile("bar.sync %0, 256;" ::"r"(1 + g) : "memory");
+      asm volatile("bar.sync 1, 256;" ::: "memory");
       const float2 o01 = px[row], o23 = px[SA_TE + row];
       out[0] = o01.x; out[1] = o01.y; out[2] = o23.x; out[3] = o23.y;
     }
@@ -477,17 +473,18 @@ struct S2Worker {
   }
 };
 
-template <int ENV, int H, int TPR, int GROUPS>
-__global__ void __launch_bounds__(128 * TPR * GROUPS + 64, 1) actor_split_tc_kernel(const ActorParams p, const S2Plan pl, const uint16_t* __restrict__ w2parts,
-                                                                 const float* __restrict__ w2scale) {
+template <int ENV, int H, int TPR>
+__global__ void __launch_bounds__(S2_NT, 1) actor_split_tc_kernel(const ActorParams p, const S2Plan pl, const uint16_t* __restrict__ w2parts,
+                                                                  const float* __restrict__ w2scale) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   constexpr int D = ENV == TJ_ENV_CARTPOLE ? 4 : 6;
-  constexpr int WW = 4 * TPR * GROUPS;                        // worker warps, then the issuing warp and the copy warp
-  using M = S2Smem<D, H, TPR, GROUPS>;
+  constexpr int WW = S2_NT / 32 - 2;                          // worker warps, then the issuing warp and the copy warp
+  using M = S2Smem<D, H, TPR>;
+  constexpr int GROUPS = M::GROUPS;
   const M m(smem_raw);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // a pair of blocks walks tiles of 256 envs, each block its 128 of them
-  constexpr int BLOCKS = GROUPS == 2 ? 2 : 1;
+  constexpr int BLOCKS = M::PAIR ? 2 : 1;
   const int n_tiles = (p.N + SA_TE * BLOCKS - 1) / (SA_TE * BLOCKS), walker = (int)blockIdx.x / BLOCKS, walkers = (int)gridDim.x / BLOCKS;
   const bool on_policy = p.C == 0;
   const uint32_t tmem = m.set_up();
@@ -497,18 +494,18 @@ __global__ void __launch_bounds__(128 * TPR * GROUPS + 64, 1) actor_split_tc_ker
   __syncthreads();
   if (warp == WW + 1) {
     if (lane == 0) {
-      if constexpr (GROUPS == 2) m.copy_half(w2parts);
+      if constexpr (M::PAIR) m.copy_half(w2parts);
       else m.copy(w2parts, (uint32_t)my_tiles * (uint32_t)pl.n_pass);
     }
     __syncwarp();
   } else if (warp == WW) {
-    if constexpr (GROUPS == 2) {
+    if constexpr (M::PAIR) {
       if (cluster_rank() == 0) m.issue_pair(tmem, my_tiles, pl.n_pass);
     } else {
-      m.issue(tmem, my_tiles, pl.n_pass);
+      m.issue(tmem, (uint32_t)my_tiles * (uint32_t)pl.n_pass);
     }
   } else {
-    S2Worker<D, H, TPR, GROUPS> wk(m, tmem, __ldg(w2scale + 1));
+    S2Worker<D, H, TPR> wk(m, tmem, __ldg(w2scale + 1));
     const int g = wk.g, half = wk.half, row = wk.row;
     unsigned long long n_episodes = 0;
     double ret_sum = 0.0;
@@ -655,7 +652,7 @@ __global__ void __launch_bounds__(S2_NT, 1) td_split_tc_kernel(const TdParams p,
                                                               const uint16_t* __restrict__ parts_target,
                                                               const float* __restrict__ scale_target) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  const S2Smem<D, H, 2, 1> m(smem_raw);
+  const S2Smem<D, H, 2> m(smem_raw);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int net = (int)(blockIdx.x & 1u), tile = (int)(blockIdx.x >> 1);   // the cluster is blocks 2 t and 2 t + 1
   const int j = tile * SA_TE + (tid & (SA_TE - 1));
@@ -672,9 +669,9 @@ __global__ void __launch_bounds__(S2_NT, 1) td_split_tc_kernel(const TdParams p,
     if (lane == 0) m.copy(net ? parts_target : parts_online, 1u);
     __syncwarp();
   } else if (warp == 8) {
-    m.issue(tmem, 1, 1);
+    m.issue(tmem, 1u);
   } else {
-    S2Worker<D, H, 2, 1> wk(m, tmem, __ldg((net ? scale_target : scale_online) + 1));
+    S2Worker<D, H, 2> wk(m, tmem, __ldg((net ? scale_target : scale_online) + 1));
     const float* x = net ? p.next_obs : p.obs;
     float obs[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (live) {
@@ -740,20 +737,19 @@ cudaError_t launch_pairs(void (*kernel)(P...), int grid, int threads, size_t sme
 }
 
 template <int ENV, int H>
-cudaError_t launch_split(const ActorParams& p, const S2Plan& pl, const uint16_t* w2parts, const float* w2scale, int grid, int groups, cudaStream_t s) {
+cudaError_t launch_split(const ActorParams& p, const S2Plan& pl, const uint16_t* w2parts, const float* w2scale, int grid, bool pairs, cudaStream_t s) {
   constexpr int D = ENV == TJ_ENV_CARTPOLE ? 4 : 6;
-  if (groups == 1)
-    return launch_chained(actor_split_tc_kernel<ENV, H, 2, 1>, grid, S2Smem<D, H, 2, 1>::NT, S2Smem<D, H, 2, 1>::bytes(), s, p, pl, w2parts, w2scale);
-  return launch_pairs(actor_split_tc_kernel<ENV, H, 1, 2>, grid, S2Smem<D, H, 1, 2>::NT, S2Smem<D, H, 1, 2>::bytes(), s, p, pl, w2parts, w2scale);
+  if (pairs) return launch_pairs(actor_split_tc_kernel<ENV, H, 1>, grid, S2_NT, S2Smem<D, H, 1>::bytes(), s, p, pl, w2parts, w2scale);
+  return launch_chained(actor_split_tc_kernel<ENV, H, 2>, grid, S2_NT, S2Smem<D, H, 2>::bytes(), s, p, pl, w2parts, w2scale);
 }
 
 template <int ENV>
-cudaError_t launch_split_env(const ActorParams& p, const S2Plan& pl, const uint16_t* w2parts, const float* w2scale, int grid, int groups, cudaStream_t s) {
+cudaError_t launch_split_env(const ActorParams& p, const S2Plan& pl, const uint16_t* w2parts, const float* w2scale, int grid, bool pairs, cudaStream_t s) {
   switch (p.H) {
-    case 64: return launch_split<ENV, 64>(p, pl, w2parts, w2scale, grid, groups, s);
-    case 128: return launch_split<ENV, 128>(p, pl, w2parts, w2scale, grid, groups, s);
-    case 192: return launch_split<ENV, 192>(p, pl, w2parts, w2scale, grid, groups, s);
-    case 256: return launch_split<ENV, 256>(p, pl, w2parts, w2scale, grid, groups, s);
+    case 64: return launch_split<ENV, 64>(p, pl, w2parts, w2scale, grid, pairs, s);
+    case 128: return launch_split<ENV, 128>(p, pl, w2parts, w2scale, grid, pairs, s);
+    case 192: return launch_split<ENV, 192>(p, pl, w2parts, w2scale, grid, pairs, s);
+    case 256: return launch_split<ENV, 256>(p, pl, w2parts, w2scale, grid, pairs, s);
     default: return cudaErrorInvalidConfiguration;
   }
 }
@@ -774,8 +770,8 @@ cudaError_t launch_actor_split(int env_kind, const ActorParams& p, const uint16_
   if (p.N <= 0) return cudaSuccess;
   if (!split_actor_supported(env_kind, p.D, p.H, p.Aout)) return cudaErrorInvalidConfiguration;
   const int n_tiles = (p.N + SA_TE - 1) / SA_TE;
-  const int groups = n_tiles > sm_count && sm_count > 1 ? 2 : 1;    // more tiles than SMs: pairs of blocks with two tiles each in flight
-  const int grid = groups == 2 ? sm_count & ~1 : (n_tiles < sm_count ? n_tiles : sm_count);
+  const bool pairs = n_tiles > sm_count && sm_count > 1;     // more tiles than SMs: pairs of blocks with two tiles each in flight
+  const int grid = pairs ? sm_count & ~1 : (n_tiles < sm_count ? n_tiles : sm_count);
   S2Plan pl{};
   pl.n_pass = p.n_steps;
   if (p.C > 0) {
@@ -787,15 +783,15 @@ cudaError_t launch_actor_split(int env_kind, const ActorParams& p, const uint16_
     pl.seg0 = (int)((p.t0 / p.T) % p.G);
     pl.n_pass += (pl.pos0 + p.n_steps) / p.T;
   }
-  return env_kind == TJ_ENV_CARTPOLE ? launch_split_env<TJ_ENV_CARTPOLE>(p, pl, w2parts, w2scale, grid, groups, s)
-                                     : launch_split_env<TJ_ENV_ACROBOT>(p, pl, w2parts, w2scale, grid, groups, s);
+  return env_kind == TJ_ENV_CARTPOLE ? launch_split_env<TJ_ENV_CARTPOLE>(p, pl, w2parts, w2scale, grid, pairs, s)
+                                     : launch_split_env<TJ_ENV_ACROBOT>(p, pl, w2parts, w2scale, grid, pairs, s);
 }
 
 int td_split_grid(int n) { return (n + SA_TE - 1) / SA_TE; }
 
 template <int D, int H>
 static cudaError_t launch_td_split_dh(const TdParams& p, const uint16_t* po, const float* so, const uint16_t* pt, const float* st, cudaStream_t s) {
-  return launch_pairs(td_split_tc_kernel<D, H>, 2 * td_split_grid(p.n), S2_NT, S2Smem<D, H, 2, 1>::bytes(), s, p, po, so, pt, st);
+  return launch_pairs(td_split_tc_kernel<D, H>, 2 * td_split_grid(p.n), S2_NT, S2Smem<D, H, 2>::bytes(), s, p, po, so, pt, st);
 }
 
 template <int D>
