@@ -389,9 +389,10 @@ cudaError_t launch_af(const ActorParams& p, const AfPlan& q, int src, int grid, 
 cudaError_t launch_actor_fma(int env_kind, const ActorParams& p, int sm_count, cudaStream_t s) {
   if (p.Ap != 4) return cudaErrorInvalidConfiguration;        // at most four outputs: one float4 per row of the head
   const int sms = sm_count > 0 ? sm_count : 148, Hp = p.Hp;
-  // Environments per block: the call spread over the SMs in as few rounds as 56 per SM allow.  (More per round need 8 x 8 tiles: 16,384
-  // Acrobot envs, hidden 256, four steps: 262 us with two rounds of 8 x 4 tiles, 333-410 us with 8 x 8 on 224 or 448 threads, whose
-  // accumulators leave too few registers to keep operand loads in flight; 352 us before, 32 envs x 128 threads.)
+  // Environments per block: the call spread over the SMs in as few rounds as 56 per SM allow.  (More per round need 8 x 8 tiles.  With one
+  // input's operands in flight on 224 threads of 255 registers they take 252 us for four steps of 16,384 Acrobot envs, hidden 256, against 261
+  // with two rounds of 8 x 4, and 277 against 409 at 4,096 envs, hidden 512, but 99-121 against 99 at 6,000 envs, where they pad; with more
+  // threads or loads in flight they spill, 333-410 us.)
   const int rounds = (p.N + sms * 56 - 1) / (sms * 56);
   int want = (p.N + sms * rounds - 1) / (sms * rounds);
   // Two blocks per SM where both fit with W2 in shared memory: one steps its environments while the other multiplies (4,096 CartPole

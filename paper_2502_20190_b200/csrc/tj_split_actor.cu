@@ -136,7 +136,8 @@ struct S2Smem {
   static constexpr int NKC = H / SA_KC, NSTREAM = 2 * NKC;
   static constexpr int W_SLOTS = PAIR ? NSTREAM : SA_SLOTS;
   // A slots: one ring that the groups' passes go through in turn.  A worker waits only for the chunks whose slots it takes over, so
-  // the one two rounds of the ring back must be known to be used up: the ring holds more than half of two passes' chunks
+  // the one two rounds of the ring back must be known to be used up: the ring holds more than half of two passes' chunks, and products are
+  // signalled complete in the order of their issue, so a worker that has seen a pass or a chunk end knows every earlier chunk used up
   static constexpr int AS = PAIR && H > 192 ? 5 : S2_A_SLOTS;
   static_assert(2 * AS > NKC || !PAIR, "the phase of a slot's barrier is unambiguous");
   static constexpr uint32_t ACC_COLS = H <= 128 ? 128 : 256;
